@@ -10,7 +10,7 @@
 #include "internal.h"
 
 void jf_build_tables(int k, DGTab *T);
-void jf_build_powtab(double gamma, PowTab *P);
+void jf_build_powtab(double gamma, double R, double p0, PowTab *P);
 void jf_background(const jfnk_physics *ph, double z, double U[4], double dU[4]);
 double jf_insert_coef(const jfnk_physics *ph, double z);
 double jf_background_theta(const jfnk_physics *ph, double z);
@@ -112,13 +112,8 @@ int check_args(const jfnk_grid *g, int k, const jfnk_physics *p) {
 }
 
 __global__ void k_eos(const double *E, size_t n, PhysC pc, const PowTab *pt, double *p) {
-    __shared__ PowTab spt;
-    const double *src = reinterpret_cast<const double *>(pt);
-    double *dst = reinterpret_cast<double *>(&spt);
-    for (int i = threadIdx.x; i < (int)(sizeof(PowTab) / sizeof(double)); i += blockDim.x) dst[i] = src[i];
-    __syncthreads();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = pressure(D64{E[i]}, pc, &spt).x;
+    if (i < n) p[i] = pressure(D64{E[i]}, pc, pt).x;
 }
 
 __global__ void k_init_state(const double *thp, const double *prow, const double *throw_, const double *ubv,
@@ -366,7 +361,7 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
     std::vector<double> ub(4 * nrow), dub(4 * nrow), uh(4 * nf), duh(4 * nf);
     PowTab pt;
     {
-        jf_build_powtab(c->pc.gamma, &pt);
+        jf_build_powtab(c->pc.gamma, c->pc.R, c->pc.p0, &pt);
         std::vector<double> pr(nrow), tr(nrow);
         for (int ez = 0; ez < g->nz; ++ez)
             for (int b = 0; b < n1; ++b) {

@@ -64,13 +64,6 @@ template <> struct Loader<TL32, 2> {
     JF_D TL32 operator()(size_t i) const { return TL32{U[i], y[i]}; }
 };
 
-__device__ __forceinline__ void load_powtab(PowTab *s, const PowTab *g) {
-    const double *src = reinterpret_cast<const double *>(g);
-    double *dst = reinterpret_cast<double *>(s);
-    const int n = sizeof(PowTab) / sizeof(double);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
-}
-
 // background values: FP64 tables for D64, FP32 copies for TL32
 JF_D D64 bgs(const double *d, const float *, size_t i, D64) { return D64{d[i]}; }
 JF_D TLc bgs(const double *, const float *f, size_t i, TL32) { return TLc{f[i]}; }
@@ -118,11 +111,8 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
                                            typename OutT<T>::type *symz, unsigned blk, double *tr_out,
                                            const double *tr_in) {
     typedef typename OutT<T>::type O;
-    __shared__ PowTab spt;
-    if (IN != 2) load_powtab(&spt, K.pt);   // the FP32 tangent power needs no table
     Loader<T, IN> ld = ld0;
     ld.prepare();
-    __syncthreads();
     constexpr int NP = NP1 * NP1;
     const int nx = K.nx, nz = K.nz;
     const size_t N1 = (size_t)K.n_el * NP;
@@ -131,7 +121,6 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
     const long long t = (long long)blk * blockDim.x + threadIdx.x;
     if (t >= nvert + nhorz) return;
     const T zero = mk(0.0, T{});
-    const auto half = mkc(0.5, 0.5f, T{});
     T H[4], Phi[4], sL[3], sR[3];
     if (t < nvert) {
         const int s = (int)(t % NP1);
@@ -187,21 +176,17 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
             gL[v] = mkc(K.two_hx, K.two_hxf, T{}) * dL;
             gR[v] = mkc(K.two_hx, K.two_hxf, T{}) * dR;
         }
-        T UL[4], UR[4], Gh[4];
+        T UL[4], UR[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             UL[v] = trL[v] + bgs(K.ubv, K.ubvf, v * nrow + J, T{});
             UR[v] = trR[v] + bgs(K.ubv, K.ubvf, v * nrow + J, T{});
         }
-        if (wallL) {
-            mirror<T, 0>(UR, Gh);
-            hllc<T, 0>(Gh, UR, K.pc, &spt, H);
-        } else if (wallR) {
-            mirror<T, 0>(UL, Gh);
-            hllc<T, 0>(UL, Gh, K.pc, &spt, H);
-        } else {
-            hllc<T, 0>(UL, UR, K.pc, &spt, H);
-        }
+        wall_states<T, 0>(UL, UR, wallL, wallR);
+        Side<T> SL, SR;
+        side_of(UL, K.pc, K.pt, SL);
+        side_of(UR, K.pc, K.pt, SR);
+        hllc_s<T, 0>(SL, SR, H);
         const double *hb = wallL ? K.hbxw : (wallR ? K.hbxw + 4 * nrow : K.hbx);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
@@ -211,20 +196,18 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
 #pragma unroll
         for (int c = 0; c < 3; ++c) sL[c] = sR[c] = zero;
         if (VISC && !wallL && !wallR) {
-            T FL[4], FR[4], Jp[4], AL[4], AR[4];
-            viscous(UL, gL, K.pc, FL);
-            viscous(UR, gR, K.pc, FR);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) Jp[v] = trL[v] - trR[v];
-            viscous(UL, Jp, K.pc, AL);
-            viscous(UR, Jp, K.pc, AR);
             // interior penalty on the jumps of u, w, theta: eta {A(U)} [U]
             const auto eta = mkc(K.eta_x, K.eta_xf, T{});
+            const auto hmu = mkc(0.5 * K.mu, 0.5f * K.pc.muf, T{});
+            const T J0 = trL[0] - trR[0];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                sL[c] = half * AL[c + 1];
-                sR[c] = half * AR[c + 1];
-                Phi[c + 1] = Phi[c + 1] - half * (FL[c + 1] + FR[c + 1]) + eta * (sL[c] + sR[c]);
+                const int v = c + 1;
+                const T pL = SL.U[v] * SL.ir, pR = SR.U[v] * SR.ir;
+                const T Jv = trL[v] - trR[v];
+                sL[c] = hmu * visc_c(pL, J0, Jv);
+                sR[c] = hmu * visc_c(pR, J0, Jv);
+                Phi[v] = Phi[v] - hmu * (visc_c(pL, gL[0], gL[v]) + visc_c(pR, gR[0], gR[v])) + eta * (sL[c] + sR[c]);
             }
         }
         const size_t fb = ((size_t)ez * (nx + 1) + fx) * NP1 + s;
@@ -282,21 +265,17 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
             gB[v] = mkc(K.two_hz, K.two_hzf, T{}) * dB + bgs(K.dubh, K.dubhf, (size_t)v * (nz + 1) + fz, T{});
             gT[v] = mkc(K.two_hz, K.two_hzf, T{}) * dT + bgs(K.dubh, K.dubhf, (size_t)v * (nz + 1) + fz, T{});
         }
-        T UB[4], UT[4], Gh[4];
+        T UB[4], UT[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             UB[v] = trB[v] + bgs(K.ubh, K.ubhf, (size_t)v * (nz + 1) + fz, T{});
             UT[v] = trT[v] + bgs(K.ubh, K.ubhf, (size_t)v * (nz + 1) + fz, T{});
         }
-        if (wallB) {
-            mirror<T, 1>(UT, Gh);
-            hllc<T, 1>(Gh, UT, K.pc, &spt, H);
-        } else if (wallT) {
-            mirror<T, 1>(UB, Gh);
-            hllc<T, 1>(UB, Gh, K.pc, &spt, H);
-        } else {
-            hllc<T, 1>(UB, UT, K.pc, &spt, H);
-        }
+        wall_states<T, 1>(UB, UT, wallB, wallT);
+        Side<T> SB, ST;
+        side_of(UB, K.pc, K.pt, SB);
+        side_of(UT, K.pc, K.pt, ST);
+        hllc_s<T, 1>(SB, ST, H);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             if (IN != 2) H[v] = H[v] - bg<T>(K.hbz, (size_t)v * (nz + 1) + fz);
@@ -305,19 +284,18 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
 #pragma unroll
         for (int c = 0; c < 3; ++c) sL[c] = sR[c] = zero;
         if (VISC && !wallB && !wallT) {
-            T FB[4], FT[4], Jp[4], AB[4], AT[4];
-            viscous(UB, gB, K.pc, FB);
-            viscous(UT, gT, K.pc, FT);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) Jp[v] = trB[v] - trT[v];
-            viscous(UB, Jp, K.pc, AB);
-            viscous(UT, Jp, K.pc, AT);
+            // interior penalty on the jumps of u, w, theta: eta {A(U)} [U]
             const auto eta = mkc(K.eta_z, K.eta_zf, T{});
+            const auto hmu = mkc(0.5 * K.mu, 0.5f * K.pc.muf, T{});
+            const T J0 = trB[0] - trT[0];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                sL[c] = half * AB[c + 1];
-                sR[c] = half * AT[c + 1];
-                Phi[c + 1] = Phi[c + 1] - half * (FB[c + 1] + FT[c + 1]) + eta * (sL[c] + sR[c]);
+                const int v = c + 1;
+                const T pL = SB.U[v] * SB.ir, pR = ST.U[v] * ST.ir;
+                const T Jv = trB[v] - trT[v];
+                sL[c] = hmu * visc_c(pL, J0, Jv);
+                sR[c] = hmu * visc_c(pR, J0, Jv);
+                Phi[v] = Phi[v] - hmu * (visc_c(pL, gB[0], gB[v]) + visc_c(pR, gT[0], gT[v])) + eta * (sL[c] + sR[c]);
             }
         }
         const size_t fb = ((size_t)fz * nx + ex) * NP1 + s;
@@ -336,7 +314,7 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
 
 template <class T, int IN, int NP1, bool VISC>
 struct k_faces_b {
-    static constexpr int TPB = 256, MINB = 4;
+    static constexpr int TPB = 256, MINB = VISC ? 2 : 4;
     static constexpr bool GROUP = !VISC && std::is_same<T, D64>::value;   // a grouped twin is built (lock-step ensembles)
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGK> K,
                                                JfArg<Loader<T, IN>> ld0, JfArg<typename OutT<T>::type *> phix,
@@ -349,7 +327,7 @@ struct k_faces_b {
     }
 };
 template <class T, int IN, int NP1, bool VISC>
-__global__ void __launch_bounds__(256, 4) k_faces(DGK K, Loader<T, IN> ld0, typename OutT<T>::type *phix,
+__global__ void __launch_bounds__(256, VISC ? 2 : 4) k_faces(DGK K, Loader<T, IN> ld0, typename OutT<T>::type *phix,
                                                typename OutT<T>::type *symx, typename OutT<T>::type *phiz,
                                                typename OutT<T>::type *symz, double *tr_out, const double *tr_in) {
     k_faces_b<T, IN, NP1, VISC>::run(blockIdx.x, gridDim.x, K, ld0, phix, symx, phiz, symz, tr_out, tr_in);
@@ -372,7 +350,6 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
     typedef typename OutT<T>::type O;
     constexpr int NP = NP1 * NP1;
     constexpr int EPB = EPBOf<NP1, TV>::value;
-    __shared__ PowTab spt;
     __shared__ O sg[2][EPB][4][NP];
     __shared__ T su[VISC ? EPB : 1][4][NP];
     // weak-form derivative and lift tables with the 2/h factors folded in:
@@ -386,7 +363,6 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
         sce[0] = e0;
         sce[1] = e0 != 0.0 ? A.adt / e0 : 0.0;
     }
-    if (IN != 2) load_powtab(&spt, K.pt);
     Loader<T, IN> ld = ld0;
     ld.prepare();
     if (threadIdx.x < NP) {
@@ -442,20 +418,22 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
     }
     __syncthreads();
     if (active) {
-        const T ir = mkc(1.0, 1.0f, T{}) / U[0];
-        const T p = pressure(U[3], K.pc, &spt);
+        const T ir = jrcp(U[0]);
+        const T p = pressure(U[3], K.pc, K.pt);
+        const T u = U[1] * ir, w = U[2] * ir;
         T Fx[4], Fz[4];
-        flux_c<T, 0>(U, U[1] * ir, p, Fx);
-        flux_c<T, 1>(U, U[2] * ir, p, Fz);
-        if (IN != 2) {
+        flux_xz(U, u, w, p, Fx, Fz);
+        if (IN != 2) {   // minus the background's fluxes; the mass fluxes are linear
+            Fx[0] = Up[1];
+            Fz[0] = Up[2];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
+            for (int v = 1; v < 4; ++v) {
                 Fx[v] = Fx[v] - bg<T>(K.fbx, v * nrow + J);
                 Fz[v] = Fz[v] - bg<T>(K.fbz, v * nrow + J);
             }
         }
         if (VISC) {
-            T dx[4], dz[4], Gx[4], Gz[4];
+            T dx[4], dz[4];
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 T sx = mk(0.0, T{}), sz = mk(0.0, T{});
@@ -467,12 +445,12 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
                 dx[v] = mkc(K.two_hx, K.two_hxf, T{}) * sx;
                 dz[v] = mkc(K.two_hz, K.two_hzf, T{}) * sz + bgs(K.dubv, K.dubvf, v * nrow + J, T{});
             }
-            viscous(U, dx, K.pc, Gx);
-            viscous(U, dz, K.pc, Gz);
+            const auto mu = mkc(K.mu, K.pc.muf, T{});
+            const T phi[4] = {u, u, w, U[3] * ir};
 #pragma unroll
             for (int v = 1; v < 4; ++v) {
-                Fx[v] = Fx[v] - Gx[v];
-                Fz[v] = Fz[v] - Gz[v];
+                Fx[v] = Fx[v] - mu * visc_c(phi[v], dx[0], dx[v]);
+                Fz[v] = Fz[v] - mu * visc_c(phi[v], dz[0], dz[v]);
             }
         }
 #pragma unroll
@@ -722,13 +700,13 @@ struct k_dgtl_b {
                 Up[v] = sn[1][le][v][node];
                 U[v] = Up[v] + TLc{K.ubvf[v * nrow + J]};
             }
-            const TL32 ir = TLc{1.0f} / U[0];
+            const TL32 ir = jrcp(U[0]);
             const TL32 p = pressure(U[3], K.pc, nullptr);
+            const TL32 u = U[1] * ir, w = U[2] * ir;
             TL32 Fx[4], Fz[4];
-            flux_c<TL32, 0>(U, U[1] * ir, p, Fx);
-            flux_c<TL32, 1>(U, U[2] * ir, p, Fz);
+            flux_xz(U, u, w, p, Fx, Fz);
             if (VISC) {
-                TL32 dx[4], dz[4], Gx[4], Gz[4];
+                TL32 dx[4], dz[4];
     #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     TL32 sx = mk(0.0, TL32{}), sz = mk(0.0, TL32{});
@@ -740,12 +718,12 @@ struct k_dgtl_b {
                     dx[v] = TLc{K.two_hxf} * sx;
                     dz[v] = TLc{K.two_hzf} * sz + TLc{K.dubvf[v * nrow + J]};
                 }
-                viscous(U, dx, K.pc, Gx);
-                viscous(U, dz, K.pc, Gz);
+                const TLc mu = TLc{K.pc.muf};
+                const TL32 phi[4] = {u, u, w, U[3] * ir};
     #pragma unroll
                 for (int v = 1; v < 4; ++v) {
-                    Fx[v] = Fx[v] - Gx[v];
-                    Fz[v] = Fz[v] - Gz[v];
+                    Fx[v] = Fx[v] - mu * visc_c(phi[v], dx[0], dx[v]);
+                    Fz[v] = Fz[v] - mu * visc_c(phi[v], dz[0], dz[v]);
                 }
             }
     #pragma unroll
@@ -768,7 +746,6 @@ struct k_dgtl_b {
                 if (VISC) td = jfma(TLc{pd[q]}, u, td);
             }
         };
-        const TLc half = TLc{0.5f};
         const int nxf = (Ev + 1) * NP1, nzf = 2 * Ev * NP1;
         for (int t = threadIdx.x; t < nxf + nzf; t += blockDim.x) {
             TL32 trL[4], trR[4], gL[4], gR[4], UL[4], UR[4], H[4], Phi[4], sLv[3], sRv[3];
@@ -792,31 +769,25 @@ struct k_dgtl_b {
                     UL[v] = aL + TLc{K.ubvf[v * nrow + J]};
                     UR[v] = aR + TLc{K.ubvf[v * nrow + J]};
                 }
-                TL32 Gh[4];
-                if (wallL) {
-                    mirror<TL32, 0>(UR, Gh);
-                    hllc<TL32, 0>(Gh, UR, K.pc, nullptr, H);
-                } else if (wallR) {
-                    mirror<TL32, 0>(UL, Gh);
-                    hllc<TL32, 0>(UL, Gh, K.pc, nullptr, H);
-                } else {
-                    hllc<TL32, 0>(UL, UR, K.pc, nullptr, H);
-                }
+                wall_states<TL32, 0>(UL, UR, wallL, wallR);
+                Side<TL32> SL, SR;
+                side_of(UL, K.pc, nullptr, SL);
+                side_of(UR, K.pc, nullptr, SR);
+                hllc_s<TL32, 0>(SL, SR, H);
     #pragma unroll
                 for (int v = 0; v < 4; ++v) Phi[v] = H[v];
                 if (VISC && !wallL && !wallR) {
-                    TL32 FL[4], FR[4], Jp[4], AL[4], AR[4];
-                    viscous(UL, gL, K.pc, FL);
-                    viscous(UR, gR, K.pc, FR);
-    #pragma unroll
-                    for (int v = 0; v < 4; ++v) Jp[v] = trL[v] - trR[v];
-                    viscous(UL, Jp, K.pc, AL);
-                    viscous(UR, Jp, K.pc, AR);
+                    const TLc hmu = TLc{0.5f * K.pc.muf};
+                    const TL32 J0 = trL[0] - trR[0];
     #pragma unroll
                     for (int q = 0; q < 3; ++q) {
-                        sLv[q] = half * AL[q + 1];
-                        sRv[q] = half * AR[q + 1];
-                        Phi[q + 1] = Phi[q + 1] - half * (FL[q + 1] + FR[q + 1]) + TLc{K.eta_xf} * (sLv[q] + sRv[q]);
+                        const int v = q + 1;
+                        const TL32 pL = UL[v] * SL.ir, pR = UR[v] * SR.ir;
+                        const TL32 Jv = trL[v] - trR[v];
+                        sLv[q] = hmu * visc_c(pL, J0, Jv);
+                        sRv[q] = hmu * visc_c(pR, J0, Jv);
+                        Phi[v] = Phi[v] - hmu * (visc_c(pL, gL[0], gL[v]) + visc_c(pR, gR[0], gR[v])) +
+                                 TLc{K.eta_xf} * (sLv[q] + sRv[q]);
                     }
                 } else {
     #pragma unroll
@@ -857,31 +828,25 @@ struct k_dgtl_b {
                     UL[v] = aB + TLc{K.ubhf[(size_t)v * (nz + 1) + fz]};
                     UR[v] = aT + TLc{K.ubhf[(size_t)v * (nz + 1) + fz]};
                 }
-                TL32 Gh[4];
-                if (wallB) {
-                    mirror<TL32, 1>(UR, Gh);
-                    hllc<TL32, 1>(Gh, UR, K.pc, nullptr, H);
-                } else if (wallT) {
-                    mirror<TL32, 1>(UL, Gh);
-                    hllc<TL32, 1>(UL, Gh, K.pc, nullptr, H);
-                } else {
-                    hllc<TL32, 1>(UL, UR, K.pc, nullptr, H);
-                }
+                wall_states<TL32, 1>(UL, UR, wallB, wallT);
+                Side<TL32> SL, SR;
+                side_of(UL, K.pc, nullptr, SL);
+                side_of(UR, K.pc, nullptr, SR);
+                hllc_s<TL32, 1>(SL, SR, H);
     #pragma unroll
                 for (int v = 0; v < 4; ++v) Phi[v] = H[v];
                 if (VISC && !wallB && !wallT) {
-                    TL32 FB[4], FT[4], Jp[4], AB[4], AT[4];
-                    viscous(UL, gB, K.pc, FB);
-                    viscous(UR, gT, K.pc, FT);
-    #pragma unroll
-                    for (int v = 0; v < 4; ++v) Jp[v] = trL[v] - trR[v];
-                    viscous(UL, Jp, K.pc, AB);
-                    viscous(UR, Jp, K.pc, AT);
+                    const TLc hmu = TLc{0.5f * K.pc.muf};
+                    const TL32 J0 = trL[0] - trR[0];
     #pragma unroll
                     for (int q = 0; q < 3; ++q) {
-                        sLv[q] = half * AB[q + 1];
-                        sRv[q] = half * AT[q + 1];
-                        Phi[q + 1] = Phi[q + 1] - half * (FB[q + 1] + FT[q + 1]) + TLc{K.eta_zf} * (sLv[q] + sRv[q]);
+                        const int v = q + 1;
+                        const TL32 pL = UL[v] * SL.ir, pR = UR[v] * SR.ir;
+                        const TL32 Jv = trL[v] - trR[v];
+                        sLv[q] = hmu * visc_c(pL, J0, Jv);
+                        sRv[q] = hmu * visc_c(pR, J0, Jv);
+                        Phi[v] = Phi[v] - hmu * (visc_c(pL, gB[0], gB[v]) + visc_c(pR, gT[0], gT[v])) +
+                                 TLc{K.eta_zf} * (sLv[q] + sRv[q]);
                     }
                 } else {
     #pragma unroll
@@ -952,26 +917,23 @@ __global__ void __launch_bounds__(128, VISC ? 5 : 8) k_dgtl(DGK K, DGArgs A, flo
 // D64 functions so that U' = 0 cancels bit for bit
 __global__ void k_bg_dg(DGK K, double *fbx, double *fbz, double *hbx, double *hbxw, double *hbz) {
     jf_pdl_enter();
-    __shared__ PowTab spt;
-    load_powtab(&spt, K.pt);
-    __syncthreads();
     const int nrow = K.nz * K.tab.np1;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nrow) {
-        D64 U[4], G[4], F[4], H[4];
+        D64 U[4], G[4], Fx[4], Fz[4], H[4];
         for (int v = 0; v < 4; ++v) U[v] = D64{K.ubv[v * nrow + i]};
-        const D64 ir = D64{1.0} / U[0];
-        const D64 p = pressure(U[3], K.pc, &spt);
-        flux_c<D64, 0>(U, U[1] * ir, p, F);
-        for (int v = 0; v < 4; ++v) fbx[v * nrow + i] = F[v].x;
-        flux_c<D64, 1>(U, U[2] * ir, p, F);
-        for (int v = 0; v < 4; ++v) fbz[v * nrow + i] = F[v].x;
-        hllc<D64, 0>(U, U, K.pc, &spt, H);
+        const D64 ir = jrcp(U[0]);
+        flux_xz(U, U[1] * ir, U[2] * ir, pressure(U[3], K.pc, K.pt), Fx, Fz);
+        for (int v = 0; v < 4; ++v) {
+            fbx[v * nrow + i] = Fx[v].x;
+            fbz[v * nrow + i] = Fz[v].x;
+        }
+        hllc<D64, 0>(U, U, K.pc, K.pt, H);
         for (int v = 0; v < 4; ++v) hbx[v * nrow + i] = H[v].x;
         mirror<D64, 0>(U, G);
-        hllc<D64, 0>(G, U, K.pc, &spt, H);
+        hllc<D64, 0>(G, U, K.pc, K.pt, H);
         for (int v = 0; v < 4; ++v) hbxw[v * nrow + i] = H[v].x;
-        hllc<D64, 0>(U, G, K.pc, &spt, H);
+        hllc<D64, 0>(U, G, K.pc, K.pt, H);
         for (int v = 0; v < 4; ++v) hbxw[(4 + v) * nrow + i] = H[v].x;
     } else if (i < nrow + K.nz + 1) {
         const int j = i - nrow;
@@ -980,11 +942,11 @@ __global__ void k_bg_dg(DGK K, double *fbx, double *fbz, double *hbx, double *hb
         for (int v = 0; v < 4; ++v) U[v] = D64{K.ubh[v * nf + j]};
         mirror<D64, 1>(U, G);
         if (j == 0)
-            hllc<D64, 1>(G, U, K.pc, &spt, H);
+            hllc<D64, 1>(G, U, K.pc, K.pt, H);
         else if (j == K.nz)
-            hllc<D64, 1>(U, G, K.pc, &spt, H);
+            hllc<D64, 1>(U, G, K.pc, K.pt, H);
         else
-            hllc<D64, 1>(U, U, K.pc, &spt, H);
+            hllc<D64, 1>(U, U, K.pc, K.pt, H);
         for (int v = 0; v < 4; ++v) hbz[v * nf + j] = H[v].x;
     }
 }
@@ -1156,7 +1118,7 @@ struct DGMember {
 constexpr int GRP_FACE_THREADS = 128;
 
 template <int NP1, bool VISC>
-__global__ void __launch_bounds__(256, 4) k_faces_grp(const DGMember *mem, int nm) {
+__global__ void __launch_bounds__(256, VISC ? 2 : 4) k_faces_grp(const DGMember *mem, int nm) {
     jf_pdl_enter();
     int m = 0;
     while (m + 1 < nm && blockIdx.x >= mem[m + 1].fb0) ++m;   // members in block order

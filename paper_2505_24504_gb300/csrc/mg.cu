@@ -56,12 +56,6 @@ JF_D S rk_stage(const RKS &rk, S x, S dt, S bmg, size_t gi) {
 JF_D D64 bgs(const double *d, const float *, size_t i, D64) { return D64{d[i]}; }
 JF_D TLc bgs(const double *, const float *f, size_t i, TL32) { return TLc{f[i]}; }
 
-__device__ __forceinline__ void load_pt(PowTab *s, const PowTab *g) {
-    const double *src = reinterpret_cast<const double *>(g);
-    double *dst = reinterpret_cast<double *>(s);
-    for (int i = threadIdx.x; i < (int)(sizeof(PowTab) / sizeof(double)); i += blockDim.x) dst[i] = src[i];
-}
-
 // Level state loaders, addressed by (variable, cell, I, J):
 // IN 0 u; IN 1 u + eps x (FP64, eps on the device); IN 2 TL32 (u, x).
 template <class T, int IN> struct FLoad;
@@ -126,26 +120,7 @@ template <> struct SOf<TL32> { typedef float type; };
 JF_D double oval(D64 a) { return a.x; }
 JF_D float oval(TL32 a) { return a.d; }
 
-template <class T, int D>
-JF_D void face_flux(const T UL[4], const T UR[4], bool wallL, bool wallR, const double *hb, size_t hs,
-                    size_t hi, bool sub, const FVK &K, const PowTab *pt, T H[4]) {
-    T G[4];
-    if (wallL) {
-        mirror<T, D>(UR, G);
-        hllc<T, D>(G, UR, K.pc, pt, H);
-    } else if (wallR) {
-        mirror<T, D>(UL, G);
-        hllc<T, D>(UL, G, K.pc, pt, H);
-    } else {
-        hllc<T, D>(UL, UR, K.pc, pt, H);
-    }
-    if (sub) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) H[v] = H[v] - mk(hb[v * hs + hi], T{});
-    }
-}
-
-// the same two-point flux from precomputed sides (1/rho of each side reused)
+// two-point viscous flux mu {rho} (phi_R - phi_L)/d, phi = u, w, theta (coef = mu / 2d)
 template <class T, class C>
 JF_D void visc2_s(const Side<T> &L, const Side<T> &R, C coef, T V[4]) {
     const T c = coef * (L.U[0] + R.U[0]);
@@ -154,62 +129,13 @@ JF_D void visc2_s(const Side<T> &L, const Side<T> &R, C coef, T V[4]) {
     for (int v = 1; v < 4; ++v) V[v] = c * (R.U[v] * R.ir - L.U[v] * L.ir);
 }
 
-template <class T, class C>
-JF_D void visc2(const T UL[4], const T UR[4], C coef, T V[4]) {
-    const T irL = mkc(1.0, 1.0f, T{}) / UL[0], irR = mkc(1.0, 1.0f, T{}) / UR[0];
-    const T c = coef * (UL[0] + UR[0]);
-    V[0] = mk(0.0, T{});
+template <class T>
+JF_D void sel_side(bool c, const Side<T> &A, const Side<T> &B, Side<T> &S) {
 #pragma unroll
-    for (int v = 1; v < 4; ++v) V[v] = c * (UR[v] * irR - UL[v] * irL);
-}
-
-// f_low (or its tangent) at one cell (I, Jz) by one thread: HLLC^pert on the four
-// faces, gravity source, two-point viscous flux (large levels: enough cells to
-// fill the GPU, and fewer instructions per cell than the four-lane form).
-template <class T, int IN, bool VISC>
-JF_D void fv_cell_op(const FVK &K, const FLoad<T, IN> &ld, const PowTab *spt, size_t c, int I, int Jz, T f[4]) {
-    const int NX = K.NX, NZ = K.NZ;
-    const bool sub = (IN < 2);
-    T U[4], Un[4][4];   // own state and the W, E, S, N neighbours
-    int nb[4] = {-1, -1, -1, -1};
-    int nI[4] = {I - 1, I + 1, I, I}, nJ[4] = {Jz, Jz, Jz - 1, Jz + 1};
-    if (I > 0) nb[0] = Jz * NX + I - 1;
-    else if (K.periodic) { nb[0] = Jz * NX + NX - 1; nI[0] = NX - 1; }
-    if (I < NX - 1) nb[1] = Jz * NX + I + 1;
-    else if (K.periodic) { nb[1] = Jz * NX; nI[1] = 0; }
-    if (Jz > 0) nb[2] = (Jz - 1) * NX + I;
-    if (Jz < NZ - 1) nb[3] = (Jz + 1) * NX + I;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        U[v] = ld(v, c, I, Jz) + bgs(K.ub, K.ubf, v * NZ + Jz, T{});
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-            Un[q][v] = nb[q] >= 0 ? ld(v, (size_t)nb[q], nI[q], nJ[q]) + bgs(K.ub, K.ubf, v * NZ + nJ[q], T{}) : U[v];
-    }
-    T HW[4], HE[4], HS[4], HN[4];
-    face_flux<T, 0>(Un[0], U, nb[0] < 0, false, nb[0] < 0 ? K.hbxw : K.hbx, NZ, Jz, sub, K, spt, HW);
-    face_flux<T, 0>(U, Un[1], false, nb[1] < 0, nb[1] < 0 ? K.hbxw + 4 * NZ : K.hbx, NZ, Jz, sub, K, spt, HE);
-    face_flux<T, 1>(Un[2], U, nb[2] < 0, false, K.hbz, NZ + 1, Jz, sub, K, spt, HS);
-    face_flux<T, 1>(U, Un[3], false, nb[3] < 0, K.hbz, NZ + 1, Jz + 1, sub, K, spt, HN);
-    const auto iHx = mkc(K.iHx, K.iHxf, T{}), iHz = mkc(K.iHz, K.iHzf, T{});
-#pragma unroll
-    for (int v = 0; v < 4; ++v) f[v] = -((HE[v] - HW[v]) * iHx + (HN[v] - HS[v]) * iHz);
-    const T up0 = ld(0, c, I, Jz);
-    f[2] = f[2] - mkc(K.g, K.gf, T{}) * up0;   // -g rho' (tangent: -g x_rho)
-    if (VISC) {
-        T VW[4], VE[4], VS[4], VN[4];
-        const T zero = mk(0.0, T{});
-        const auto cx = mkc(K.vcx, K.vcxf, T{}), cz = mkc(K.vcz, K.vczf, T{});
-        if (nb[0] >= 0) visc2(Un[0], U, cx, VW); else { for (int v = 0; v < 4; ++v) VW[v] = zero; }
-        if (nb[1] >= 0) visc2(U, Un[1], cx, VE); else { for (int v = 0; v < 4; ++v) VE[v] = zero; }
-        if (nb[2] >= 0) visc2(Un[2], U, cz, VS); else { for (int v = 0; v < 4; ++v) VS[v] = zero; }
-        if (nb[3] >= 0) visc2(U, Un[3], cz, VN); else { for (int v = 0; v < 4; ++v) VN[v] = zero; }
-#pragma unroll
-        for (int v = 1; v < 4; ++v) f[v] = f[v] + (VE[v] - VW[v]) * iHx + (VN[v] - VS[v]) * iHz;
-    }
+    for (int v = 0; v < 4; ++v) S.U[v] = sel(c, A.U[v], B.U[v]);
+    S.ir = sel(c, A.ir, B.ir);
+    S.p = sel(c, A.p, B.p);
+    S.c = sel(c, A.c, B.c);
 }
 
 JF_D D64 shfl_x(D64 a, int m) { return D64{__shfl_xor_sync(0xffffffffu, a.x, m)}; }
@@ -273,18 +199,21 @@ JF_D T fv_cell_op4(const FVK &K, const FLoad<T, IN> &ld, const PowTab *spt, size
         swap12(N);
     }
     if (wall) N[1] = -U[1];   // slip-wall ghost: normal momentum reversed
+    // lanes of a warp hold left and right faces: the two sides are put in order by
+    // selects, so that one evaluation serves both (a branch would run it twice)
+    Side<T> own, nbr, L, R;
+    side_of(U, K.pc, spt, own);
+    side_of(N, K.pc, spt, nbr);
+    sel_side(right, own, nbr, L);
+    sel_side(right, nbr, own, R);
     T H[4];
-    if (right) hllc<T, 0>(U, N, K.pc, spt, H);
-    else hllc<T, 0>(N, U, K.pc, spt, H);
+    hllc_s<T, 0>(L, R, H);
     T V[4];
     if (VISC) {
+        visc2_s(L, R, zf ? mkc(K.vcz, K.vczf, T{}) : mkc(K.vcx, K.vcxf, T{}), V);
         if (wall) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) V[v] = mk(0.0, T{});
-        } else if (right) {
-            visc2(U, N, zf ? mkc(K.vcz, K.vczf, T{}) : mkc(K.vcx, K.vcxf, T{}), V);
-        } else {
-            visc2(N, U, zf ? mkc(K.vcz, K.vczf, T{}) : mkc(K.vcx, K.vcxf, T{}), V);
         }
     }
     if (zf) {
@@ -327,9 +256,8 @@ JF_D S gprime_of(const FLoad<T, IN> &ld, S x, T f, const double *fu, size_t gi, 
     return x - (S)adtf * (S)oval(f);
 }
 
-// One thread (L = 1) or four lanes (L = 4, lane q owns variable q) per cell of
-// an NX x NZ level.
-template <class T, int IN, int MODE, bool VISC, int L>
+// Four lanes per cell of an NX x NZ level, lane q owns variable q.
+template <class T, int IN, int MODE, bool VISC>
 struct k_fv_b {
     static constexpr int TPB = 256, MINB = 0;
     static constexpr bool GROUP = !VISC && std::is_same<T, TL32>::value;   // a grouped twin is built (lock-step ensembles)
@@ -341,56 +269,45 @@ struct k_fv_b {
                                                JfArg<RKS> rk) {
         jf_pdl_enter();
         typedef typename SOf<T>::type S;
-        __shared__ PowTab spt;
-        if (IN < 2) load_pt(&spt, K.pt);   // the FP32 tangent power needs no table
         FLoad<T, IN> ld = ld0;
         ld.prepare();
-        __syncthreads();
         const float adtf = IN >= 2 ? K.adtf : 0.0f;
         const size_t n1 = (size_t)K.NX * K.NZ;
         const size_t t = (size_t)jf_bid * blockDim.x + threadIdx.x;
-        const int q = L == 4 ? (int)(t & 3) : 0;
-        const size_t cell = L == 4 ? (t >> 2) : t;
+        const int v = (int)(t & 3);
+        const size_t cell = t >> 2;
         const bool live = cell < n1;
-        if (L == 1 && !live) return;
         const size_t c = live ? cell : n1 - 1;   // idle lanes still join the shuffles
         const int I = (int)(c % K.NX), Jz = (int)(c / K.NX);
-        T f[4];
-        if (L == 4) f[0] = fv_cell_op4<T, IN, VISC>(K, ld, &spt, c, I, Jz, q);
-        else fv_cell_op<T, IN, VISC>(K, ld, &spt, c, I, Jz, f);
+        const T f = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, v);
         if (!live) return;
-    #pragma unroll
-        for (int k = 0; k < (L == 4 ? 1 : 4); ++k) {
-            const int v = L == 4 ? q : k;
-            const size_t gi = (size_t)v * n1 + c;
-            if (MODE == FV_RES) {
-                out[gi] = (S)oval(f[k]);
-            } else {
-                const S x = (S)ld.dir(v, c, I, Jz);
-                const S gx = gprime_of<T, IN, S>(ld, x, f[k], fu, gi, adt, adtf, ld.step());
-                if (MODE == FV_SMOOTH)
-                    out[gi] = store_round<S>(rk_stage<S>(rk, x, dtau[c], b[gi] - gx, gi), bf16);
-                else
-                    out[gi] = gx - b[gi];
-            }
+        const size_t gi = (size_t)v * n1 + c;
+        if (MODE == FV_RES) {
+            out[gi] = (S)oval(f);
+        } else {
+            const S x = (S)ld.dir(v, c, I, Jz);
+            const S gx = gprime_of<T, IN, S>(ld, x, f, fu, gi, adt, adtf, ld.step());
+            if (MODE == FV_SMOOTH)
+                out[gi] = store_round<S>(rk_stage<S>(rk, x, dtau[c], b[gi] - gx, gi), bf16);
+            else
+                out[gi] = gx - b[gi];
         }
     }
 };
-template <class T, int IN, int MODE, bool VISC, int L>
+template <class T, int IN, int MODE, bool VISC>
 __global__ void __launch_bounds__(256) k_fv(FVK K, FLoad<T, IN> ld0, const typename SOf<T>::type *xin,
                                             const typename SOf<T>::type *b, const typename SOf<T>::type *dtau,
                                             const double *fu, double adt, typename SOf<T>::type *out,
                                             int bf16, RKS rk) {
-    k_fv_b<T, IN, MODE, VISC, L>::run(blockIdx.x, gridDim.x, K, ld0, xin, b, dtau, fu, adt, out, bf16, rk);
+    k_fv_b<T, IN, MODE, VISC>::run(blockIdx.x, gridDim.x, K, ld0, xin, b, dtau, fu, adt, out, bf16, rk);
 }
 
 // Defect and restriction in one pass: the defect g'x - b of every child cell of
 // a coarse cell, averaged into b_c; when x_c is given, also the coarse level's
-// first pseudo-time step x_c = dtau_c b_c.  L = 1: one thread per coarse cell
-// loops over its fac x fac children.  L = 4, FAC2: 2 x 2 agglomeration with
+// first pseudo-time step x_c = dtau_c b_c.  FAC2: 2 x 2 agglomeration with
 // sixteen lanes per coarse cell (four lanes per child, children summed by
-// shuffles); L = 4 otherwise: four lanes per coarse cell loop over the children.
-template <class T, int IN, bool VISC, int L, bool FAC2>
+// shuffles); otherwise four lanes per coarse cell loop over the children.
+template <class T, int IN, bool VISC, bool FAC2>
 struct k_fv_defect_restrict_b {
     static constexpr int TPB = 256, MINB = 0;
     static constexpr bool GROUP = !VISC && std::is_same<T, TL32>::value;   // a grouped twin is built (lock-step ensembles)
@@ -401,41 +318,13 @@ struct k_fv_defect_restrict_b {
                                                JfArg<const typename SOf<T>::type *> dtau_c, JfArg<int> bf16) {
         jf_pdl_enter();
         typedef typename SOf<T>::type S;
-        __shared__ PowTab spt;
-        if (IN < 2) load_pt(&spt, K.pt);
         FLoad<T, IN> ld = ld0;
         ld.prepare();
-        __syncthreads();
         const int NXc = K.NX / fac, NZc = K.NZ / fac;
         const size_t nc = (size_t)NXc * NZc, n1 = (size_t)K.NX * K.NZ;
         const size_t t = (size_t)jf_bid * blockDim.x + threadIdx.x;
         const double eps = ld.step();
         const float adtf = IN >= 2 ? K.adtf : 0.0f;
-        if (L == 1) {
-            if (t >= nc) return;
-            const int Ic = (int)(t % NXc), Jc = (int)(t / NXc);
-            S acc[4] = {0, 0, 0, 0};
-            for (int jj = 0; jj < fac; ++jj)
-                for (int ii = 0; ii < fac; ++ii) {
-                    const int I = Ic * fac + ii, Jz = Jc * fac + jj;
-                    const size_t c = (size_t)Jz * K.NX + I;
-                    T f[4];
-                    fv_cell_op<T, IN, VISC>(K, ld, &spt, c, I, Jz, f);
-    #pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        const size_t gi = (size_t)v * n1 + c;
-                        acc[v] += gprime_of<T, IN, S>(ld, (S)ld.dir(v, c, I, Jz), f[v], fu, gi, adt, adtf, eps) - b[gi];
-                    }
-                }
-            const S inv = (S)1 / (S)(fac * fac);
-    #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const S bv = store_round<S>(acc[v] * inv, bf16);
-                bc[(size_t)v * nc + t] = bv;
-                if (xc) xc[(size_t)v * nc + t] = store_round<S>(dtau_c[t] * bv, bf16);
-            }
-            return;
-        }
         const int q = (int)(t & 3);
         const size_t g = FAC2 ? (t >> 4) : (t >> 2);
         const bool live = g < nc;
@@ -446,7 +335,7 @@ struct k_fv_defect_restrict_b {
             const int ch = (int)((t >> 2) & 3);
             const int I = 2 * Ic + (ch & 1), Jz = 2 * Jc + (ch >> 1);
             const size_t c = (size_t)Jz * K.NX + I;
-            const T fq = fv_cell_op4<T, IN, VISC>(K, ld, &spt, c, I, Jz, q);
+            const T fq = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, q);
             const size_t gi = (size_t)q * n1 + c;
             const S d = gprime_of<T, IN, S>(ld, (S)ld.dir(q, c, I, Jz), fq, fu, gi, adt, adtf, eps) - b[gi];
             const S d2 = d + __shfl_xor_sync(0xffffffffu, d, 4);
@@ -457,7 +346,7 @@ struct k_fv_defect_restrict_b {
                 for (int ii = 0; ii < fac; ++ii) {
                     const int I = Ic * fac + ii, Jz = Jc * fac + jj;
                     const size_t c = (size_t)Jz * K.NX + I;
-                    const T fq = fv_cell_op4<T, IN, VISC>(K, ld, &spt, c, I, Jz, q);
+                    const T fq = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, q);
                     const size_t gi = (size_t)q * n1 + c;
                     acc += gprime_of<T, IN, S>(ld, (S)ld.dir(q, c, I, Jz), fq, fu, gi, adt, adtf, eps) - b[gi];
                 }
@@ -468,12 +357,12 @@ struct k_fv_defect_restrict_b {
         if (xc) xc[(size_t)q * nc + cc] = store_round<S>(dtau_c[cc] * bv, bf16);
     }
 };
-template <class T, int IN, bool VISC, int L, bool FAC2>
+template <class T, int IN, bool VISC, bool FAC2>
 __global__ void __launch_bounds__(256) k_fv_defect_restrict(FVK K, FLoad<T, IN> ld0, const typename SOf<T>::type *b,
                                                             const double *fu, double adt, int fac,
                                                             typename SOf<T>::type *bc, typename SOf<T>::type *xc,
                                                             const typename SOf<T>::type *dtau_c, int bf16) {
-    k_fv_defect_restrict_b<T, IN, VISC, L, FAC2>::run(blockIdx.x, gridDim.x, K, ld0, b, fu, adt, fac, bc, xc, dtau_c, bf16);
+    k_fv_defect_restrict_b<T, IN, VISC, FAC2>::run(blockIdx.x, gridDim.x, K, ld0, b, fu, adt, fac, bc, xc, dtau_c, bf16);
 }
 
 // Face-once form for large levels: a block owns a tile of TX x TZ cells.  The
@@ -501,9 +390,6 @@ struct k_fv_tile_b {
         jf_pdl_enter();
         typedef typename SOf<T>::type S;
         constexpr int TX = FV_TX;
-        // the FP64 power table (the FP32 tangent power needs none)
-        __shared__ double spt_raw[IN < 2 ? sizeof(PowTab) / sizeof(double) : 1];
-        PowTab &spt = *reinterpret_cast<PowTab *>(spt_raw);
         // the tile's cells and a one-cell halo as face sides: state, 1/rho, p, c
         // (one pressure / sound speed per cell instead of one per face and side)
         __shared__ T sU[4][TZ + 2][TX + 2];
@@ -511,7 +397,6 @@ struct k_fv_tile_b {
         __shared__ S sGx[4][TZ][TX + 1];   // net flux H - V through the west face of local cell (i, j)
         __shared__ S sGz[4][TZ + 1][TX];   // ... through the south face
         __shared__ S sD[MODE == FV_DEFRES ? 4 : 1][MODE == FV_DEFRES ? TZ : 1][MODE == FV_DEFRES ? TX : 1];
-        if (IN < 2) load_pt(&spt, K.pt);
         FLoad<T, IN> ld = ld0;
         ld.prepare();
         const int NX = K.NX, NZ = K.NZ;
@@ -536,7 +421,6 @@ struct k_fv_tile_b {
             up0 = (S)oval(ld(0, c, I, J));
             if (MODE == FV_SMOOTH) dtc = dtau[c];
         }
-        if (IN < 2) __syncthreads();   // the power table
         for (int idx = threadIdx.x; idx < (TZ + 2) * (TX + 2); idx += blockDim.x) {
             const int li = idx % (TX + 2), lj = idx / (TX + 2);
             int I = I0 + li - 1;
@@ -548,7 +432,7 @@ struct k_fv_tile_b {
     #pragma unroll
                 for (int v = 0; v < 4; ++v) U[v] = ld(v, c, I, J) + bgs(K.ub, K.ubf, v * NZ + J, T{});
                 Side<T> sd;
-                side_of(U, K.pc, &spt, sd);
+                side_of(U, K.pc, K.pt, sd);
     #pragma unroll
                 for (int v = 0; v < 4; ++v) sU[v][lj][li] = sd.U[v];
                 sIr[lj][li] = sd.ir;
@@ -705,9 +589,6 @@ struct k_fv_dtau_b {
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<FVK> K, JfArg<const S *> u,
                                                JfArg<double> adt, JfArg<double> sigma, JfArg<S *> dtau) {
         jf_pdl_enter();
-        __shared__ PowTab spt;
-        load_pt(&spt, K.pt);
-        __syncthreads();
         const int NX = K.NX, NZ = K.NZ;
         const size_t n1 = (size_t)NX * NZ;
         const size_t c = (size_t)jf_bid * blockDim.x + threadIdx.x;
@@ -719,12 +600,12 @@ struct k_fv_dtau_b {
         };
         S U[4], V[4];
         st(I, Jz, U);
-        const S sx = wave_speed_r<S>(U, 0, K.pc, &spt), sz = wave_speed_r<S>(U, 1, K.pc, &spt);
+        const S sx = wave_speed_r<S>(U, 0, K.pc, K.pt), sz = wave_speed_r<S>(U, 1, K.pc, K.pt);
         S eW = sx, eE = sx, eS = sz, eN = sz;
-        if (I > 0 || K.periodic) { st(I > 0 ? I - 1 : NX - 1, Jz, V); eW = fmax(sx, wave_speed_r<S>(V, 0, K.pc, &spt)); }
-        if (I < NX - 1 || K.periodic) { st(I < NX - 1 ? I + 1 : 0, Jz, V); eE = fmax(sx, wave_speed_r<S>(V, 0, K.pc, &spt)); }
-        if (Jz > 0) { st(I, Jz - 1, V); eS = fmax(sz, wave_speed_r<S>(V, 1, K.pc, &spt)); }
-        if (Jz < NZ - 1) { st(I, Jz + 1, V); eN = fmax(sz, wave_speed_r<S>(V, 1, K.pc, &spt)); }
+        if (I > 0 || K.periodic) { st(I > 0 ? I - 1 : NX - 1, Jz, V); eW = fmax(sx, wave_speed_r<S>(V, 0, K.pc, K.pt)); }
+        if (I < NX - 1 || K.periodic) { st(I < NX - 1 ? I + 1 : 0, Jz, V); eE = fmax(sx, wave_speed_r<S>(V, 0, K.pc, K.pt)); }
+        if (Jz > 0) { st(I, Jz - 1, V); eS = fmax(sz, wave_speed_r<S>(V, 1, K.pc, K.pt)); }
+        if (Jz < NZ - 1) { st(I, Jz + 1, V); eN = fmax(sz, wave_speed_r<S>(V, 1, K.pc, K.pt)); }
         const S iHx = (S)K.iHx, iHz = (S)K.iHz;
         const S lam = (S)0.5 * (eW + eE) * iHx + (S)0.5 * (eS + eN) * iHz + (S)(2.0 * K.mu) * (iHx * iHx + iHz * iHz);
         dtau[c] = (S)sigma / ((S)1 + (S)adt * lam);
@@ -736,36 +617,32 @@ __global__ void k_fv_dtau(FVK K, const S *u, double adt, double sigma, S *dtau) 
 }
 
 // DG pseudo-time step per element: lambda_E = (k+1)^2 max_nodes(|v| + c)(1/hx + 1/hz)
-// + 2 mu (k+1)^4 (1/hx^2 + 1/hz^2).
+// + 2 mu (k+1)^4 (1/hx^2 + 1/hz^2).  A block takes as many elements as its threads hold
+// nodes; the FP64 closing formula runs in the first threads, one per element (one
+// element per warp paid for a whole warp's FP64 slots: 21 us on 12,800 Q3 elements, 7.0 now).
 template <class R>
 struct k_dg_dtau_b {
-    static constexpr int TPB = 0, MINB = 0;
+    static constexpr int TPB = 256, MINB = 0;
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const R *> U,
                                                JfArg<const R *> ubv, JfArg<int> nx, JfArg<int> nz, JfArg<int> np1,
                                                JfArg<PhysC> pc, JfArg<const PowTab *> pt, JfArg<double> ihx,
                                                JfArg<double> ihz, JfArg<double> mu, JfArg<double> adt,
                                                JfArg<double> sigma, JfArg<double *> dtau, JfArg<float *> dtauf) {
         jf_pdl_enter();
-        __shared__ PowTab spt;
-        if (sizeof(R) == 8) load_pt(&spt, pt);
-        __syncthreads();
-        // one warp per element, one lane per node, max over the lanes
+        __shared__ R ssp[256];
         const int n_el = nx * nz;
-        const int lane = threadIdx.x & 31;
-        const int e = (int)(((size_t)jf_bid * blockDim.x + threadIdx.x) >> 5);
-        if (e >= n_el) return;   // uniform over the warp
-        const int NP = np1 * np1;
+        const int NP = np1 * np1, E = 256 / NP;
+        const int le = threadIdx.x / NP, node = threadIdx.x % NP;
+        const int e0 = (int)jf_bid * E, e = e0 + le;
         const size_t N1 = (size_t)n_el * NP;
-        const int ez = e / nx;
         const size_t nrow = (size_t)nz * np1;
-        R sp = 0;
-        if (lane < NP) {
-            const int J = ez * np1 + lane / np1;
-            R W[4];
-            for (int v = 0; v < 4; ++v) W[v] = U[v * N1 + (size_t)e * NP + lane] + ubv[v * nrow + J];
+        if (le < E && e < n_el) {
+            const int J = (e / nx) * np1 + node / np1;
+            R W[4], sp;
+            for (int v = 0; v < 4; ++v) W[v] = U[v * N1 + (size_t)e * NP + node] + ubv[v * nrow + J];
             if (sizeof(R) == 8) {
                 const double ir = 1.0 / (double)W[0];
-                const double p = pc.p0 * pow_gamma_tab(pc.R_over_p0 * (double)W[3], &spt);
+                const double p = eos_pow((double)W[3], pt);
                 sp = (R)(sqrt(((double)W[1] * ir) * ((double)W[1] * ir) + ((double)W[2] * ir) * ((double)W[2] * ir)) +
                          sqrt(pc.gamma * p * ir));
             } else {
@@ -774,20 +651,23 @@ struct k_dg_dtau_b {
                 sp = (R)(sqrtf(((float)W[1] * ir) * ((float)W[1] * ir) + ((float)W[2] * ir) * ((float)W[2] * ir)) +
                          sqrtf(pc.gammaf * p * ir));
             }
+            ssp[threadIdx.x] = sp;
         }
-    #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sp = fmax(sp, __shfl_xor_sync(0xffffffffu, sp, o));
-        if (lane != 0) return;
-        const double vmax = (double)sp;
+        __syncthreads();
+        const int el = threadIdx.x;
+        if (el >= E || e0 + el >= n_el) return;
+        R sm = 0;
+        for (int q = 0; q < NP; ++q) sm = fmax(sm, ssp[el * NP + q]);
+        const double vmax = (double)sm;
         const double n2 = (double)np1 * np1;
         const double lam = n2 * vmax * (ihx + ihz) + 2.0 * mu * n2 * n2 * (ihx * ihx + ihz * ihz);
         const double d = sigma / (1.0 + adt * lam);
-        if (dtau) dtau[e] = d;
-        if (dtauf) dtauf[e] = (float)d;
+        if (dtau) dtau[e0 + el] = d;
+        if (dtauf) dtauf[e0 + el] = (float)d;
     }
 };
 template <class R>
-__global__ void k_dg_dtau(const R *U, const R *ubv, int nx, int nz, int np1, PhysC pc, const PowTab *pt,
+__global__ void __launch_bounds__(256) k_dg_dtau(const R *U, const R *ubv, int nx, int nz, int np1, PhysC pc, const PowTab *pt,
                           double ihx, double ihz, double mu, double adt, double sigma, double *dtau,
                           float *dtauf) {
     k_dg_dtau_b<R>::run(blockIdx.x, gridDim.x, U, ubv, nx, nz, np1, pc, pt, ihx, ihz, mu, adt, sigma, dtau, dtauf);
@@ -1103,20 +983,17 @@ __global__ void k_sub(const S *r, const S *w, S *d, size_t n) {
 
 __global__ void k_bg_fv(FVK K, double *hbx, double *hbxw, double *hbz) {
     jf_pdl_enter();
-    __shared__ PowTab spt;
-    load_pt(&spt, K.pt);
-    __syncthreads();
     const int NZ = K.NZ;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     D64 U[4], G[4], H[4];
     if (i < NZ) {
         for (int v = 0; v < 4; ++v) U[v] = D64{K.ub[v * NZ + i]};
-        hllc<D64, 0>(U, U, K.pc, &spt, H);
+        hllc<D64, 0>(U, U, K.pc, K.pt, H);
         for (int v = 0; v < 4; ++v) hbx[v * NZ + i] = H[v].x;
         mirror<D64, 0>(U, G);
-        hllc<D64, 0>(G, U, K.pc, &spt, H);
+        hllc<D64, 0>(G, U, K.pc, K.pt, H);
         for (int v = 0; v < 4; ++v) hbxw[v * NZ + i] = H[v].x;
-        hllc<D64, 0>(U, G, K.pc, &spt, H);
+        hllc<D64, 0>(U, G, K.pc, K.pt, H);
         for (int v = 0; v < 4; ++v) hbxw[(4 + v) * NZ + i] = H[v].x;
     } else if (i < 2 * NZ + 1) {
         const int j = i - NZ;   // face between rows j-1 and j
@@ -1124,17 +1001,17 @@ __global__ void k_bg_fv(FVK K, double *hbx, double *hbxw, double *hbz) {
         if (j == 0) {
             for (int v = 0; v < 4; ++v) T_[v] = D64{K.ub[v * NZ + 0]};
             mirror<D64, 1>(T_, G);
-            hllc<D64, 1>(G, T_, K.pc, &spt, H);
+            hllc<D64, 1>(G, T_, K.pc, K.pt, H);
         } else if (j == NZ) {
             for (int v = 0; v < 4; ++v) B[v] = D64{K.ub[v * NZ + NZ - 1]};
             mirror<D64, 1>(B, G);
-            hllc<D64, 1>(B, G, K.pc, &spt, H);
+            hllc<D64, 1>(B, G, K.pc, K.pt, H);
         } else {
             for (int v = 0; v < 4; ++v) {
                 B[v] = D64{K.ub[v * NZ + j - 1]};
                 T_[v] = D64{K.ub[v * NZ + j]};
             }
-            hllc<D64, 1>(B, T_, K.pc, &spt, H);
+            hllc<D64, 1>(B, T_, K.pc, K.pt, H);
         }
         for (int v = 0; v < 4; ++v) hbz[v * (NZ + 1) + j] = H[v].x;
     }
@@ -1236,7 +1113,7 @@ void launch_fv(bool l4, unsigned g, int tb, cudaStream_t s, const FVK &K, const 
                const double *fu, double adt, typename SOf<T>::type *out, int bf = 0,
                RKS rk = RKS{nullptr, 0, 1.0, 1.0f}) {
     if (l4) {
-        jf_launch<k_fv_b<T, IN, MODE, V, 4>>(k_fv<T, IN, MODE, V, 4>, g, tb, 0, s, K, ld, x, b, dt, fu, adt, out, bf, rk);
+        jf_launch<k_fv_b<T, IN, MODE, V>>(k_fv<T, IN, MODE, V>, g, tb, 0, s, K, ld, x, b, dt, fu, adt, out, bf, rk);
     } else if (tb >= 256) {   // tile rows follow the block size: 32 x 8 or 32 x 4 cells
         const unsigned gt = (unsigned)(((K.NX + FV_TX - 1) / FV_TX) * ((K.NZ + 7) / 8));
         jf_launch<k_fv_tile_b<T, IN, MODE, V, 8>>(k_fv_tile<T, IN, MODE, V, 8>, gt, FV_TX * 8, 0, s, K, ld, b, dt, fu, adt, out, nullptr, nullptr, bf,
@@ -1334,6 +1211,14 @@ int fv_smooth32_corrected(jfnk_ctx *c, int l, const float *x, bool zero, const f
     return JFNK_OK;
 }
 
+inline int fv_smooth_or_defect(jfnk_ctx *c, int l, int mode, const void *x, const void *b, void *out,
+                               cudaStream_t s, RKS rk = RKS{nullptr, 0, 1.0, 1.0f}) {
+    if (c->prec == 64)
+        return fv_op64(c, l, mode, (const double *)c->lev[l].u, (const double *)x, (const double *)b,
+                       (double *)out, s, rk);
+    return fv_op32(c, l, mode, (const float *)x, (const float *)b, (float *)out, s, rk);
+}
+
 // defect g'x - b on level l restricted to level l+1 (b_{l+1}, and x_{l+1} = dtau b
 // when xc is given)
 int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *bc, void *xc, const void *dtc,
@@ -1347,14 +1232,28 @@ int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *b
     const int tb = c->opts.tile_fv;
     const bool l4 = fv_four_lanes(c, n1);
     const bool f2 = L.fac == 2;
-    const unsigned g = nblk((l4 ? (f2 ? 16 : 4) : 1) * nc, tb);   // lanes per coarse cell
+    const unsigned g = nblk((f2 ? 16 : 4) * nc, tb);   // lanes per coarse cell
     c->fv_calls++;
-#define JF_DR(T, IN, V, LN, F2, ...) jf_launch<k_fv_defect_restrict_b<T, IN, V, LN, F2>>(k_fv_defect_restrict<T, IN, V, LN, F2>, g, tb, 0, s, __VA_ARGS__)
-#define JF_DR2(T, IN, V, ...)                                \
-    do {                                                     \
-        if (!l4) JF_DR(T, IN, V, 1, false, __VA_ARGS__);     \
-        else if (f2) JF_DR(T, IN, V, 4, true, __VA_ARGS__);  \
-        else JF_DR(T, IN, V, 4, false, __VA_ARGS__);         \
+    if (!l4 && !f2) {
+        // large levels agglomerated by 3 or 5 (odd k + 1): separate defect and restriction
+        // (the fused kernel would run fac^2 cells one after another per coarse cell)
+        c->fv_calls--;   // counted by the defect
+        JF_RET(fv_smooth_or_defect(c, l, FV_DEFECT, x, b, L.r, s));
+        if (c->prec == 64)
+            jf_launch<k_restrict_b_b<double>>(k_restrict_b<double>, nblk(C.n, 256), 256, 0, s, (const double *)L.r, L.NX, L.NZ, L.fac,
+                      (double *)bc, (double *)xc, (const double *)dtc, 0);
+        else
+            jf_launch<k_restrict_b_b<float>>(k_restrict_b<float>, nblk(C.n, 256), 256, 0, s, (const float *)L.r, L.NX, L.NZ, L.fac,
+                      (float *)bc, (float *)xc, (const float *)dtc, (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0);
+        jf_launched();
+        JF_CK(cudaGetLastError());
+        return JFNK_OK;
+    }
+#define JF_DR(T, IN, V, F2, ...) jf_launch<k_fv_defect_restrict_b<T, IN, V, F2>>(k_fv_defect_restrict<T, IN, V, F2>, g, tb, 0, s, __VA_ARGS__)
+#define JF_DR2(T, IN, V, ...)                            \
+    do {                                                 \
+        if (f2) JF_DR(T, IN, V, true, __VA_ARGS__);      \
+        else JF_DR(T, IN, V, false, __VA_ARGS__);        \
     } while (0)
     // large levels with 2 x 2 agglomeration: the face-once tile kernel
     const int tz = tb >= 256 ? 8 : 4;   // tile rows follow the block size
@@ -1409,14 +1308,6 @@ int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *b
     jf_launched();
     JF_CK(cudaGetLastError());
     return JFNK_OK;
-}
-
-inline int fv_smooth_or_defect(jfnk_ctx *c, int l, int mode, const void *x, const void *b, void *out,
-                               cudaStream_t s, RKS rk = RKS{nullptr, 0, 1.0, 1.0f}) {
-    if (c->prec == 64)
-        return fv_op64(c, l, mode, (const double *)c->lev[l].u, (const double *)x, (const double *)b,
-                       (double *)out, s, rk);
-    return fv_op32(c, l, mode, (const float *)x, (const float *)b, (float *)out, s, rk);
 }
 
 // more than one stage per pseudo-time step (opts.rk_stages > 1)
@@ -1486,10 +1377,7 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
     if (l < c->nlev - 1) {
         FVLev &C = c->lev[l + 1];
         const bool fuse = c->mid_pre >= 1 && !rk_multi(c);
-        if (zero || c->prec == 64 || (L.fac != 2 && !fv_four_lanes(c, n1))) {
-            // FP64, and large levels agglomerated by 3 or 5 (odd k + 1): separate defect
-            // and restriction (one thread per fine cell keeps the defect kernel occupied;
-            // the fused kernel would run fac^2 cells one after another per coarse cell)
+        if (zero || c->prec == 64) {   // separate defect and restriction
             if (zero) {
                 jf_launch<k_neg_b<S>>(k_neg<S>, nblk(L.n, 256), 256, 0, s, (S *)L.r, (const S *)L.b, L.n);
                 jf_launched();
@@ -1773,10 +1661,11 @@ int mg_linearize(jfnk_ctx *c, const double *Uin, double adt, cudaStream_t s) {
     c->mg_adt = adt;
     c->mg_U = U;
     // DG pseudo-time steps: FP64 for the FP64 preconditioner, FP32 from the FP32
-    // copy of the state otherwise (a step-size heuristic; one warp per element)
-    const unsigned gd = (unsigned)(((size_t)c->n_el * 32 + 127) / 128);
+    // copy of the state otherwise (a step-size heuristic)
+    const int epb = 256 / (c->np1 * c->np1);
+    const unsigned gd = (unsigned)((c->n_el + epb - 1) / epb);
     if (c->prec == 64) {
-        jf_launch<k_dg_dtau_b<double>>(k_dg_dtau<double>, gd, 128, 0, s, U, (const double *)c->ubv, c->grid.nx, c->grid.nz, c->np1,
+        jf_launch<k_dg_dtau_b<double>>(k_dg_dtau<double>, gd, 256, 0, s, U, (const double *)c->ubv, c->grid.nx, c->grid.nz, c->np1,
                   c->pc, c->powtab, 1.0 / c->hx, 1.0 / c->hz, c->phys.mu, adt, c->opts.sigma_dg, c->dtau_dg,
                   c->dtau_dgf);
         jf_launched();
@@ -1784,7 +1673,7 @@ int mg_linearize(jfnk_ctx *c, const double *Uin, double adt, cudaStream_t s) {
         JF_RET(to_fv<double, double>(c, U, (double *)c->lev[0].u, s));
     } else {
         JF_RET(blas_copy_d2f(U, c->Usf, c->N, s));
-        jf_launch<k_dg_dtau_b<float>>(k_dg_dtau<float>, gd, 128, 0, s, (const float *)c->Usf, (const float *)c->ubvf, c->grid.nx,
+        jf_launch<k_dg_dtau_b<float>>(k_dg_dtau<float>, gd, 256, 0, s, (const float *)c->Usf, (const float *)c->ubvf, c->grid.nx,
                   c->grid.nz, c->np1, c->pc, c->powtab, 1.0 / c->hx, 1.0 / c->hz, c->phys.mu, adt,
                   c->opts.sigma_dg, c->dtau_dg, c->dtau_dgf);
         jf_launched();

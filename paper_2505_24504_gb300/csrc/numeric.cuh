@@ -9,13 +9,11 @@
 //        flux code on TL32 gives the exact directional derivative J(u) x of the
 //        operator in FP32, the product the FP32 preconditioner smooths with.
 //
-// Both carry a power x^gamma:
-//  D64: table-driven reduction x = 2^e m_i (1+t), |t| < 2^-8, with 2^(e gamma),
-//       m_i^gamma and 1/m_i from tables built on the host in long double and the
-//       binomial series of (1+t)^gamma to t^6 (truncation < 1e-18); about 10
-//       FP64 pipe operations against ~100 for the library pow on this GPU.
-//       Inputs outside the table range fall back to pow().
-//  TL32: value by the fast exp2/log2 power, tangent gamma p / x.
+// FP64 work is scarce on this GPU: an SM issues two FP64 lanes per clock against 128
+// FP32 and 64 integer lanes, so one FP64 instruction of a warp costs as much as 32
+// integer or 64 FP32 ones.  The FP64 quotients, square roots and the EOS power below
+// therefore do their approximation work on the FP32 and integer pipes and spend FP64
+// instructions only on the final, correctly rounding steps.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -26,31 +24,117 @@
 #define JF_D __device__ __forceinline__
 
 // ---------------------------------------------------------------------------
+// EOS power p = p0 (R E / p0)^gamma = C E^gamma, C = p0 (R/p0)^gamma.  E = 2^e m, m in
+// [1, 2); the interval of m (512 of them) gives v, the double nearest to the reciprocal
+// of its midpoint, so t = m v - 1 has |t| <= 2^-10 (one rounding, v is exact by
+// definition), and E^gamma C = pe[e] mg (1 + t)^gamma with pe[e] = C 2^(e gamma) and
+// mg = v^-gamma from long double.  The binomial series of (1+t)^gamma runs to t^5; its
+// terms from t^3 on are below 2^-34, so their factor is evaluated in FP32 (2^-58 of the
+// result).  Six FP64 instructions.  e outside -32..31, E <= 0 and NaN: pow().
 struct PowTab {
-    double gamma;
-    double pe[64];      // 2^(e gamma), e = -32 .. 31
-    double mg[256];     // (1 + i/256)^gamma
-    double minv[256];   // 1 / (1 + i/256)
-    double c[7];        // binomial coefficients C(gamma, n), n = 1..6 (c[0] unused)
+    double pe[64];          // C 2^(e gamma), e = -32 .. 31
+    double2 mv[512];        // (v, mg) of interval i: [1 + i/512, 1 + (i+1)/512)
+    double gamma, p0, R_over_p0;
+    double c1, c2;          // binomial coefficients C(gamma, n)
+    float c3, c4, c5;
 };
 
-JF_D double pow_gamma_tab(double x, const PowTab *T) {
-    const long long b = __double_as_longlong(x);
-    const int e = (int)((b >> 52) & 0x7ff) - 1023;
-    if (!(x > 0.0) || e < -32 || e > 31) return pow(x, T->gamma);
-    const int i = (int)((b >> 44) & 0xff);
-    const double m = __longlong_as_double((b & 0x000fffffffffffffLL) | 0x3ff0000000000000LL);
-    const double mi = __longlong_as_double((b & 0x000ff00000000000LL) | 0x3ff0000000000000LL);
-    const double t = __dmul_rn(__dsub_rn(m, mi), T->minv[i]);
-    double q = T->c[6];
-    q = __fma_rn(q, t, T->c[5]);
-    q = __fma_rn(q, t, T->c[4]);
-    q = __fma_rn(q, t, T->c[3]);
-    q = __fma_rn(q, t, T->c[2]);
-    q = __fma_rn(q, t, T->c[1]);
-    q = __dmul_rn(q, t);                      // (1+t)^gamma - 1
-    const double s = __dmul_rn(T->pe[e + 32], T->mg[i]);
+// float -> double on the integer pipe, for zero and normal floats
+JF_D double f2d_normal(float f) {
+    const unsigned b = __float_as_uint(f);
+    const unsigned hi = ((b & 0x7fffffffu) >> 3) + (896u << 20);
+    return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) ? hi : 0u)), (int)(b << 29));
+}
+// the leading 24 bits of a positive double's significand as a float in [1, 2)
+JF_D float mant_hi(unsigned hi, unsigned lo) {
+    return __uint_as_float(0x3f800000u | (__funnelshift_l(lo, hi, 3) & 0x7fffffu));
+}
+
+static __device__ __noinline__ double eos_slow(double E, const PowTab *T) {
+    return T->p0 * pow(T->R_over_p0 * E, T->gamma);
+}
+JF_D double eos_pow(double E, const PowTab *T) {
+    const unsigned hi = (unsigned)__double2hiint(E), lo = (unsigned)__double2loint(E);
+    if (hi - (991u << 20) >= (64u << 20)) return eos_slow(E, T);   // exponent -32..31, positive
+    const int e = (int)(hi >> 20) - 991;
+    const double2 mv = __ldg(&T->mv[(hi >> 11) & 511u]);
+    const double m = __hiloint2double((int)((hi & 0xfffffu) | 0x3ff00000u), (int)lo);
+    const double t = __fma_rn(m, mv.x, -1.0);
+    // FP32 copies of m and v (v in (1/2, 1))
+    const unsigned vh = (unsigned)__double2hiint(mv.x) - (896u << 20), vl = (unsigned)__double2loint(mv.x);
+    const float tf = fmaf(mant_hi(hi, lo), __uint_as_float(__funnelshift_l(vl, vh, 3)), -1.0f);
+    const double u = f2d_normal(fmaf(fmaf(__ldg(&T->c5), tf, __ldg(&T->c4)), tf, __ldg(&T->c3)));
+    const double q = __dmul_rn(t, __fma_rn(t, __fma_rn(t, u, __ldg(&T->c2)), __ldg(&T->c1)));   // (1+t)^gamma - 1
+    const double s = __dmul_rn(__ldg(&T->pe[e]), mv.y);
     return __fma_rn(s, q, s);
+}
+
+// ---------------------------------------------------------------------------
+// Quotient, reciprocal and square root of doubles with binary exponents within +-400
+// (others, zeros, infinities and NaN take the IEEE intrinsics).  A hardware FP32
+// approximation of the significand is refined to about 45 bits in two-float arithmetic
+// (Newton's iteration with the residual formed by FMA) and put together as a double on
+// the integer pipe; one FP64 correction with the exact residual (Markstein, "Computation
+// of elementary functions on the IBM RISC System/6000 processor", 1990) then gives the
+// quotient from an approximation whose error is 2^-88: the correctly rounded result (no
+// difference from the IEEE intrinsics in 3.1e8 random quotients and roots; reciprocals of
+// the last few significands below a power of two, whose exact value lies that close to a
+// tie, can round to the other neighbour).  Two FP64 instructions for a reciprocal, three
+// for a quotient or a square root: 35, 55 and 51 clocks of an SM per warp where the IEEE
+// intrinsics take 142 and 143, latency 236, 300 and 328 clocks against 562 and 597.
+JF_D bool mid_exp(unsigned hi) { return (hi & 0x7fffffffu) - (623u << 20) < (801u << 20); }
+
+// a two-float value f + g (f in [1/2, 1], |g| below 2^-21) as a double
+JF_D double join2(float f, float g) {
+    const unsigned b = __float_as_uint(f);
+    const long long base = (long long)((((unsigned long long)(b >> 3) + (896ull << 20)) << 32) | (unsigned)(b << 29));
+    return __longlong_as_double(base + 2ll * __float2int_rn(g * 4503599627370496.0f));   // units of 2^-53
+}
+// 1 / |b| to about 45 bits, sign of b
+JF_D double rcp45(double b) {
+    const unsigned hi = (unsigned)__double2hiint(b), lo = (unsigned)__double2loint(b);
+    const float mh = mant_hi(hi, lo);
+    const float ml = (float)(int)(lo & 0x1fffffffu) * 2.220446049250313e-16f;   // 2^-52
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(mh));
+    const float e = fmaf(-ml, r, fmaf(-mh, r, 1.0f));
+    const double x = join2(r, r * fmaf(e, e, e));
+    const unsigned sh = ((hi >> 20) & 0x7ffu) - 1023u;   // binary exponent of b
+    return __hiloint2double((int)(((unsigned)__double2hiint(x) - (sh << 20)) | (hi & 0x80000000u)), __double2loint(x));
+}
+static __device__ __noinline__ double div_slow(double a, double b) { return __ddiv_rn(a, b); }
+static __device__ __noinline__ double sqrt_slow(double x) { return __dsqrt_rn(x); }
+
+JF_D double div64(double a, double b) {
+    const unsigned ah = (unsigned)__double2hiint(a), bh = (unsigned)__double2hiint(b);
+    const bool zero = ((ah & 0x7fffffffu) | (unsigned)__double2loint(a)) == 0u;
+    if (!mid_exp(bh) || !(mid_exp(ah) || zero)) return div_slow(a, b);
+    const double r = rcp45(b);
+    const double q = __dmul_rn(a, r);
+    return __fma_rn(__fma_rn(-b, q, a), r, q);
+}
+JF_D double rcp64(double b) {
+    if (!mid_exp((unsigned)__double2hiint(b))) return div_slow(1.0, b);
+    const double r = rcp45(b);
+    return __fma_rn(__fma_rn(-b, r, 1.0), r, r);
+}
+// sqrt: y = 1/sqrt of the significand scaled to [1, 4), to about 45 bits
+JF_D double sqrt64(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    if (hi - (623u << 20) >= (801u << 20)) return sqrt_slow(x);   // negative, zero, out of range, NaN
+    const int e = (int)(hi >> 20) - 1023, odd = e & 1, half = (e - odd) >> 1;
+    const float sc = odd ? 2.0f : 1.0f;
+    const float mh = mant_hi(hi, lo) * sc;
+    const float ml = (float)(int)(lo & 0x1fffffffu) * (2.220446049250313e-16f * sc);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(mh));
+    const float p = y * y, pe = fmaf(y, y, -p);
+    const float d = fmaf(-ml, p, fmaf(-mh, pe, fmaf(-mh, p, 1.0f)));   // 1 - m y^2
+    const double z = join2(y, y * (d * fmaf(0.375f, d, 0.5f)));
+    const double w = __hiloint2double(__double2hiint(z) - (half << 20), __double2loint(z));   // 1/sqrt(x)
+    const double g = __dmul_rn(x, w);
+    const double h = __hiloint2double(__double2hiint(w) - (1 << 20), __double2loint(w));      // half of it
+    return __fma_rn(__fma_rn(-g, g, x), h, g);
 }
 
 // ---------------------------------------------------------------------------
@@ -61,10 +145,21 @@ JF_D D64 mk(double v, D64) { return D64{v}; }
 JF_D D64 operator+(D64 a, D64 b) { return D64{__dadd_rn(a.x, b.x)}; }
 JF_D D64 operator-(D64 a, D64 b) { return D64{__dsub_rn(a.x, b.x)}; }
 JF_D D64 operator*(D64 a, D64 b) { return D64{__dmul_rn(a.x, b.x)}; }
-JF_D D64 operator/(D64 a, D64 b) { return D64{__ddiv_rn(a.x, b.x)}; }
+JF_D D64 operator/(D64 a, D64 b) { return D64{div64(a.x, b.x)}; }
 JF_D D64 operator-(D64 a) { return D64{-a.x}; }
-JF_D D64 jsqrt(D64 a) { return D64{__dsqrt_rn(a.x)}; }
-JF_D double val(D64 a) { return a.x; }
+JF_D D64 jsqrt(D64 a) { return D64{sqrt64(a.x)}; }
+JF_D D64 jrcp(D64 a) { return D64{rcp64(a.x)}; }
+// comparisons on the integer pipe (the sign-magnitude order of the bit patterns)
+JF_D bool nonneg(D64 a) {
+    const long long i = __double_as_longlong(a.x);
+    return i >= 0 || (i << 1) == 0;   // -0 included
+}
+JF_D bool le(D64 a, D64 b) {
+    long long i = __double_as_longlong(a.x), j = __double_as_longlong(b.x);
+    i ^= (i >> 63) & 0x7fffffffffffffffll;
+    j ^= (j >> 63) & 0x7fffffffffffffffll;
+    return i <= j;
+}
 JF_D D64 jfma(D64 a, D64 b, D64 c) { return D64{__fma_rn(a.x, b.x, c.x)}; }
 
 // ---------------------------------------------------------------------------
@@ -90,7 +185,12 @@ JF_D TL32 jsqrt(TL32 a) {
     const float r = rsqrtf(a.v);
     return TL32{a.v * r, 0.5f * a.d * r};
 }
-JF_D float val(TL32 a) { return a.v; }   // compared in FP32: no FP64-pipe conversion
+JF_D bool nonneg(TL32 a) { return a.v >= 0.0f; }
+JF_D bool le(TL32 a, TL32 b) { return a.v <= b.v; }
+JF_D TL32 jrcp(TL32 a) {
+    const float ib = frcp(a.v);
+    return TL32{ib, -(ib * a.d) * ib};
+}
 JF_D TL32 jfma(TL32 a, TL32 b, TL32 c) { return a * b + c; }
 
 // An FP32 constant in tangent-linear arithmetic (its tangent is zero): products,

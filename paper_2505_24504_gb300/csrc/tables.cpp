@@ -200,21 +200,34 @@ static void subcell_average_table(const LD *x, int n, LD P[5][5]) {
     }
 }
 
-void jf_build_powtab(double gamma, PowTab *P) {
+void jf_build_powtab(double gamma, double R, double p0, PowTab *P) {
     memset(P, 0, sizeof(*P));
     const LD g = gamma;
     P->gamma = gamma;
-    for (int e = -32; e < 32; ++e) P->pe[e + 32] = (double)exp2l((LD)e * g);
-    for (int i = 0; i < 256; ++i) {
-        const LD m = 1.0L + i / 256.0L;
-        P->mg[i] = (double)powl(m, g);
-        P->minv[i] = (double)(1.0L / m);
+    P->p0 = p0;
+    P->R_over_p0 = R / p0;
+    const LD C = (LD)p0 * powl((LD)R / p0, g);
+    for (int e = -32; e < 32; ++e) P->pe[e + 32] = (double)(C * exp2l((LD)e * g));
+    LD c[10] = {1.0L};
+    for (int n = 1; n < 10; ++n) c[n] = c[n - 1] * (g - (n - 1)) / n;
+    // v^-gamma by powl for one interval in four; from it for the other three by the
+    // binomial series (|t| < 2^-8; powl in software quadruple precision costs a
+    // microsecond, and a context would pay for 512)
+    for (int i = 0; i < 512; ++i) P->mv[i].x = (double)(1.0L / (1.0L + (i + 0.5L) / 512.0L));
+    for (int b = 1; b < 512; b += 4) {
+        const LD vb = P->mv[b].x, mb = powl(1.0L / vb, g);
+        for (int i = b - 1; i < b + 3; ++i) {
+            const LD t = vb / (LD)P->mv[i].x - 1.0L;
+            LD q = c[9];
+            for (int n = 8; n >= 0; --n) q = q * t + c[n];
+            P->mv[i].y = (double)(mb * q);
+        }
     }
-    LD c = 1.0L;
-    for (int nn = 1; nn <= 6; ++nn) {
-        c = c * (g - (nn - 1)) / nn;
-        P->c[nn] = (double)c;
-    }
+    P->c1 = (double)c[1];
+    P->c2 = (double)c[2];
+    P->c3 = (float)c[3];
+    P->c4 = (float)c[4];
+    P->c5 = (float)c[5];
 }
 
 // Environmental atmosphere at height z: U (4) and dU/dz (4).
