@@ -159,7 +159,7 @@ size_t workspace(const jfnk_grid *g, int k, const jfnk_opts *o, const jfnk_physi
         b += sS * n * 6 + sS * n / 4;
     }
     b += 8 * 4096 * 32 + 8 * 256;
-    b += 8 * (fx + fz) * (visc ? 16 : 8);   // face traces of the Newton iterate
+    b += 8 * (fx + fz) * (visc ? 33 : 12) + 8 * N + 8 * npt * (visc ? 19 : 5);   // linearisation of the DG operator
     if (nlev_out) *nlev_out = nl;
     return b;
 }
@@ -501,8 +501,11 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
     A_(c->partial, 8 * (size_t)c->nb_red * 32);
     {
         const size_t nfp = (size_t)g->nz * (g->nx + 1) * c->np1 + (size_t)(g->nz + 1) * g->nx * c->np1;
-        A_(c->trU, 8 * nfp * (ph->mu != 0.0 ? 16 : 8));
-        c->tr_valid = 0;
+        A_(c->lin.tr, 8 * nfp * (visc ? 20 : 8));
+        A_(c->lin.H, 8 * nfp * (visc ? 13 : 4));
+        A_(c->lin.U, 8 * N);
+        A_(c->lin.F, 8 * c->npt * (visc ? 19 : 5));
+        c->lin_valid = 0;
     }
     A_(c->scal, 8 * (size_t)S_COUNT);
     A_(c->ticket, 256);
@@ -576,27 +579,28 @@ int jv_product(jfnk_ctx *c, const double *U, const double *fU, const double *y, 
                double *Jy, void *stream) {
     if (!c || !U || !y || !Jy || Jy == U || Jy == y || (fU && Jy == fU)) return JFNK_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    if (!fU) {
+    const bool own = fU == nullptr;
+    if (own) {
         DGArgs a = {};
         a.U = U;
         a.out0 = c->fU;
+        a.lin_out = !(eps > 0.0);
         JF_RET(dg_apply(c, DG_RES, a, s));
         fU = c->fU;
-    }
-    double *epsp = c->scal + S_EPS;
-    if (eps > 0.0) {
-        JF_CK(cudaMemcpyAsync(epsp, &eps, sizeof(double), cudaMemcpyHostToDevice, s));
-        JF_CK(cudaStreamSynchronize(s));   // eps lives on the caller's stack
-    } else {
-        JF_RET(red_dot(c, y, y, c->N, epsp, RED_EPS, s));
     }
     DGArgs a = {};
     a.U = U;
     a.y = y;
     a.fU = fU;
-    a.eps = epsp;
     a.adt = adt;
     a.out0 = Jy;
+    if (eps > 0.0) {
+        a.eps_val = eps;
+    } else {
+        JF_RET(red_dot(c, y, y, c->N, c->scal + S_EPS, RED_EPS, s));
+        a.eps = c->scal + S_EPS;
+        a.lin = own;   // f(U) and its linearisation were just evaluated
+    }
     return dg_apply(c, DG_JV, a, s);
 }
 
@@ -607,10 +611,13 @@ int mg_precondition(jfnk_ctx *c, const double *U, double adt, const double *r, d
         JF_CK(cudaMemcpyAsync(z, r, 8 * c->N, cudaMemcpyDeviceToDevice, s));
         return JFNK_OK;
     }
-    DGArgs a = {};
-    a.U = U;
-    a.out0 = c->fU;
-    JF_RET(dg_apply(c, DG_RES, a, s));
+    if (c->prec == 64) {   // f(U) of the FD products; the FP32 tangent products need none
+        DGArgs a = {};
+        a.U = U;
+        a.out0 = c->fU;
+        a.lin_out = 1;
+        JF_RET(dg_apply(c, DG_RES, a, s));
+    }
     JF_RET(mg_linearize(c, U, adt, s));
     if (c->prec == 64) return mg_apply(c, r, z, s);
     JF_RET(mg_apply(c, r, c->Z, s));
@@ -665,17 +672,21 @@ int jfnk_time_operator(jfnk_ctx *c, int which, const double *U, const double *y,
     a.U = U;
     a.adt = 1.0;
     if (which == 1) {
-        // f(U), its face traces and eps once, outside the timed launches; the timed
-        // products take the form the solver's Arnoldi steps use (stored traces of U)
+        // f(U), its linearisation and eps once, outside the timed launches; the timed
+        // products take the form the solver's Arnoldi steps use
         a.out0 = c->fU;
-        a.tr_out = c->trU;
+        a.lin_out = 1;
         rc = dg_apply(c, DG_RES, a, s);
-        a.tr_out = nullptr;
+        a.lin_out = 0;
         if (!rc) rc = red_dot(c, y, y, c->N, c->scal + S_EPS, RED_EPS, s);
         a.y = y;
         a.fU = c->fU;
         a.eps = c->scal + S_EPS;
-        a.tr_in = c->trU;
+        a.lin = 1;
+        if (!rc && c->prec != 64) {   // FP32 directions, as the FP32 preconditioner's z_j
+            rc = blas_copy_d2f(y, (float *)c->pz, c->N, s);
+            a.yf = (const float *)c->pz;
+        }
     }
     if (which == 2) {
         rc = blas_copy_d2f(y, (float *)c->pz, c->N, s);
@@ -732,6 +743,7 @@ int jfnk_autotune(jfnk_ctx *c, const double *U, const double *y, int reps, int *
         DGArgs a = {};
         a.U = U;
         a.out0 = c->fU;
+        a.lin_out = 1;
         int rc = dg_apply(c, DG_RES, a, s);
         if (!rc) rc = mg_linearize(c, U, 1.0, s);
         best_mg = 1e300;

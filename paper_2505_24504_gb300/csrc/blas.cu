@@ -657,30 +657,26 @@ __device__ __forceinline__ double f2d_bits(float f) {
     return __longlong_as_double((long long)r);
 }
 
-// y = (double) x and eps = sqrt(2^-52)/|y| (for the FD product) in one launch.
-// The squares are summed in FP32 within a thread (eps needs a few digits), the
-// per-thread partials in FP64.
-struct k_f2d_eps_b {
+// eps = sqrt(2^-52)/|x| of the FD product from an FP32 direction.  The squares are
+// summed in FP32 within a thread (eps needs a few digits), the per-thread partials in
+// FP64.
+struct k_eps32_b {
     static constexpr int TPB = RB, MINB = 0;
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const float *> x,
-                                               JfArg<double *> y, JfArg<size_t> n, JfArg<double *> part,
-                                               JfArg<unsigned *> ticket, JfArg<double *> eps) {
+                                               JfArg<size_t> n, JfArg<double *> part, JfArg<unsigned *> ticket,
+                                               JfArg<double *> eps) {
         jf_pdl_enter();
         float acc = 0.0f, acc2 = 0.0f;
         const size_t stride = (size_t)jf_nblk * RB;
-        const size_t n4 = n / 4;   // float4 in, two double2 out (x, y 16-byte aligned)
+        const size_t n4 = n / 4;   // x 16-byte aligned
         const float4 *x4 = reinterpret_cast<const float4 *>(x);
-        double2 *y2 = reinterpret_cast<double2 *>(y);
         for (size_t i = (size_t)jf_bid * RB + threadIdx.x; i < n4; i += stride) {
             const float4 f = x4[i];
-            y2[2 * i] = make_double2(f2d_bits(f.x), f2d_bits(f.y));
-            y2[2 * i + 1] = make_double2(f2d_bits(f.z), f2d_bits(f.w));
             acc = fmaf(f.y, f.y, fmaf(f.x, f.x, acc));
             acc2 = fmaf(f.w, f.w, fmaf(f.z, f.z, acc2));
         }
         for (size_t i = 4 * n4 + (size_t)jf_bid * RB + threadIdx.x; i < n; i += stride) {
             const float f = x[i];
-            y[i] = f2d_bits(f);
             acc = fmaf(f, f, acc);
         }
         const double tsum = block_sum((double)acc + (double)acc2);
@@ -693,9 +689,8 @@ struct k_f2d_eps_b {
         }
     }
 };
-__global__ void __launch_bounds__(RB) k_f2d_eps(const float *x, double *y, size_t n, double *part, unsigned *ticket,
-                                                double *eps) {
-    k_f2d_eps_b::run(blockIdx.x, gridDim.x, x, y, n, part, ticket, eps);
+__global__ void __launch_bounds__(RB) k_eps32(const float *x, size_t n, double *part, unsigned *ticket, double *eps) {
+    k_eps32_b::run(blockIdx.x, gridDim.x, x, n, part, ticket, eps);
 }
 
 struct YV {
@@ -1017,10 +1012,10 @@ int blas_mupdate_norm(jfnk_ctx *c, const double *V, int nv, size_t ldv, const do
     return JFNK_OK;
 }
 
-int blas_f2d_eps(jfnk_ctx *c, const float *x, double *y, size_t n, double *eps_out, cudaStream_t s) {
-    if (((uintptr_t)x & 15) || ((uintptr_t)y & 15)) return JFNK_EINVAL;
+int blas_eps32(jfnk_ctx *c, const float *x, size_t n, double *eps_out, cudaStream_t s) {
+    if ((uintptr_t)x & 15) return JFNK_EINVAL;
     const int nb = nblocks_red(c, n);
-    jf_launch<k_f2d_eps_b>(k_f2d_eps, nb, RB, 0, s, x, y, n, c->partial, c->ticket, eps_out);
+    jf_launch<k_eps32_b>(k_eps32, nb, RB, 0, s, x, n, c->partial, c->ticket, eps_out);
     jf_launched();
     JF_CK(cudaGetLastError());
     return JFNK_OK;

@@ -21,6 +21,11 @@
 
 namespace {
 
+// the 1D tables the operator kernels read
+struct TabK {
+    int np1;
+    double lp[5], lm[5], dlp[5], dlm[5], Dn[5][5];
+};
 struct DGK {
     int nx, nz, n_el, periodic;
     double two_hx, two_hz, g, mu, eta_x, eta_z;
@@ -34,7 +39,7 @@ struct DGK {
     const PowTab *pt;
     const double *ubv, *dubv, *fbx, *fbz, *hbx, *hbxw, *ubh, *dubh, *hbz;
     const float *ubvf, *dubvf, *ubhf, *dubhf;
-    DGTab tab;
+    TabK tab;
 };
 
 template <class T> struct OutT;
@@ -52,9 +57,11 @@ template <> struct Loader<D64, 0> {
     JF_D D64 operator()(size_t i) const { return D64{U[i]}; }
 };
 template <> struct Loader<D64, 1> {
-    const double *U, *y, *epsp;   // eps is a device scalar written by a reduction
+    const double *U, *y, *epsp;   // eps: a device scalar written by a reduction, or given
     double eps;
-    JF_D void prepare() { eps = *epsp; }
+    JF_D void prepare() {
+        if (epsp) eps = *epsp;
+    }
     JF_D D64 operator()(size_t i) const { return D64{__fma_rn(eps, y[i], U[i])}; }
 };
 template <> struct Loader<TL32, 2> {
@@ -85,31 +92,13 @@ JF_D void line_trace(const Loader<T, IN> &ld, size_t i0, size_t st, const double
         if (VISC) d = jfma(mkc(pd[q], pdf[q], T{}), u, d);
     }
 }
-// The same traces of the FD state U + eps y from the stored traces of U (Newton
-// iterate, written by the residual) and the traces of y: tr(U + eps y) =
-// tr(U) + eps tr(y) -- the U part is then the same bits as in f(U).
-template <int NP1, bool VISC>
-JF_D void line_trace_fd(const Loader<D64, 1> &ld, size_t i0, size_t st, const double *pa, const double *pd,
-                        double trU, double dU, D64 &a, D64 &d) {
-    double ay = 0.0, dy = 0.0;
-#pragma unroll
-    for (int q = 0; q < NP1; ++q) {
-        const double y = ld.y[i0 + q * st];
-        ay = __fma_rn(pa[q], y, ay);
-        if (VISC) dy = __fma_rn(pd[q], y, dy);
-    }
-    a = D64{__fma_rn(ld.eps, ay, trU)};
-    d = D64{VISC ? __fma_rn(ld.eps, dy, dU) : 0.0};
-}
-
 // Body of the face kernel for block `blk` of one operator evaluation; K is the
 // launch parameter (single operator) or a member's descriptor in global memory
 // (grouped launch over ensemble members).
 template <class T, int IN, int NP1, bool VISC>
 __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld0, typename OutT<T>::type *phix,
                                            typename OutT<T>::type *symx, typename OutT<T>::type *phiz,
-                                           typename OutT<T>::type *symz, unsigned blk, double *tr_out,
-                                           const double *tr_in) {
+                                           typename OutT<T>::type *symz, unsigned blk, const LinPtr &lin) {
     typedef typename OutT<T>::type O;
     Loader<T, IN> ld = ld0;
     ld.prepare();
@@ -120,6 +109,7 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
     const long long nhorz = (long long)(nz + 1) * nx * NP1;
     const long long t = (long long)blk * blockDim.x + threadIdx.x;
     if (t >= nvert + nhorz) return;
+    const size_t nfp = (size_t)(nvert + nhorz);
     const T zero = mk(0.0, T{});
     T H[4], Phi[4], sL[3], sR[3];
     if (t < nvert) {
@@ -141,36 +131,13 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
         }
         // traces: L at xi = +1 (row s), R at xi = -1
         T trL[4], trR[4], gL[4], gR[4];
-        const size_t nfp = (size_t)(nvert + nhorz);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             T aL, aR, dL, dR;
             const size_t iL0 = (size_t)v * N1 + (size_t)eL * NP + s * NP1;
             const size_t iR0 = (size_t)v * N1 + (size_t)eR * NP + s * NP1;
-            bool done = false;
-            if constexpr (IN == 1) {
-                if (tr_in) {
-                    line_trace_fd<NP1, VISC>(ld, iL0, 1, K.tab.lp, K.tab.dlp, tr_in[(2 * v) * nfp + t],
-                                             VISC ? tr_in[(8 + 2 * v) * nfp + t] : 0.0, aL, dL);
-                    line_trace_fd<NP1, VISC>(ld, iR0, 1, K.tab.lm, K.tab.dlm, tr_in[(2 * v + 1) * nfp + t],
-                                             VISC ? tr_in[(9 + 2 * v) * nfp + t] : 0.0, aR, dR);
-                    done = true;
-                }
-            }
-            if (!done) {
-                line_trace<T, IN, NP1, VISC>(ld, iL0, 1, K.tab.lp, K.tlp, K.tab.dlp, K.tdlp, aL, dL);
-                line_trace<T, IN, NP1, VISC>(ld, iR0, 1, K.tab.lm, K.tlm, K.tab.dlm, K.tdlm, aR, dR);
-            }
-            if constexpr (IN == 0) {
-                if (tr_out) {
-                    tr_out[(2 * v) * nfp + t] = outv(aL);
-                    tr_out[(2 * v + 1) * nfp + t] = outv(aR);
-                    if (VISC) {
-                        tr_out[(8 + 2 * v) * nfp + t] = outv(dL);
-                        tr_out[(9 + 2 * v) * nfp + t] = outv(dR);
-                    }
-                }
-            }
+            line_trace<T, IN, NP1, VISC>(ld, iL0, 1, K.tab.lp, K.tlp, K.tab.dlp, K.tdlp, aL, dL);
+            line_trace<T, IN, NP1, VISC>(ld, iR0, 1, K.tab.lm, K.tlm, K.tab.dlm, K.tdlm, aR, dR);
             trL[v] = aL;
             trR[v] = aR;
             gL[v] = mkc(K.two_hx, K.two_hxf, T{}) * dL;
@@ -182,11 +149,31 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
             UL[v] = trL[v] + bgs(K.ubv, K.ubvf, v * nrow + J, T{});
             UR[v] = trR[v] + bgs(K.ubv, K.ubvf, v * nrow + J, T{});
         }
+        if constexpr (IN == 0) {
+            if (lin.tr) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    lin.tr[(2 * v) * nfp + t] = outv(UL[v]);
+                    lin.tr[(2 * v + 1) * nfp + t] = outv(UR[v]);
+                    if (VISC) {
+                        lin.tr[(8 + 2 * v) * nfp + t] = outv(gL[v]);
+                        lin.tr[(9 + 2 * v) * nfp + t] = outv(gR[v]);
+                        lin.tr[(16 + v) * nfp + t] = outv(trL[v] - trR[v]);
+                    }
+                }
+            }
+        }
         wall_states<T, 0>(UL, UR, wallL, wallR);
         Side<T> SL, SR;
         side_of(UL, K.pc, K.pt, SL);
         side_of(UR, K.pc, K.pt, SR);
         hllc_s<T, 0>(SL, SR, H);
+        if constexpr (IN == 0) {
+            if (lin.tr) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) lin.H[v * nfp + t] = outv(H[v]);
+            }
+        }
         const double *hb = wallL ? K.hbxw : (wallR ? K.hbxw + 4 * nrow : K.hbx);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
@@ -207,7 +194,15 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
                 const T Jv = trL[v] - trR[v];
                 sL[c] = hmu * visc_c(pL, J0, Jv);
                 sR[c] = hmu * visc_c(pR, J0, Jv);
-                Phi[v] = Phi[v] - hmu * (visc_c(pL, gL[0], gL[v]) + visc_c(pR, gR[0], gR[v])) + eta * (sL[c] + sR[c]);
+                const T V = visc_face(hmu, eta, pL, pR, gL, gR, v, sL[c], sR[c]);
+                Phi[v] = Phi[v] - V;
+                if constexpr (IN == 0) {
+                    if (lin.tr) {
+                        lin.H[(4 + c) * nfp + t] = outv(V);
+                        lin.H[(7 + c) * nfp + t] = outv(sL[c]);
+                        lin.H[(10 + c) * nfp + t] = outv(sR[c]);
+                    }
+                }
             }
         }
         const size_t fb = ((size_t)ez * (nx + 1) + fx) * NP1 + s;
@@ -230,36 +225,13 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
         const int eB = (wallB ? 0 : fz - 1) * nx + ex;
         const int eT = (wallT ? nz - 1 : fz) * nx + ex;
         T trB[4], trT[4], gB[4], gT[4];
-        const size_t nfp = (size_t)(nvert + nhorz);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             T aB, aT, dB, dT;
             const size_t iB0 = (size_t)v * N1 + (size_t)eB * NP + s;
             const size_t iT0 = (size_t)v * N1 + (size_t)eT * NP + s;
-            bool done = false;
-            if constexpr (IN == 1) {
-                if (tr_in) {
-                    line_trace_fd<NP1, VISC>(ld, iB0, NP1, K.tab.lp, K.tab.dlp, tr_in[(2 * v) * nfp + t],
-                                             VISC ? tr_in[(8 + 2 * v) * nfp + t] : 0.0, aB, dB);
-                    line_trace_fd<NP1, VISC>(ld, iT0, NP1, K.tab.lm, K.tab.dlm, tr_in[(2 * v + 1) * nfp + t],
-                                             VISC ? tr_in[(9 + 2 * v) * nfp + t] : 0.0, aT, dT);
-                    done = true;
-                }
-            }
-            if (!done) {
-                line_trace<T, IN, NP1, VISC>(ld, iB0, NP1, K.tab.lp, K.tlp, K.tab.dlp, K.tdlp, aB, dB);
-                line_trace<T, IN, NP1, VISC>(ld, iT0, NP1, K.tab.lm, K.tlm, K.tab.dlm, K.tdlm, aT, dT);
-            }
-            if constexpr (IN == 0) {
-                if (tr_out) {
-                    tr_out[(2 * v) * nfp + t] = outv(aB);
-                    tr_out[(2 * v + 1) * nfp + t] = outv(aT);
-                    if (VISC) {
-                        tr_out[(8 + 2 * v) * nfp + t] = outv(dB);
-                        tr_out[(9 + 2 * v) * nfp + t] = outv(dT);
-                    }
-                }
-            }
+            line_trace<T, IN, NP1, VISC>(ld, iB0, NP1, K.tab.lp, K.tlp, K.tab.dlp, K.tdlp, aB, dB);
+            line_trace<T, IN, NP1, VISC>(ld, iT0, NP1, K.tab.lm, K.tlm, K.tab.dlm, K.tdlm, aT, dT);
             trB[v] = aB;
             trT[v] = aT;
             gB[v] = mkc(K.two_hz, K.two_hzf, T{}) * dB + bgs(K.dubh, K.dubhf, (size_t)v * (nz + 1) + fz, T{});
@@ -271,11 +243,31 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
             UB[v] = trB[v] + bgs(K.ubh, K.ubhf, (size_t)v * (nz + 1) + fz, T{});
             UT[v] = trT[v] + bgs(K.ubh, K.ubhf, (size_t)v * (nz + 1) + fz, T{});
         }
+        if constexpr (IN == 0) {
+            if (lin.tr) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    lin.tr[(2 * v) * nfp + t] = outv(UB[v]);
+                    lin.tr[(2 * v + 1) * nfp + t] = outv(UT[v]);
+                    if (VISC) {
+                        lin.tr[(8 + 2 * v) * nfp + t] = outv(gB[v]);
+                        lin.tr[(9 + 2 * v) * nfp + t] = outv(gT[v]);
+                        lin.tr[(16 + v) * nfp + t] = outv(trB[v] - trT[v]);
+                    }
+                }
+            }
+        }
         wall_states<T, 1>(UB, UT, wallB, wallT);
         Side<T> SB, ST;
         side_of(UB, K.pc, K.pt, SB);
         side_of(UT, K.pc, K.pt, ST);
         hllc_s<T, 1>(SB, ST, H);
+        if constexpr (IN == 0) {
+            if (lin.tr) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) lin.H[v * nfp + t] = outv(H[v]);
+            }
+        }
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             if (IN != 2) H[v] = H[v] - bg<T>(K.hbz, (size_t)v * (nz + 1) + fz);
@@ -295,7 +287,15 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
                 const T Jv = trB[v] - trT[v];
                 sL[c] = hmu * visc_c(pL, J0, Jv);
                 sR[c] = hmu * visc_c(pR, J0, Jv);
-                Phi[v] = Phi[v] - hmu * (visc_c(pL, gB[0], gB[v]) + visc_c(pR, gT[0], gT[v])) + eta * (sL[c] + sR[c]);
+                const T V = visc_face(hmu, eta, pL, pR, gB, gT, v, sL[c], sR[c]);
+                Phi[v] = Phi[v] - V;
+                if constexpr (IN == 0) {
+                    if (lin.tr) {
+                        lin.H[(4 + c) * nfp + t] = outv(V);
+                        lin.H[(7 + c) * nfp + t] = outv(sL[c]);
+                        lin.H[(10 + c) * nfp + t] = outv(sR[c]);
+                    }
+                }
             }
         }
         const size_t fb = ((size_t)fz * nx + ex) * NP1 + s;
@@ -320,36 +320,29 @@ struct k_faces_b {
                                                JfArg<Loader<T, IN>> ld0, JfArg<typename OutT<T>::type *> phix,
                                                JfArg<typename OutT<T>::type *> symx,
                                                JfArg<typename OutT<T>::type *> phiz,
-                                               JfArg<typename OutT<T>::type *> symz, JfArg<double *> tr_out,
-                                               JfArg<const double *> tr_in) {
+                                               JfArg<typename OutT<T>::type *> symz, JfArg<LinPtr> lin) {
         jf_pdl_enter();
-        faces_body<T, IN, NP1, VISC>(K, ld0, phix, symx, phiz, symz, jf_bid, tr_out, tr_in);
+        faces_body<T, IN, NP1, VISC>(K, ld0, phix, symx, phiz, symz, jf_bid, lin);
     }
 };
 template <class T, int IN, int NP1, bool VISC>
 __global__ void __launch_bounds__(256, VISC ? 2 : 4) k_faces(DGK K, Loader<T, IN> ld0, typename OutT<T>::type *phix,
                                                typename OutT<T>::type *symx, typename OutT<T>::type *phiz,
-                                               typename OutT<T>::type *symz, double *tr_out, const double *tr_in) {
-    k_faces_b<T, IN, NP1, VISC>::run(blockIdx.x, gridDim.x, K, ld0, phix, symx, phiz, symz, tr_out, tr_in);
+                                               typename OutT<T>::type *symz, LinPtr lin) {
+    k_faces_b<T, IN, NP1, VISC>::run(blockIdx.x, gridDim.x, K, ld0, phix, symx, phiz, symz, lin);
 }
 
 // ---------------------------------------------------------------------------
-// elements per volume block: TV = 2 -> ~128 threads, TV = 1 -> ~64 threads
-template <int NP1, int TV> struct EPBOf {
-    static constexpr int NP = NP1 * NP1;
-    static constexpr int T = TV == 2 ? 128 : 64;
-    static constexpr int value = (T / NP) > 0 ? (T / NP) : 1;
-};
-
-template <class T, int IN, int MODE, int NP1, bool VISC, int TV>
+// blockDim.x / NP elements per volume block (at most 128 threads)
+template <class T, int IN, int MODE, int NP1, bool VISC>
 __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &ld0, const DGArgs &A,
                                             const typename OutT<T>::type *phix,
                                             const typename OutT<T>::type *symx,
                                             const typename OutT<T>::type *phiz,
-                                            const typename OutT<T>::type *symz, unsigned blk) {
+                                            const typename OutT<T>::type *symz, unsigned blk, const LinPtr &lin) {
     typedef typename OutT<T>::type O;
     constexpr int NP = NP1 * NP1;
-    constexpr int EPB = EPBOf<NP1, TV>::value;
+    constexpr int EPB = 128 / NP;
     __shared__ O sg[2][EPB][4][NP];
     __shared__ T su[VISC ? EPB : 1][4][NP];
     // weak-form derivative and lift tables with the 2/h factors folded in:
@@ -359,7 +352,7 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
     __shared__ O sl[8][NP1];
     __shared__ double sce[2];   // eps and adt / eps of the FD modes: one IEEE division per block
     if ((MODE == DG_JV || MODE == DG_SMOOTH64) && threadIdx.x == 0) {
-        const double e0 = *A.eps;
+        const double e0 = A.eps ? *A.eps : A.eps_val;
         sce[0] = e0;
         sce[1] = e0 != 0.0 ? A.adt / e0 : 0.0;
     }
@@ -379,8 +372,9 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
     const int le = threadIdx.x / NP;
     const int node = threadIdx.x % NP;
     const int a = node % NP1, b = node / NP1;
-    const int e = (int)blk * EPB + le;
-    const bool active = (le < EPB) && (e < K.n_el);
+    const int epb = blockDim.x / NP;
+    const int e = (int)blk * epb + le;
+    const bool active = (le < epb) && (e < K.n_el);
     const int nx = K.nx, nz = K.nz;
     const int ez = active ? e / nx : 0, ex = active ? e % nx : 0;
     const size_t N1 = (size_t)K.n_el * NP;
@@ -423,6 +417,17 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
         const T u = U[1] * ir, w = U[2] * ir;
         T Fx[4], Fz[4];
         flux_xz(U, u, w, p, Fx, Fz);
+        const size_t gl = (size_t)e * NP + node;
+        if constexpr (IN == 0) {
+            if (lin.tr) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) lin.U[v * N1 + gl] = outv(U[v]);
+#pragma unroll
+                for (int v = 1; v < 4; ++v) lin.F[(v - 1) * N1 + gl] = outv(Fx[v]);
+                lin.F[3 * N1 + gl] = outv(Fz[2]);
+                lin.F[4 * N1 + gl] = outv(Fz[3]);
+            }
+        }
         if (IN != 2) {   // minus the background's fluxes; the mass fluxes are linear
             Fx[0] = Up[1];
             Fz[0] = Up[2];
@@ -449,8 +454,24 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
             const T phi[4] = {u, u, w, U[3] * ir};
 #pragma unroll
             for (int v = 1; v < 4; ++v) {
-                Fx[v] = Fx[v] - mu * visc_c(phi[v], dx[0], dx[v]);
-                Fz[v] = Fz[v] - mu * visc_c(phi[v], dz[0], dz[v]);
+                const T gx = mu * visc_c(phi[v], dx[0], dx[v]), gz = mu * visc_c(phi[v], dz[0], dz[v]);
+                Fx[v] = Fx[v] - gx;
+                Fz[v] = Fz[v] - gz;
+                if constexpr (IN == 0) {
+                    if (lin.tr) {
+                        lin.F[(12 + v) * N1 + gl] = outv(gx);
+                        lin.F[(15 + v) * N1 + gl] = outv(gz);
+                    }
+                }
+            }
+            if constexpr (IN == 0) {
+                if (lin.tr) {
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        lin.F[(5 + v) * N1 + gl] = outv(dx[v]);
+                        lin.F[(9 + v) * N1 + gl] = outv(dz[v]);
+                    }
+                }
             }
         }
 #pragma unroll
@@ -521,7 +542,7 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
     }
 }
 
-template <class T, int IN, int MODE, int NP1, bool VISC, int TV>
+template <class T, int IN, int MODE, int NP1, bool VISC>
 struct k_volume_b {
     static constexpr int TPB = 128, MINB = 8;
     static constexpr bool GROUP = !VISC && std::is_same<T, D64>::value && MODE != DG_SMOOTH64;   // a grouped twin is built (lock-step ensembles)
@@ -530,18 +551,18 @@ struct k_volume_b {
                                                JfArg<const typename OutT<T>::type *> phix,
                                                JfArg<const typename OutT<T>::type *> symx,
                                                JfArg<const typename OutT<T>::type *> phiz,
-                                               JfArg<const typename OutT<T>::type *> symz) {
+                                               JfArg<const typename OutT<T>::type *> symz, JfArg<LinPtr> lin) {
         jf_pdl_enter();
-        volume_body<T, IN, MODE, NP1, VISC, TV>(K, ld0, A, phix, symx, phiz, symz, jf_bid);
+        volume_body<T, IN, MODE, NP1, VISC>(K, ld0, A, phix, symx, phiz, symz, jf_bid, lin);
     }
 };
-template <class T, int IN, int MODE, int NP1, bool VISC, int TV>
+template <class T, int IN, int MODE, int NP1, bool VISC>
 __global__ void __launch_bounds__(128, 8) k_volume(DGK K, Loader<T, IN> ld0, DGArgs A,
                                                    const typename OutT<T>::type *phix,
                                                    const typename OutT<T>::type *symx,
                                                    const typename OutT<T>::type *phiz,
-                                                   const typename OutT<T>::type *symz) {
-    k_volume_b<T, IN, MODE, NP1, VISC, TV>::run(blockIdx.x, gridDim.x, K, ld0, A, phix, symx, phiz, symz);
+                                                   const typename OutT<T>::type *symz, LinPtr lin) {
+    k_volume_b<T, IN, MODE, NP1, VISC>::run(blockIdx.x, gridDim.x, K, ld0, A, phix, symx, phiz, symz, lin);
 }
 
 // ---------------------------------------------------------------------------
@@ -786,8 +807,7 @@ struct k_dgtl_b {
                         const TL32 Jv = trL[v] - trR[v];
                         sLv[q] = hmu * visc_c(pL, J0, Jv);
                         sRv[q] = hmu * visc_c(pR, J0, Jv);
-                        Phi[v] = Phi[v] - hmu * (visc_c(pL, gL[0], gL[v]) + visc_c(pR, gR[0], gR[v])) +
-                                 TLc{K.eta_xf} * (sLv[q] + sRv[q]);
+                        Phi[v] = Phi[v] - visc_face(hmu, TLc{K.eta_xf}, pL, pR, gL, gR, v, sLv[q], sRv[q]);
                     }
                 } else {
     #pragma unroll
@@ -845,8 +865,7 @@ struct k_dgtl_b {
                         const TL32 Jv = trL[v] - trR[v];
                         sLv[q] = hmu * visc_c(pL, J0, Jv);
                         sRv[q] = hmu * visc_c(pR, J0, Jv);
-                        Phi[v] = Phi[v] - hmu * (visc_c(pL, gB[0], gB[v]) + visc_c(pR, gT[0], gT[v])) +
-                                 TLc{K.eta_zf} * (sLv[q] + sRv[q]);
+                        Phi[v] = Phi[v] - visc_face(hmu, TLc{K.eta_zf}, pL, pR, gB, gT, v, sLv[q], sRv[q]);
                     }
                 } else {
     #pragma unroll
@@ -981,28 +1000,35 @@ DGK make_K(jfnk_ctx *c) {
     K.dubvf = c->dubvf;
     K.ubhf = c->ubhf;
     K.dubhf = c->dubhf;
-    K.tab = c->tab;
+    K.tab.np1 = c->np1;
+    for (int q = 0; q < 5; ++q) {
+        K.tab.lp[q] = c->tab.lp[q];
+        K.tab.lm[q] = c->tab.lm[q];
+        K.tab.dlp[q] = c->tab.dlp[q];
+        K.tab.dlm[q] = c->tab.dlm[q];
+        for (int r = 0; r < 5; ++r) K.tab.Dn[r][q] = c->tab.Dn[r][q];
+    }
     K.two_hxf = (float)K.two_hx;
     K.two_hzf = (float)K.two_hz;
     K.eta_xf = (float)K.eta_x;
     K.eta_zf = (float)K.eta_z;
     for (int r = 0; r < 5; ++r)
         for (int q = 0; q < 5; ++q) {
-            K.Dx[r][q] = K.two_hx * K.tab.Dw[r][q];
-            K.Dz[r][q] = K.two_hz * K.tab.Dw[r][q];
+            K.Dx[r][q] = K.two_hx * c->tab.Dw[r][q];
+            K.Dz[r][q] = K.two_hz * c->tab.Dw[r][q];
             K.Dxf[r][q] = (float)K.Dx[r][q];
             K.Dzf[r][q] = (float)K.Dz[r][q];
             K.Dnf[r][q] = (float)K.tab.Dn[r][q];
         }
     for (int q = 0; q < 5; ++q) {
-        K.lift[0][q] = K.two_hx * K.tab.lmw[q];
-        K.lift[1][q] = K.two_hx * K.tab.lpw[q];
-        K.lift[2][q] = K.two_hx * K.two_hx * K.tab.dlmw[q];
-        K.lift[3][q] = K.two_hx * K.two_hx * K.tab.dlpw[q];
-        K.lift[4][q] = K.two_hz * K.tab.lmw[q];
-        K.lift[5][q] = K.two_hz * K.tab.lpw[q];
-        K.lift[6][q] = K.two_hz * K.two_hz * K.tab.dlmw[q];
-        K.lift[7][q] = K.two_hz * K.two_hz * K.tab.dlpw[q];
+        K.lift[0][q] = K.two_hx * c->tab.lmw[q];
+        K.lift[1][q] = K.two_hx * c->tab.lpw[q];
+        K.lift[2][q] = K.two_hx * K.two_hx * c->tab.dlmw[q];
+        K.lift[3][q] = K.two_hx * K.two_hx * c->tab.dlpw[q];
+        K.lift[4][q] = K.two_hz * c->tab.lmw[q];
+        K.lift[5][q] = K.two_hz * c->tab.lpw[q];
+        K.lift[6][q] = K.two_hz * K.two_hz * c->tab.dlmw[q];
+        K.lift[7][q] = K.two_hz * K.two_hz * c->tab.dlpw[q];
         for (int r = 0; r < 8; ++r) K.liftf[r][q] = (float)K.lift[r][q];
     }
     for (int a = 0; a < 5; ++a) {
@@ -1013,6 +1039,21 @@ DGK make_K(jfnk_ctx *c) {
     }
     return K;
 }
+
+// adds the two launches' times of a timed evaluation (jfnk_time_operator)
+int timing_close(jfnk_ctx *c, cudaStream_t s) {
+    if (!c->timing) return JFNK_OK;
+    JF_CK(cudaEventRecord(c->tev[2], s));
+    JF_CK(cudaEventSynchronize(c->tev[2]));
+    float m0 = 0.f, m1 = 0.f;
+    JF_CK(cudaEventElapsedTime(&m0, c->tev[0], c->tev[1]));
+    JF_CK(cudaEventElapsedTime(&m1, c->tev[1], c->tev[2]));
+    c->t_faces_ms += m0;
+    c->t_volume_ms += m1;
+    return JFNK_OK;
+}
+
+#include "dg_fd.cuh"
 
 template <class T, int IN, int MODE, int NP1, bool VISC>
 int launch(jfnk_ctx *c, const DGK &K, const Loader<T, IN> &ld, const DGArgs &a, cudaStream_t s) {
@@ -1031,31 +1072,16 @@ int launch(jfnk_ctx *c, const DGK &K, const Loader<T, IN> &ld, const DGArgs &a, 
     }
     const long long nf = (long long)K.nz * (K.nx + 1) * NP1 + (long long)(K.nz + 1) * K.nx * NP1;
     if (c->timing) JF_CK(cudaEventRecord(c->tev[0], s));
-    const int tf = c->opts.tile_faces;
+    const LinPtr lin = IN == 0 && a.lin_out ? c->lin : LinPtr{};
+    const int tf = spread_threads(c->opts.tile_faces, (size_t)nf, c->n_sm);
     jf_launch<k_faces_b<T, IN, NP1, VISC>>(k_faces<T, IN, NP1, VISC>, (unsigned)((nf + tf - 1) / tf), tf, 0, s, K, ld, phix, symx, phiz, symz,
-              a.tr_out, a.tr_in); jf_launched();
+              lin); jf_launched();
     if (c->timing) JF_CK(cudaEventRecord(c->tev[1], s));
-    if (c->opts.tile_volume == 1) {
-        constexpr int EPB = EPBOf<NP1, 1>::value;
-        const int nb = (K.n_el + EPB - 1) / EPB;
-        jf_launch<k_volume_b<T, IN, MODE, NP1, VISC, 1>>(k_volume<T, IN, MODE, NP1, VISC, 1>, nb, EPB * NP1 * NP1, 0, s, K, ld, a, phix, symx, phiz, symz);
-    } else {
-        constexpr int EPB = EPBOf<NP1, 2>::value;
-        const int nb = (K.n_el + EPB - 1) / EPB;
-        jf_launch<k_volume_b<T, IN, MODE, NP1, VISC, 2>>(k_volume<T, IN, MODE, NP1, VISC, 2>, nb, EPB * NP1 * NP1, 0, s, K, ld, a, phix, symx, phiz, symz);
-    }
+    const int epb = spread_elements<NP1>(c->opts.tile_volume, K.n_el, c->n_sm);
+    jf_launch<k_volume_b<T, IN, MODE, NP1, VISC>>(k_volume<T, IN, MODE, NP1, VISC>, (unsigned)((K.n_el + epb - 1) / epb), epb * NP1 * NP1, 0, s, K, ld, a, phix, symx, phiz, symz, lin);
     jf_launched();
     JF_CK(cudaGetLastError());
-    if (c->timing) {
-        JF_CK(cudaEventRecord(c->tev[2], s));
-        JF_CK(cudaEventSynchronize(c->tev[2]));
-        float m0 = 0.f, m1 = 0.f;
-        JF_CK(cudaEventElapsedTime(&m0, c->tev[0], c->tev[1]));
-        JF_CK(cudaEventElapsedTime(&m1, c->tev[1], c->tev[2]));
-        c->t_faces_ms += m0;
-        c->t_volume_ms += m1;
-    }
-    return JFNK_OK;
+    return timing_close(c, s);
 }
 
 // FP32 tangent modes: one fused launch (k_dgtl); a.first1 selects the defect at
@@ -1089,9 +1115,13 @@ int dispatch_mode(jfnk_ctx *c, int mode, const DGArgs &a, cudaStream_t s) {
     switch (mode) {
         case DG_RES: return launch<D64, 0, DG_RES, NP1, VISC>(c, K, Loader<D64, 0>{a.U}, a, s);
         case DG_G: return launch<D64, 0, DG_G, NP1, VISC>(c, K, Loader<D64, 0>{a.U}, a, s);
-        case DG_JV: return launch<D64, 1, DG_JV, NP1, VISC>(c, K, Loader<D64, 1>{a.U, a.y, a.eps, 0.0}, a, s);
+        case DG_JV:
+            if (a.lin && a.yf) return launch_fd<float, DG_JV, NP1, VISC>(c, a, a.yf, s);
+            if (a.lin) return launch_fd<double, DG_JV, NP1, VISC>(c, a, a.y, s);
+            return launch<D64, 1, DG_JV, NP1, VISC>(c, K, Loader<D64, 1>{a.U, a.y, a.eps, a.eps_val}, a, s);
         case DG_SMOOTH64:
-            return launch<D64, 1, DG_SMOOTH64, NP1, VISC>(c, K, Loader<D64, 1>{a.U, a.y, a.eps, 0.0}, a, s);
+            if (a.lin) return launch_fd<double, DG_SMOOTH64, NP1, VISC>(c, a, a.y, s);
+            return launch<D64, 1, DG_SMOOTH64, NP1, VISC>(c, K, Loader<D64, 1>{a.U, a.y, a.eps, a.eps_val}, a, s);
         case DG_TLJV:
             if (c->opts.dg_fused == 2 && !a.out1f)
                 return launch<TL32, 2, DG_TLJV, NP1, VISC>(c, K, Loader<TL32, 2>{a.Uf, a.yf}, a, s);
@@ -1123,7 +1153,7 @@ __global__ void __launch_bounds__(256, VISC ? 2 : 4) k_faces_grp(const DGMember 
     int m = 0;
     while (m + 1 < nm && blockIdx.x >= mem[m + 1].fb0) ++m;   // members in block order
     const DGMember &M = mem[m];
-    faces_body<D64, 0, NP1, VISC>(M.K, M.ld, M.phix, M.symx, M.phiz, M.symz, blockIdx.x - M.fb0, nullptr, nullptr);
+    faces_body<D64, 0, NP1, VISC>(M.K, M.ld, M.phix, M.symx, M.phiz, M.symz, blockIdx.x - M.fb0, LinPtr{});
 }
 
 template <int NP1, bool VISC>
@@ -1132,7 +1162,7 @@ __global__ void __launch_bounds__(128, 8) k_volume_grp(const DGMember *mem, int 
     int m = 0;
     while (m + 1 < nm && blockIdx.x >= mem[m + 1].vb0) ++m;
     const DGMember &M = mem[m];
-    volume_body<D64, 0, DG_RES, NP1, VISC, 2>(M.K, M.ld, M.A, M.phix, M.symx, M.phiz, M.symz, blockIdx.x - M.vb0);
+    volume_body<D64, 0, DG_RES, NP1, VISC>(M.K, M.ld, M.A, M.phix, M.symx, M.phiz, M.symz, blockIdx.x - M.vb0, LinPtr{});
 }
 
 template <int NP1, bool VISC>
@@ -1140,7 +1170,7 @@ void launch_grp(const DGMember *dmem, const std::vector<DGMember> &h, int first,
     const DGMember &last = h[first + cnt - 1];
     const long long nfl = (long long)last.K.nz * (last.K.nx + 1) * NP1 + (long long)(last.K.nz + 1) * last.K.nx * NP1;
     const unsigned fb = last.fb0 + (unsigned)((nfl + GRP_FACE_THREADS - 1) / GRP_FACE_THREADS);
-    constexpr int EPB = EPBOf<NP1, 2>::value;
+    constexpr int EPB = 128 / (NP1 * NP1);
     const unsigned vb = last.vb0 + (unsigned)((last.K.n_el + EPB - 1) / EPB);
     jf_launch_now(k_faces_grp<NP1, VISC>, fb, GRP_FACE_THREADS, 0, s, dmem + first, cnt);
     jf_launch_now(k_volume_grp<NP1, VISC>, vb, EPB * NP1 * NP1, 0, s, dmem + first, cnt);
@@ -1187,8 +1217,9 @@ int dg_apply(jfnk_ctx *c, int mode, const DGArgs &a_in, cudaStream_t s) {
     a.adtf = (float)a.adt;
     a.alphaf = (float)a.alpha;
     c->dg_calls++;
-    // the stored traces belong to the cached f(U): any other writer of the cache drops them
-    if (a.out0 == c->fU || a.out1 == c->fU) c->tr_valid = a.tr_out == c->trU ? 1 : 0;
+    // the linearisation belongs to the cached f(U): any other writer of the cache drops it
+    if (a.out0 == c->fU || a.out1 == c->fU) c->lin_valid = a.lin_out;
+    if (a.lin && !c->lin_valid) return JFNK_EINVAL;
     switch (c->np1) {
         case 2: return dg_dispatch<2>(c, mode, a, s);
         case 3: return dg_dispatch<3>(c, mode, a, s);

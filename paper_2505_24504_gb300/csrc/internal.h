@@ -211,6 +211,16 @@ struct FVLev {
     uint16_t *xb, *bb;   // bf16 storage of x and b on the coarsest level (prec 16)
 };
 
+// Linearisation of the DG operator at a state U, written by the residual at U and read by
+// the finite-difference products about it (per face point: state traces of both sides,
+// normal derivatives and jumps when viscous; fluxes; per node: state, fluxes, gradients).
+struct LinPtr {
+    double *tr;   // [8, or 20 viscous][face points]
+    double *H;    // [4, or 13][face points]: HLLC flux, viscous part, symmetry terms
+    double *U;    // [4][nodes]
+    double *F;    // [5, or 19][nodes]: F_x (1..3), F_z (2, 3); gradients and viscous fluxes
+};
+
 struct jfnk_ctx {
     jfnk_grid grid;
     int k, np1, n_el;
@@ -250,8 +260,8 @@ struct jfnk_ctx {
     FVLev lev[JF_MAXLEV];
     // reductions
     double *partial;     // scratch partial sums
-    double *trU;         // face traces of the Newton iterate (values, and derivatives when viscous)
-    int tr_valid;        // trU and fU come from the same residual evaluation
+    LinPtr lin;          // linearisation of the DG operator at the state of the last residual
+    int lin_valid;       // lin and fU come from the same residual evaluation
     unsigned *ticket;    // arrival counter of the single-launch reductions (0 between launches)
     int nb_red;          // partial-sum blocks
     int n_sm;            // streaming multiprocessors of the context's device
@@ -291,7 +301,7 @@ struct jfnk_ctx {
 };
 
 // device scalar slots in ctx->scal
-enum { S_NORM = 0, S_EPS = 1, S_W1 = 2, S_FLAG = 3, S_INV = 4, S_EPSDG = 5, S_EPSFV = 8, S_NRM_FV = 24, S_H = 64, S_H2 = 128, S_COUNT = 256 };
+enum { S_NORM = 0, S_EPS = 1, S_W1 = 2, S_FLAG = 3, S_INV = 4, S_EPSDG = 5, S_CEPS = 6, S_EPSFV = 8, S_NRM_FV = 24, S_H = 64, S_H2 = 128, S_COUNT = 256 };
 
 // number of kernels this library has launched (diagnostic counter); the
 // thread-local twin lets a graph capture count only its own thread's launches
@@ -347,7 +357,7 @@ struct DGArgs {
     const double *r;       // FP64 right-hand side (SMOOTH64)
     const float *rf;       // FP32 right-hand side (TLSMOOTH)
     const double *Ubs;     // Ubar_s (G)
-    const double *eps;     // device scalar eps (JV, SMOOTH64)
+    const double *eps;     // device scalar eps (JV, SMOOTH64); null: eps_val
     const double *dtau;    // [n_el] (smoothing)
     const float *dtauf;    // [n_el] (FP32 smoothing)
     double adt;
@@ -355,8 +365,9 @@ struct DGArgs {
     float alphaf;
     void *out0;
     double *out1;
-    double *tr_out;        // FP64 residual / G: store the face traces of U here (may be null)
-    const double *tr_in;   // FP64 FD product: face traces of U from the residual at U (may be null)
+    double eps_val;        // eps of a FD product when the device scalar is null
+    int lin_out;           // FP64 residual / G: store the context's linearisation at U
+    int lin;               // FD product about the stored linearisation (direction yf, else y)
     float *out1f;          // FP32 defect at the first step from zero: z = dtau r is formed from rf and
                            // dtauf on the fly (yf unused) and written here
     const TransferOut *tro;   // with out1f: also T^mf of the defect to the finest FV level (host struct,
@@ -394,13 +405,32 @@ constexpr int GS_FUSED_MAX = 16;   // basis vectors of the fused CGS2 kernels
 int blas_cgs2(jfnk_ctx *c, const double *V, const float *V32, int nv, size_t ldv, double *w, float *w32, size_t n,
               double *h1, double *h2, double *w1sq, double *nrm, double *flag, cudaStream_t s);
 int blas_time_cgs2(jfnk_ctx *c, int reps, double *ms, cudaStream_t s);
-int blas_f2d_eps(jfnk_ctx *c, const float *x, double *y, size_t n, double *eps_out, cudaStream_t s);
+int blas_eps32(jfnk_ctx *c, const float *x, size_t n, double *eps_out, cudaStream_t s);
 int blas_scale_copy(const double *w, const double *nrm_dev, double *v, size_t n, cudaStream_t s);
 int blas_axpby(double a, const double *x, double b, const double *y, double *z, size_t n, cudaStream_t s);
 int blas_zcomb(const void *Z, int prec32, int nz, size_t n, const double *yv, double *x, cudaStream_t s);
 int blas_copy_d2f(const double *x, float *y, size_t n, cudaStream_t s);
 int blas_copy_f2d(const float *x, double *y, size_t n, cudaStream_t s);
 int blas_scale(double a, const double *x, double *y, size_t n, cudaStream_t s);
+
+// Launch shapes: a kernel whose blocks do not cooperate takes smaller blocks when the
+// tuned ones leave SMs without work (one SM runs an FP64 warp instruction every 19
+// clocks, so on small grids the work per SM, not the number of warps, sets the time).
+// Recorded launches (lock-step ensembles) keep the tuned shape, which members share.
+inline int spread_threads(int tile, size_t n, int n_sm) {
+    if (t_jf_rec) return tile;
+    while (tile > 32 && n < (size_t)tile * 2 * n_sm) tile /= 2;
+    return tile;
+}
+template <int NP1>
+inline int spread_elements(int tile_volume, int n_el, int n_sm) {
+    constexpr int NP = NP1 * NP1;
+    auto fit = [](int threads) { return threads / NP > 0 ? threads / NP : 1; };
+    int t = tile_volume == 2 ? 128 : 64;
+    if (!t_jf_rec)
+        while (t > 32 && n_el < fit(t) * 2 * n_sm) t /= 2;
+    return fit(t);
+}
 
 // preconditioner (mg.cu)
 int mg_linearize(jfnk_ctx *c, const double *U, double adt, cudaStream_t s);

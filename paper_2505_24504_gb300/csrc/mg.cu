@@ -1418,6 +1418,10 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
     return JFNK_OK;
 }
 
+// FP64 DG products about the linearisation the last residual stored (the state the
+// preconditioner is linearised at); a given numerator of eps takes the general form
+inline int fd_lin(const jfnk_ctx *c) { return c->opts.precond_fd_eps == 0.0; }
+
 template <class S>
 int dg_smooth_step(jfnk_ctx *c, const S *r, S *&z, S *&z2, bool &zero, cudaStream_t s);
 
@@ -1440,6 +1444,7 @@ int dg_smooth_step<double>(jfnk_ctx *c, const double *r, double *&z, double *&z2
     a.dtau = c->dtau_dg;
     a.adt = c->mg_adt;
     a.out0 = z2;
+    a.lin = fd_lin(c);
     JF_RET(dg_apply(c, DG_SMOOTH64, a, s));
     double *t = z;
     z = z2;
@@ -1485,6 +1490,7 @@ int dg_defect<double>(jfnk_ctx *c, const double *r, const double *z, double *d, 
     a.eps = c->scal + S_EPSDG;
     a.adt = c->mg_adt;
     a.out0 = c->w2;
+    a.lin = fd_lin(c);
     JF_RET(dg_apply(c, DG_JV, a, s));
     jf_launch<k_sub_b<double>>(k_sub<double>, nblk(c->N, 256), 256, 0, s, r, c->w2, d, c->N); jf_launched();
     JF_CK(cudaGetLastError());
@@ -1551,6 +1557,7 @@ int dg_rk_step(jfnk_ctx *c, const S *r, S *&z, S *&z2, S *&z3, bool &zero, cudaS
                 A.r = (const double *)r;
                 A.eps = c->scal + S_EPSDG;
                 A.dtau = c->dtau_dg;
+                A.lin = fd_lin(c);
                 JF_RET(dg_apply(c, DG_SMOOTH64, A, s));
             } else {
                 A.Uf = c->Usf;

@@ -72,42 +72,46 @@ JF_D void mirror_side(const Side<T> &A, Side<T> &G) {
 // the branch selects is evaluated.
 // With q_K = rho_K (S_K - u_K) the star flux is, identically, the flux of the star state
 // through the contact: mass M = rho* S*, normal momentum M S* + p_K + q_K (S* - u_K),
-// tangential momentum M v_t, M theta.  In this form nothing large cancels (F_K and
-// S_K (U*_K - U_K) do in the other) and a wall (S* = 0) gets exactly no mass flux; it
-// takes half the operations: the whole flux about 57 FP64 instructions instead of 119.
+// tangential momentum M v_t, M theta.  All speeds are taken relative to the sides, with
+// d = u_R - u_L: S_L - u_L = min(-c_L, d - c_R), S_R - u_R = max(c_L - d, c_R),
+// S* - u_L = ((p_R - p_L) - d q_R) / (q_L - q_R).  In this form nothing large cancels
+// (F_K and S_K (U*_K - U_K) do in the textbook one), and the whole flux takes about 51
+// FP64 instructions instead of 119.
 // With the quotients, roots and powers of numeric.cuh the FP64 residual's face kernel
-// fell from 48.6 to 29.9 us on 103,360 Q3 face points, from 46.9 to 26.6 us on the
-// 50,016 viscous Q2 ones, and from 26 to 16 us where one SM's latency chain sets the
+// fell from 48.6 to 28.0 us on 103,360 Q3 face points, from 46.9 to 26.0 us on the
+// 50,016 viscous Q2 ones, and from 26 to 15 us where one SM's latency chain sets the
 // time (20 x 10 elements, Q2).
 template <class T, int D>
 JF_D void hllc_s(const Side<T> &L, const Side<T> &R, T H[4]) {
     constexpr int iN = 1 + D, iT = 2 - D;
     const T uL = L.U[iN] * L.ir, uR = R.U[iN] * R.ir;
-    const T a1 = uL - L.c, a2 = uR - R.c;
-    const T SL = sel(le(a1, a2), a1, a2);
-    const T b1 = uL + L.c, b2 = uR + R.c;
-    const T SR = sel(le(b2, b1), b1, b2);
-    const T qL = L.U[0] * (SL - uL), qR = R.U[0] * (SR - uR);
-    const T Sst = ((R.p - L.p) + (uL * qL - uR * qR)) / (qL - qR);
-    const bool sl = nonneg(SL);
+    const T d = uR - uL;
+    const T x = d - R.c, y = L.c - d;
+    const T dL = sel(le(-L.c, x), -L.c, x);   // S_L - u_L
+    const T dR = sel(le(R.c, y), y, R.c);     // S_R - u_R
+    const T qL = L.U[0] * dL, qR = R.U[0] * dR;
+    const T sL = jfma(-d, qR, R.p - L.p) / (qL - qR);   // S* - u_L
+    const T Sst = uL + sL;
+    const bool sl = le(-dL, uL);              // 0 <= S_L
     const bool left = nonneg(Sst) || sl;
-    const bool pure = sl || (!left && !nonneg(SR));
-    const T un = sel(left, uL, uR), ir = sel(left, L.ir, R.ir), p = sel(left, L.p, R.p);
+    const bool pure = sl || (!left && !le(-dR, uR));
+    const T ir = sel(left, L.ir, R.ir), p = sel(left, L.p, R.p);
     const T Ut = sel(left, L.U[iT], R.U[iT]), U3 = sel(left, L.U[3], R.U[3]);
     if (pure) {
-        const T Un = sel(left, L.U[iN], R.U[iN]);
+        const T Un = sel(left, L.U[iN], R.U[iN]), un = sel(left, uL, uR);
         H[0] = Un;
         H[iN] = jfma(Un, un, p);
         H[iT] = Ut * un;
         H[3] = U3 * un;
         return;
     }
-    const T S = sel(left, SL, SR), q = sel(left, qL, qR);
-    const T M = q / (S - Sst) * Sst;
+    const T q = sel(left, qL, qR), s = sel(left, sL, sL - d);   // s = S* - u_K
+    const T M = q / (sel(left, dL, dR) - s) * Sst;
+    const T Mi = M * ir;
     H[0] = M;
-    H[iN] = jfma(M, Sst, jfma(q, Sst - un, p));
-    H[iT] = M * (Ut * ir);
-    H[3] = M * (U3 * ir);
+    H[iN] = jfma(M, Sst, jfma(q, s, p));
+    H[iT] = Mi * Ut;
+    H[3] = Mi * U3;
 }
 
 template <class T, int D>
@@ -140,6 +144,14 @@ JF_D void wall_states(T UL[4], T UR[4], bool wallL, bool wallR) {
 // v = 1, 2, 3 from phi = U_v / rho.
 template <class T>
 JF_D T visc_c(T phi, T dU0, T dUv) { return jfma(-phi, dU0, dUv); }
+
+// Viscous part V of a face's term Phi = H - V, component v: the mean of the two sides'
+// viscous fluxes (hmu = mu / 2, phi = U_v / rho, g the normal derivatives) less the
+// interior penalty eta {A(U)} [U] on the jumps of u, w, theta (sL, sR = 1/2 A(U_side) [U]).
+template <class T, class C, class E>
+JF_D T visc_face(C hmu, E eta, T pL, T pR, const T gL[4], const T gR[4], int v, T sL, T sR) {
+    return hmu * (visc_c(pL, gL[0], gL[v]) + visc_c(pR, gR[0], gR[v])) - eta * (sL + sR);
+}
 
 // |v . e_D| + c for pseudo-time step sizes (plain double, not on the residual path).
 JF_D double wave_speed(const double U[4], int D, const PhysC &P, const PowTab *pt) {

@@ -53,30 +53,21 @@ struct Phases {
     }
 };
 
-// z_j of the flexible basis as an FP64 pointer; FP32 storage is converted and
-// eps of the FD product computed in the same pass (*eps_ready = true)
-const double *z_as_double(jfnk_ctx *c, int j, double *tmp, cudaStream_t s, int *rc, bool *eps_ready) {
-    *rc = JFNK_OK;
-    *eps_ready = false;
-    if (c->prec == 64 || !c->mg_on) return (const double *)c->Z + (size_t)j * c->N;
-    *rc = blas_f2d_eps(c, (const float *)c->Z + (size_t)j * c->N, tmp, c->N, c->scal + S_EPS, s);
-    *eps_ready = true;
-    return tmp;
-}
-
-// w = G'(U) y with eps = sqrt(eps_mach)/|y| computed on the device (skipped
-// when the caller already wrote eps to S_EPS)
-int apply_jv(jfnk_ctx *c, const double *U, double adt, const double *y, double *w, cudaStream_t s,
-             bool eps_ready = false) {
-    if (!eps_ready) JF_RET(red_dot(c, y, y, c->N, c->scal + S_EPS, RED_EPS, s));
+// w = G'(U) y about the linearisation of the last residual (U is its state), with
+// eps = sqrt(eps_mach)/|y| computed on the device; y in FP64, or in FP32 (yf) as the FP32
+// preconditioner writes it
+int apply_jv(jfnk_ctx *c, const double *U, double adt, const double *y, const float *yf, double *w, cudaStream_t s) {
+    if (yf) JF_RET(blas_eps32(c, yf, c->N, c->scal + S_EPS, s));
+    else JF_RET(red_dot(c, y, y, c->N, c->scal + S_EPS, RED_EPS, s));
     DGArgs a = {};
     a.U = U;
     a.y = y;
+    a.yf = yf;
     a.fU = c->fU;
     a.eps = c->scal + S_EPS;
     a.adt = adt;
     a.out0 = w;
-    a.tr_in = c->tr_valid ? c->trU : nullptr;   // U is the iterate of the last residual
+    a.lin = 1;
     return dg_apply(c, DG_JV, a, s);
 }
 
@@ -96,7 +87,6 @@ int arnoldi_step_work(jfnk_ctx *c, const double *U, double adt, int j, cudaStrea
     const size_t N = c->N;
     double *V = c->V;
     double *vj = V + (size_t)j * N, *w = V + (size_t)(j + 1) * N;
-    int rc;
     if (ph) ph->mark(0, s);
     if (c->mg_on) {
         JF_RET(mg_apply(c, vj, (char *)c->Z + (size_t)j * N * (c->prec == 64 ? 8 : 4), s,
@@ -104,11 +94,9 @@ int arnoldi_step_work(jfnk_ctx *c, const double *U, double adt, int j, cudaStrea
     } else {
         JF_CK(jf_memcpy((double *)c->Z + (size_t)j * N, vj, 8 * N, cudaMemcpyDeviceToDevice, s));
     }
-    bool eps_ready = false;
-    const double *zj = z_as_double(c, j, c->w1, s, &rc, &eps_ready);
-    JF_RET(rc);
     if (ph) ph->mark(1, s);
-    JF_RET(apply_jv(c, U, adt, zj, w, s, eps_ready));
+    if (c->prec == 64 || !c->mg_on) JF_RET(apply_jv(c, U, adt, (const double *)c->Z + (size_t)j * N, nullptr, w, s));
+    else JF_RET(apply_jv(c, U, adt, nullptr, (const float *)c->Z + (size_t)j * N, w, s));
     if (ph) ph->mark(2, s);
     // classical Gram-Schmidt; the update kernel also reduces |w|^2, and a
     // second pass runs only when the first lost more than half of |w|
@@ -257,7 +245,7 @@ int fgmres(jfnk_ctx *c, const double *U, double adt, const double *b, double *x,
         if (conv) return JFNK_OK;
         if (*its >= maxit) return JFNK_ENOTCONV;
         // restart from the true residual r = b - G'x
-        JF_RET(apply_jv(c, U, adt, x, c->w2, s));
+        JF_RET(apply_jv(c, U, adt, x, nullptr, c->w2, s));
         JF_RET(blas_axpby(1.0, b, -1.0, c->w2, c->w2, N, s));
         r = c->w2;
         JF_RET(read_norm(c, r, &beta, s));
@@ -275,7 +263,7 @@ int eval_G(jfnk_ctx *c, const double *U, double adt, double *nrm, cudaStream_t s
     a.adt = adt;
     a.out0 = c->G;
     a.out1 = c->fU;
-    a.tr_out = c->trU;   // the FD products of this Newton iterate reuse its face traces
+    a.lin_out = 1;   // the FD products of this Newton iterate are taken about it
     JF_RET(dg_apply(c, DG_G, a, s));
     return read_norm(c, c->G, nrm, s);
 }
