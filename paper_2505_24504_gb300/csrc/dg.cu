@@ -1,18 +1,17 @@
 // DG operator f = M^-1 L_h(U') on the GPU (Sec. 2.1; well-balanced form of Sec. 4).
 //
 // Two launches per evaluation:
-//  k_faces   one thread per face point.  Traces of U' from both sides (and the
-//            normal-gradient traces for the viscous terms), HLLC^pert =
-//            HLLC(U'+Ubar) - HLLC(Ubar), symmetric interior penalty terms, slip
-//            walls by a mirrored ghost.  Every face flux is computed once and
-//            stored: Phi = H - {F_v.n} + eta [U] for the lift with l_a(+-1), and
-//            the two symmetry terms 1/2 A(U_side) [U] for the lift with l_a'(+-1).
-//  k_volume  a block holds EPB elements, one thread per node.  Fluxes
-//            F_c^pert - F_v at the node, the weak-form derivative by sum
-//            factorisation over the (k+1) nodes of the row / column (tables in
-//            shared memory), gravity source, lift of the stored face terms and
-//            the mode's epilogue (residual, FD product, Newton residual G or a
-//            pseudo-time smoothing step).
+//  k_dg_flux the first blocks take the face points, one thread each: traces of U' from
+//            both sides (and the normal-gradient traces for the viscous terms),
+//            HLLC^pert = HLLC(U'+Ubar) - HLLC(Ubar), symmetric interior penalty terms,
+//            slip walls by a mirrored ghost.  Every face flux is computed once and
+//            stored: Phi = H - {F_v.n} + eta [U] for the lift with l_a(+-1), and the two
+//            symmetry terms 1/2 A(U_side) [U] for the lift with l_a'(+-1).  The other
+//            blocks hold some elements each, one thread per node: fluxes F_c^pert - F_v,
+//            the weak-form derivative by sum factorisation over the (k+1) nodes of the
+//            row / column (tables in shared memory), gravity source.
+//  k_dg_lift adds the lifts of the stored face terms and runs the mode's epilogue
+//            (residual, FD product, Newton residual G or a pseudo-time smoothing step).
 // The same kernels run on D64 (FP64 residual and finite-difference products)
 // and on TL32 (FP32 tangent-linear products for the FP32 preconditioner).
 #include <vector>
@@ -92,9 +91,18 @@ JF_D void line_trace(const Loader<T, IN> &ld, size_t i0, size_t st, const double
         if (VISC) d = jfma(mkc(pd[q], pdf[q], T{}), u, d);
     }
 }
-// Body of the face kernel for block `blk` of one operator evaluation; K is the
-// launch parameter (single operator) or a member's descriptor in global memory
-// (grouped launch over ensemble members).
+template <class T>
+JF_D void swap_d(bool c, T &a, T &b) {
+    const T t = a;
+    a = sel(c, b, a);
+    b = sel(c, t, b);
+}
+
+// Face terms of block `blk` of one operator evaluation, one thread per face point; K is
+// the launch parameter (single operator) or a member's descriptor in global memory
+// (grouped launch over ensemble members).  Vertical and horizontal faces run the same
+// code: the momentum components are exchanged for the latter (the same arithmetic,
+// component for component, in half the instructions and without a divergent block).
 template <class T, int IN, int NP1, bool VISC>
 __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld0, typename OutT<T>::type *phix,
                                            typename OutT<T>::type *symx, typename OutT<T>::type *phiz,
@@ -105,269 +113,142 @@ __device__ __forceinline__ void faces_body(const DGK &K, const Loader<T, IN> &ld
     constexpr int NP = NP1 * NP1;
     const int nx = K.nx, nz = K.nz;
     const size_t N1 = (size_t)K.n_el * NP;
-    const long long nvert = (long long)nz * (nx + 1) * NP1;
-    const long long nhorz = (long long)(nz + 1) * nx * NP1;
+    const long long nvert = (long long)nz * (nx + 1) * NP1, nfp = nvert + (long long)(nz + 1) * nx * NP1;
     const long long t = (long long)blk * blockDim.x + threadIdx.x;
-    if (t >= nvert + nhorz) return;
-    const size_t nfp = (size_t)(nvert + nhorz);
-    const T zero = mk(0.0, T{});
-    T H[4], Phi[4], sL[3], sR[3];
-    if (t < nvert) {
-        const int s = (int)(t % NP1);
-        const int fx = (int)((t / NP1) % (nx + 1));
-        const int ez = (int)(t / (NP1 * (nx + 1)));
-        const int J = ez * NP1 + s;
-        const size_t nrow = (size_t)nz * NP1;
-        int eL, eR;
-        bool wallL = false, wallR = false;
-        if (K.periodic) {
-            eL = ez * nx + (fx + nx - 1) % nx;
-            eR = ez * nx + fx % nx;
-        } else {
-            wallL = (fx == 0);
-            wallR = (fx == nx);
-            eL = ez * nx + (wallL ? 0 : fx - 1);
-            eR = ez * nx + (wallR ? nx - 1 : fx);
-        }
-        // traces: L at xi = +1 (row s), R at xi = -1
-        T trL[4], trR[4], gL[4], gR[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            T aL, aR, dL, dR;
-            const size_t iL0 = (size_t)v * N1 + (size_t)eL * NP + s * NP1;
-            const size_t iR0 = (size_t)v * N1 + (size_t)eR * NP + s * NP1;
-            line_trace<T, IN, NP1, VISC>(ld, iL0, 1, K.tab.lp, K.tlp, K.tab.dlp, K.tdlp, aL, dL);
-            line_trace<T, IN, NP1, VISC>(ld, iR0, 1, K.tab.lm, K.tlm, K.tab.dlm, K.tdlm, aR, dR);
-            trL[v] = aL;
-            trR[v] = aR;
-            gL[v] = mkc(K.two_hx, K.two_hxf, T{}) * dL;
-            gR[v] = mkc(K.two_hx, K.two_hxf, T{}) * dR;
-        }
-        T UL[4], UR[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            UL[v] = trL[v] + bgs(K.ubv, K.ubvf, v * nrow + J, T{});
-            UR[v] = trR[v] + bgs(K.ubv, K.ubvf, v * nrow + J, T{});
-        }
-        if constexpr (IN == 0) {
-            if (lin.tr) {
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    lin.tr[(2 * v) * nfp + t] = outv(UL[v]);
-                    lin.tr[(2 * v + 1) * nfp + t] = outv(UR[v]);
-                    if (VISC) {
-                        lin.tr[(8 + 2 * v) * nfp + t] = outv(gL[v]);
-                        lin.tr[(9 + 2 * v) * nfp + t] = outv(gR[v]);
-                        lin.tr[(16 + v) * nfp + t] = outv(trL[v] - trR[v]);
-                    }
-                }
-            }
-        }
-        wall_states<T, 0>(UL, UR, wallL, wallR);
-        Side<T> SL, SR;
-        side_of(UL, K.pc, K.pt, SL);
-        side_of(UR, K.pc, K.pt, SR);
-        hllc_s<T, 0>(SL, SR, H);
-        if constexpr (IN == 0) {
-            if (lin.tr) {
-#pragma unroll
-                for (int v = 0; v < 4; ++v) lin.H[v * nfp + t] = outv(H[v]);
-            }
-        }
-        const double *hb = wallL ? K.hbxw : (wallR ? K.hbxw + 4 * nrow : K.hbx);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            if (IN != 2) H[v] = H[v] - bg<T>(hb, v * nrow + J);
-            Phi[v] = H[v];
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) sL[c] = sR[c] = zero;
-        if (VISC && !wallL && !wallR) {
-            // interior penalty on the jumps of u, w, theta: eta {A(U)} [U]
-            const auto eta = mkc(K.eta_x, K.eta_xf, T{});
-            const auto hmu = mkc(0.5 * K.mu, 0.5f * K.pc.muf, T{});
-            const T J0 = trL[0] - trR[0];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const int v = c + 1;
-                const T pL = SL.U[v] * SL.ir, pR = SR.U[v] * SR.ir;
-                const T Jv = trL[v] - trR[v];
-                sL[c] = hmu * visc_c(pL, J0, Jv);
-                sR[c] = hmu * visc_c(pR, J0, Jv);
-                const T V = visc_face(hmu, eta, pL, pR, gL, gR, v, sL[c], sR[c]);
-                Phi[v] = Phi[v] - V;
-                if constexpr (IN == 0) {
-                    if (lin.tr) {
-                        lin.H[(4 + c) * nfp + t] = outv(V);
-                        lin.H[(7 + c) * nfp + t] = outv(sL[c]);
-                        lin.H[(10 + c) * nfp + t] = outv(sR[c]);
-                    }
-                }
-            }
-        }
-        const size_t fb = ((size_t)ez * (nx + 1) + fx) * NP1 + s;
-        const size_t fs = (size_t)nz * (nx + 1) * NP1;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) phix[v * fs + fb] = (O)outv(Phi[v]);
-        if (VISC) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                symx[(size_t)c * fs + fb] = (O)outv(sL[c]);
-                symx[(size_t)(3 + c) * fs + fb] = (O)outv(sR[c]);
-            }
-        }
+    if (t >= nfp) return;
+    const bool zf = t >= nvert;
+    const int u = (int)(zf ? t - nvert : t);
+    const int s = u % NP1, c = u / NP1;
+    int eL, eR, ib;              // elements of the two sides (L: west / below), background index
+    bool wallL, wallR;
+    if (!zf) {
+        const int fx = c % (nx + 1), ez = c / (nx + 1);
+        wallL = fx == 0 && !K.periodic;
+        wallR = fx == nx && !K.periodic;
+        eL = ez * nx + (fx == 0 ? (K.periodic ? nx - 1 : 0) : fx - 1);
+        eR = ez * nx + (fx == nx ? (K.periodic ? 0 : nx - 1) : fx);
+        ib = ez * NP1 + s;
     } else {
-        const long long u = t - nvert;
-        const int s = (int)(u % NP1);
-        const int ex = (int)((u / NP1) % nx);
-        const int fz = (int)(u / (NP1 * nx));
-        const bool wallB = (fz == 0), wallT = (fz == nz);
-        const int eB = (wallB ? 0 : fz - 1) * nx + ex;
-        const int eT = (wallT ? nz - 1 : fz) * nx + ex;
-        T trB[4], trT[4], gB[4], gT[4];
+        const int ex = c % nx, fz = c / nx;
+        wallL = fz == 0;
+        wallR = fz == nz;
+        eL = (wallL ? 0 : fz - 1) * nx + ex;
+        eR = (wallR ? nz - 1 : fz) * nx + ex;
+        ib = fz;
+    }
+    const int nb = zf ? nz + 1 : nz * NP1;   // stride of the background tables
+    const double *ub = zf ? K.ubh : K.ubv;
+    const float *ubf = zf ? K.ubhf : K.ubvf;
+    const int st = zf ? NP1 : 1, i0 = zf ? s : s * NP1;
+    const auto two_h = mkc(zf ? K.two_hz : K.two_hx, zf ? K.two_hzf : K.two_hxf, T{});
+    T UL[4], UR[4], gL[4], gR[4], J[4];   // states, normal derivatives and jumps
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            T aB, aT, dB, dT;
-            const size_t iB0 = (size_t)v * N1 + (size_t)eB * NP + s;
-            const size_t iT0 = (size_t)v * N1 + (size_t)eT * NP + s;
-            line_trace<T, IN, NP1, VISC>(ld, iB0, NP1, K.tab.lp, K.tlp, K.tab.dlp, K.tdlp, aB, dB);
-            line_trace<T, IN, NP1, VISC>(ld, iT0, NP1, K.tab.lm, K.tlm, K.tab.dlm, K.tdlm, aT, dT);
-            trB[v] = aB;
-            trT[v] = aT;
-            gB[v] = mkc(K.two_hz, K.two_hzf, T{}) * dB + bgs(K.dubh, K.dubhf, (size_t)v * (nz + 1) + fz, T{});
-            gT[v] = mkc(K.two_hz, K.two_hzf, T{}) * dT + bgs(K.dubh, K.dubhf, (size_t)v * (nz + 1) + fz, T{});
+    for (int v = 0; v < 4; ++v) {
+        T aL, aR, dL, dR;
+        line_trace<T, IN, NP1, VISC>(ld, v * N1 + (size_t)eL * NP + i0, st, K.tab.lp, K.tlp, K.tab.dlp, K.tdlp, aL, dL);
+        line_trace<T, IN, NP1, VISC>(ld, v * N1 + (size_t)eR * NP + i0, st, K.tab.lm, K.tlm, K.tab.dlm, K.tdlm, aR, dR);
+        UL[v] = aL + bgs(ub, ubf, (size_t)v * nb + ib, T{});
+        UR[v] = aR + bgs(ub, ubf, (size_t)v * nb + ib, T{});
+        if (VISC) {
+            gL[v] = two_h * dL;
+            gR[v] = two_h * dR;
+            if (zf) {   // the background varies with z only
+                gL[v] = gL[v] + bgs(K.dubh, K.dubhf, (size_t)v * nb + ib, T{});
+                gR[v] = gR[v] + bgs(K.dubh, K.dubhf, (size_t)v * nb + ib, T{});
+            }
+            J[v] = aL - aR;
         }
-        T UB[4], UT[4];
+    }
+    if constexpr (IN == 0) {
+        if (lin.tr) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            UB[v] = trB[v] + bgs(K.ubh, K.ubhf, (size_t)v * (nz + 1) + fz, T{});
-            UT[v] = trT[v] + bgs(K.ubh, K.ubhf, (size_t)v * (nz + 1) + fz, T{});
-        }
-        if constexpr (IN == 0) {
-            if (lin.tr) {
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    lin.tr[(2 * v) * nfp + t] = outv(UB[v]);
-                    lin.tr[(2 * v + 1) * nfp + t] = outv(UT[v]);
-                    if (VISC) {
-                        lin.tr[(8 + 2 * v) * nfp + t] = outv(gB[v]);
-                        lin.tr[(9 + 2 * v) * nfp + t] = outv(gT[v]);
-                        lin.tr[(16 + v) * nfp + t] = outv(trB[v] - trT[v]);
-                    }
+            for (int v = 0; v < 4; ++v) {
+                lin.tr[(2 * v) * nfp + t] = outv(UL[v]);
+                lin.tr[(2 * v + 1) * nfp + t] = outv(UR[v]);
+                if (VISC) {
+                    lin.tr[(8 + 2 * v) * nfp + t] = outv(gL[v]);
+                    lin.tr[(9 + 2 * v) * nfp + t] = outv(gR[v]);
+                    lin.tr[(16 + v) * nfp + t] = outv(J[v]);
                 }
             }
         }
-        wall_states<T, 1>(UB, UT, wallB, wallT);
-        Side<T> SB, ST;
-        side_of(UB, K.pc, K.pt, SB);
-        side_of(UT, K.pc, K.pt, ST);
-        hllc_s<T, 1>(SB, ST, H);
-        if constexpr (IN == 0) {
-            if (lin.tr) {
+    }
+    swap_d(zf, UL[1], UL[2]);
+    swap_d(zf, UR[1], UR[2]);
+    wall_states<T, 0>(UL, UR, wallL, wallR);
+    Side<T> L, R;
+    side_of(UL, K.pc, K.pt, L);
+    side_of(UR, K.pc, K.pt, R);
+    T H[4];
+    hllc_s<T, 0>(L, R, H);
+    swap_d(zf, H[1], H[2]);
+    if constexpr (IN == 0) {
+        if (lin.tr) {
 #pragma unroll
-                for (int v = 0; v < 4; ++v) lin.H[v * nfp + t] = outv(H[v]);
-            }
+            for (int v = 0; v < 4; ++v) lin.H[v * nfp + t] = outv(H[v]);
         }
+    }
+    const double *hb = zf ? K.hbz : (wallL ? K.hbxw : (wallR ? K.hbxw + 4 * (size_t)nb : K.hbx));
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            if (IN != 2) H[v] = H[v] - bg<T>(K.hbz, (size_t)v * (nz + 1) + fz);
-            Phi[v] = H[v];
-        }
+    for (int v = 0; v < 4; ++v)
+        if (IN != 2) H[v] = H[v] - bg<T>(hb, (size_t)v * nb + ib);
+    O *phi = zf ? phiz : phix;
+    const size_t fs = zf ? (size_t)(nfp - nvert) : (size_t)nvert;
+    if (VISC) {
+        O *sym = zf ? symz : symx;
+        if (wallL || wallR) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) sL[c] = sR[c] = zero;
-        if (VISC && !wallB && !wallT) {
-            // interior penalty on the jumps of u, w, theta: eta {A(U)} [U]
-            const auto eta = mkc(K.eta_z, K.eta_zf, T{});
+            for (int q = 0; q < 6; ++q) sym[(size_t)q * fs + u] = 0;
+        } else {
+            swap_d(zf, L.U[1], L.U[2]);   // back to (u, w)
+            swap_d(zf, R.U[1], R.U[2]);
+            const auto eta = mkc(zf ? K.eta_z : K.eta_x, zf ? K.eta_zf : K.eta_xf, T{});
             const auto hmu = mkc(0.5 * K.mu, 0.5f * K.pc.muf, T{});
-            const T J0 = trB[0] - trT[0];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const int v = c + 1;
-                const T pL = SB.U[v] * SB.ir, pR = ST.U[v] * ST.ir;
-                const T Jv = trB[v] - trT[v];
-                sL[c] = hmu * visc_c(pL, J0, Jv);
-                sR[c] = hmu * visc_c(pR, J0, Jv);
-                const T V = visc_face(hmu, eta, pL, pR, gB, gT, v, sL[c], sR[c]);
-                Phi[v] = Phi[v] - V;
+            for (int q = 0; q < 3; ++q) {
+                const int v = q + 1;
+                const T pL = L.U[v] * L.ir, pR = R.U[v] * R.ir;
+                const T sL = hmu * visc_c(pL, J[0], J[v]), sR = hmu * visc_c(pR, J[0], J[v]);
+                const T V = visc_face(hmu, eta, pL, pR, gL, gR, v, sL, sR);
+                H[v] = H[v] - V;
                 if constexpr (IN == 0) {
                     if (lin.tr) {
-                        lin.H[(4 + c) * nfp + t] = outv(V);
-                        lin.H[(7 + c) * nfp + t] = outv(sL[c]);
-                        lin.H[(10 + c) * nfp + t] = outv(sR[c]);
+                        lin.H[(4 + q) * nfp + t] = outv(V);
+                        lin.H[(7 + q) * nfp + t] = outv(sL);
+                        lin.H[(10 + q) * nfp + t] = outv(sR);
                     }
                 }
-            }
-        }
-        const size_t fb = ((size_t)fz * nx + ex) * NP1 + s;
-        const size_t fs = (size_t)(nz + 1) * nx * NP1;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) phiz[v * fs + fb] = (O)outv(Phi[v]);
-        if (VISC) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                symz[(size_t)c * fs + fb] = (O)outv(sL[c]);
-                symz[(size_t)(3 + c) * fs + fb] = (O)outv(sR[c]);
+                sym[(size_t)q * fs + u] = (O)outv(sL);
+                sym[(size_t)(3 + q) * fs + u] = (O)outv(sR);
             }
         }
     }
-}
-
-template <class T, int IN, int NP1, bool VISC>
-struct k_faces_b {
-    static constexpr int TPB = 256, MINB = VISC ? 2 : 4;
-    static constexpr bool GROUP = !VISC && std::is_same<T, D64>::value;   // a grouped twin is built (lock-step ensembles)
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGK> K,
-                                               JfArg<Loader<T, IN>> ld0, JfArg<typename OutT<T>::type *> phix,
-                                               JfArg<typename OutT<T>::type *> symx,
-                                               JfArg<typename OutT<T>::type *> phiz,
-                                               JfArg<typename OutT<T>::type *> symz, JfArg<LinPtr> lin) {
-        jf_pdl_enter();
-        faces_body<T, IN, NP1, VISC>(K, ld0, phix, symx, phiz, symz, jf_bid, lin);
-    }
-};
-template <class T, int IN, int NP1, bool VISC>
-__global__ void __launch_bounds__(256, VISC ? 2 : 4) k_faces(DGK K, Loader<T, IN> ld0, typename OutT<T>::type *phix,
-                                               typename OutT<T>::type *symx, typename OutT<T>::type *phiz,
-                                               typename OutT<T>::type *symz, LinPtr lin) {
-    k_faces_b<T, IN, NP1, VISC>::run(blockIdx.x, gridDim.x, K, ld0, phix, symx, phiz, symz, lin);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) phi[v * fs + u] = (O)outv(H[v]);
 }
 
 // ---------------------------------------------------------------------------
-// blockDim.x / NP elements per volume block (at most 128 threads)
-template <class T, int IN, int MODE, int NP1, bool VISC>
-__device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &ld0, const DGArgs &A,
-                                            const typename OutT<T>::type *phix,
-                                            const typename OutT<T>::type *symx,
-                                            const typename OutT<T>::type *phiz,
-                                            const typename OutT<T>::type *symz, unsigned blk, const LinPtr &lin) {
+// Node fluxes and their weak-form derivatives with the gravity source: the operator
+// without the lifted face terms, into `part` ([4][nodes]).  blockDim.x / NP elements per
+// block (at most 128 threads), one thread per node.
+template <class T, int IN, int NP1, bool VISC>
+__device__ __forceinline__ void nodes_body(const DGK &K, const Loader<T, IN> &ld0, typename OutT<T>::type *part,
+                                           unsigned blk, const LinPtr &lin) {
     typedef typename OutT<T>::type O;
     constexpr int NP = NP1 * NP1;
     constexpr int EPB = 128 / NP;
     __shared__ O sg[2][EPB][4][NP];
-    __shared__ T su[VISC ? EPB : 1][4][NP];
-    // weak-form derivative and lift tables with the 2/h factors folded in:
-    // sDx = (2/hx) Dw, sDz = (2/hz) Dw; sl[0..3] x-lifts, sl[4..7] z-lifts
+    __shared__ T su[VISC ? EPB : 1][4][VISC ? NP : 1];
+    // weak-form derivative tables with the 2/h factors folded in: sDx = (2/hx) Dw, sDz = (2/hz) Dw
     __shared__ O sDx[NP1][NP1], sDz[NP1][NP1];
     __shared__ O sDn[NP1][NP1];
-    __shared__ O sl[8][NP1];
-    __shared__ double sce[2];   // eps and adt / eps of the FD modes: one IEEE division per block
-    if ((MODE == DG_JV || MODE == DG_SMOOTH64) && threadIdx.x == 0) {
-        const double e0 = A.eps ? *A.eps : A.eps_val;
-        sce[0] = e0;
-        sce[1] = e0 != 0.0 ? A.adt / e0 : 0.0;
-    }
     Loader<T, IN> ld = ld0;
     ld.prepare();
-    if (threadIdx.x < NP) {
-        const int r = threadIdx.x / NP1, q = threadIdx.x % NP1;
+    for (int i = threadIdx.x; i < NP; i += blockDim.x) {
+        const int r = i / NP1, q = i % NP1;
         sDx[r][q] = pick<O>(K.Dx[r][q], K.Dxf[r][q]);
         sDz[r][q] = pick<O>(K.Dz[r][q], K.Dzf[r][q]);
         sDn[r][q] = pick<O>(K.tab.Dn[r][q], K.Dnf[r][q]);
-    }
-    if (threadIdx.x < NP1) {
-        const int q = threadIdx.x;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) sl[r][q] = pick<O>(K.lift[r][q], K.liftf[r][q]);
     }
     const int le = threadIdx.x / NP;
     const int node = threadIdx.x % NP;
@@ -376,31 +257,10 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
     const int e = (int)blk * epb + le;
     const bool active = (le < epb) && (e < K.n_el);
     const int nx = K.nx, nz = K.nz;
-    const int ez = active ? e / nx : 0, ex = active ? e % nx : 0;
+    const int ez = active ? e / nx : 0;
     const size_t N1 = (size_t)K.n_el * NP;
     const size_t nrow = (size_t)nz * NP1;
     const int J = ez * NP1 + b;
-    // FP32 tangent modes: face terms and the epilogue's operands are loaded now so
-    // that their latency overlaps the flux work below (the FP64 modes are bound by
-    // FP64 arithmetic and keep their registers for it)
-    constexpr bool PF = (IN == 2);
-    const size_t fsx = (size_t)nz * (nx + 1) * NP1, fsz = (size_t)(nz + 1) * nx * NP1;
-    const size_t iL = ((size_t)ez * (nx + 1) + ex) * NP1 + b, iR = iL + NP1;
-    const size_t iB = ((size_t)ez * nx + ex) * NP1 + a, iT = iB + (size_t)nx * NP1;
-    O pxl[4], pxr[4], pzb[4], pzt[4];
-    float ef[4], edt = 0.0f;   // operands of the FP32 smoothing mode
-    if (PF && active) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            pxl[v] = phix[v * fsx + iL];
-            pxr[v] = phix[v * fsx + iR];
-            pzb[v] = phiz[v * fsz + iB];
-            pzt[v] = phiz[v * fsz + iT];
-            if (MODE == DG_TLSMOOTH || (MODE == DG_TLJV && A.rf)) ef[v] = A.rf[(size_t)v * N1 + (size_t)e * NP + node];
-        }
-        if (MODE == DG_TLSMOOTH) edt = A.dtauf[e];
-    }
-    __syncthreads();
     T Up[4], U[4];
     if (active) {
 #pragma unroll
@@ -410,7 +270,7 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
             if (VISC) su[le][v][node] = Up[v];
         }
     }
-    __syncthreads();
+    if (VISC) __syncthreads();
     if (active) {
         const T ir = jrcp(U[0]);
         const T p = pressure(U[3], K.pc, K.pt);
@@ -482,11 +342,6 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
     }
     __syncthreads();
     if (!active) return;
-    const O lmxa = sl[0][a], lpxa = sl[1][a], dlmxa = sl[2][a], dlpxa = sl[3][a];
-    const O lmzb = sl[4][b], lpzb = sl[5][b], dlmzb = sl[6][b], dlpzb = sl[7][b];
-    const double eps = (MODE == DG_JV || MODE == DG_SMOOTH64) ? sce[0] : 0.0;
-    const double ceps = (MODE == DG_JV || MODE == DG_SMOOTH64) ? sce[1] : 0.0;
-    const float adtf = (MODE == DG_TLJV || MODE == DG_TLSMOOTH) ? A.adtf : 0.0f;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
         O f = 0;
@@ -496,18 +351,82 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
             f = fma(sDz[b][q], sg[1][le][v][q * NP1 + a], f);
         }
         if (v == 2) f = fma(-pick<O>(K.g, K.gf), (O)outv(Up[0]), f);
-        f = fma(lmxa, PF ? pxl[v] : phix[v * fsx + iL], f);
-        f = fma(-lpxa, PF ? pxr[v] : phix[v * fsx + iR], f);
-        f = fma(lmzb, PF ? pzb[v] : phiz[v * fsz + iB], f);
-        f = fma(-lpzb, PF ? pzt[v] : phiz[v * fsz + iT], f);
+        part[(size_t)v * N1 + (size_t)e * NP + node] = f;
+    }
+}
+
+// Both in one launch: the first `nface` blocks take the face points, the others the
+// nodes; neither needs the other (the lift below adds them).  Bound by the FP64 pipe:
+// 95 instructions a face point and 57 a Q3 node take 40.5 of the 48.1 us of Q3 160 x 80
+// (Q4 320 x 160: 257 of 264).  As a face launch and a volume launch with the lifts the
+// pair took 28.0 + 34.3 us against 48.1 + 12.6 now; the gain is on small grids, where each
+// launch pays a latency chain of some thousand clocks (Q2 20 x 10: 14.4 us a residual
+// then, 11.5 now, most of it the host's).
+template <class T, int IN, int NP1, bool VISC>
+struct k_dg_flux_b {
+    static constexpr int TPB = 128, MINB = VISC ? 4 : 7;
+    static constexpr bool GROUP = !VISC && std::is_same<T, D64>::value;   // a grouped twin is built (lock-step ensembles)
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGK> K, JfArg<unsigned> nface,
+                                               JfArg<Loader<T, IN>> ld0, JfArg<typename OutT<T>::type *> part,
+                                               JfArg<typename OutT<T>::type *> phix,
+                                               JfArg<typename OutT<T>::type *> symx,
+                                               JfArg<typename OutT<T>::type *> phiz,
+                                               JfArg<typename OutT<T>::type *> symz, JfArg<LinPtr> lin) {
+        jf_pdl_enter();
+        if (jf_bid < nface) faces_body<T, IN, NP1, VISC>(K, ld0, phix, symx, phiz, symz, jf_bid, lin);
+        else nodes_body<T, IN, NP1, VISC>(K, ld0, part, jf_bid - nface, lin);
+    }
+};
+template <class T, int IN, int NP1, bool VISC>
+__global__ void __launch_bounds__(128, VISC ? 4 : 7)
+    k_dg_flux(DGK K, unsigned nface, Loader<T, IN> ld0, typename OutT<T>::type *part, typename OutT<T>::type *phix,
+              typename OutT<T>::type *symx, typename OutT<T>::type *phiz, typename OutT<T>::type *symz, LinPtr lin) {
+    k_dg_flux_b<T, IN, NP1, VISC>::run(blockIdx.x, gridDim.x, K, nface, ld0, part, phix, symx, phiz, symz, lin);
+}
+
+// Adds the lifts of the face terms to `part` and runs the mode's epilogue, one thread
+// per node.
+template <class T, int MODE, int NP1, bool VISC>
+__device__ __forceinline__ void lift_body(const DGK &K, const DGArgs &A, const typename OutT<T>::type *part,
+                                          const typename OutT<T>::type *phix, const typename OutT<T>::type *symx,
+                                          const typename OutT<T>::type *phiz, const typename OutT<T>::type *symz,
+                                          unsigned blk) {
+    typedef typename OutT<T>::type O;
+    constexpr int NP = NP1 * NP1;
+    constexpr bool FD = MODE == DG_JV || MODE == DG_SMOOTH64;
+    __shared__ O sl[8][NP1];    // sl[0..3] x-lifts, sl[4..7] z-lifts
+    __shared__ double sce[2];   // eps and adt / eps of the FD modes: one quotient per block
+    for (int i = threadIdx.x; i < 8 * NP1; i += blockDim.x)
+        sl[i / NP1][i % NP1] = pick<O>(K.lift[i / NP1][i % NP1], K.liftf[i / NP1][i % NP1]);
+    if (FD && threadIdx.x == 0) {
+        const double e0 = A.eps ? *A.eps : A.eps_val;
+        sce[0] = e0;
+        sce[1] = e0 != 0.0 ? div64(A.adt, e0) : 0.0;
+    }
+    const int N1 = K.n_el * NP, n = (int)blk * (int)blockDim.x + (int)threadIdx.x;
+    __syncthreads();
+    if (n >= N1) return;
+    const int e = n / NP, node = n % NP, a = node % NP1, b = node / NP1;
+    const int nx = K.nx, nz = K.nz, ez = e / nx, ex = e - ez * nx;
+    const int fsx = nz * (nx + 1) * NP1, fsz = (nz + 1) * nx * NP1;
+    const int iL = (ez * (nx + 1) + ex) * NP1 + b, iR = iL + NP1;
+    const int iB = (ez * nx + ex) * NP1 + a, iT = iB + nx * NP1;
+    const double eps = FD ? sce[0] : 0.0, ceps = FD ? sce[1] : 0.0;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        const size_t gi = (size_t)v * N1 + n;
+        O f = part[gi];
+        f = fma(sl[0][a], phix[(size_t)v * fsx + iL], f);
+        f = fma(-sl[1][a], phix[(size_t)v * fsx + iR], f);
+        f = fma(sl[4][b], phiz[(size_t)v * fsz + iB], f);
+        f = fma(-sl[5][b], phiz[(size_t)v * fsz + iT], f);
         if (VISC && v > 0) {
             const int c = v - 1;
-            f = fma(dlmxa, symx[(size_t)(3 + c) * fsx + iL], f);
-            f = fma(dlpxa, symx[(size_t)c * fsx + iR], f);
-            f = fma(dlmzb, symz[(size_t)(3 + c) * fsz + iB], f);
-            f = fma(dlpzb, symz[(size_t)c * fsz + iT], f);
+            f = fma(sl[2][a], symx[(size_t)(3 + c) * fsx + iL], f);
+            f = fma(sl[3][a], symx[(size_t)c * fsx + iR], f);
+            f = fma(sl[6][b], symz[(size_t)(3 + c) * fsz + iB], f);
+            f = fma(sl[7][b], symz[(size_t)c * fsz + iT], f);
         }
-        const size_t gi = (size_t)v * N1 + (size_t)e * NP + node;
         if (MODE == DG_RES) {
             ((double *)A.out0)[gi] = (double)f;
         } else if (MODE == DG_JV) {
@@ -526,43 +445,40 @@ __device__ __forceinline__ void volume_body(const DGK &K, const Loader<T, IN> &l
                 ((double *)A.out0)[gi] = A.z0mode == 1 ? ((const double *)A.z0)[gi] + st : st;
             }
         } else if (MODE == DG_TLJV) {
-            const float z = (float)outv(Up[v]);   // the loader's tangent input is y
-            const float jz = z - adtf * (float)f;
-            ((float *)A.out0)[gi] = A.rf ? ef[v] - jz : jz;   // with r given: the defect r - G'z
+            const float z = A.yf[gi];
+            const float jz = z - A.adtf * (float)f;
+            ((float *)A.out0)[gi] = A.rf ? A.rf[gi] - jz : jz;   // with r given: the defect r - G'z
         } else {  // DG_TLSMOOTH
-            const float z = (float)outv(Up[v]);
-            const float Jz = z - adtf * (float)f;
+            const float z = A.yf[gi];
+            const float Jz = z - A.adtf * (float)f;
             if (A.z0mode == 0) {
-                ((float *)A.out0)[gi] = z + edt * (ef[v] - Jz);
+                ((float *)A.out0)[gi] = z + A.dtauf[e] * (A.rf[gi] - Jz);
             } else {
-                const float st = (A.alphaf * edt) * (ef[v] - Jz);
+                const float st = (A.alphaf * A.dtauf[e]) * (A.rf[gi] - Jz);
                 ((float *)A.out0)[gi] = A.z0mode == 1 ? ((const float *)A.z0)[gi] + st : st;
             }
         }
     }
 }
-
-template <class T, int IN, int MODE, int NP1, bool VISC>
-struct k_volume_b {
+template <class T, int MODE, int NP1, bool VISC>
+struct k_dg_lift_b {
     static constexpr int TPB = 128, MINB = 8;
     static constexpr bool GROUP = !VISC && std::is_same<T, D64>::value && MODE != DG_SMOOTH64;   // a grouped twin is built (lock-step ensembles)
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGK> K,
-                                               JfArg<Loader<T, IN>> ld0, JfArg<DGArgs> A,
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGK> K, JfArg<DGArgs> A,
+                                               JfArg<const typename OutT<T>::type *> part,
                                                JfArg<const typename OutT<T>::type *> phix,
                                                JfArg<const typename OutT<T>::type *> symx,
                                                JfArg<const typename OutT<T>::type *> phiz,
-                                               JfArg<const typename OutT<T>::type *> symz, JfArg<LinPtr> lin) {
+                                               JfArg<const typename OutT<T>::type *> symz) {
         jf_pdl_enter();
-        volume_body<T, IN, MODE, NP1, VISC>(K, ld0, A, phix, symx, phiz, symz, jf_bid, lin);
+        lift_body<T, MODE, NP1, VISC>(K, A, part, phix, symx, phiz, symz, jf_bid);
     }
 };
-template <class T, int IN, int MODE, int NP1, bool VISC>
-__global__ void __launch_bounds__(128, 8) k_volume(DGK K, Loader<T, IN> ld0, DGArgs A,
-                                                   const typename OutT<T>::type *phix,
-                                                   const typename OutT<T>::type *symx,
-                                                   const typename OutT<T>::type *phiz,
-                                                   const typename OutT<T>::type *symz, LinPtr lin) {
-    k_volume_b<T, IN, MODE, NP1, VISC>::run(blockIdx.x, gridDim.x, K, ld0, A, phix, symx, phiz, symz, lin);
+template <class T, int MODE, int NP1, bool VISC>
+__global__ void __launch_bounds__(128, 8)
+    k_dg_lift(DGK K, DGArgs A, const typename OutT<T>::type *part, const typename OutT<T>::type *phix,
+              const typename OutT<T>::type *symx, const typename OutT<T>::type *phiz, const typename OutT<T>::type *symz) {
+    k_dg_lift_b<T, MODE, NP1, VISC>::run(blockIdx.x, gridDim.x, K, A, part, phix, symx, phiz, symz);
 }
 
 // ---------------------------------------------------------------------------
@@ -1073,12 +989,17 @@ int launch(jfnk_ctx *c, const DGK &K, const Loader<T, IN> &ld, const DGArgs &a, 
     const long long nf = (long long)K.nz * (K.nx + 1) * NP1 + (long long)(K.nz + 1) * K.nx * NP1;
     if (c->timing) JF_CK(cudaEventRecord(c->tev[0], s));
     const LinPtr lin = IN == 0 && a.lin_out ? c->lin : LinPtr{};
-    const int tf = spread_threads(c->opts.tile_faces, (size_t)nf, c->n_sm);
-    jf_launch<k_faces_b<T, IN, NP1, VISC>>(k_faces<T, IN, NP1, VISC>, (unsigned)((nf + tf - 1) / tf), tf, 0, s, K, ld, phix, symx, phiz, symz,
-              lin); jf_launched();
+    const int epb = spread_elements<NP1>(c->opts.tile_volume, K.n_el, c->n_sm), tb = epb * NP1 * NP1;
+    const unsigned nface = (unsigned)((nf + tb - 1) / tb), nnode = (unsigned)((K.n_el + epb - 1) / epb);
+    // the operator without its lifts, closed in place
+    O *part = MODE == DG_G ? (O *)a.out1 : (O *)a.out0;
+    jf_launch<k_dg_flux_b<T, IN, NP1, VISC>>(k_dg_flux<T, IN, NP1, VISC>, nface + nnode, tb, 0, s, K, nface, ld, part, phix, symx, phiz, symz,
+              lin);
+    jf_launched();
     if (c->timing) JF_CK(cudaEventRecord(c->tev[1], s));
-    const int epb = spread_elements<NP1>(c->opts.tile_volume, K.n_el, c->n_sm);
-    jf_launch<k_volume_b<T, IN, MODE, NP1, VISC>>(k_volume<T, IN, MODE, NP1, VISC>, (unsigned)((K.n_el + epb - 1) / epb), epb * NP1 * NP1, 0, s, K, ld, a, phix, symx, phiz, symz, lin);
+    const int tl = spread_threads(128, c->npt, c->n_sm);
+    jf_launch<k_dg_lift_b<T, MODE, NP1, VISC>>(k_dg_lift<T, MODE, NP1, VISC>, (unsigned)((c->npt + tl - 1) / tl), tl, 0, s, K, a, (const O *)part,
+              (const O *)phix, (const O *)symx, (const O *)phiz, (const O *)symz);
     jf_launched();
     JF_CK(cudaGetLastError());
     return timing_close(c, s);
@@ -1136,44 +1057,51 @@ int dispatch_mode(jfnk_ctx *c, int mode, const DGArgs &a, cudaStream_t s) {
 
 // ---- one launch per operator across ensemble members ---------------------
 // A member's share of a grouped residual launch: its operator constants, state,
-// output and face buffers, and the first face / volume block of the launch that
-// belongs to it.
+// output and face buffers, its face block count and the first flux / lift block of the
+// launch that belongs to it.
 struct DGMember {
     DGK K;
     Loader<D64, 0> ld;
     DGArgs A;
     double *phix, *symx, *phiz, *symz;
-    unsigned fb0, vb0;
+    unsigned nface, fb0, lb0;
 };
-constexpr int GRP_FACE_THREADS = 128;
+// flux and lift blocks of one member (128-thread blocks, 128 / NP elements each)
+inline void group_blocks(const DGK &K, unsigned &nface, unsigned &nflux, unsigned &nlift) {
+    const int n1 = K.tab.np1, np = n1 * n1, epb = 128 / np, tb = epb * np;
+    const long long nf = (long long)K.nz * (K.nx + 1) * n1 + (long long)(K.nz + 1) * K.nx * n1;
+    nface = (unsigned)((nf + tb - 1) / tb);
+    nflux = nface + (unsigned)((K.n_el + epb - 1) / epb);
+    nlift = (unsigned)(((long long)K.n_el * np + 127) / 128);
+}
 
 template <int NP1, bool VISC>
-__global__ void __launch_bounds__(256, VISC ? 2 : 4) k_faces_grp(const DGMember *mem, int nm) {
+__global__ void __launch_bounds__(128, VISC ? 4 : 7) k_flux_grp(const DGMember *mem, int nm) {
     jf_pdl_enter();
     int m = 0;
     while (m + 1 < nm && blockIdx.x >= mem[m + 1].fb0) ++m;   // members in block order
     const DGMember &M = mem[m];
-    faces_body<D64, 0, NP1, VISC>(M.K, M.ld, M.phix, M.symx, M.phiz, M.symz, blockIdx.x - M.fb0, LinPtr{});
+    const unsigned bid = blockIdx.x - M.fb0;
+    if (bid < M.nface) faces_body<D64, 0, NP1, VISC>(M.K, M.ld, M.phix, M.symx, M.phiz, M.symz, bid, LinPtr{});
+    else nodes_body<D64, 0, NP1, VISC>(M.K, M.ld, (double *)M.A.out0, bid - M.nface, LinPtr{});
 }
 
 template <int NP1, bool VISC>
-__global__ void __launch_bounds__(128, 8) k_volume_grp(const DGMember *mem, int nm) {
+__global__ void __launch_bounds__(128, 8) k_lift_grp(const DGMember *mem, int nm) {
     jf_pdl_enter();
     int m = 0;
-    while (m + 1 < nm && blockIdx.x >= mem[m + 1].vb0) ++m;
+    while (m + 1 < nm && blockIdx.x >= mem[m + 1].lb0) ++m;
     const DGMember &M = mem[m];
-    volume_body<D64, 0, DG_RES, NP1, VISC>(M.K, M.ld, M.A, M.phix, M.symx, M.phiz, M.symz, blockIdx.x - M.vb0, LinPtr{});
+    lift_body<D64, DG_RES, NP1, VISC>(M.K, M.A, (const double *)M.A.out0, M.phix, M.symx, M.phiz, M.symz, blockIdx.x - M.lb0);
 }
 
 template <int NP1, bool VISC>
 void launch_grp(const DGMember *dmem, const std::vector<DGMember> &h, int first, int cnt, cudaStream_t s) {
     const DGMember &last = h[first + cnt - 1];
-    const long long nfl = (long long)last.K.nz * (last.K.nx + 1) * NP1 + (long long)(last.K.nz + 1) * last.K.nx * NP1;
-    const unsigned fb = last.fb0 + (unsigned)((nfl + GRP_FACE_THREADS - 1) / GRP_FACE_THREADS);
-    constexpr int EPB = 128 / (NP1 * NP1);
-    const unsigned vb = last.vb0 + (unsigned)((last.K.n_el + EPB - 1) / EPB);
-    jf_launch_now(k_faces_grp<NP1, VISC>, fb, GRP_FACE_THREADS, 0, s, dmem + first, cnt);
-    jf_launch_now(k_volume_grp<NP1, VISC>, vb, EPB * NP1 * NP1, 0, s, dmem + first, cnt);
+    unsigned nface, nflux, nlift;
+    group_blocks(last.K, nface, nflux, nlift);
+    jf_launch_now(k_flux_grp<NP1, VISC>, last.fb0 + nflux, 128 / (NP1 * NP1) * (NP1 * NP1), 0, s, dmem + first, cnt);
+    jf_launch_now(k_lift_grp<NP1, VISC>, last.lb0 + nlift, 128, 0, s, dmem + first, cnt);
     jf_launched(2);
 }
 
@@ -1246,13 +1174,13 @@ int dg_residual_grouped(jfnk_ctx *const *ctx, int n, const double *const *U, dou
     if ((int)order.size() != n) return JFNK_EINVAL;
     std::vector<DGMember> h(n);
     std::vector<int> gstart;
-    unsigned fb = 0, vb = 0;
+    unsigned fb = 0, lb = 0;
     for (int q = 0; q < n; ++q) {
         jfnk_ctx *c = ctx[order[q]];
         if (q == 0 || c->np1 != ctx[order[q - 1]]->np1 ||
             (c->phys.mu != 0.0) != (ctx[order[q - 1]]->phys.mu != 0.0)) {
             gstart.push_back(q);
-            fb = vb = 0;
+            fb = lb = 0;
         }
         DGMember &M = h[q];
         M.K = make_K(c);
@@ -1265,12 +1193,11 @@ int dg_residual_grouped(jfnk_ctx *const *ctx, int n, const double *const *U, dou
         M.phiz = (double *)c->phiz;
         M.symz = (double *)c->symz;
         M.fb0 = fb;
-        M.vb0 = vb;
-        const int n1 = c->np1;
-        const long long nf = (long long)c->grid.nz * (c->grid.nx + 1) * n1 + (long long)(c->grid.nz + 1) * c->grid.nx * n1;
-        fb += (unsigned)((nf + GRP_FACE_THREADS - 1) / GRP_FACE_THREADS);
-        const int epb = (128 / (n1 * n1)) > 0 ? 128 / (n1 * n1) : 1;
-        vb += (unsigned)((c->n_el + epb - 1) / epb);
+        M.lb0 = lb;
+        unsigned nflux, nlift;
+        group_blocks(M.K, M.nface, nflux, nlift);
+        fb += nflux;
+        lb += nlift;
         c->dg_calls++;
     }
     JF_CK(cudaMemcpyAsync(dmem, h.data(), sizeof(DGMember) * (size_t)n, cudaMemcpyHostToDevice, s));

@@ -94,12 +94,6 @@ struct DGF {
 };
 
 constexpr int FD_MINB = 7;   // 72 registers: 28 warps an SM, no spills
-JF_D void swap_d(bool c, D64 &a, D64 &b) {
-    const D64 t = a;
-    a = sel(c, b, a);
-    b = sel(c, t, b);
-}
-
 // Difference of the face terms at U + eps y and U, one thread per face point (the linear
 // index of the residual's face kernel).  Vertical and horizontal faces run the same code:
 // the momentum components are exchanged for the latter.

@@ -428,7 +428,7 @@ inline int spread_elements(int tile_volume, int n_el, int n_sm) {
     auto fit = [](int threads) { return threads / NP > 0 ? threads / NP : 1; };
     int t = tile_volume == 2 ? 128 : 64;
     if (!t_jf_rec)
-        while (t > 32 && n_el < fit(t) * 2 * n_sm) t /= 2;
+        while (t > 32 && n_el < fit(t) * 4 * n_sm) t /= 2;
     return fit(t);
 }
 
