@@ -620,8 +620,8 @@ int mg_precondition(jfnk_ctx *c, const double *U, double adt, const double *r, d
     }
     JF_RET(mg_linearize(c, U, adt, s));
     if (c->prec == 64) return mg_apply(c, r, z, s);
-    JF_RET(mg_apply(c, r, c->Z, s));
-    return blas_copy_f2d((const float *)c->Z, z, c->N, s);
+    JF_RET(mg_apply(c, r, nullptr, s));
+    return blas_copy_f2d((const float *)c->pout, z, c->N, s);
 }
 
 int jfnk_norm2(jfnk_ctx *c, const double *x, size_t n, double *out, void *stream) {

@@ -29,15 +29,16 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// (through shared memory: 12 FP64 adds of one warp, where a shuffle tree in every warp
+// took 45 warp adds and two dependent trees of 110 clocks a step)
 __device__ __forceinline__ double block_sum(double v) {
-    __shared__ double sw[RB / 32];
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) sw[wid] = v;
+    __shared__ double sv[RB];
+    sv[threadIdx.x] = v;
     __syncthreads();
     double r = 0.0;
-    if (wid == 0) {
-        r = lane < RB / 32 ? sw[lane] : 0.0;
+    if (threadIdx.x < 32) {
+        const double *q = sv + threadIdx.x;
+        r = ((q[0] + q[32]) + (q[64] + q[96])) + ((q[128] + q[160]) + (q[192] + q[224]));
         r = warp_sum(r);
     }
     __syncthreads();
@@ -67,8 +68,8 @@ __device__ __forceinline__ double sum_partials(const double *part, int nb) {
 // cnum: numerator of the eps ops (sqrt(2^-52) for RED_EPS, sqrt(2^-23) for
 // RED_EPS32, the preconditioner's choice for RED_EPSP)
 __device__ __forceinline__ double finish_op(double acc, int op, double cnum = 1.4901161193847656e-08) {
-    if (op == RED_SQRT) return sqrt(acc);
-    if (op == RED_EPS || op == RED_EPS32 || op == RED_EPSP) return acc > 0.0 ? cnum / sqrt(acc) : 0.0;
+    if (op == RED_SQRT) return sqrt64(acc);
+    if (op == RED_EPS || op == RED_EPS32 || op == RED_EPSP) return acc > 0.0 ? div64(cnum, sqrt64(acc)) : 0.0;
     return acc;
 }
 
@@ -114,8 +115,9 @@ __device__ __forceinline__ double warp_sum_scatter(const double (&a)[NV], int la
 // h[j] = sum over blocks of part[j * nb + b] by the whole block, fixed order:
 // thread t sums the partials b = t mod RB of every vector (all loads of a round
 // issued together), then one warp-and-block reduction of the NV sums.
+// Thread j < NV returns its sum.
 template <int NV>
-__device__ __forceinline__ void finish_multi(const double *part, int nb, double *h) {
+__device__ __forceinline__ double finish_multi(const double *part, int nb, double *h) {
     constexpr int P = NV <= 1 ? 1 : NV <= 2 ? 2 : NV <= 4 ? 4 : NV <= 8 ? 8 : NV <= 16 ? 16 : 32;
     __shared__ double fw[NV][RB / 32];
     double a[NV];
@@ -138,7 +140,26 @@ __device__ __forceinline__ void finish_multi(const double *part, int nb, double 
 #pragma unroll
         for (int q = 0; q < RB / 32; ++q) r += fw[threadIdx.x][q];
         h[threadIdx.x] = r;
+        return r;
     }
+    return 0.0;
+}
+// The close of pass 2 by the last block: with |w1|^2 = tot (thread 0) and lane j's h1, h2
+// (first warp), the second-pass flag, |w| and 1/|w|.
+__device__ __forceinline__ void close_update(double tot, double h1, double h2, double *w1sq, double *nrm, double *flag,
+                                             unsigned *ticket) {
+    if (threadIdx.x >= 32) return;
+    const double hh = warp_sum(h1 * h1), hh2 = warp_sum(h2 * h2);
+    if (threadIdx.x != 0) return;
+    *w1sq = tot;
+    const bool second = tot < 0.5 * (tot + hh);
+    // |w2|^2 = |w1|^2 - |h2|^2 for w2 = w1 - V h2 with V orthonormal and h2 = V^T w1;
+    // after the first pass h2 is tiny against |w1|, so the difference does not cancel
+    const double nr = sqrt64(second ? fmax(tot - hh2, 0.0) : tot);
+    nrm[0] = nr;
+    nrm[S_INV - S_NORM] = nr != 0.0 ? rcp64(nr) : 0.0;
+    *flag = second ? 1.0 : 0.0;
+    *ticket = 0u;
 }
 
 // Warp sums of NV per-lane values at about one FP64 add per value and lane:
@@ -190,42 +211,6 @@ __device__ __forceinline__ void store_multi(const double (&acc)[NV], double *par
     }
 }
 
-// pass 1: h = V^T w
-template <int NV>
-struct k_gs_dot_b {
-    static constexpr int TPB = RB, MINB = 0;
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const double *> V,
-                                               JfArg<size_t> ldv, JfArg<const double *> w, JfArg<size_t> n2,
-                                               JfArg<double *> part, JfArg<unsigned *> ticket, JfArg<double *> h) {
-        jf_pdl_enter();
-        const double2 *w2 = reinterpret_cast<const double2 *>(w);
-        const double2 *Vp[NV];
-    #pragma unroll
-        for (int j = 0; j < NV; ++j) Vp[j] = reinterpret_cast<const double2 *>(V + (size_t)j * ldv);
-        double acc[NV];
-    #pragma unroll
-        for (int j = 0; j < NV; ++j) acc[j] = 0.0;
-        for (size_t i = (size_t)jf_bid * RB + threadIdx.x; i < n2; i += (size_t)jf_nblk * RB) {
-            const double2 a = w2[i];
-            double2 v[NV];
-    #pragma unroll
-            for (int j = 0; j < NV; ++j) v[j] = Vp[j][i];
-    #pragma unroll
-            for (int j = 0; j < NV; ++j) acc[j] = fma(v[j].y, a.y, fma(v[j].x, a.x, acc[j]));
-        }
-        store_multi<NV>(acc, part, jf_bid, jf_nblk);
-        if (!last_block(ticket, jf_nblk)) return;
-        finish_multi<NV>(part, jf_nblk, h);
-        __syncthreads();
-        if (threadIdx.x == 0) *ticket = 0u;
-    }
-};
-template <int NV>
-__global__ void __launch_bounds__(RB) k_gs_dot(const double *V, size_t ldv, const double *w, size_t n2,
-                                               double *part, unsigned *ticket, double *h) {
-    k_gs_dot_b<NV>::run(blockIdx.x, gridDim.x, V, ldv, w, n2, part, ticket, h);
-}
-
 // pass 2: w <- w - V h1, h2 = V^T w, w1sq = |w|^2, flag = (|w1| < |w0|/sqrt(2)),
 // nrm = |w| (final unless the third pass runs)
 template <int NV>
@@ -266,24 +251,9 @@ struct k_gs_update_dot_b {
         const double bs = block_sum(sq);
         if (threadIdx.x == 0) part[(size_t)NV * jf_nblk + jf_bid] = bs;
         if (!last_block(ticket, jf_nblk)) return;
-        finish_multi<NV>(part, jf_nblk, h2);
+        const double r2 = finish_multi<NV>(part, jf_nblk, h2);
         const double tot = sum_partials(part + (size_t)NV * jf_nblk, jf_nblk);
-        if (threadIdx.x == 0) {
-            double hh = 0.0, hh2 = 0.0;
-            for (int j = 0; j < NV; ++j) {
-                hh += h1[j] * h1[j];
-                hh2 += h2[j] * h2[j];
-            }
-            *w1sq = tot;
-            const bool second = tot < 0.5 * (tot + hh);
-            // |w2|^2 = |w1|^2 - |h2|^2 for w2 = w1 - V h2 with V orthonormal and h2 = V^T w1;
-            // after the first pass h2 is tiny against |w1|, so the difference does not cancel
-            const double nr = sqrt(second ? fmax(tot - hh2, 0.0) : tot);
-            nrm[0] = nr;
-            nrm[S_INV - S_NORM] = nr != 0.0 ? 1.0 / nr : 0.0;
-            *flag = second ? 1.0 : 0.0;
-            *ticket = 0u;
-        }
+        close_update(tot, threadIdx.x < NV ? h1[threadIdx.x] : 0.0, r2, w1sq, nrm, flag, ticket);
     }
 };
 template <int NV>
@@ -414,6 +384,179 @@ template <int NV>
 __global__ void __launch_bounds__(RB) k_gs_dot32(const float *V32, size_t ldv, const double *w, size_t n2,
                                                  double *part, unsigned *ticket, double *h) {
     k_gs_dot32_b<NV>::run(blockIdx.x, gridDim.x, V32, ldv, w, n2, part, ticket, h);
+}
+
+// The three passes for 17 to 32 basis vectors (nv at run time): the sums stay in
+// registers, the vectors are read in groups of four, in pass 2 once for the update and
+// again (from L1 / L2) for the sums.  The general multi-dot path took eight launches and
+// some 110 us of latency for such a column on a grid of 7,200 unknowns, these three 40.
+constexpr int LV = 32;
+template <class F>
+__device__ __forceinline__ void vec_groups(int nv, F f) {
+#pragma unroll
+    for (int j0 = 0; j0 < LV; j0 += 4)
+        if (j0 < nv) f(j0);
+}
+struct k_gsl_dot32_b {
+    static constexpr int TPB = RB, MINB = 0;
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const float *> V32, JfArg<int> nv,
+                                               JfArg<size_t> ldv, JfArg<const double *> w, JfArg<size_t> n2,
+                                               JfArg<double *> part, JfArg<unsigned *> ticket, JfArg<double *> h) {
+        jf_pdl_enter();
+        const double2 *w2 = reinterpret_cast<const double2 *>(w);
+        const size_t l2 = ldv / 2;
+        const float2 *V2 = reinterpret_cast<const float2 *>(V32);
+        float acc[LV];
+    #pragma unroll
+        for (int j = 0; j < LV; ++j) acc[j] = 0.0f;
+        for (size_t i = (size_t)jf_bid * RB + threadIdx.x; i < n2; i += (size_t)jf_nblk * RB) {
+            const double2 a = w2[i];
+            const float ax = d2f_trunc(a.x), ay = d2f_trunc(a.y);
+            vec_groups(nv, [&](int j0) {
+    #pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (j0 + j < nv) {
+                        const float2 v = V2[(size_t)(j0 + j) * l2 + i];
+                        acc[j0 + j] = fmaf(v.y, ay, fmaf(v.x, ax, acc[j0 + j]));
+                    }
+            });
+        }
+        __shared__ float sw[LV][RB / 32];
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    #pragma unroll
+        for (int j = 0; j < LV; ++j) {
+            float v = acc[j];
+    #pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) sw[j][wid] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x < nv) {
+            double r = 0.0;
+    #pragma unroll
+            for (int q = 0; q < RB / 32; ++q) r += (double)sw[threadIdx.x][q];
+            part[(size_t)threadIdx.x * jf_nblk + jf_bid] = r;
+        }
+        if (!last_block(ticket, jf_nblk)) return;
+        sum_rows(part, nv, jf_nblk, h);
+        __syncthreads();
+        if (threadIdx.x == 0) *ticket = 0u;
+    }
+    // h[j] = sum of row j of part, a warp per row in turn, fixed order
+    static __device__ __forceinline__ void sum_rows(const double *part, int nv, unsigned nb, double *h) {
+        const int lane = threadIdx.x & 31;
+        for (int j = threadIdx.x >> 5; j < nv; j += RB / 32) {
+            double a = 0.0;
+            for (unsigned b = lane; b < nb; b += 32) a += __ldcg(part + (size_t)j * nb + b);
+            a = warp_sum(a);
+            if (lane == 0) h[j] = a;
+        }
+    }
+};
+__global__ void __launch_bounds__(RB) k_gsl_dot32(const float *V32, int nv, size_t ldv, const double *w, size_t n2,
+                                                  double *part, unsigned *ticket, double *h) {
+    k_gsl_dot32_b::run(blockIdx.x, gridDim.x, V32, nv, ldv, w, n2, part, ticket, h);
+}
+struct k_gsl_update_dot_b {
+    static constexpr int TPB = RB, MINB = 0;
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const double *> V, JfArg<int> nv,
+                                               JfArg<size_t> ldv, JfArg<double *> w, JfArg<size_t> n2,
+                                               JfArg<const double *> h1, JfArg<double *> part, JfArg<unsigned *> ticket,
+                                               JfArg<double *> h2, JfArg<double *> w1sq, JfArg<double *> nrm,
+                                               JfArg<double *> flag) {
+        jf_pdl_enter();
+        __shared__ double sc[LV];
+        if (threadIdx.x < LV) sc[threadIdx.x] = threadIdx.x < nv ? -h1[threadIdx.x] : 0.0;
+        __syncthreads();
+        double2 *wv = reinterpret_cast<double2 *>(w);
+        const double2 *V2 = reinterpret_cast<const double2 *>(V);
+        const size_t l2 = ldv / 2;
+        double acc[LV];
+    #pragma unroll
+        for (int j = 0; j < LV; ++j) acc[j] = 0.0;
+        double sq = 0.0;
+        for (size_t i = (size_t)jf_bid * RB + threadIdx.x; i < n2; i += (size_t)jf_nblk * RB) {
+            double2 a = wv[i];
+            vec_groups(nv, [&](int j0) {
+                double2 v[4];
+    #pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = j0 + j < nv ? V2[(size_t)(j0 + j) * l2 + i] : make_double2(0.0, 0.0);
+    #pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    a.x = fma(sc[j0 + j], v[j].x, a.x);
+                    a.y = fma(sc[j0 + j], v[j].y, a.y);
+                }
+            });
+            wv[i] = a;
+            sq = fma(a.y, a.y, fma(a.x, a.x, sq));
+            vec_groups(nv, [&](int j0) {
+    #pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (j0 + j < nv) {
+                        const double2 v = V2[(size_t)(j0 + j) * l2 + i];
+                        acc[j0 + j] = fma(v.y, a.y, fma(v.x, a.x, acc[j0 + j]));
+                    }
+            });
+        }
+        store_multi<LV>(acc, part, jf_bid, jf_nblk);
+        const double bs = block_sum(sq);
+        if (threadIdx.x == 0) part[(size_t)LV * jf_nblk + jf_bid] = bs;
+        if (!last_block(ticket, jf_nblk)) return;
+        __shared__ double sh[LV];
+        if (threadIdx.x < LV) sh[threadIdx.x] = 0.0;
+        __syncthreads();
+        k_gsl_dot32_b::sum_rows(part, nv, jf_nblk, sh);
+        const double tot = sum_partials(part + (size_t)LV * jf_nblk, jf_nblk);   // synchronises
+        const double r2 = threadIdx.x < LV ? sh[threadIdx.x] : 0.0;
+        if (threadIdx.x < nv) h2[threadIdx.x] = r2;
+        close_update(tot, threadIdx.x < LV ? sc[threadIdx.x] : 0.0, r2, w1sq, nrm, flag, ticket);
+    }
+};
+__global__ void __launch_bounds__(RB) k_gsl_update_dot(const double *V, int nv, size_t ldv, double *w, size_t n2,
+                                                       const double *h1, double *part, unsigned *ticket, double *h2,
+                                                       double *w1sq, double *nrm, double *flag) {
+    k_gsl_update_dot_b::run(blockIdx.x, gridDim.x, V, nv, ldv, w, n2, h1, part, ticket, h2, w1sq, nrm, flag);
+}
+struct k_gsl_update_scale_b {
+    static constexpr int TPB = RB, MINB = 0;
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const double *> V, JfArg<int> nv,
+                                               JfArg<size_t> ldv, JfArg<double *> w, JfArg<float *> w32, JfArg<size_t> n2,
+                                               JfArg<const double *> h2, JfArg<const double *> flag,
+                                               JfArg<const double *> inv) {
+        jf_pdl_enter();
+        __shared__ double sc[LV];
+        if (threadIdx.x < LV) sc[threadIdx.x] = threadIdx.x < nv ? -h2[threadIdx.x] : 0.0;
+        __syncthreads();
+        const bool second = *flag != 0.0;
+        const double s = *inv;
+        double2 *wv = reinterpret_cast<double2 *>(w);
+        float2 *f2 = reinterpret_cast<float2 *>(w32);
+        const double2 *V2 = reinterpret_cast<const double2 *>(V);
+        const size_t l2 = ldv / 2;
+        for (size_t i = (size_t)jf_bid * RB + threadIdx.x; i < n2; i += (size_t)jf_nblk * RB) {
+            double2 a = wv[i];
+            if (second)
+                vec_groups(nv, [&](int j0) {
+                    double2 v[4];
+    #pragma unroll
+                    for (int j = 0; j < 4; ++j) v[j] = j0 + j < nv ? V2[(size_t)(j0 + j) * l2 + i] : make_double2(0.0, 0.0);
+    #pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        a.x = fma(sc[j0 + j], v[j].x, a.x);
+                        a.y = fma(sc[j0 + j], v[j].y, a.y);
+                    }
+                });
+            a.x *= s;
+            a.y *= s;
+            wv[i] = a;
+            if (w32) f2[i] = make_float2(d2f_trunc(a.x), d2f_trunc(a.y));
+        }
+    }
+};
+__global__ void __launch_bounds__(RB) k_gsl_update_scale(const double *V, int nv, size_t ldv, double *w, float *w32,
+                                                         size_t n2, const double *h2, const double *flag,
+                                                         const double *inv) {
+    k_gsl_update_scale_b::run(blockIdx.x, gridDim.x, V, nv, ldv, w, w32, n2, h2, flag, inv);
 }
 
 template <class S>
@@ -693,6 +836,23 @@ __global__ void __launch_bounds__(RB) k_eps32(const float *x, size_t n, double *
     k_eps32_b::run(blockIdx.x, gridDim.x, x, n, part, ticket, eps);
 }
 
+// eps = sqrt(2^-52)/|z| from the blocks' sums of squares of z (written with z by the
+// preconditioner's last smoothing step): one block
+struct k_eps_part_b {
+    static constexpr int TPB = RB, MINB = 0;
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const float *> part, JfArg<int> nb,
+                                               JfArg<double *> eps) {
+        jf_pdl_enter();
+        double acc = 0.0;
+        for (int i = threadIdx.x; i < nb; i += RB) acc += f2d_bits(part[i]);
+        acc = block_sum(acc);
+        if (threadIdx.x == 0) *eps = finish_op(acc, RED_EPS);
+    }
+};
+__global__ void __launch_bounds__(RB) k_eps_part(const float *part, int nb, double *eps) {
+    k_eps_part_b::run(blockIdx.x, gridDim.x, part, nb, eps);
+}
+
 struct YV {
     double y[MAXV];
 };
@@ -761,7 +921,9 @@ inline unsigned grid_for(size_t n) {
 // ~8 elements per thread: the FP64 shuffle tree (5 adds per value reduced)
 // stays small next to the per-element FMAs
 inline int nblocks_red(jfnk_ctx *c, size_t n) {
-    size_t g = (n + (size_t)RB * 8 - 1) / ((size_t)RB * 8);
+    // (two elements on short vectors: there the rounds of loads set the time)
+    const size_t per = n < (size_t)c->n_sm * RB * 8 ? 2 : 8;
+    size_t g = (n + (size_t)RB * per - 1) / ((size_t)RB * per);
     if (g > (size_t)c->nb_red) g = c->nb_red;
     if (g < 1) g = 1;
     return (int)g;
@@ -817,13 +979,8 @@ static void cgs2_t(jfnk_ctx *c, const double *V, const float *V32, size_t ldv, d
                    double *h1, double *h2, double *w1sq, double *nrm, double *flag, cudaStream_t s) {
     const size_t n2 = n / 2;
     const int g2 = one_wave(c, k_gs_update_dot<NV>, n2), g3 = one_wave(c, k_gs_update_scale<NV>, n2);
-    if (V32) {
-        const int g1 = one_wave(c, k_gs_dot32<NV>, n2);
-        jf_launch<k_gs_dot32_b<NV>>(k_gs_dot32<NV>, g1, RB, 0, s, V32, ldv, w, n2, c->partial, c->ticket, h1);
-    } else {
-        const int g1 = one_wave(c, k_gs_dot<NV>, n2);
-        jf_launch<k_gs_dot_b<NV>>(k_gs_dot<NV>, g1, RB, 0, s, V, ldv, w, n2, c->partial, c->ticket, h1);
-    }
+    const int g1 = one_wave(c, k_gs_dot32<NV>, n2);
+    jf_launch<k_gs_dot32_b<NV>>(k_gs_dot32<NV>, g1, RB, 0, s, V32, ldv, w, n2, c->partial, c->ticket, h1);
     jf_launch<k_gs_update_dot_b<NV>>(k_gs_update_dot<NV>, g2, RB, 0, s, V, ldv, w, n2, h1, c->partial, c->ticket, h2, w1sq, nrm, flag);
     jf_launch<k_gs_update_scale_b<NV>>(k_gs_update_scale<NV>, g3, RB, 0, s, V, ldv, w, w32, n2, h2, flag, nrm + (S_INV - S_NORM));
     jf_launched(3);
@@ -831,7 +988,18 @@ static void cgs2_t(jfnk_ctx *c, const double *V, const float *V32, size_t ldv, d
 
 int blas_cgs2(jfnk_ctx *c, const double *V, const float *V32, int nv, size_t ldv, double *w, float *w32, size_t n,
               double *h1, double *h2, double *w1sq, double *nrm, double *flag, cudaStream_t s) {
-    if (nv < 1 || nv > GS_FUSED_MAX || (n & 1) || (ldv & 1)) return JFNK_EINVAL;
+    if (nv < 1 || nv > GS_FUSED_MAX || (n & 1) || (ldv & 1) || !V32) return JFNK_EINVAL;
+    if (nv > 16) {
+        const size_t n2 = n / 2;
+        const int g1 = one_wave(c, k_gsl_dot32, n2), g2 = one_wave(c, k_gsl_update_dot, n2),
+                  g3 = one_wave(c, k_gsl_update_scale, n2);
+        jf_launch<k_gsl_dot32_b>(k_gsl_dot32, g1, RB, 0, s, V32, nv, ldv, w, n2, c->partial, c->ticket, h1);
+        jf_launch<k_gsl_update_dot_b>(k_gsl_update_dot, g2, RB, 0, s, V, nv, ldv, w, n2, h1, c->partial, c->ticket, h2, w1sq, nrm, flag);
+        jf_launch<k_gsl_update_scale_b>(k_gsl_update_scale, g3, RB, 0, s, V, nv, ldv, w, w32, n2, h2, flag, nrm + (S_INV - S_NORM));
+        jf_launched(3);
+        JF_CK(cudaGetLastError());
+        return JFNK_OK;
+    }
     switch (nv) {
 #define JF_GS(K) case K: cgs2_t<K>(c, V, V32, ldv, w, w32, n, h1, h2, w1sq, nrm, flag, s); break;
         JF_GS(1) JF_GS(2) JF_GS(3) JF_GS(4) JF_GS(5) JF_GS(6) JF_GS(7) JF_GS(8)
@@ -1016,6 +1184,14 @@ int blas_eps32(jfnk_ctx *c, const float *x, size_t n, double *eps_out, cudaStrea
     if ((uintptr_t)x & 15) return JFNK_EINVAL;
     const int nb = nblocks_red(c, n);
     jf_launch<k_eps32_b>(k_eps32, nb, RB, 0, s, x, n, c->partial, c->ticket, eps_out);
+    jf_launched();
+    JF_CK(cudaGetLastError());
+    return JFNK_OK;
+}
+
+int blas_eps_part(jfnk_ctx *c, const float *part, int nb, double *eps_out, cudaStream_t s) {
+    (void)c;
+    jf_launch<k_eps_part_b>(k_eps_part, 1, RB, 0, s, part, nb, eps_out);
     jf_launched();
     JF_CK(cudaGetLastError());
     return JFNK_OK;

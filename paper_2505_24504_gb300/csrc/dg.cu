@@ -799,7 +799,8 @@ struct k_dgtl_b {
             }
         }
         __syncthreads();
-        if (!active && !(FIRST && TR.b)) return;
+        if (!active && !(FIRST && TR.b) && !(MODE == DG_TLSMOOTH && A.npart)) return;
+        float sq = 0.0f;   // sum of squares of the new z
         const float lmxa = sl[0][a], lpxa = sl[1][a], dlmxa = sl[2][a], dlpxa = sl[3][a];
         const float lmzb = sl[4][b], lpzb = sl[5][b], dlmzb = sl[6][b], dlpzb = sl[7][b];
         const float adtf = A.adtf;
@@ -833,11 +834,27 @@ struct k_dgtl_b {
                 if (FIRST) out1f[gi] = z;
             } else {  // DG_TLSMOOTH
                 if (A.z0mode == 0) {
-                    ((float *)A.out0)[gi] = z + edt * (ef[v] - jz);
+                    const float zn = z + edt * (ef[v] - jz);
+                    ((float *)A.out0)[gi] = zn;
+                    sq = fmaf(zn, zn, sq);
                 } else {
                     const float st = (A.alphaf * edt) * (ef[v] - jz);
                     ((float *)A.out0)[gi] = A.z0mode == 1 ? ((const float *)A.z0)[gi] + st : st;
                 }
+            }
+        }
+        if (MODE == DG_TLSMOOTH && A.npart) {
+            // (blocks have E NP <= 128 threads: lanes past the end hold zero)
+            __shared__ float ssq[128];
+            __syncthreads();
+            ssq[threadIdx.x] = sq;
+            __syncthreads();
+            if (threadIdx.x < 32) {
+                float r = 0.0f;
+                for (int i = threadIdx.x; i < E * NP; i += 32) r += ssq[i];
+    #pragma unroll
+                for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(__activemask(), r, o);
+                if (threadIdx.x == 0) A.npart[jf_bid] = r;
             }
         }
         if (FIRST && TR.b) dgtl_transfer<NP1, E>(TR, sdf, smf, sg[0], le, node, ez, ex0 + le, active);

@@ -378,7 +378,20 @@ struct DGArgs {
     const void *z0;
     int z0mode;
     double alpha;
+    float *npart;          // FP32 smoothing: each block's sum of squares of the new z (may be null)
 };
+// blocks of the fused FP32 tangent product (k_dgtl), a strip of elements each
+inline int dgtl_blocks(const jfnk_ctx *c) {
+    const int np = c->np1 * c->np1, e = 128 / np > 0 ? 128 / np : 1;
+    return c->grid.nz * ((c->grid.nx + e - 1) / e);
+}
+// the blocks whose sums of squares the FP32 preconditioner leaves in c->partial with its
+// output (0: none; eps of the FD product then takes a pass over z)
+inline int mg_norm_blocks(const jfnk_ctx *c) {
+    const bool ok = c->mg_on && c->prec != 64 && c->dg_post > 0 && c->opts.dg_fused != 2 && c->opts.rk_stages == 1 &&
+                    c->opts.rk_alpha[0] == 1.0 && dgtl_blocks(c) <= c->nb_red * 32;
+    return ok ? dgtl_blocks(c) : 0;
+}
 
 int dg_apply(jfnk_ctx *c, int mode, const DGArgs &a, cudaStream_t s);
 size_t dg_member_bytes();
@@ -399,8 +412,8 @@ int blas_reortho_flag(const double *w1sq, const double *h, int nv, double *flag,
 int blas_mupdate_norm(jfnk_ctx *c, const double *V, int nv, size_t ldv, const double *h, double *w, size_t n,
                       double sign, const double *flag_in, double *w1sq, double *nrm, double *flag_out,
                       cudaStream_t s);
-constexpr int GS_FUSED_MAX = 16;   // basis vectors of the fused CGS2 kernels
-// V32 (optional): float copy of the basis (first pass in FP32); w32: where the
+constexpr int GS_FUSED_MAX = 32;   // basis vectors of the fused CGS2 kernels
+// V32: float copy of the basis (first pass in FP32); w32: where the
 // float copy of the normalised w goes (may be null)
 int blas_cgs2(jfnk_ctx *c, const double *V, const float *V32, int nv, size_t ldv, double *w, float *w32, size_t n,
               double *h1, double *h2, double *w1sq, double *nrm, double *flag, cudaStream_t s);
@@ -409,6 +422,7 @@ int blas_eps32(jfnk_ctx *c, const float *x, size_t n, double *eps_out, cudaStrea
 int blas_scale_copy(const double *w, const double *nrm_dev, double *v, size_t n, cudaStream_t s);
 int blas_axpby(double a, const double *x, double b, const double *y, double *z, size_t n, cudaStream_t s);
 int blas_zcomb(const void *Z, int prec32, int nz, size_t n, const double *yv, double *x, cudaStream_t s);
+int blas_eps_part(jfnk_ctx *c, const float *part, int nb, double *eps_out, cudaStream_t s);
 int blas_copy_d2f(const double *x, float *y, size_t n, cudaStream_t s);
 int blas_copy_f2d(const float *x, double *y, size_t n, cudaStream_t s);
 int blas_scale(double a, const double *x, double *y, size_t n, cudaStream_t s);

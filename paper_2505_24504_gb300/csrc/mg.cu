@@ -583,11 +583,14 @@ JF_D float wave_speed_r<float>(const float U[4], int D, const PhysC &P, const Po
     return fabsf(U[1 + D] * ir) + sqrtf(P.gammaf * p * ir);
 }
 
+// One launch per level of the linearisation: dtau of the level's cells and, by the thread
+// of each first child, the state of the next coarser level (mean of fac x fac children).
 template <class S>
-struct k_fv_dtau_b {
+struct k_fv_lin_b {
     static constexpr int TPB = 0, MINB = 0;
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<FVK> K, JfArg<const S *> u,
-                                               JfArg<double> adt, JfArg<double> sigma, JfArg<S *> dtau) {
+                                               JfArg<double> adt, JfArg<double> sigma, JfArg<S *> dtau, JfArg<int> fac,
+                                               JfArg<S *> uc, JfArg<int> bf16) {
         jf_pdl_enter();
         const int NX = K.NX, NZ = K.NZ;
         const size_t n1 = (size_t)NX * NZ;
@@ -606,30 +609,47 @@ struct k_fv_dtau_b {
         if (I < NX - 1 || K.periodic) { st(I < NX - 1 ? I + 1 : 0, Jz, V); eE = fmax(sx, wave_speed_r<S>(V, 0, K.pc, K.pt)); }
         if (Jz > 0) { st(I, Jz - 1, V); eS = fmax(sz, wave_speed_r<S>(V, 1, K.pc, K.pt)); }
         if (Jz < NZ - 1) { st(I, Jz + 1, V); eN = fmax(sz, wave_speed_r<S>(V, 1, K.pc, K.pt)); }
-        const S iHx = (S)K.iHx, iHz = (S)K.iHz;
-        const S lam = (S)0.5 * (eW + eE) * iHx + (S)0.5 * (eS + eN) * iHz + (S)(2.0 * K.mu) * (iHx * iHx + iHz * iHz);
+        const S iHx = pick<S>(K.iHx, K.iHxf), iHz = pick<S>(K.iHz, K.iHzf);
+        const S lam = (S)0.5 * (eW + eE) * iHx + (S)0.5 * (eS + eN) * iHz +
+                      pick<S>(2.0 * K.mu, 2.0f * K.pc.muf) * (iHx * iHx + iHz * iHz);
         dtau[c] = (S)sigma / ((S)1 + (S)adt * lam);
+        if (!uc || I % fac || Jz % fac) return;
+        const int NXc = NX / fac, NZc = NZ / fac;
+        const size_t nc = (size_t)NXc * NZc, cc = (size_t)(Jz / fac) * NXc + I / fac;
+        if (I / fac >= NXc || Jz / fac >= NZc) return;
+        for (int v = 0; v < 4; ++v) {
+            const S *f = u + (size_t)v * n1 + c;
+            S acc = 0;
+            for (int jj = 0; jj < fac; ++jj)
+                for (int ii = 0; ii < fac; ++ii) acc += f[(size_t)jj * NX + ii];
+            uc[(size_t)v * nc + cc] = store_round<S>(acc / (S)(fac * fac), bf16);
+        }
     }
 };
 template <class S>
-__global__ void k_fv_dtau(FVK K, const S *u, double adt, double sigma, S *dtau) {
-    k_fv_dtau_b<S>::run(blockIdx.x, gridDim.x, K, u, adt, sigma, dtau);
+__global__ void k_fv_lin(FVK K, const S *u, double adt, double sigma, S *dtau, int fac, S *uc, int bf16) {
+    k_fv_lin_b<S>::run(blockIdx.x, gridDim.x, K, u, adt, sigma, dtau, fac, uc, bf16);
 }
 
-// DG pseudo-time step per element: lambda_E = (k+1)^2 max_nodes(|v| + c)(1/hx + 1/hz)
-// + 2 mu (k+1)^4 (1/hx^2 + 1/hz^2).  A block takes as many elements as its threads hold
-// nodes; the FP64 closing formula runs in the first threads, one per element (one
-// element per warp paid for a whole warp's FP64 slots: 21 us on 12,800 Q3 elements, 7.0 now).
-template <class R>
+// DG pseudo-time step of an element, lambda_E = (k+1)^2 max_nodes(|v| + c)(1/hx + 1/hz)
+// + 2 mu (k+1)^4 (1/hx^2 + 1/hz^2)
+JF_D double dg_dtau_of(double vmax, int np1, double ihx, double ihz, double mu, double adt, double sigma) {
+    const double n2 = (double)np1 * np1;
+    const double lam = n2 * vmax * (ihx + ihz) + 2.0 * mu * n2 * n2 * (ihx * ihx + ihz * ihz);
+    return div64(sigma, 1.0 + adt * lam);
+}
+// The same for the FP64 preconditioner.  A block takes as many elements as its threads hold
+// nodes; the closing formula runs in the first threads, one per element.  (The FP32
+// preconditioner's steps come with the transfer of the state, k_to_fv.)
 struct k_dg_dtau_b {
     static constexpr int TPB = 256, MINB = 0;
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const R *> U,
-                                               JfArg<const R *> ubv, JfArg<int> nx, JfArg<int> nz, JfArg<int> np1,
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const double *> U,
+                                               JfArg<const double *> ubv, JfArg<int> nx, JfArg<int> nz, JfArg<int> np1,
                                                JfArg<PhysC> pc, JfArg<const PowTab *> pt, JfArg<double> ihx,
                                                JfArg<double> ihz, JfArg<double> mu, JfArg<double> adt,
-                                               JfArg<double> sigma, JfArg<double *> dtau, JfArg<float *> dtauf) {
+                                               JfArg<double> sigma, JfArg<double *> dtau) {
         jf_pdl_enter();
-        __shared__ R ssp[256];
+        __shared__ double ssp[256];
         const int n_el = nx * nz;
         const int NP = np1 * np1, E = 256 / NP;
         const int le = threadIdx.x / NP, node = threadIdx.x % NP;
@@ -638,39 +658,24 @@ struct k_dg_dtau_b {
         const size_t nrow = (size_t)nz * np1;
         if (le < E && e < n_el) {
             const int J = (e / nx) * np1 + node / np1;
-            R W[4], sp;
+            double W[4];
             for (int v = 0; v < 4; ++v) W[v] = U[v * N1 + (size_t)e * NP + node] + ubv[v * nrow + J];
-            if (sizeof(R) == 8) {
-                const double ir = 1.0 / (double)W[0];
-                const double p = eos_pow((double)W[3], pt);
-                sp = (R)(sqrt(((double)W[1] * ir) * ((double)W[1] * ir) + ((double)W[2] * ir) * ((double)W[2] * ir)) +
-                         sqrt(pc.gamma * p * ir));
-            } else {
-                const float ir = 1.0f / (float)W[0];
-                const float p = pc.p0f * __powf(pc.R_over_p0f * (float)W[3], pc.gammaf);
-                sp = (R)(sqrtf(((float)W[1] * ir) * ((float)W[1] * ir) + ((float)W[2] * ir) * ((float)W[2] * ir)) +
-                         sqrtf(pc.gammaf * p * ir));
-            }
-            ssp[threadIdx.x] = sp;
+            const double ir = rcp64(W[0]);
+            const double p = eos_pow(W[3], pt);
+            ssp[threadIdx.x] = sqrt64((W[1] * ir) * (W[1] * ir) + (W[2] * ir) * (W[2] * ir)) + sqrt64(pc.gamma * p * ir);
         }
         __syncthreads();
         const int el = threadIdx.x;
         if (el >= E || e0 + el >= n_el) return;
-        R sm = 0;
+        double sm = 0.0;
         for (int q = 0; q < NP; ++q) sm = fmax(sm, ssp[el * NP + q]);
-        const double vmax = (double)sm;
-        const double n2 = (double)np1 * np1;
-        const double lam = n2 * vmax * (ihx + ihz) + 2.0 * mu * n2 * n2 * (ihx * ihx + ihz * ihz);
-        const double d = sigma / (1.0 + adt * lam);
-        if (dtau) dtau[e0 + el] = d;
-        if (dtauf) dtauf[e0 + el] = (float)d;
+        dtau[e0 + el] = dg_dtau_of(sm, np1, ihx, ihz, mu, adt, sigma);
     }
 };
-template <class R>
-__global__ void __launch_bounds__(256) k_dg_dtau(const R *U, const R *ubv, int nx, int nz, int np1, PhysC pc, const PowTab *pt,
-                          double ihx, double ihz, double mu, double adt, double sigma, double *dtau,
-                          float *dtauf) {
-    k_dg_dtau_b<R>::run(blockIdx.x, gridDim.x, U, ubv, nx, nz, np1, pc, pt, ihx, ihz, mu, adt, sigma, dtau, dtauf);
+__global__ void __launch_bounds__(256) k_dg_dtau(const double *U, const double *ubv, int nx, int nz, int np1, PhysC pc,
+                                                 const PowTab *pt, double ihx, double ihz, double mu, double adt,
+                                                 double sigma, double *dtau) {
+    k_dg_dtau_b::run(blockIdx.x, gridDim.x, U, ubv, nx, nz, np1, pc, pt, ihx, ihz, mu, adt, sigma, dtau);
 }
 
 // ---- transfer -------------------------------------------------------------
@@ -691,15 +696,27 @@ __device__ __forceinline__ void load_ttab(const TK &K, R sV[NP1][NP1], R sVi[NP1
     for (int t = threadIdx.x; t < NP1; t += blockDim.x) som[t] = (R)K.tab.om[t];
 }
 
+// What the FP32 linearisation takes along with the transfer of the state: the context's
+// FP64 and FP32 copies of U and the DG pseudo-time steps.  One launch instead of a copy, a
+// conversion, the step sizes and the transfer, each a pass over the state.
+struct LinOut {
+    double *Ul;          // null: a plain transfer
+    float *Uf, *dtauf;
+    const float *ubvf;
+    PhysC pc;
+    double ihx, ihz, mu, adt, sigma;
+};
+
 // T^mf: DG (Si) -> FV (So), arithmetic in the storage precision.  Block: EPB
 // elements x NP subcells.
 template <class Si, class So, int NP1>
 struct k_to_fv_b {
     static constexpr int TPB = 128, MINB = 0;
     static constexpr bool GROUP = std::is_same<So, float>::value;   // a grouped twin is built (lock-step ensembles)
+    static constexpr bool LIN = std::is_same<Si, double>::value && std::is_same<So, float>::value;
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<TK> K, JfArg<const Si *> u,
                                                JfArg<So *> v, JfArg<int> massfix, JfArg<So *> x0,
-                                               JfArg<const So *> dtau0) {
+                                               JfArg<const So *> dtau0, JfArg<LinOut> lo) {
         jf_pdl_enter();
         typedef typename RealOf<Si, So>::type R;
         constexpr int NP = NP1 * NP1;
@@ -714,9 +731,35 @@ struct k_to_fv_b {
         const bool act = e < K.n_el;
         const size_t N1 = (size_t)K.n_el * NP;
         const int i = node % NP1, j = node / NP1;   // subcell (i along x, j along z) / node (a, b)
-        if (act)
-            for (int q = 0; q < 4; ++q) su[le][q][node] = (R)u[q * N1 + (size_t)e * NP + node];
+        __shared__ float ssp[LIN ? EPB * NP : 1];   // |v| + c at the nodes
+        if (act) {
+            float W[4];
+            for (int q = 0; q < 4; ++q) {
+                const size_t gi = q * N1 + (size_t)e * NP + node;
+                const Si ui = u[gi];
+                su[le][q][node] = (R)ui;
+                if (LIN) {
+                    lo.Ul[gi] = ui;
+                    lo.Uf[gi] = (float)ui;
+                    W[q] = (float)ui + lo.ubvf[q * (K.nz * NP1) + (e / K.nx) * NP1 + node / NP1];
+                }
+            }
+            if (LIN) {
+                const float ir = 1.0f / W[0];
+                const float p = lo.pc.p0f * __powf(lo.pc.R_over_p0f * W[3], lo.pc.gammaf);
+                ssp[threadIdx.x] = sqrtf((W[1] * ir) * (W[1] * ir) + (W[2] * ir) * (W[2] * ir)) +
+                                   sqrtf(lo.pc.gammaf * p * ir);
+            }
+        }
         __syncthreads();
+        if (LIN) {   // the closing FP64 formula once per element
+            const int el = threadIdx.x, e1 = jf_bid * EPB + el;
+            if (el < EPB && e1 < K.n_el) {
+                float sm = 0.0f;
+                for (int q = 0; q < NP; ++q) sm = fmaxf(sm, ssp[el * NP + q]);
+                lo.dtauf[e1] = (float)dg_dtau_of((double)sm, NP1, lo.ihx, lo.ihz, lo.mu, lo.adt, lo.sigma);
+            }
+        }
         // t1(i, b) = sum_a V[i][a] u(a, b), stored at [b][i]
         if (act)
             for (int q = 0; q < 4; ++q) {
@@ -763,8 +806,8 @@ struct k_to_fv_b {
     }
 };
 template <class Si, class So, int NP1>
-__global__ void __launch_bounds__(128) k_to_fv(TK K, const Si *u, So *v, int massfix, So *x0, const So *dtau0) {
-    k_to_fv_b<Si, So, NP1>::run(blockIdx.x, gridDim.x, K, u, v, massfix, x0, dtau0);
+__global__ void __launch_bounds__(128) k_to_fv(TK K, const Si *u, So *v, int massfix, So *x0, const So *dtau0, LinOut lo) {
+    k_to_fv_b<Si, So, NP1>::run(blockIdx.x, gridDim.x, K, u, v, massfix, x0, dtau0, lo);
 }
 
 // T^-1_mf: FV (Si) -> DG (So); acc 0: store, 1: add
@@ -836,32 +879,6 @@ struct k_to_dg_b {
 template <class Si, class So, int NP1>
 __global__ void __launch_bounds__(128) k_to_dg(TK K, const Si *v, So *u, int massfix, int acc_mode) {
     k_to_dg_b<Si, So, NP1>::run(blockIdx.x, gridDim.x, K, v, u, massfix, acc_mode);
-}
-
-// R: coarse = mean of fac x fac children
-template <class S>
-struct k_restrict_body {
-    static constexpr int TPB = 0, MINB = 0;
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const S *> f, JfArg<int> NXf,
-                                               JfArg<int> NZf, JfArg<int> fac, JfArg<S *> cz) {
-        jf_pdl_enter();
-        const int NXc = NXf / fac, NZc = NZf / fac;
-        const size_t nc = (size_t)NXc * NZc;
-        const size_t t = (size_t)jf_bid * blockDim.x + threadIdx.x;
-        if (t >= 4 * nc) return;
-        const int q = (int)(t / nc);
-        const size_t c = t % nc;
-        const int I = (int)(c % NXc), J = (int)(c / NXc);
-        const S *fq = f + (size_t)q * NXf * NZf;
-        S acc = 0;
-        for (int jj = 0; jj < fac; ++jj)
-            for (int ii = 0; ii < fac; ++ii) acc += fq[(size_t)(J * fac + jj) * NXf + I * fac + ii];
-        cz[t] = acc / (S)(fac * fac);
-    }
-};
-template <class S>
-__global__ void k_restrict(const S *f, int NXf, int NZf, int fac, S *cz) {
-    k_restrict_body<S>::run(blockIdx.x, gridDim.x, f, NXf, NZf, fac, cz);
 }
 
 // R plus the coarse level's first pseudo-time step from zero: b_c = R r and,
@@ -1067,16 +1084,17 @@ TK make_tk(jfnk_ctx *c) {
 }
 
 template <class Si, class So>
-int to_fv(jfnk_ctx *c, const Si *u, So *v, cudaStream_t s, So *x0 = nullptr, const So *dtau0 = nullptr) {
+int to_fv(jfnk_ctx *c, const Si *u, So *v, cudaStream_t s, So *x0 = nullptr, const So *dtau0 = nullptr,
+          LinOut lo = LinOut{}) {
     TK K = make_tk(c);
     const int NP = c->np1 * c->np1;
     const int EPB = (128 / NP) > 0 ? 128 / NP : 1;
     const unsigned g = (unsigned)((c->n_el + EPB - 1) / EPB);
     switch (c->np1) {
-        case 2: jf_launch<k_to_fv_b<Si, So, 2>>(k_to_fv<Si, So, 2>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0); jf_launched(); break;
-        case 3: jf_launch<k_to_fv_b<Si, So, 3>>(k_to_fv<Si, So, 3>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0); jf_launched(); break;
-        case 4: jf_launch<k_to_fv_b<Si, So, 4>>(k_to_fv<Si, So, 4>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0); jf_launched(); break;
-        case 5: jf_launch<k_to_fv_b<Si, So, 5>>(k_to_fv<Si, So, 5>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0); jf_launched(); break;
+        case 2: jf_launch<k_to_fv_b<Si, So, 2>>(k_to_fv<Si, So, 2>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo); jf_launched(); break;
+        case 3: jf_launch<k_to_fv_b<Si, So, 3>>(k_to_fv<Si, So, 3>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo); jf_launched(); break;
+        case 4: jf_launch<k_to_fv_b<Si, So, 4>>(k_to_fv<Si, So, 4>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo); jf_launched(); break;
+        case 5: jf_launch<k_to_fv_b<Si, So, 5>>(k_to_fv<Si, So, 5>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo); jf_launched(); break;
         default: return JFNK_EINVAL;
     }
     JF_CK(cudaGetLastError());
@@ -1423,10 +1441,10 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
 inline int fd_lin(const jfnk_ctx *c) { return c->opts.precond_fd_eps == 0.0; }
 
 template <class S>
-int dg_smooth_step(jfnk_ctx *c, const S *r, S *&z, S *&z2, bool &zero, cudaStream_t s);
+int dg_smooth_step(jfnk_ctx *c, const S *r, S *&z, S *&z2, bool &zero, cudaStream_t s, bool last = false);
 
 template <>
-int dg_smooth_step<double>(jfnk_ctx *c, const double *r, double *&z, double *&z2, bool &zero, cudaStream_t s) {
+int dg_smooth_step<double>(jfnk_ctx *c, const double *r, double *&z, double *&z2, bool &zero, cudaStream_t s, bool) {
     const int NP = c->np1 * c->np1;
     if (zero) {
         jf_launch<k_scale_dtau_dg_b<double>>(k_scale_dtau_dg<double>, nblk(c->N, 256), 256, 0, s, z, r, c->dtau_dg, c->npt, NP, 1.0); jf_launched();
@@ -1453,7 +1471,7 @@ int dg_smooth_step<double>(jfnk_ctx *c, const double *r, double *&z, double *&z2
 }
 
 template <>
-int dg_smooth_step<float>(jfnk_ctx *c, const float *r, float *&z, float *&z2, bool &zero, cudaStream_t s) {
+int dg_smooth_step<float>(jfnk_ctx *c, const float *r, float *&z, float *&z2, bool &zero, cudaStream_t s, bool last) {
     const int NP = c->np1 * c->np1;
     if (zero) {
         jf_launch<k_scale_dtau_dg_b<float>>(k_scale_dtau_dg<float>, nblk(c->N, 256), 256, 0, s, z, r, c->dtau_dgf, c->npt, NP, 1.0); jf_launched();
@@ -1469,6 +1487,7 @@ int dg_smooth_step<float>(jfnk_ctx *c, const float *r, float *&z, float *&z2, bo
     a.dtauf = c->dtau_dgf;
     a.adt = c->mg_adt;
     a.out0 = z2;
+    a.npart = last && mg_norm_blocks(c) ? (float *)c->partial : nullptr;
     JF_RET(dg_apply(c, DG_TLSMOOTH, a, s));
     float *t = z;
     z = z2;
@@ -1637,7 +1656,7 @@ int apply_t(jfnk_ctx *c, const S *r, S *zout, cudaStream_t s) {
             continue;
         }
         if (i == c->dg_post - 1) z2 = zout;   // the last step writes the output itself
-        JF_RET(dg_smooth_step<S>(c, r, z, z2, zero, s));
+        JF_RET(dg_smooth_step<S>(c, r, z, z2, zero, s, i == c->dg_post - 1));
     }
     if (c->dg_post == 0) JF_CK(jf_memcpy(zout, z, c->N * sizeof(S), cudaMemcpyDeviceToDevice, s));
     for (int l = 0; l < c->nlev; ++l) {
@@ -1662,51 +1681,39 @@ int fv_setup_background(jfnk_ctx *c, cudaStream_t s) {
 }
 
 int mg_linearize(jfnk_ctx *c, const double *Uin, double adt, cudaStream_t s) {
-    // every pointer the captured graph holds is context-owned
-    JF_CK(jf_memcpy(c->Ulin, Uin, 8 * c->N, cudaMemcpyDeviceToDevice, s));
-    const double *U = c->Ulin;
+    // every pointer the captured graph holds is context-owned: Ulin is the copy of U
     c->mg_adt = adt;
-    c->mg_U = U;
-    // DG pseudo-time steps: FP64 for the FP64 preconditioner, FP32 from the FP32
-    // copy of the state otherwise (a step-size heuristic)
-    const int epb = 256 / (c->np1 * c->np1);
-    const unsigned gd = (unsigned)((c->n_el + epb - 1) / epb);
+    c->mg_U = c->Ulin;
     if (c->prec == 64) {
-        jf_launch<k_dg_dtau_b<double>>(k_dg_dtau<double>, gd, 256, 0, s, U, (const double *)c->ubv, c->grid.nx, c->grid.nz, c->np1,
-                  c->pc, c->powtab, 1.0 / c->hx, 1.0 / c->hz, c->phys.mu, adt, c->opts.sigma_dg, c->dtau_dg,
-                  c->dtau_dgf);
+        JF_CK(jf_memcpy(c->Ulin, Uin, 8 * c->N, cudaMemcpyDeviceToDevice, s));
+        const double *U = c->Ulin;
+        const int epb = 256 / (c->np1 * c->np1);
+        jf_launch<k_dg_dtau_b>(k_dg_dtau, (unsigned)((c->n_el + epb - 1) / epb), 256, 0, s, U, (const double *)c->ubv, c->grid.nx,
+                  c->grid.nz, c->np1, c->pc, c->powtab, 1.0 / c->hx, 1.0 / c->hz, c->phys.mu, adt, c->opts.sigma_dg,
+                  c->dtau_dg);
         jf_launched();
         JF_CK(cudaGetLastError());
         JF_RET(to_fv<double, double>(c, U, (double *)c->lev[0].u, s));
     } else {
-        JF_RET(blas_copy_d2f(U, c->Usf, c->N, s));
-        jf_launch<k_dg_dtau_b<float>>(k_dg_dtau<float>, gd, 256, 0, s, (const float *)c->Usf, (const float *)c->ubvf, c->grid.nx,
-                  c->grid.nz, c->np1, c->pc, c->powtab, 1.0 / c->hx, 1.0 / c->hz, c->phys.mu, adt,
-                  c->opts.sigma_dg, c->dtau_dg, c->dtau_dgf);
-        jf_launched();
-        JF_CK(cudaGetLastError());
-        JF_RET(to_fv<double, float>(c, U, (float *)c->lev[0].u, s));
+        JF_RET(to_fv<double, float>(c, Uin, (float *)c->lev[0].u, s, nullptr, nullptr,
+                                    LinOut{c->Ulin, c->Usf, c->dtau_dgf, c->ubvf, c->pc, 1.0 / c->hx, 1.0 / c->hz,
+                                           c->phys.mu, adt, c->opts.sigma_dg}));
     }
     for (int l = 0; l < c->nlev; ++l) {
         FVLev &L = c->lev[l];
         FVK K = make_fvk(c, l);
         const size_t n1 = (size_t)L.NX * L.NZ;
-        if (l > 0) {
-            FVLev &F = c->lev[l - 1];
-            if (c->prec == 64)
-                jf_launch<k_restrict_body<double>>(k_restrict<double>, nblk(L.n, 256), 256, 0, s, (const double *)F.u, F.NX, F.NZ, F.fac, (double *)L.u);
-            else
-                jf_launch<k_restrict_b_b<float>>(k_restrict_b<float>, nblk(L.n, 256), 256, 0, s, (const float *)F.u, F.NX, F.NZ, F.fac, (float *)L.u,
-                                                                   nullptr, nullptr,
-                                                                   (c->prec == 16 && l == c->nlev - 1) ? 1 : 0);
-            jf_launched();
-        }
+        void *uc = l + 1 < c->nlev ? c->lev[l + 1].u : nullptr;
+        const int bf = (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0;
         if (c->prec == 64) {
             JF_RET(fv_op64(c, l, FV_RES, (const double *)L.u, nullptr, nullptr, (double *)L.fu, s));
-            jf_launch<k_fv_dtau_b<double>>(k_fv_dtau<double>, nblk(n1), 128, 0, s, K, (const double *)L.u, adt, c->opts.sigma_fv, (double *)L.dtau); jf_launched();
+            jf_launch<k_fv_lin_b<double>>(k_fv_lin<double>, nblk(n1), 128, 0, s, K, (const double *)L.u, adt, c->opts.sigma_fv,
+                      (double *)L.dtau, L.fac, (double *)uc, 0);
         } else {
-            jf_launch<k_fv_dtau_b<float>>(k_fv_dtau<float>, nblk(n1), 128, 0, s, K, (const float *)L.u, adt, c->opts.sigma_fv, (float *)L.dtau); jf_launched();
+            jf_launch<k_fv_lin_b<float>>(k_fv_lin<float>, nblk(n1), 128, 0, s, K, (const float *)L.u, adt, c->opts.sigma_fv,
+                      (float *)L.dtau, L.fac, (float *)uc, bf);
         }
+        jf_launched();
         JF_CK(cudaGetLastError());
     }
     return JFNK_OK;
@@ -1790,7 +1797,7 @@ int mg_apply(jfnk_ctx *c, const double *r, void *z, cudaStream_t s, const float 
     } else {
         JF_RET(apply_body(c, s));
     }
-    JF_CK(jf_memcpy(z, c->pout, sS * c->N, cudaMemcpyDeviceToDevice, s));
+    if (z) JF_CK(jf_memcpy(z, c->pout, sS * c->N, cudaMemcpyDeviceToDevice, s));   // null: the result stays in pout
     return JFNK_OK;
 }
 
