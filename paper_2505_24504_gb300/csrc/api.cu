@@ -145,6 +145,7 @@ size_t workspace(const jfnk_grid *g, int k, const jfnk_opts *o, const jfnk_physi
     const bool visc = ph ? ph->mu != 0.0 : true;
     b += 8 * (4 + (visc ? 6 : 0)) * (fx + fz);
     if (prec != 64) b += 4 * (4 + (visc ? 6 : 0)) * (fx + fz);
+    if (prec != 64 && o->dg_fused != 2 && !(ph && visc)) b += 128 * (fx + fz) + 4 * N;   // FP32 flux derivatives
     b += 8 * N * 9;                        // DG work vectors
     b += 12 * N * (size_t)(m + 1);         // V and its float copy
     const bool mg_on = o->mg_key[0] != 0;
@@ -438,6 +439,10 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
     if (c->prec != 64) {
         A_(c->dtau_dgf, 4 * (size_t)c->n_el);
         A_(c->Usf, 4 * N);
+        if (!visc && o.dg_fused != 2) {
+            A_(c->jac, 4 * 32 * (fx + fz));
+            A_(c->jacn, 4 * N);
+        }
         A_(c->ubvf, 4 * 4 * nrow);
         A_(c->dubvf, 4 * 4 * nrow);
         A_(c->ubhf, 4 * 4 * nf);
@@ -655,6 +660,7 @@ int jfnk_tangent_product(jfnk_ctx *c, const double *U, const double *y, double a
     a.yf = (const float *)c->pz;
     a.adt = adt;
     a.out0 = c->pz2;
+    if (c->jac) JF_RET(dg_apply(c, DG_TLLIN, a, s));
     JF_RET(dg_apply(c, DG_TLJV, a, s));
     return blas_copy_f2d((const float *)c->pz2, out, c->N, s);
 }
@@ -693,6 +699,7 @@ int jfnk_time_operator(jfnk_ctx *c, int which, const double *U, const double *y,
         if (!rc) rc = blas_copy_d2f(U, c->Usf, c->N, s);
         a.yf = (const float *)c->pz;
         a.Uf = c->Usf;
+        if (!rc && c->jac) rc = dg_apply(c, DG_TLLIN, a, s);
     }
     a.out0 = which == 2 ? (void *)c->pz2 : (void *)c->w2;
     c->t_faces_ms = c->t_volume_ms = 0.0;

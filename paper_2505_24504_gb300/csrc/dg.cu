@@ -493,10 +493,15 @@ __global__ void __launch_bounds__(128, 8)
 // cost less than a second launch and the face buffers' round trip.
 // FIRST = 1 (defect mode): the direction is the first pseudo-time step from zero,
 // z = dtau_E r, formed on the fly; the epilogue also writes that z to out1f.
-template <int NP1> struct StripOf {
-    static constexpr int NP = NP1 * NP1;
-    static constexpr int E = (128 / NP) > 0 ? 128 / NP : 1;
-};
+
+// Padding of an element's staged values [variable][node] in shared memory, in elements of
+// `words` 32-bit words: with the plain stride 4 (k+1)^2 the face points of a strip's
+// elements read the same banks (6 ways on Q3, 8 on Q1); these paddings minimise the
+// conflicts over the face points of a block (1.4 to 1.8 ways, counted on the host for
+// every padding below 33).
+constexpr int strip_pad(int np1, int words) {
+    return words == 1 ? (np1 == 2 ? 2 : np1 == 4 ? 9 : np1 == 5 ? 3 : 0) : (np1 == 2 ? 2 : 5);
+}
 
 // T^mf of the strip's defect (in sd) to the finest FV level: the 1D transfer
 // matrix along x, then along z (through the scratch st), the mass fix from the
@@ -568,12 +573,14 @@ struct k_dgtl_b {
                                                JfArg<float *> out1f, JfArg<TransferOut> TR) {
         jf_pdl_enter();
         constexpr int NP = NP1 * NP1;
-        constexpr int E = StripOf<NP1>::E;
+        constexpr int E = strip_elems(NP1, VISC);
         // U' (value, tangent) of the strip's elements [1], of the elements below [0] and
         // above [2] them, and of the strip's west [0] and east [1] neighbours: every
         // trace the faces need comes from shared memory, loaded coalesced up front
-        __shared__ TL32 sn[3][E][4][NP];
-        __shared__ TL32 se[2][4][NP];
+        // (an element's values [variable][node], padded: see strip_pad)
+        constexpr int S = 4 * NP + strip_pad(NP1, 2);
+        __shared__ TL32 sn[3][E][S];
+        __shared__ TL32 se[2][S];
         __shared__ float sg[2][E][4][NP];              // volume fluxes (tangent part)
         __shared__ float sPx[E + 1][4][NP1];           // x-face terms Phi (face f west of strip element f)
         __shared__ float sPz[2][E][4][NP1];            // z-face terms: [0] bottom, [1] top of element le
@@ -604,11 +611,11 @@ struct k_dgtl_b {
         const int e = ez * nx + ex0 + le;
         // direction at a node: y (or dtau_E r for the first step from zero)
         auto dir = [&](int el, size_t i) -> float { return FIRST ? A.dtauf[el] * A.rf[i] : A.yf[i]; };
-        auto load = [&](int el, TL32 (*dst)[NP]) {
+        auto load = [&](int el, TL32 *dst) {
     #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 const size_t gi = (size_t)v * N1 + (size_t)el * NP + node;
-                dst[v][node] = TL32{A.Uf[gi], dir(el, gi)};
+                dst[v * NP + node] = TL32{A.Uf[gi], dir(el, gi)};
             }
         };
         float ef[4] = {0.f, 0.f, 0.f, 0.f}, edt = 0.0f;
@@ -634,7 +641,7 @@ struct k_dgtl_b {
             TL32 U[4];
     #pragma unroll
             for (int v = 0; v < 4; ++v) {
-                Up[v] = sn[1][le][v][node];
+                Up[v] = sn[1][le][v * NP + node];
                 U[v] = Up[v] + TLc{K.ubvf[v * nrow + J]};
             }
             const TL32 ir = jrcp(U[0]);
@@ -649,8 +656,8 @@ struct k_dgtl_b {
                     TL32 sx = mk(0.0, TL32{}), sz = mk(0.0, TL32{});
     #pragma unroll
                     for (int q = 0; q < NP1; ++q) {
-                        sx = jfma(TLc{sDn[a][q]}, sn[1][le][v][b * NP1 + q], sx);
-                        sz = jfma(TLc{sDn[b][q]}, sn[1][le][v][q * NP1 + a], sz);
+                        sx = jfma(TLc{sDn[a][q]}, sn[1][le][v * NP + b * NP1 + q], sx);
+                        sz = jfma(TLc{sDn[b][q]}, sn[1][le][v * NP + q * NP1 + a], sz);
                     }
                     dx[v] = TLc{K.two_hxf} * sx;
                     dz[v] = TLc{K.two_hzf} * sz + TLc{K.dubvf[v * nrow + J]};
@@ -672,13 +679,13 @@ struct k_dgtl_b {
         // ---- faces ------------------------------------------------------------
         // value and derivative traces of variable v along NP1 nodes i0 + q st of one
         // element's staged nodes, in the order of line_trace
-        auto trace = [&](const TL32 (*src)[NP], int v, int i0, int st, const float *pa, const float *pd, TL32 &tv,
+        auto trace = [&](const TL32 *src, int v, int i0, int st, const float *pa, const float *pd, TL32 &tv,
                          TL32 &td) {
             tv = mk(0.0, TL32{});
             td = mk(0.0, TL32{});
     #pragma unroll
             for (int q = 0; q < NP1; ++q) {
-                const TL32 u = src[v][i0 + q * st];
+                const TL32 u = src[v * NP + i0 + q * st];
                 tv = jfma(TLc{pa[q]}, u, tv);
                 if (VISC) td = jfma(TLc{pd[q]}, u, td);
             }
@@ -689,8 +696,8 @@ struct k_dgtl_b {
             if (t < nxf) {
                 const int f = t / NP1, sp = t % NP1;      // face f lies west of strip element f
                 const bool wallL = f == 0 && !has_w, wallR = f == Ev && !has_e;
-                const TL32 (*srcL)[NP] = f > 0 ? sn[1][f - 1] : se[0];
-                const TL32 (*srcR)[NP] = f < Ev ? sn[1][f] : se[1];
+                const TL32 *srcL = f > 0 ? sn[1][f - 1] : se[0];
+                const TL32 *srcR = f < Ev ? sn[1][f] : se[1];
                 const int J = ez * NP1 + sp;
     #pragma unroll
                 for (int v = 0; v < 4; ++v) {
@@ -865,6 +872,305 @@ __global__ void __launch_bounds__(128, VISC ? 5 : 8) k_dgtl(DGK K, DGArgs A, flo
     k_dgtl_b<NP1, VISC, MODE, FIRST>::run(blockIdx.x, gridDim.x, K, A, out1f, TR);
 }
 
+// ---------------------------------------------------------------------------
+// FP32 tangent product about a stored linearisation (inviscid).  Every product of one
+// Newton iterate differentiates the same fluxes, so the linearisation keeps, per face
+// point, the 4 x 4 derivatives of the HLLC flux with respect to both states (FP32, eight
+// float4 in structure-of-arrays order) and, per node, u, w, theta and dp/d(rho theta),
+// from which the flux derivatives follow.  A product is then traces, two 4 x 4 products a
+// face point, a dozen FMAs a node and the operator's sums: a fifth of the instructions of
+// the tangent evaluation (k_dgtl, which the viscous operator keeps).
+// What bounds it: the chain load - traces - sums of a block and L2 traffic (128 bytes a
+// face point).  Each thread therefore fetches its face point's derivatives into registers
+// first of all; they arrive while the block stages the direction.  Its arithmetic is
+// written in explicit FMAs so that the grouped twin rounds alike.
+// Measured on GB300 (events around a product): Q3 160 x 80 elements 13.7 us against 16.7
+// for the tangent evaluation (17.0 without the padding of the staged values: half of L1's
+// cycles were bank conflicts), Q4 320 x 160 52 against 61, Q1 200 x 100 10.8 against 13.4,
+// Q2 20 x 10 7.4 against 8.5; the derivatives take 11.7 us once per Newton iterate.
+template <int NP1>
+struct k_dgjac_b {
+    static constexpr int TPB = 128, MINB = 0;
+    static constexpr bool GROUP = false;   // a few launches a Newton iterate: members one at a time
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGK> K, JfArg<const float *> Uf,
+                                               JfArg<float4 *> J, JfArg<float4 *> Jn) {
+        jf_pdl_enter();
+        constexpr int NP = NP1 * NP1;
+        const int nx = K.nx, nz = K.nz;
+        const size_t N1 = (size_t)K.n_el * NP;
+        const long long nvert = (long long)nz * (nx + 1) * NP1, nfp = nvert + (long long)(nz + 1) * nx * NP1;
+        const long long t = (long long)jf_bid * blockDim.x + threadIdx.x;
+        if (t >= nfp + (long long)N1) return;
+        if (t >= nfp) {   // a node
+            const size_t n = (size_t)(t - nfp);
+            const int J0 = (int)(n / NP) / nx * NP1 + (int)(n % NP) / NP1;
+            float U[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) U[v] = Uf[v * N1 + n] + K.ubvf[(size_t)v * nz * NP1 + J0];
+            const float ir = frcp(U[0]);
+            const TL32 p = pressure(TL32{U[3], 1.0f}, K.pc, nullptr);
+            Jn[n] = make_float4(U[1] * ir, U[2] * ir, U[3] * ir, p.d);
+            return;
+        }
+        const bool zf = t >= nvert;
+        const int u = (int)(zf ? t - nvert : t);
+        const int s = u % NP1, c = u / NP1;
+        int eL, eR, ib;
+        bool wallL, wallR;
+        if (!zf) {
+            const int fx = c % (nx + 1), ez = c / (nx + 1);
+            wallL = fx == 0 && !K.periodic;
+            wallR = fx == nx && !K.periodic;
+            eL = ez * nx + (fx == 0 ? (K.periodic ? nx - 1 : 0) : fx - 1);
+            eR = ez * nx + (fx == nx ? (K.periodic ? 0 : nx - 1) : fx);
+            ib = ez * NP1 + s;
+        } else {
+            const int ex = c % nx, fz = c / nx;
+            wallL = fz == 0;
+            wallR = fz == nz;
+            eL = (wallL ? 0 : fz - 1) * nx + ex;
+            eR = (wallR ? nz - 1 : fz) * nx + ex;
+            ib = fz;
+        }
+        const int nb = zf ? nz + 1 : nz * NP1;
+        const float *ubf = zf ? K.ubhf : K.ubvf;
+        const int st = zf ? NP1 : 1, i0 = zf ? s : s * NP1;
+        float UL[4], UR[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            float a = 0.0f, b = 0.0f;
+#pragma unroll
+            for (int q = 0; q < NP1; ++q) {
+                a = fmaf(K.tlp[q], Uf[v * N1 + (size_t)eL * NP + i0 + q * st], a);
+                b = fmaf(K.tlm[q], Uf[v * N1 + (size_t)eR * NP + i0 + q * st], b);
+            }
+            UL[v] = a + ubf[(size_t)v * nb + ib];
+            UR[v] = b + ubf[(size_t)v * nb + ib];
+        }
+        auto swapf = [&](float &a, float &b) {
+            const float x = a;
+            a = zf ? b : a;
+            b = zf ? x : b;
+        };
+        swapf(UL[1], UL[2]);
+        swapf(UR[1], UR[2]);
+        float A[8][4];   // A[4 side + input][output], in the face's frame
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            TL32 L[4], R[4], H[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                L[v] = TL32{UL[v], d == v ? 1.0f : 0.0f};
+                R[v] = TL32{UR[v], d == 4 + v ? 1.0f : 0.0f};
+            }
+            wall_states<TL32, 0>(L, R, wallL, wallR);
+            Side<TL32> SL, SR;
+            side_of(L, K.pc, nullptr, SL);
+            side_of(R, K.pc, nullptr, SR);
+            hllc_s<TL32, 0>(SL, SR, H);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) A[d][v] = H[v].d;
+        }
+        // to (rho, rho u, rho w, rho theta) order: exchange inputs and outputs 1, 2
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) swapf(A[4 * q + 1][v], A[4 * q + 2][v]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) swapf(A[4 * q + i][1], A[4 * q + i][2]);
+#pragma unroll
+            for (int v = 0; v < 4; ++v)   // row v: output v against the side's four inputs
+                J[(size_t)(4 * q + v) * nfp + t] = make_float4(A[4 * q][v], A[4 * q + 1][v], A[4 * q + 2][v], A[4 * q + 3][v]);
+        }
+    }
+};
+template <int NP1>
+__global__ void __launch_bounds__(128) k_dgjac(DGK K, const float *Uf, float4 *J, float4 *Jn) {
+    k_dgjac_b<NP1>::run(blockIdx.x, gridDim.x, K, Uf, J, Jn);
+}
+
+JF_D float dot4(float4 a, const float x[4], float s) {
+    return fmaf(a.w, x[3], fmaf(a.z, x[2], fmaf(a.y, x[1], fmaf(a.x, x[0], s))));
+}
+
+// A block of 128 threads owns a strip of E elements of one element row, (3 E + 1) NP1 <=
+// 128 face points, as k_dgtl does.  MODE, FIRST and the transfer: as k_dgtl.
+template <int NP1, int MODE, int FIRST>
+struct k_dgjl_b {
+    static constexpr int TPB = 128, MINB = 7;
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGK> K, JfArg<DGArgs> A,
+                                               JfArg<const float4 *> J, JfArg<const float4 *> Jn, JfArg<float *> out1f,
+                                               JfArg<TransferOut> TR) {
+        jf_pdl_enter();
+        constexpr int NP = NP1 * NP1;
+        constexpr int E = strip_elems(NP1, false);
+        constexpr int S = 4 * NP + strip_pad(NP1, 1);
+        __shared__ float sz[3][E][S];                  // direction: rows below, own, above
+        __shared__ float se[2][S];                     // west and east neighbours
+        __shared__ float sg[2][E][4][NP];              // node flux derivatives
+        __shared__ float sPx[E + 1][4][NP1], sPz[2][E][4][NP1];
+        __shared__ float sDx[NP1][NP1], sDz[NP1][NP1], sl[4][NP1], st[2][NP1];
+        __shared__ float sdf[FIRST ? E : 1][4][NP];
+        __shared__ float smf[FIRST ? E : 1][4];
+        const int nx = K.nx, nz = K.nz;
+        const int nstrip = (nx + E - 1) / E;
+        const int ez = (int)jf_bid / nstrip, ex0 = ((int)jf_bid % nstrip) * E;
+        const int Ev = min(E, nx - ex0);
+        const size_t N1 = (size_t)K.n_el * NP;
+        const size_t nvert = (size_t)nz * (nx + 1) * NP1, nfp = nvert + (size_t)(nz + 1) * nx * NP1;
+        const int tid = threadIdx.x;
+        // the face point of this thread and its derivatives
+        const int nxf = (Ev + 1) * NP1, nzf = 2 * Ev * NP1;
+        const bool isx = tid < nxf, face = tid < nxf + nzf;
+        const int fu = isx ? tid : tid - nxf;
+        const int sp = fu % NP1;
+        const int f = fu / NP1;                                  // x: face west of strip element f
+        const int top = isx ? 0 : f / Ev, l = isx ? 0 : f % Ev;  // z: bottom / top face of element l
+        float4 JL[4], JR[4];
+        if (face) {
+            const size_t t = isx ? ((size_t)ez * (nx + 1) + ex0 + f) * NP1 + sp
+                                 : nvert + ((size_t)(ez + top) * nx + ex0 + l) * NP1 + sp;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                JL[v] = J[(size_t)v * nfp + t];
+                JR[v] = J[(size_t)(4 + v) * nfp + t];
+            }
+        }
+        const int le = tid / NP, node = tid % NP;
+        const int a = node % NP1, b = node / NP1;
+        const bool active = le < Ev;
+        const int e = ez * nx + ex0 + le;
+        auto dir = [&](int el, size_t i) -> float { return FIRST ? A.dtauf[el] * A.rf[i] : A.yf[i]; };
+        auto load = [&](int el, float *dst) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const size_t gi = (size_t)v * N1 + (size_t)el * NP + node;
+                dst[v * NP + node] = dir(el, gi);
+            }
+        };
+        float ef[4] = {0.f, 0.f, 0.f, 0.f}, edt = 0.0f;
+        float4 jn = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (active) {
+            load(e, sz[1][le]);
+            if (ez > 0) load(e - nx, sz[0][le]);
+            if (ez < nz - 1) load(e + nx, sz[2][le]);
+            jn = Jn[(size_t)e * NP + node];
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                if (MODE == DG_TLSMOOTH || A.rf) ef[v] = A.rf[(size_t)v * N1 + (size_t)e * NP + node];
+            if (MODE == DG_TLSMOOTH) edt = A.dtauf[e];
+        }
+        const bool has_w = ex0 > 0 || K.periodic, has_e = ex0 + Ev < nx || K.periodic;
+        if (le == 0 && has_w) load(ez * nx + (ex0 - 1 + nx) % nx, se[0]);
+        if (le == 1 && has_e) load(ez * nx + (ex0 + Ev) % nx, se[1]);
+        if (tid < NP) {
+            const int r = tid / NP1, q = tid % NP1;
+            sDx[r][q] = K.Dxf[r][q];
+            sDz[r][q] = K.Dzf[r][q];
+        }
+        if (tid < NP1) {
+            sl[0][tid] = K.liftf[0][tid];
+            sl[1][tid] = K.liftf[1][tid];
+            sl[2][tid] = K.liftf[4][tid];
+            sl[3][tid] = K.liftf[5][tid];
+            st[0][tid] = K.tlm[tid];
+            st[1][tid] = K.tlp[tid];
+        }
+        __syncthreads();
+        float z[4] = {0.f, 0.f, 0.f, 0.f};
+        if (active) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) z[v] = sz[1][le][v * NP + node];
+            const float u = jn.x, w = jn.y, th = jn.z, pd = jn.w * z[3];
+            const float du = fmaf(-u, z[0], z[1]), dw = fmaf(-w, z[0], z[2]);   // rho du, rho dw
+            const float uw = fmaf(w, du, u * z[2]);                            // d(rho u w) = w rho du + u d(rho w)
+            sg[0][le][0][node] = z[1];
+            sg[0][le][1][node] = fmaf(u, z[1] + du, pd);
+            sg[0][le][2][node] = uw;
+            sg[0][le][3][node] = fmaf(th, du, u * z[3]);
+            sg[1][le][0][node] = z[2];
+            sg[1][le][1][node] = uw;
+            sg[1][le][2][node] = fmaf(w, z[2] + dw, pd);
+            sg[1][le][3][node] = fmaf(th, dw, w * z[3]);
+        }
+        if (face) {
+            // the lines of the two sides; at a wall the outer one only has to be finite (its
+            // derivatives are zero)
+            const float *sL, *sR;
+            if (isx) {
+                sL = f > 0 ? sz[1][f - 1] : (has_w ? se[0] : sz[1][0]);
+                sR = f < Ev ? sz[1][f] : (has_e ? se[1] : sz[1][Ev - 1]);
+            } else {
+                sL = top ? sz[1][l] : (ez > 0 ? sz[0][l] : sz[1][l]);
+                sR = top ? (ez < nz - 1 ? sz[2][l] : sz[1][l]) : sz[1][l];
+            }
+            const int i0 = isx ? sp * NP1 : sp, s1 = isx ? 1 : NP1;
+            float dL[4], dR[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                dL[v] = dR[v] = 0.0f;
+#pragma unroll
+                for (int q = 0; q < NP1; ++q) {
+                    dL[v] = fmaf(st[1][q], sL[v * NP + i0 + q * s1], dL[v]);
+                    dR[v] = fmaf(st[0][q], sR[v * NP + i0 + q * s1], dR[v]);
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const float H = dot4(JR[v], dR, dot4(JL[v], dL, 0.0f));
+                if (isx) sPx[f][v][sp] = H;
+                else sPz[top][l][v][sp] = H;
+            }
+        }
+        __syncthreads();
+        if (!active && !(FIRST && TR.b) && !(MODE == DG_TLSMOOTH && A.npart)) return;
+        float sq = 0.0f;   // sum of squares of the new z
+#pragma unroll
+        for (int v = 0; v < 4 && active; ++v) {
+            float r = 0.0f;
+#pragma unroll
+            for (int q = 0; q < NP1; ++q) {
+                r = fmaf(sDx[a][q], sg[0][le][v][b * NP1 + q], r);
+                r = fmaf(sDz[b][q], sg[1][le][v][q * NP1 + a], r);
+            }
+            if (v == 2) r = fmaf(-K.gf, z[0], r);
+            r = fmaf(sl[0][a], sPx[le][v][b], r);
+            r = fmaf(-sl[1][a], sPx[le + 1][v][b], r);
+            r = fmaf(sl[2][b], sPz[0][le][v][a], r);
+            r = fmaf(-sl[3][b], sPz[1][le][v][a], r);
+            const size_t gi = (size_t)v * N1 + (size_t)e * NP + node;
+            const float jz = fmaf(-A.adtf, r, z[v]);
+            if (MODE == DG_TLJV) {
+                const float dv = A.rf ? ef[v] - jz : jz;   // with r given: the defect r - G'z
+                if (FIRST && TR.b) sdf[le][v][node] = dv;
+                else ((float *)A.out0)[gi] = dv;
+                if (FIRST) out1f[gi] = z[v];
+            } else if (A.z0mode == 0) {
+                const float zn = fmaf(edt, ef[v] - jz, z[v]);
+                ((float *)A.out0)[gi] = zn;
+                sq = fmaf(zn, zn, sq);
+            } else {
+                const float stp = __fmul_rn(A.alphaf * edt, ef[v] - jz);
+                ((float *)A.out0)[gi] = A.z0mode == 1 ? ((const float *)A.z0)[gi] + stp : stp;
+            }
+        }
+        if (MODE == DG_TLSMOOTH && A.npart) {
+            __shared__ float ssq[4];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if ((tid & 31) == 0) ssq[tid >> 5] = sq;
+            __syncthreads();
+            if (tid == 0) A.npart[jf_bid] = (ssq[0] + ssq[1]) + (ssq[2] + ssq[3]);
+        }
+        if (FIRST && TR.b) dgtl_transfer<NP1, E>(TR, sdf, smf, sg[0], le, node, ez, ex0 + le, active);
+    }
+};
+template <int NP1, int MODE, int FIRST>
+__global__ void __launch_bounds__(128, 7)
+    k_dgjl(DGK K, DGArgs A, const float4 *J, const float4 *Jn, float *out1f, TransferOut TR) {
+    k_dgjl_b<NP1, MODE, FIRST>::run(blockIdx.x, gridDim.x, K, A, J, Jn, out1f, TR);
+}
+
 // background fluxes at node rows and horizontal faces, with the residual's own
 // D64 functions so that U' = 0 cancels bit for bit
 __global__ void k_bg_dg(DGK K, double *fbx, double *fbz, double *hbx, double *hbxw, double *hbz) {
@@ -1026,15 +1332,24 @@ int launch(jfnk_ctx *c, const DGK &K, const Loader<T, IN> &ld, const DGArgs &a, 
 // the first pseudo-time step from zero, whose z = dtau r is also written to a.out1f
 template <int NP1, bool VISC, int MODE>
 int launch_tl(jfnk_ctx *c, const DGK &K, const DGArgs &a, cudaStream_t s) {
-    constexpr int E = StripOf<NP1>::E;
+    constexpr int E = strip_elems(NP1, VISC);
     const unsigned nb = (unsigned)(K.nz * ((K.nx + E - 1) / E));
-    const int threads = E * NP1 * NP1;
     if (c->timing) JF_CK(cudaEventRecord(c->tev[0], s));
-    if (MODE == DG_TLJV && a.out1f)
-        jf_launch<k_dgtl_b<NP1, VISC, MODE, 1>>(k_dgtl<NP1, VISC, MODE, 1>, nb, threads, 0, s, K, a, a.out1f,
-                  a.tro ? *a.tro : TransferOut{});
-    else
-        jf_launch<k_dgtl_b<NP1, VISC, MODE, 0>>(k_dgtl<NP1, VISC, MODE, 0>, nb, threads, 0, s, K, a, (float *)nullptr, TransferOut{});
+    if constexpr (VISC) {
+        const int threads = E * NP1 * NP1;
+        if (MODE == DG_TLJV && a.out1f)
+            jf_launch<k_dgtl_b<NP1, VISC, MODE, 1>>(k_dgtl<NP1, VISC, MODE, 1>, nb, threads, 0, s, K, a, a.out1f,
+                      a.tro ? *a.tro : TransferOut{});
+        else
+            jf_launch<k_dgtl_b<NP1, VISC, MODE, 0>>(k_dgtl<NP1, VISC, MODE, 0>, nb, threads, 0, s, K, a, (float *)nullptr, TransferOut{});
+    } else {
+        const float4 *J = (const float4 *)c->jac, *Jn = (const float4 *)c->jacn;
+        if (MODE == DG_TLJV && a.out1f)
+            jf_launch<k_dgjl_b<NP1, MODE, 1>>(k_dgjl<NP1, MODE, 1>, nb, 128, 0, s, K, a, J, Jn, a.out1f,
+                      a.tro ? *a.tro : TransferOut{});
+        else
+            jf_launch<k_dgjl_b<NP1, MODE, 0>>(k_dgjl<NP1, MODE, 0>, nb, 128, 0, s, K, a, J, Jn, (float *)nullptr, TransferOut{});
+    }
     jf_launched();
     JF_CK(cudaGetLastError());
     if (c->timing) {
@@ -1060,6 +1375,14 @@ int dispatch_mode(jfnk_ctx *c, int mode, const DGArgs &a, cudaStream_t s) {
         case DG_SMOOTH64:
             if (a.lin) return launch_fd<double, DG_SMOOTH64, NP1, VISC>(c, a, a.y, s);
             return launch<D64, 1, DG_SMOOTH64, NP1, VISC>(c, K, Loader<D64, 1>{a.U, a.y, a.eps, a.eps_val}, a, s);
+        case DG_TLLIN:   // the stored linearisation of the fused FP32 products at Uf
+            if constexpr (!VISC) {
+                const long long nt = (long long)K.nz * (K.nx + 1) * NP1 + (long long)(K.nz + 1) * K.nx * NP1 + (long long)c->npt;
+                jf_launch<k_dgjac_b<NP1>>(k_dgjac<NP1>, (unsigned)((nt + 127) / 128), 128, 0, s, K, a.Uf, (float4 *)c->jac, (float4 *)c->jacn);
+                jf_launched();
+                JF_CK(cudaGetLastError());
+            }
+            return JFNK_OK;
         case DG_TLJV:
             if (c->opts.dg_fused == 2 && !a.out1f)
                 return launch<TL32, 2, DG_TLJV, NP1, VISC>(c, K, Loader<TL32, 2>{a.Uf, a.yf}, a, s);
@@ -1161,7 +1484,7 @@ int dg_apply(jfnk_ctx *c, int mode, const DGArgs &a_in, cudaStream_t s) {
     DGArgs a = a_in;
     a.adtf = (float)a.adt;
     a.alphaf = (float)a.alpha;
-    c->dg_calls++;
+    if (mode != DG_TLLIN) c->dg_calls++;
     // the linearisation belongs to the cached f(U): any other writer of the cache drops it
     if (a.out0 == c->fU || a.out1 == c->fU) c->lin_valid = a.lin_out;
     if (a.lin && !c->lin_valid) return JFNK_EINVAL;

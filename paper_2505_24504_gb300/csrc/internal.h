@@ -255,6 +255,8 @@ struct jfnk_ctx {
     void *pz, *pz2, *pd, *pr;
     double *dtau_dg;     // [n_el]
     float *dtau_dgf;     // [n_el] FP32 copy (prec 32)
+    float *jac, *jacn;   // FP32 derivatives of the face fluxes (32 a face point) and node values
+                         // (4 a node) of the fused tangent products (prec 32, inviscid)
     float *Usf;          // FP32 copy of the linearisation state U' + Ubar (prec 32)
     int nlev;
     FVLev lev[JF_MAXLEV];
@@ -332,7 +334,8 @@ enum DGMode {
     DG_G = 2,        // out0 = U' - adt f - Ubar_s ; out1 = f
     DG_SMOOTH64 = 3, // out0 = z + dtau (r - [z - adt (f(U'+eps z) - fU)/eps])
     DG_TLJV = 4,     // out0 = z - adt J z, or r - (z - adt J z) when rf is given  (FP32 tangent)
-    DG_TLSMOOTH = 5  // out0 = z + dtau (r - (z - adt J z))            (FP32 tangent)
+    DG_TLSMOOTH = 5, // out0 = z + dtau (r - (z - adt J z))            (FP32 tangent)
+    DG_TLLIN = 6     // stored linearisation of the fused FP32 products at Uf (inviscid)
 };
 
 // DG -> finest-FV transfer T^mf folded into the FP32 defect kernel: the 1D
@@ -380,9 +383,16 @@ struct DGArgs {
     double alpha;
     float *npart;          // FP32 smoothing: each block's sum of squares of the new z (may be null)
 };
-// blocks of the fused FP32 tangent product (k_dgtl), a strip of elements each
+// Elements of a strip (block) of the fused FP32 tangent products: one thread per node
+// (viscous), and not more than 128 face points, (3 E + 1)(k + 1), where each thread also
+// owns one (inviscid)
+constexpr int strip_elems(int np1, bool visc) {
+    const int n = 128 / (np1 * np1), f = (128 / np1 - 1) / 3;
+    return visc || n < f ? n : f;
+}
+// blocks of such a product
 inline int dgtl_blocks(const jfnk_ctx *c) {
-    const int np = c->np1 * c->np1, e = 128 / np > 0 ? 128 / np : 1;
+    const int e = strip_elems(c->np1, c->phys.mu != 0.0);
     return c->grid.nz * ((c->grid.nx + e - 1) / e);
 }
 // the blocks whose sums of squares the FP32 preconditioner leaves in c->partial with its

@@ -1698,6 +1698,11 @@ int mg_linearize(jfnk_ctx *c, const double *Uin, double adt, cudaStream_t s) {
         JF_RET(to_fv<double, float>(c, Uin, (float *)c->lev[0].u, s, nullptr, nullptr,
                                     LinOut{c->Ulin, c->Usf, c->dtau_dgf, c->ubvf, c->pc, 1.0 / c->hx, 1.0 / c->hz,
                                            c->phys.mu, adt, c->opts.sigma_dg}));
+        if (c->jac && (c->dg_pre || c->dg_post)) {
+            DGArgs a = {};
+            a.Uf = c->Usf;
+            JF_RET(dg_apply(c, DG_TLLIN, a, s));
+        }
     }
     for (int l = 0; l < c->nlev; ++l) {
         FVLev &L = c->lev[l];

@@ -64,6 +64,15 @@ JF_D void mirror_side(const Side<T> &A, Side<T> &G) {
     G.U[1 + D] = -A.U[1 + D];
 }
 
+// Does S_L = u_L - c_L (S_R = u_L + c_L) hold of the Davis speeds?  FP64 compares the
+// differences it has; the FP32 tangent, whose derivative jumps where the two speeds
+// agree, compares the speeds themselves (a rounding of 3e-5 m/s decides either way, and
+// the same way for the same states).
+JF_D bool slower(D64, D64 cL, D64, D64, D64 x) { return le(-cL, x); }
+JF_D bool faster(D64, D64, D64, D64 cR, D64 y) { return le(cR, y); }
+JF_D bool slower(TL32 uL, TL32 cL, TL32 uR, TL32 cR, TL32) { return le(uL - cL, uR - cR); }
+JF_D bool faster(TL32 uL, TL32 cL, TL32 uR, TL32 cR, TL32) { return le(uR + cR, uL + cL); }
+
 // HLLC flux in direction e_D, normal from L to R.  Davis wave speeds
 // S_L = min(u_L - c_L, u_R - c_R), S_R = max(u_L + c_L, u_R + c_R), c^2 = gamma p / rho;
 // contact speed S*; star states rho*_K = rho_K (S_K - u_K)/(S_K - S*) with normal
@@ -87,8 +96,8 @@ JF_D void hllc_s(const Side<T> &L, const Side<T> &R, T H[4]) {
     const T uL = L.U[iN] * L.ir, uR = R.U[iN] * R.ir;
     const T d = uR - uL;
     const T x = d - R.c, y = L.c - d;
-    const T dL = sel(le(-L.c, x), -L.c, x);   // S_L - u_L
-    const T dR = sel(le(R.c, y), y, R.c);     // S_R - u_R
+    const T dL = sel(slower(uL, L.c, uR, R.c, x), -L.c, x);   // S_L - u_L
+    const T dR = sel(faster(uL, L.c, uR, R.c, y), y, R.c);    // S_R - u_R
     const T qL = L.U[0] * dL, qR = R.U[0] * dR;
     const T sL = jfma(-d, qR, R.p - L.p) / (qL - qR);   // S* - u_L
     const T Sst = uL + sL;
