@@ -503,15 +503,15 @@ constexpr int strip_pad(int np1, int words) {
     return words == 1 ? (np1 == 2 ? 2 : np1 == 4 ? 9 : np1 == 5 ? 3 : 0) : (np1 == 2 ? 2 : 5);
 }
 
-// T^mf of the strip's defect (in sd) to the finest FV level: the 1D transfer
-// matrix along x, then along z (through the scratch st), the mass fix from the
-// subcell values (mean against the modified Newton-Cotes quadrature), written to
-// b and, when x0 is given, x0 = dtau b.  The arithmetic and its order are those of
-// the stand-alone transfer kernel.  All threads of the block call it.
+// T^mf of the strip's defect (in sd) to the finest FV level: the 1D transfer matrix along
+// x, then along z (through the scratch st), the mass fix (mean of the subcell values
+// against the modified Newton-Cotes quadrature, both tensor products, so they follow the
+// two sweeps: row sums smf, then their sum), written to b and, when x0 is given, x0 = dtau b.
+// All threads of the block call it.
 template <int NP1, int E>
-__device__ __forceinline__ void dgtl_transfer(const TransferOut &TR, float (*sd)[4][NP1 * NP1], float (*smf)[4],
-                                              float (*st)[4][NP1 * NP1], int le, int node, int ez, int ex,
-                                              bool active) {
+__device__ __forceinline__ void dgtl_transfer(const TransferOut &TR, float (*sd)[4][NP1 * NP1],
+                                              float (*smf)[4][2][NP1], float (*st)[4][NP1 * NP1], int le, int node,
+                                              int ez, int ex, bool active) {
     constexpr int NP = NP1 * NP1;
     const int i = node % NP1, j = node / NP1;
     __syncthreads();   // sd complete; sg (scratch st) no longer read
@@ -525,6 +525,20 @@ __device__ __forceinline__ void dgtl_transfer(const TransferOut &TR, float (*sd)
         }
     }
     __syncthreads();
+    // row sums of t1: lane (q, j) of an element's first 4 NP1 threads, or in turn
+    if (active)
+        for (int r = node; r < 4 * NP1; r += NP) {
+            const int q = r / NP1, row = r % NP1;
+            float m = 0.0f, w = 0.0f;
+#pragma unroll
+            for (int k = 0; k < NP1; ++k) {
+                const float x = st[le][q][row * NP1 + k];
+                m += x;
+                w = fmaf(TR.om[k], x, w);
+            }
+            smf[le][q][0][row] = m;
+            smf[le][q][1][row] = w;
+        }
     float Tu[4] = {0.f, 0.f, 0.f, 0.f};
     if (active) {
 #pragma unroll
@@ -536,29 +550,19 @@ __device__ __forceinline__ void dgtl_transfer(const TransferOut &TR, float (*sd)
         }
     }
     __syncthreads();
-    if (active) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) sd[le][q][node] = Tu[q];
-    }
-    __syncthreads();
-    if (active && node < 4) {
-        const int q = node;
-        float mfv = 0.0f, mnc = 0.0f;
-        for (int jj = 0; jj < NP1; ++jj)
-            for (int ii = 0; ii < NP1; ++ii) {
-                const float x = sd[le][q][jj * NP1 + ii];
-                mfv += x;
-                mnc = fmaf(TR.om[ii] * TR.om[jj], x, mnc);
-            }
-        smf[le][q] = TR.massfix ? (mfv / (float)NP - mnc) : 0.0f;
-    }
-    __syncthreads();
     if (!active) return;
     const size_t I = (size_t)ex * NP1 + i, Jr = (size_t)ez * NP1 + j;
     const size_t cell = Jr * TR.NX + I, ncell = (size_t)TR.NX * TR.NZ;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const float val = Tu[q] - smf[le][q];
+        float shift = 0.0f;
+        if (TR.massfix) {
+#pragma unroll
+            for (int b = 0; b < NP1; ++b) shift = fmaf(TR.vm[b], smf[le][q][0][b], shift);
+#pragma unroll
+            for (int b = 0; b < NP1; ++b) shift = fmaf(-TR.vo[b], smf[le][q][1][b], shift);
+        }
+        const float val = Tu[q] - shift;
         const size_t gi = (size_t)q * ncell + cell;
         TR.b[gi] = val;
         if (TR.x0) TR.x0[gi] = TR.dtau0[cell] * val;   // first pseudo-time step from zero
@@ -588,7 +592,7 @@ struct k_dgtl_b {
         __shared__ float sSz[VISC ? 2 : 1][VISC ? E : 1][6][NP1];
         __shared__ float sDx[NP1][NP1], sDz[NP1][NP1], sDn[NP1][NP1], sl[8][NP1];
         __shared__ float sdf[FIRST ? E : 1][4][NP];    // the defect, for the transfer (FIRST)
-        __shared__ float smf[FIRST ? E : 1][4];        // mass-fix shift per element and variable
+        __shared__ float smf[FIRST ? E : 1][4][2][NP1];   // row sums of the mass fix
         const int nx = K.nx, nz = K.nz;
         const int nstrip = (nx + E - 1) / E;
         const int ez = (int)jf_bid / nstrip, ex0 = ((int)jf_bid % nstrip) * E;
@@ -1011,7 +1015,7 @@ struct k_dgjl_b {
         __shared__ float sPx[E + 1][4][NP1], sPz[2][E][4][NP1];
         __shared__ float sDx[NP1][NP1], sDz[NP1][NP1], sl[4][NP1], st[2][NP1];
         __shared__ float sdf[FIRST ? E : 1][4][NP];
-        __shared__ float smf[FIRST ? E : 1][4];
+        __shared__ float smf[FIRST ? E : 1][4][2][NP1];   // row sums of the mass fix
         const int nx = K.nx, nz = K.nz;
         const int nstrip = (nx + E - 1) / E;
         const int ez = (int)jf_bid / nstrip, ex0 = ((int)jf_bid % nstrip) * E;

@@ -18,7 +18,7 @@
 // caller's own, larger eps takes the general form.
 // Measured on GB300 (events around the launches): Q3 160 x 80 elements 31.8 + 11.6 us,
 // the general form 33.0 + 40.7 (and 48.8 + 47.4 before the primitives of numeric.cuh);
-// viscous Q2 256 x 32 35.9 + 8.1 against 49.0 + 30.9, Q4 320 x 160 150 + 37 against
+// viscous Q2 256 x 32 31.3 + 8.7 against 49.0 + 30.9, Q4 320 x 160 150 + 37 against
 // 191 + 267.  The 103,360 face points and 204,800 nodes take 21.5 us of FP64 issue.
 
 // ---- two-float arithmetic -----------------------------------------------------
@@ -94,6 +94,7 @@ struct DGF {
 };
 
 constexpr int FD_MINB = 7;   // 72 registers: 28 warps an SM, no spills
+constexpr int FD_MINV = 6;   // viscous, 80 registers: 31.3 us on Q2 256 x 32, 36.4 with 118 and no spills
 // Difference of the face terms at U + eps y and U, one thread per face point (the linear
 // index of the residual's face kernel).  Vertical and horizontal faces run the same code:
 // the momentum components are exchanged for the latter.
@@ -289,7 +290,7 @@ JF_D void fd_nodes(const DGF &K, const Y *y, double eps, float2 *part, unsigned 
 // The first block also leaves alpha dt / eps for the lift.
 template <class Y, int NP1, bool VISC>
 struct k_fd_flux_b {
-    static constexpr int TPB = 128, MINB = VISC ? 4 : FD_MINB;
+    static constexpr int TPB = 128, MINB = VISC ? FD_MINV : FD_MINB;
     static constexpr bool GROUP = !VISC;   // a grouped twin is built (lock-step ensembles)
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGF> K, JfArg<unsigned> nface,
                                                JfArg<const Y *> y, JfArg<const double *> epsp, JfArg<double> adt,
@@ -303,7 +304,7 @@ struct k_fd_flux_b {
     }
 };
 template <class Y, int NP1, bool VISC>
-__global__ void __launch_bounds__(128, VISC ? 4 : FD_MINB)
+__global__ void __launch_bounds__(128, VISC ? FD_MINV : FD_MINB)
     k_fd_flux(DGF K, unsigned nface, const Y *y, const double *epsp, double adt, double *cepsp, float2 *part,
               float2 *phix, float2 *symx, float2 *phiz, float2 *symz) {
     k_fd_flux_b<Y, NP1, VISC>::run(blockIdx.x, gridDim.x, K, nface, y, epsp, adt, cepsp, part, phix, symx, phiz, symz);

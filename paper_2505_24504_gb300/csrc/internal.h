@@ -345,6 +345,7 @@ enum DGMode {
 struct TransferOut {
     float V[5][5];
     float om[5];
+    float vm[5], vo[5];   // sum_j V[j][b] / (k+1)^2 and sum_j om_j V[j][b]: the mass fix's z functionals
     int massfix;
     int NX, NZ;
     float *b, *x0;

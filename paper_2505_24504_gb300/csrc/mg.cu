@@ -823,7 +823,7 @@ struct k_to_dg_b {
         constexpr int EPB = (128 / NP) > 0 ? 128 / NP : 1;
         __shared__ R sv[EPB][4][NP];
         __shared__ R st[EPB][4][NP];
-        __shared__ R sc[EPB][4];
+        __shared__ R sc[EPB][4][2][NP1];
         __shared__ R sV[NP1][NP1], sVi[NP1][NP1], som[NP1];
         load_ttab<R, NP1>(K, sV, sVi, som);
         const int le = threadIdx.x / NP, node = threadIdx.x % NP;
@@ -853,25 +853,38 @@ struct k_to_dg_b {
                 for (int jj = 0; jj < NP1; ++jj) acc = fma(sVi[b][jj], st[le][q][jj * NP1 + a], acc);
                 Ti[q] = acc;
             }
-        if (act && node < 4) {
-            // m_E(T^-1 v)/|E| from the subcell values (T T^-1 v = v) by the midpoint weights,
-            // m_E(v)/|E| the subcell mean
-            const int q = node;
-            R mfv = 0, mnc = 0;
-            for (int jj = 0; jj < NP1; ++jj)
+        // m_E(T^-1 v)/|E| from the subcell values (T T^-1 v = v) by the midpoint weights,
+        // m_E(v)/|E| the subcell mean: row sums, then (below) their weighted sum
+        if (act && massfix)
+            for (int r = node; r < 4 * NP1; r += NP) {
+                const int q = r / NP1, row = r % NP1;
+                R m = 0, w = 0;
+    #pragma unroll
                 for (int ii = 0; ii < NP1; ++ii) {
-                    const R x = sv[le][q][jj * NP1 + ii];
-                    mfv += x;
-                    mnc = fma(som[ii] * som[jj], x, mnc);
+                    const R x = sv[le][q][row * NP1 + ii];
+                    m += x;
+                    w = fma(som[ii], x, w);
                 }
-            sc[le][q] = massfix ? (mnc - mfv / (R)NP) : (R)0;
-        }
+                sc[le][q][0][row] = m;
+                sc[le][q][1][row] = w;
+            }
         __syncthreads();
         if (!act) return;
         const size_t N1 = (size_t)K.n_el * NP;
+    #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const size_t gi = q * N1 + (size_t)e * NP + node;
-            const R val = Ti[q] - sc[le][q];
+            R shift = 0;
+            if (massfix) {
+                R mfv = 0;
+    #pragma unroll
+                for (int jj = 0; jj < NP1; ++jj) {
+                    mfv += sc[le][q][0][jj];
+                    shift = fma(som[jj], sc[le][q][1][jj], shift);
+                }
+                shift -= mfv * ((R)1 / (R)NP);
+            }
+            const R val = Ti[q] - shift;
             u[gi] = acc_mode ? (So)((R)u[gi] + val) : (So)val;
         }
     }
@@ -1625,6 +1638,15 @@ int apply_t(jfnk_ctx *c, const S *r, S *zout, cudaStream_t s) {
         for (int i = 0; i < 5; ++i) {
             for (int a = 0; a < 5; ++a) tro.V[i][a] = (float)K.tab.V[i][a];
             tro.om[i] = (float)K.tab.om[i];
+        }
+        for (int b = 0; b < c->np1; ++b) {
+            double m = 0.0, o = 0.0;
+            for (int j = 0; j < c->np1; ++j) {
+                m += K.tab.V[j][b];
+                o += K.tab.om[j] * K.tab.V[j][b];
+            }
+            tro.vm[b] = (float)(m / (c->np1 * c->np1));
+            tro.vo[b] = (float)o;
         }
         tro.massfix = c->opts.massfix && !c->opts.transfer_l2;
         tro.NX = c->lev[0].NX;
