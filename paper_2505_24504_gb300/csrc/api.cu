@@ -158,6 +158,7 @@ size_t workspace(const jfnk_grid *g, int k, const jfnk_opts *o, const jfnk_physi
         const size_t n = 4 * (size_t)NX[l] * NZ[l];
         b += 8 * (4 * (size_t)NZ[l] * 4 + 4);
         b += sS * n * 6 + sS * n / 4;
+        if (prec != 64 && n / 4 <= FV_STORED) b += 320 * (n / 4);   // stored stencil
     }
     b += 8 * 4096 * 32 + 8 * 256;
     b += 8 * (fx + fz) * (visc ? 33 : 12) + 8 * N + 8 * npt * (visc ? 19 : 5);   // linearisation of the DG operator
@@ -479,6 +480,7 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
         A_(L.b, sS * L.n);
         A_(L.r, sS * L.n);
         A_(L.dtau, sS * L.n / 4);
+        if (c->prec != 64 && L.n / 4 <= FV_STORED) A_(L.st, 320 * (L.n / 4));
         std::vector<double> ub(4 * (size_t)NZ[l]);
         for (int J = 0; J < NZ[l]; ++J) {
             double U[4], dU[4];

@@ -23,9 +23,10 @@
 // programmatic stream serialisation and each first waits (griddepcontrol.wait)
 // for its predecessor grid to complete with its memory writes visible, so no
 // read or write moves ahead of that point.  The successor is released when the
-// predecessor completes (no early trigger: blocks that wait early would hold
-// SM resources the predecessor still needs); what is saved is part of the
-// launch latency between dependent kernels.  JFNK_PDL=0 in the environment
+// predecessor completes (no early trigger: blocks that wait early hold SM resources
+// that running kernels need; even from grids of at most 80 blocks it cost the ensemble
+// 6 % and a Q2 20 x 10 step 19 %); what is saved is part of the launch latency between
+// dependent kernels.  JFNK_PDL=0 in the environment
 // launches them with plain stream ordering.
 #ifdef __CUDACC__
 __device__ __forceinline__ void jf_pdl_enter() {
@@ -195,6 +196,13 @@ struct DGTab {
     double om[5];        // modified Newton-Cotes weights on [0,1] at the subcell centres
 };
 
+// FP32 levels of at most this many cells keep their tangent's stencil (320 bytes a cell).
+// There a launch is a latency chain and the stencil shortens it: a step of the inertia
+// gravity wave (levels of 3,840, 960 and 240 cells) takes 6.96 ms against 7.40, of the
+// viscous density current 8.76 against 8.86, of the 819,200-unknown warm bubble 16.76
+// against 16.86.  At 51,200 cells reading the stencil costs more than the fluxes it
+// saves (preconditioner of the warm bubble 169 us against 155), at 12,800 the two agree.
+constexpr size_t FV_STORED = 4096;
 struct FVLev {
     int NX, NZ;
     int fac;             // agglomeration factor to the next coarser level (0: coarsest)
@@ -208,6 +216,7 @@ struct FVLev {
     // level vectors; element type is double (prec 64) or float (prec 32/16)
     void *u, *fu, *x, *x2, *b, *r;
     void *dtau;          // [NZ][NX]
+    float *st;           // stored stencil of the tangent: 80 floats a cell (FP32, at most FV_STORED cells)
     uint16_t *xb, *bb;   // bf16 storage of x and b on the coarsest level (prec 16)
 };
 

@@ -34,6 +34,7 @@ struct FVK {
     const PowTab *pt;
     const double *ub, *hbx, *hbxw, *hbz;
     const float *ubf;
+    const float4 *st;                    // stored stencil of the FP32 tangent (small levels), or null
 };
 
 // One stage of the pseudo-time smoother (Sec. 3.5) in the FV smoothing kernels:
@@ -161,6 +162,55 @@ JF_D T reduce_scatter4(const T f[4], int q) {
     return keep + shfl_x(send, 1);
 }
 
+// Neighbour of cell c = (I, Jz) across face q (0 W, 1 E, 2 S, 3 N); negative at a wall
+JF_D long fv_neighbour(const FVK &K, size_t c, int I, int Jz, int q, int &nI, int &nJ) {
+    const int NX = K.NX, NZ = K.NZ;
+    nI = I;
+    nJ = Jz;
+    if (q == 0) {
+        if (I > 0) { nI = I - 1; return (long)c - 1; }
+        if (K.periodic) { nI = NX - 1; return (long)c + NX - 1; }
+    } else if (q == 1) {
+        if (I < NX - 1) { nI = I + 1; return (long)c + 1; }
+        if (K.periodic) { nI = 0; return (long)c - (NX - 1); }
+    } else if (q == 2) {
+        if (Jz > 0) { nJ = Jz - 1; return (long)c - NX; }
+    } else {
+        if (Jz < NZ - 1) { nJ = Jz + 1; return (long)c + NX; }
+    }
+    return -1;
+}
+
+// Component q of the tangent J x at a cell from the level's stored stencil: five 4 x 4
+// blocks (own cell, W, E, S, N), block k's row q at [(4 k + q) cells + c].  The small
+// levels' launches are short chains of dependent instructions, three microseconds of
+// tangent fluxes each; the blocks, made once per linearisation, leave twenty FMAs behind
+// one load.  Lane q loads variable q of the five cells, the lanes of a cell exchange them.
+template <int IN>
+JF_D float fv_cell_st(const FVK &K, const FLoad<TL32, IN> &ld, size_t c, int I, int Jz, int q) {
+    const size_t n1 = (size_t)K.NX * K.NZ;
+    float4 row[5];
+    float x[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) row[k] = K.st[(size_t)(4 * k + q) * n1 + c];
+    x[0] = ld.dir(q, c, I, Jz);
+#pragma unroll
+    for (int k = 1; k < 5; ++k) {
+        int nI, nJ;
+        const long nb = fv_neighbour(K, c, I, Jz, k - 1, nI, nJ);
+        x[k] = nb >= 0 ? ld.dir(q, (size_t)nb, nI, nJ) : 0.0f;
+    }
+    float f = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        f = fmaf(row[k].x, __shfl_sync(0xffffffffu, x[k], 0, 4), f);
+        f = fmaf(row[k].y, __shfl_sync(0xffffffffu, x[k], 1, 4), f);
+        f = fmaf(row[k].z, __shfl_sync(0xffffffffu, x[k], 2, 4), f);
+        f = fmaf(row[k].w, __shfl_sync(0xffffffffu, x[k], 3, 4), f);
+    }
+    return f;
+}
+
 // f_low (or its tangent) at cell (I, Jz), computed by four lanes: lane q evaluates
 // face q (0 W, 1 E, 2 S, 3 N): HLLC^pert (background flux of the face row
 // subtracted), the two-point viscous flux, and lane 2 adds the gravity source.
@@ -173,19 +223,8 @@ JF_D T fv_cell_op4(const FVK &K, const FLoad<T, IN> &ld, const PowTab *spt, size
     const int NX = K.NX, NZ = K.NZ;
     const bool sub = (IN < 2);
     const bool zf = q >= 2, right = (q & 1) != 0;
-    long nb = -1;
-    int nI = I, nJ = Jz;
-    if (q == 0) {
-        if (I > 0) { nb = (long)c - 1; nI = I - 1; }
-        else if (K.periodic) { nb = (long)c + NX - 1; nI = NX - 1; }
-    } else if (q == 1) {
-        if (I < NX - 1) { nb = (long)c + 1; nI = I + 1; }
-        else if (K.periodic) { nb = (long)c - (NX - 1); nI = 0; }
-    } else if (q == 2) {
-        if (Jz > 0) { nb = (long)c - NX; nJ = Jz - 1; }
-    } else {
-        if (Jz < NZ - 1) { nb = (long)c + NX; nJ = Jz + 1; }
-    }
+    int nI, nJ;
+    const long nb = fv_neighbour(K, c, I, Jz, q, nI, nJ);
     const bool wall = nb < 0;
     T U[4], N[4];
     const T up0 = ld(0, c, I, Jz);
@@ -256,8 +295,9 @@ JF_D S gprime_of(const FLoad<T, IN> &ld, S x, T f, const double *fu, size_t gi, 
     return x - (S)adtf * (S)oval(f);
 }
 
-// Four lanes per cell of an NX x NZ level, lane q owns variable q.
-template <class T, int IN, int MODE, bool VISC>
+// Four lanes per cell of an NX x NZ level, lane q owns variable q.  ST: from the stored
+// stencil (FP32 tangent, small levels).
+template <class T, int IN, int MODE, bool VISC, bool ST>
 struct k_fv_b {
     static constexpr int TPB = 256, MINB = 0;
     static constexpr bool GROUP = !VISC && std::is_same<T, TL32>::value;   // a grouped twin is built (lock-step ensembles)
@@ -279,7 +319,9 @@ struct k_fv_b {
         const bool live = cell < n1;
         const size_t c = live ? cell : n1 - 1;   // idle lanes still join the shuffles
         const int I = (int)(c % K.NX), Jz = (int)(c / K.NX);
-        const T f = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, v);
+        T f;
+        if constexpr (ST) f = T{0.0f, fv_cell_st<IN>(K, ld, c, I, Jz, v)};
+        else f = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, v);
         if (!live) return;
         const size_t gi = (size_t)v * n1 + c;
         if (MODE == FV_RES) {
@@ -294,12 +336,12 @@ struct k_fv_b {
         }
     }
 };
-template <class T, int IN, int MODE, bool VISC>
+template <class T, int IN, int MODE, bool VISC, bool ST>
 __global__ void __launch_bounds__(256) k_fv(FVK K, FLoad<T, IN> ld0, const typename SOf<T>::type *xin,
                                             const typename SOf<T>::type *b, const typename SOf<T>::type *dtau,
                                             const double *fu, double adt, typename SOf<T>::type *out,
                                             int bf16, RKS rk) {
-    k_fv_b<T, IN, MODE, VISC>::run(blockIdx.x, gridDim.x, K, ld0, xin, b, dtau, fu, adt, out, bf16, rk);
+    k_fv_b<T, IN, MODE, VISC, ST>::run(blockIdx.x, gridDim.x, K, ld0, xin, b, dtau, fu, adt, out, bf16, rk);
 }
 
 // Defect and restriction in one pass: the defect g'x - b of every child cell of
@@ -307,7 +349,7 @@ __global__ void __launch_bounds__(256) k_fv(FVK K, FLoad<T, IN> ld0, const typen
 // first pseudo-time step x_c = dtau_c b_c.  FAC2: 2 x 2 agglomeration with
 // sixteen lanes per coarse cell (four lanes per child, children summed by
 // shuffles); otherwise four lanes per coarse cell loop over the children.
-template <class T, int IN, bool VISC, bool FAC2>
+template <class T, int IN, bool VISC, bool FAC2, bool ST>
 struct k_fv_defect_restrict_b {
     static constexpr int TPB = 256, MINB = 0;
     static constexpr bool GROUP = !VISC && std::is_same<T, TL32>::value;   // a grouped twin is built (lock-step ensembles)
@@ -335,7 +377,9 @@ struct k_fv_defect_restrict_b {
             const int ch = (int)((t >> 2) & 3);
             const int I = 2 * Ic + (ch & 1), Jz = 2 * Jc + (ch >> 1);
             const size_t c = (size_t)Jz * K.NX + I;
-            const T fq = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, q);
+            T fq;
+                    if constexpr (ST) fq = T{0.0f, fv_cell_st<IN>(K, ld, c, I, Jz, q)};
+                    else fq = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, q);
             const size_t gi = (size_t)q * n1 + c;
             const S d = gprime_of<T, IN, S>(ld, (S)ld.dir(q, c, I, Jz), fq, fu, gi, adt, adtf, eps) - b[gi];
             const S d2 = d + __shfl_xor_sync(0xffffffffu, d, 4);
@@ -346,7 +390,9 @@ struct k_fv_defect_restrict_b {
                 for (int ii = 0; ii < fac; ++ii) {
                     const int I = Ic * fac + ii, Jz = Jc * fac + jj;
                     const size_t c = (size_t)Jz * K.NX + I;
-                    const T fq = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, q);
+                    T fq;
+                    if constexpr (ST) fq = T{0.0f, fv_cell_st<IN>(K, ld, c, I, Jz, q)};
+                    else fq = fv_cell_op4<T, IN, VISC>(K, ld, K.pt, c, I, Jz, q);
                     const size_t gi = (size_t)q * n1 + c;
                     acc += gprime_of<T, IN, S>(ld, (S)ld.dir(q, c, I, Jz), fq, fu, gi, adt, adtf, eps) - b[gi];
                 }
@@ -357,12 +403,12 @@ struct k_fv_defect_restrict_b {
         if (xc) xc[(size_t)q * nc + cc] = store_round<S>(dtau_c[cc] * bv, bf16);
     }
 };
-template <class T, int IN, bool VISC, bool FAC2>
+template <class T, int IN, bool VISC, bool FAC2, bool ST>
 __global__ void __launch_bounds__(256) k_fv_defect_restrict(FVK K, FLoad<T, IN> ld0, const typename SOf<T>::type *b,
                                                             const double *fu, double adt, int fac,
                                                             typename SOf<T>::type *bc, typename SOf<T>::type *xc,
                                                             const typename SOf<T>::type *dtau_c, int bf16) {
-    k_fv_defect_restrict_b<T, IN, VISC, FAC2>::run(blockIdx.x, gridDim.x, K, ld0, b, fu, adt, fac, bc, xc, dtau_c, bf16);
+    k_fv_defect_restrict_b<T, IN, VISC, FAC2, ST>::run(blockIdx.x, gridDim.x, K, ld0, b, fu, adt, fac, bc, xc, dtau_c, bf16);
 }
 
 // Face-once form for large levels: a block owns a tile of TX x TZ cells.  The
@@ -629,6 +675,130 @@ struct k_fv_lin_b {
 template <class S>
 __global__ void k_fv_lin(FVK K, const S *u, double adt, double sigma, S *dtau, int fac, S *uc, int bf16) {
     k_fv_lin_b<S>::run(blockIdx.x, gridDim.x, K, u, adt, sigma, dtau, fac, uc, bf16);
+}
+
+// The same with the level's stored stencil (FP32): four lanes per cell, lane q on face q
+// evaluates the tangent flux for unit directions of both sides' variables.
+template <bool VISC>
+struct k_fv_linst_b {
+    static constexpr int TPB = 128, MINB = 0;
+    static constexpr bool GROUP = false;   // a few launches a Newton iterate: members one at a time
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<FVK> K, JfArg<const float *> u,
+                                               JfArg<double> adt, JfArg<double> sigma, JfArg<float *> dtau,
+                                               JfArg<int> fac, JfArg<float *> uc, JfArg<int> bf16, JfArg<float4 *> st) {
+        jf_pdl_enter();
+        const int NX = K.NX, NZ = K.NZ;
+        const size_t n1 = (size_t)NX * NZ;
+        const size_t t = (size_t)jf_bid * blockDim.x + threadIdx.x;
+        const int q = (int)(t & 3);
+        const bool live = (t >> 2) < n1;
+        const size_t c = live ? (t >> 2) : n1 - 1;   // idle lanes still join the shuffles
+        const int I = (int)(c % NX), Jz = (int)(c / NX);
+        const bool zf = q >= 2, right = (q & 1) != 0;
+        int nI, nJ;
+        const long nb = fv_neighbour(K, c, I, Jz, q, nI, nJ);
+        const bool wall = nb < 0;
+        float U[4], N[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            U[v] = u[v * n1 + c] + K.ubf[v * NZ + Jz];
+            N[v] = wall ? U[v] : u[v * n1 + (size_t)nb] + K.ubf[v * NZ + nJ];
+        }
+        // pseudo-time step: the faces' speeds summed over the lanes
+        {
+            const float so = wave_speed_r<float>(U, zf ? 1 : 0, K.pc, K.pt), sn = wave_speed_r<float>(N, zf ? 1 : 0, K.pc, K.pt);
+            float e = fmaxf(so, sn);
+            e += __shfl_xor_sync(0xffffffffu, e, 1);
+            float part = 0.5f * e * (zf ? K.iHzf : K.iHxf);
+            part += __shfl_xor_sync(0xffffffffu, part, 2);
+            const float lam = part + 2.0f * K.pc.muf * (K.iHxf * K.iHxf + K.iHzf * K.iHzf);
+            if (live && q == 0) dtau[c] = (float)sigma / (1.0f + (float)adt * lam);
+        }
+        if (live && uc && I % fac == 0 && Jz % fac == 0) {   // lane q restricts variable q
+            const int NXc = NX / fac, NZc = NZ / fac;
+            if (I / fac < NXc && Jz / fac < NZc) {
+                float acc = 0.0f;
+                for (int jj = 0; jj < fac; ++jj)
+                    for (int ii = 0; ii < fac; ++ii) acc += u[(size_t)q * n1 + c + (size_t)jj * NX + ii];
+                uc[(size_t)q * NXc * NZc + (size_t)(Jz / fac) * NXc + I / fac] = store_round<float>(acc / (float)(fac * fac), bf16);
+            }
+        }
+        auto swapf = [&](float &a, float &b) {
+            const float x = a;
+            a = zf ? b : a;
+            b = zf ? x : b;
+        };
+        swapf(U[1], U[2]);
+        swapf(N[1], N[2]);
+        const float ih = zf ? K.iHzf : K.iHxf;
+        float Co[4][4], Cn[4][4];   // [output][input] of f against the own cell and the neighbour
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            TL32 A[4], B[4], H[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                A[v] = TL32{U[v], d == v ? 1.0f : 0.0f};
+                B[v] = wall ? A[v] : TL32{N[v], d == 4 + v ? 1.0f : 0.0f};
+            }
+            if (wall) B[1] = -A[1];
+            Side<TL32> own, nbr, L, R;
+            side_of(A, K.pc, nullptr, own);
+            side_of(B, K.pc, nullptr, nbr);
+            sel_side(right, own, nbr, L);
+            sel_side(right, nbr, own, R);
+            hllc_s<TL32, 0>(L, R, H);
+            float h[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) h[v] = H[v].d;
+            if (VISC) {
+                TL32 V[4];
+                visc2_s(L, R, zf ? TLc{K.vczf} : TLc{K.vcxf}, V);
+#pragma unroll
+                for (int v = 1; v < 4; ++v) h[v] -= wall ? 0.0f : V[v].d;
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const float f = (right ? -ih : ih) * h[v];
+                if (d < 4) Co[v][d] = f;
+                else Cn[v][d - 4] = f;
+            }
+        }
+        // to (rho, rho u, rho w, rho theta) order
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            swapf(Co[1][v], Co[2][v]);
+            swapf(Cn[1][v], Cn[2][v]);
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            swapf(Co[v][1], Co[v][2]);
+            swapf(Cn[v][1], Cn[v][2]);
+        }
+        // own block: the four faces' shares; lane q keeps row q
+        float row[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                float a = Co[r][i];
+                a += __shfl_xor_sync(0xffffffffu, a, 1);
+                a += __shfl_xor_sync(0xffffffffu, a, 2);
+                if (r == q) row[i] = a;
+            }
+        }
+        if (q == 2) row[0] -= K.gf;   // -g rho'
+        if (!live) return;
+        st[(size_t)q * n1 + c] = make_float4(row[0], row[1], row[2], row[3]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            st[(size_t)(4 * (1 + q) + r) * n1 + c] = wall ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                                          : make_float4(Cn[r][0], Cn[r][1], Cn[r][2], Cn[r][3]);
+    }
+};
+template <bool VISC>
+__global__ void __launch_bounds__(128) k_fv_linst(FVK K, const float *u, double adt, double sigma, float *dtau, int fac,
+                                                  float *uc, int bf16, float4 *st) {
+    k_fv_linst_b<VISC>::run(blockIdx.x, gridDim.x, K, u, adt, sigma, dtau, fac, uc, bf16, st);
 }
 
 // DG pseudo-time step of an element, lambda_E = (k+1)^2 max_nodes(|v| + c)(1/hx + 1/hz)
@@ -1074,6 +1244,7 @@ FVK make_fvk(jfnk_ctx *c, int l) {
     K.hbxw = L.hbxw;
     K.hbz = L.hbz;
     K.ubf = L.ubf;
+    K.st = (const float4 *)L.st;
     return K;
 }
 
@@ -1143,8 +1314,15 @@ void launch_fv(bool l4, unsigned g, int tb, cudaStream_t s, const FVK &K, const 
                const typename SOf<T>::type *x, const typename SOf<T>::type *b, const typename SOf<T>::type *dt,
                const double *fu, double adt, typename SOf<T>::type *out, int bf = 0,
                RKS rk = RKS{nullptr, 0, 1.0, 1.0f}) {
+    if constexpr (std::is_same<T, TL32>::value) {
+        if (K.st) {
+            jf_launch<k_fv_b<T, IN, MODE, false, true>>(k_fv<T, IN, MODE, false, true>, g, tb, 0, s, K, ld, x, b, dt, fu, adt, out, bf, rk);
+            jf_launched();
+            return;
+        }
+    }
     if (l4) {
-        jf_launch<k_fv_b<T, IN, MODE, V>>(k_fv<T, IN, MODE, V>, g, tb, 0, s, K, ld, x, b, dt, fu, adt, out, bf, rk);
+        jf_launch<k_fv_b<T, IN, MODE, V, false>>(k_fv<T, IN, MODE, V, false>, g, tb, 0, s, K, ld, x, b, dt, fu, adt, out, bf, rk);
     } else if (tb >= 256) {   // tile rows follow the block size: 32 x 8 or 32 x 4 cells
         const unsigned gt = (unsigned)(((K.NX + FV_TX - 1) / FV_TX) * ((K.NZ + 7) / 8));
         jf_launch<k_fv_tile_b<T, IN, MODE, V, 8>>(k_fv_tile<T, IN, MODE, V, 8>, gt, FV_TX * 8, 0, s, K, ld, b, dt, fu, adt, out, nullptr, nullptr, bf,
@@ -1200,7 +1378,7 @@ int fv_op32(jfnk_ctx *c, int l, int mode, const float *x, const float *b, float 
     const bool visc = c->phys.mu != 0.0;
     c->fv_calls++;
     const int tb = c->opts.tile_fv;
-    const bool l4 = fv_four_lanes(c, n1);
+    const bool l4 = L.st || fv_four_lanes(c, n1);
     const unsigned g = nblk((l4 ? 4 : 1) * n1, tb);
     FLoad<TL32, 2> ld{(const float *)L.u, x, n1};
     const float *dt = (const float *)L.dtau;
@@ -1229,7 +1407,7 @@ int fv_smooth32_corrected(jfnk_ctx *c, int l, const float *x, bool zero, const f
     const bool visc = c->phys.mu != 0.0;
     c->fv_calls++;
     const int tb = c->opts.tile_fv;
-    const bool l4 = fv_four_lanes(c, n1);
+    const bool l4 = L.st || fv_four_lanes(c, n1);
     const unsigned g = nblk((l4 ? 4 : 1) * n1, tb);
     FLoad<TL32, 3> ld{(const float *)L.u, x, (const float *)C.x, n1, C.NX, L.fac, zero ? 1 : 0,
                       (size_t)C.NX * C.NZ};
@@ -1261,7 +1439,7 @@ int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *b
     const size_t nc = (size_t)C.NX * C.NZ;
     const bool visc = c->phys.mu != 0.0;
     const int tb = c->opts.tile_fv;
-    const bool l4 = fv_four_lanes(c, n1);
+    const bool l4 = L.st || fv_four_lanes(c, n1);
     const bool f2 = L.fac == 2;
     const unsigned g = nblk((f2 ? 16 : 4) * nc, tb);   // lanes per coarse cell
     c->fv_calls++;
@@ -1280,11 +1458,11 @@ int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *b
         JF_CK(cudaGetLastError());
         return JFNK_OK;
     }
-#define JF_DR(T, IN, V, F2, ...) jf_launch<k_fv_defect_restrict_b<T, IN, V, F2>>(k_fv_defect_restrict<T, IN, V, F2>, g, tb, 0, s, __VA_ARGS__)
-#define JF_DR2(T, IN, V, ...)                            \
-    do {                                                 \
-        if (f2) JF_DR(T, IN, V, true, __VA_ARGS__);      \
-        else JF_DR(T, IN, V, false, __VA_ARGS__);        \
+#define JF_DR(T, IN, V, F2, ST, ...) jf_launch<k_fv_defect_restrict_b<T, IN, V, F2, ST>>(k_fv_defect_restrict<T, IN, V, F2, ST>, g, tb, 0, s, __VA_ARGS__)
+#define JF_DR2(T, IN, V, ST, ...)                            \
+    do {                                                     \
+        if (f2) JF_DR(T, IN, V, true, ST, __VA_ARGS__);      \
+        else JF_DR(T, IN, V, false, ST, __VA_ARGS__);        \
     } while (0)
     // large levels with 2 x 2 agglomeration: the face-once tile kernel
     const int tz = tb >= 256 ? 8 : 4;   // tile rows follow the block size
@@ -1318,8 +1496,8 @@ int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *b
 #undef JF_DRT
 #define JF_DR4(T, IN, ...)                                   \
     do {                                                     \
-        if (visc) JF_DR2(T, IN, true, __VA_ARGS__);          \
-        else JF_DR2(T, IN, false, __VA_ARGS__);              \
+        if (visc) JF_DR2(T, IN, true, false, __VA_ARGS__);   \
+        else JF_DR2(T, IN, false, false, __VA_ARGS__);       \
     } while (0)
     if (c->prec == 64) {
         double *epsp = c->scal + S_EPSFV + l;
@@ -1330,8 +1508,12 @@ int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *b
     } else {
         FLoad<TL32, 2> ld{(const float *)L.u, (const float *)x, n1};
         const int bf = (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0;   // BF16 coarsest level
-        JF_DR4(TL32, 2, K, ld, (const float *)b, nullptr, c->mg_adt, L.fac, (float *)bc, (float *)xc,
-               (const float *)dtc, bf);
+        if (K.st)
+            JF_DR2(TL32, 2, false, true, K, ld, (const float *)b, nullptr, c->mg_adt, L.fac, (float *)bc, (float *)xc,
+                   (const float *)dtc, bf);
+        else
+            JF_DR4(TL32, 2, K, ld, (const float *)b, nullptr, c->mg_adt, L.fac, (float *)bc, (float *)xc,
+                   (const float *)dtc, bf);
     }
 #undef JF_DR4
 #undef JF_DR2
@@ -1736,6 +1918,12 @@ int mg_linearize(jfnk_ctx *c, const double *Uin, double adt, cudaStream_t s) {
             JF_RET(fv_op64(c, l, FV_RES, (const double *)L.u, nullptr, nullptr, (double *)L.fu, s));
             jf_launch<k_fv_lin_b<double>>(k_fv_lin<double>, nblk(n1), 128, 0, s, K, (const double *)L.u, adt, c->opts.sigma_fv,
                       (double *)L.dtau, L.fac, (double *)uc, 0);
+        } else if (L.st && c->phys.mu != 0.0) {
+            jf_launch<k_fv_linst_b<true>>(k_fv_linst<true>, nblk(4 * n1), 128, 0, s, K, (const float *)L.u, adt, c->opts.sigma_fv,
+                      (float *)L.dtau, L.fac, (float *)uc, bf, (float4 *)L.st);
+        } else if (L.st) {
+            jf_launch<k_fv_linst_b<false>>(k_fv_linst<false>, nblk(4 * n1), 128, 0, s, K, (const float *)L.u, adt, c->opts.sigma_fv,
+                      (float *)L.dtau, L.fac, (float *)uc, bf, (float4 *)L.st);
         } else {
             jf_launch<k_fv_lin_b<float>>(k_fv_lin<float>, nblk(n1), 128, 0, s, K, (const float *)L.u, adt, c->opts.sigma_fv,
                       (float *)L.dtau, L.fac, (float *)uc, bf);
