@@ -70,9 +70,30 @@ JF_D double join(F2 a) {
     const long long k = (long long)__float2int_rn(__fmul_rn(L, sc));
     return __longlong_as_double(__double_as_longlong(f2d_normal(H)) + k);
 }
-// direction entries: FP32 vectors are exact in the first part
-JF_D F2 y2(float y) { return F2{y, 0.0f}; }
-JF_D F2 y2(double y) { return split2(y); }
+// Direction entries as two floats.  FP32 vectors are exact in the first part.  FP64 ones
+// are scaled by the power of two that brings |y| (from eps = sqrt(eps_mach)/|y|) to about
+// one, so that a direction of any magnitude keeps its 48 bits; `es` is eps scaled back.
+template <class Y> struct Dir;
+template <> struct Dir<float> {
+    double es;
+    JF_D explicit Dir(double eps) : es(eps) {}
+    JF_D F2 operator()(float y) const { return F2{y, 0.0f}; }
+};
+template <> struct Dir<double> {
+    double es;
+    int k;
+    JF_D explicit Dir(double eps) {
+        const int hi = __double2hiint(eps), f = (hi >> 20) & 0x7ff;
+        k = f - 997;   // binary exponent of eps, plus 26
+        es = f ? __hiloint2double(hi - (k << 20), __double2loint(eps)) : eps * __hiloint2double(2020 << 20, 0);
+    }
+    JF_D F2 operator()(double y) const {
+        const int hi = __double2hiint(y), f = (hi >> 20) & 0x7ff;
+        if (f == 0x7ff) return split2(y);           // infinity, NaN
+        if (f == 0 || f + k <= 0) return F2{0.0f, 0.0f};
+        return split2(__hiloint2double(hi + (k << 20), __double2loint(y)));
+    }
+};
 JF_D double y64(float y) { return f2d_normal(y); }
 JF_D double y64(double y) { return y; }
 JF_D double y64_any(float y) { return f2d_conv(y); }   // any input (NaN, infinity, subnormal)
@@ -102,6 +123,7 @@ template <class Y, int NP1, bool VISC>
 JF_D void fd_faces(const DGF &K, const Y *y, double eps, float2 *phix, float2 *symx, float2 *phiz, float2 *symz,
                    unsigned blk) {
     constexpr int NP = NP1 * NP1;
+    const Dir<Y> dir(eps);
     const int nx = K.nx, nz = K.nz;
     const size_t N1 = (size_t)K.n_el * NP;
     const long long nvert = (long long)nz * (nx + 1) * NP1, nf = nvert + (long long)(nz + 1) * nx * NP1;
@@ -136,7 +158,7 @@ JF_D void fd_faces(const DGF &K, const Y *y, double eps, float2 *phix, float2 *s
         F2 aL{0.f, 0.f}, aR{0.f, 0.f}, dL{0.f, 0.f}, dR{0.f, 0.f};
 #pragma unroll
         for (int q = 0; q < NP1; ++q) {
-            const F2 yl = y2(y[v * N1 + bL + q * st]), yr = y2(y[v * N1 + bR + q * st]);
+            const F2 yl = dir(y[v * N1 + bL + q * st]), yr = dir(y[v * N1 + bR + q * st]);
             f2_fma(aL, f2(K.lp[q]), yl);
             f2_fma(aR, f2(K.lm[q]), yr);
             if (VISC) {
@@ -146,12 +168,12 @@ JF_D void fd_faces(const DGF &K, const Y *y, double eps, float2 *phix, float2 *s
         }
         const double tL = K.lin.tr[(2 * v) * nf + t], tR = K.lin.tr[(2 * v + 1) * nf + t];
         const double yL = join(aL), yR = join(aR);
-        UL[v] = D64{__fma_rn(eps, yL, tL)};
-        UR[v] = D64{__fma_rn(eps, yR, tR)};
+        UL[v] = D64{__fma_rn(dir.es, yL, tL)};
+        UR[v] = D64{__fma_rn(dir.es, yR, tR)};
         if (VISC) {
-            gL[v] = D64{__fma_rn(eps, join(dL), K.lin.tr[(8 + 2 * v) * nf + t])};
-            gR[v] = D64{__fma_rn(eps, join(dR), K.lin.tr[(9 + 2 * v) * nf + t])};
-            J[v] = D64{__fma_rn(eps, __dsub_rn(yL, yR), K.lin.tr[(16 + v) * nf + t])};
+            gL[v] = D64{__fma_rn(dir.es, join(dL), K.lin.tr[(8 + 2 * v) * nf + t])};
+            gR[v] = D64{__fma_rn(dir.es, join(dR), K.lin.tr[(9 + 2 * v) * nf + t])};
+            J[v] = D64{__fma_rn(dir.es, __dsub_rn(yL, yR), K.lin.tr[(16 + v) * nf + t])};
         }
     }
     swap_d(zf, UL[1], UL[2]);
@@ -201,6 +223,7 @@ JF_D void fd_nodes(const DGF &K, const Y *y, double eps, float2 *part, unsigned 
     __shared__ float2 sF[2][EPB][4][NP];              // flux differences
     __shared__ float2 sy[VISC ? EPB : 1][4][VISC ? NP : 1];
     __shared__ float2 sD[2][NP1][NP1], sDn[VISC ? 2 : 1][NP1][NP1];
+    const Dir<Y> dir(eps);
     const int epb = blockDim.x / NP;
     const int le = threadIdx.x / NP, node = threadIdx.x % NP;
     const int a = node % NP1, b = node / NP1;
@@ -217,11 +240,11 @@ JF_D void fd_nodes(const DGF &K, const Y *y, double eps, float2 *part, unsigned 
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             yv[v] = y[v * N1 + gi0];
-            if (VISC) sy[le][v][node] = f2v(y2(yv[v]));
+            if (VISC) sy[le][v][node] = f2v(dir(yv[v]));
         }
     }
     if (VISC) __syncthreads();
-    const F2 e2 = split2(eps);
+    const F2 e2 = split2(dir.es);
     if (active) {
         D64 U[4];
 #pragma unroll
@@ -231,8 +254,8 @@ JF_D void fd_nodes(const DGF &K, const Y *y, double eps, float2 *part, unsigned 
         const D64 vu = U[1] * ir, vw = U[2] * ir;
         D64 Fx[4], Fz[4];
         flux_xz(U, vu, vw, p, Fx, Fz);
-        sF[0][le][0][node] = f2v(f2_mul(e2, y2(yv[1])));   // the mass fluxes are linear
-        sF[1][le][0][node] = f2v(f2_mul(e2, y2(yv[2])));
+        sF[0][le][0][node] = f2v(f2_mul(e2, dir(yv[1])));   // the mass fluxes are linear
+        sF[1][le][0][node] = f2v(f2_mul(e2, dir(yv[2])));
         if (VISC) {
             D64 dx[4], dz[4];
 #pragma unroll
@@ -243,8 +266,8 @@ JF_D void fd_nodes(const DGF &K, const Y *y, double eps, float2 *part, unsigned 
                     f2_fma(sx, f2(sDn[0][a][q]), f2(sy[le][v][b * NP1 + q]));
                     f2_fma(sz, f2(sDn[VISC ? 1 : 0][b][q]), f2(sy[le][v][q * NP1 + a]));
                 }
-                dx[v] = D64{__fma_rn(eps, join(sx), K.lin.F[(5 + v) * N1 + gi0])};
-                dz[v] = D64{__fma_rn(eps, join(sz), K.lin.F[(9 + v) * N1 + gi0])};
+                dx[v] = D64{__fma_rn(dir.es, join(sx), K.lin.F[(5 + v) * N1 + gi0])};
+                dz[v] = D64{__fma_rn(dir.es, join(sz), K.lin.F[(9 + v) * N1 + gi0])};
             }
             const D64 phi[4] = {vu, vu, vw, U[3] * ir};
             const D64 mu = D64{K.mu};
@@ -278,7 +301,7 @@ JF_D void fd_nodes(const DGF &K, const Y *y, double eps, float2 *part, unsigned 
             f2_fma(f, f2(sD[0][a][q]), f2(sF[0][le][v][b * NP1 + q]));
             f2_fma(f, f2(sD[1][b][q]), f2(sF[1][le][v][q * NP1 + a]));
         }
-        if (v == 2) f2_fma(f, f2_neg(f2(K.g)), f2_mul(e2, y2(yv[0])));
+        if (v == 2) f2_fma(f, f2_neg(f2(K.g)), f2_mul(e2, dir(yv[0])));
         part[v * N1 + gi0] = f2v(f);
     }
 }

@@ -55,3 +55,18 @@ def test_product_about_linearisation(name, w):
         z[3] = float("nan")
         ctx.jv_product(Ug, None, z, adt, 0.0, J2)
         assert not bool(torch.isfinite(J2).all())        # NaN is not swallowed
+
+
+@pytest.mark.parametrize("e", [-330, -130, 130, 330])
+def test_direction_of_any_magnitude(e):
+    """eps is inversely proportional to |y|, so a direction scaled by a power of two gives the scaled
+    product bit for bit (also far outside the range of single precision)."""
+    import torch
+    w = synth.scaled(synth.DENSITY_CURRENT_Q2_256x32, 9, 4)
+    dg = oracle_dg(w)
+    U, y = to_gpu(perturbed_state(w, dg).ravel()), to_gpu(synth.random_perturbation(dg.shape[1:], 11).ravel())
+    ctx = gpu_context(w)
+    J1, J2 = torch.empty_like(U), torch.empty_like(U)
+    ctx.jv_product(U, None, y, 0.3 * w.dt, 0.0, J1)
+    ctx.jv_product(U, None, y * 2.0 ** e, 0.3 * w.dt, 0.0, J2)
+    assert bool(((J2 * 2.0 ** -e) == J1).all())
