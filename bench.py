@@ -52,9 +52,9 @@ FALLBACK_HBM_GBS = 6800.0
 # FP64 arithmetic per SM and clock: the nominal 1.25 TFLOP/s of a 152-SM GB300 at
 # 2.07 GHz is 2 DFMA (4 flops) per SM and clock
 FP64_FLOP_PER_SM_CLK = 4.0
-# DRAM bytes (read + write) of one FP64 FD-product face launch on this workload,
-# ncu, cold L2 (writes stay in L2)
-TRAFFIC_FACE = 13_339_136
+# DRAM bytes (read + write) of one FD product about the stored linearisation on this
+# workload (flux launch 28.02 MB, lift launch 13.15 MB), ncu, cold L2 (writes stay in L2)
+TRAFFIC_FD = 41_165_000
 
 
 def parse():
@@ -234,27 +234,25 @@ def timed_once(ctx, U, w, **kw):
 
 
 # ---------------------------------------------------------------------------
-# Algorithmic FP64 flops of the FD product, from the formulas (a divide, square
-# root or x^gamma counts one flop, an FMA two, compares and selects none):
-#  face point, stored traces of U plus eps times the traces of y:
-#    traces of y: 2 sides x 4 variables x (k+1) FMA; tr(U) + eps tr(y): 8 FMA;
-#    + background: 8; HLLC: 1/rho 2, velocities 2, pressures 2 x 3, sound speeds
-#    2 x 3, wave-speed bounds 4, S - u 2, contact speed numerator 7, denominator
-#    3, quotient 1, star factor 4, star state 5, side flux 4, F + S (U* - U) 12
-#    (58); minus the background flux: 4
-#  node, volume term: U + eps y 4 FMA; + background 4; 1/rho 1; pressure 3;
-#    velocities 2; two convective fluxes 8; minus the background fluxes 8;
-#    sum factorisation 4 variables x 2 directions x (k+1) FMA; gravity 2; lift of
-#    the four face terms 4 x 4 FMA; FD quotient and update 3 per variable
-HLLC_FLOPS = 58
+# Algorithmic flops of the FD product about a stored linearisation, from the formulas (a
+# divide, square root or x^gamma counts one flop, an FMA two, compares and selects none):
+#  face point, stored states of U plus eps times the traces of y:
+#    traces of y: 2 sides x 4 variables x (k+1) FMA; U + eps tr(y): 8 FMA; HLLC in
+#    contact form: 1/rho 2, velocities 2, pressures 2 x 3, sound speeds 2 x 3, their
+#    differences 3, rho (S - u) 2, contact speed 7, star mass 3, side factors 1, flux 6
+#    (38); minus the stored flux: 4
+#  node: U + eps y 4 FMA; 1/rho 1; pressure 3; velocities 2; fluxes 7; minus the stored
+#    fluxes 5; sum factorisation 4 variables x 2 directions x (k+1) FMA; gravity 2; lift
+#    of the four face terms 4 x 4 FMA; quotient and update 1 FMA per variable
+HLLC_FLOPS = 38
 
 
 def alg_flops_face_point(k):
-    return 2 * (2 * 4 * (k + 1)) + 2 * 8 + 8 + HLLC_FLOPS + 4
+    return 2 * (2 * 4 * (k + 1)) + 2 * 8 + HLLC_FLOPS + 4
 
 
 def alg_flops_node(k):
-    return 2 * 4 + 4 + 1 + 3 + 2 + 8 + 8 + 2 * (4 * 2 * (k + 1)) + 2 + 2 * 16 + 3 * 4
+    return 2 * 4 + 1 + 3 + 2 + 7 + 5 + 2 * (4 * 2 * (k + 1)) + 2 + 2 * 16 + 2 * 4
 
 
 def fp64_peak_tflops(sm_mhz):
@@ -871,7 +869,7 @@ def main():
         U0 = initial_state(c64, w)
         y = torch.randn(c64.N, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
         fm, vm = c64.time_operator(1, U0, y, args.profile_dg)
-        print(json.dumps({"profile": "FP64 FD product", "face_ms": fm, "volume_ms": vm, "reps": args.profile_dg}))
+        print(json.dumps({"profile": "FP64 FD product", "flux_ms": fm, "lift_ms": vm, "reps": args.profile_dg}))
         return
     if args.profile_ensemble >= 0:
         members = [m for m in synth.ensemble(args.ensemble) if args.ensemble_order in (0, m.k)]
@@ -950,7 +948,7 @@ def main():
     e2e_ms = max_over_ranks(e2e_ms, dist)
     e2e = world * ne2e / (e2e_ms / 1e3)
 
-    # ---- roofline of the dominant kernel (FP64 FD product, face kernel) --------
+    # ---- roofline of the FD product of the Arnoldi steps (FP64 fluxes) ---------
     peaks = measured_peaks()
     hbm_peak = peaks.get("hbm_gbs") or FALLBACK_HBM_GBS
     hbm_note = "of measured (MEASURED_PEAKS.json hbm_gbs)" if peaks.get("hbm_gbs") else "of fallback"
@@ -958,22 +956,23 @@ def main():
     peak64, nsm = fp64_peak_tflops(sm_mhz)
     y = torch.randn(ctx.N, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
     ctx64 = make_context(w, 64, **preset)
-    fm, vm = ctx64.time_operator(1, U0, y, 20)
+    ctx.time_operator(1, U0, y, 3)
+    fm, vm = ctx.time_operator(1, U0, y, 20)   # FP32 directions, as the Arnoldi steps pass them
     n1 = w.k + 1
     face_pts = (w.nz * (w.nx + 1) + (w.nz + 1) * w.nx) * n1
     nodes = w.n_el * n1 * n1
     fl_face, fl_node = alg_flops_face_point(w.k), alg_flops_node(w.k)
-    ach = fl_face * face_pts / (fm * 1e-3) / 1e12
-    ach_v = fl_node * nodes / (vm * 1e-3) / 1e12
-    roof = {"bound": "alu", "kernel": "k_faces<D64> FP64 FD product (face points)", "achieved": ach,
-            "peak": peak64, "unit": "TFLOP/s", "frac": ach / peak64, "traffic": TRAFFIC_FACE,
+    flops = fl_face * face_pts + fl_node * nodes
+    ach = flops / ((fm + vm) * 1e-3) / 1e12
+    roof = {"bound": "alu", "kernel": "k_fd_flux + k_fd_lift: one FD product about the stored linearisation",
+            "achieved": ach, "peak": peak64, "unit": "TFLOP/s", "frac": ach / peak64, "traffic": TRAFFIC_FD,
             "peak_source": (f"derived, not measured: {nsm} SMs (device properties) x {FP64_FLOP_PER_SM_CLK:g} FP64 "
                             f"flop/SM/clock x {sm_mhz:g} MHz"),
-            "launch_ms": fm, "flop_per_unit": fl_face, "units_per_launch": face_pts,
-            "flop_counting": "algorithmic, from the formulas (bench.py alg_flops_face_point); ncu counts 250 "
-                             "executed FP64-pipe flops per face point (IEEE divide/sqrt sequences, table power)",
-            "volume_kernel": {"achieved": ach_v, "frac": ach_v / peak64, "launch_ms": vm,
-                              "flop_per_unit": fl_node, "units_per_launch": nodes},
+            "flux_launch_ms": fm, "lift_launch_ms": vm, "flop": flops,
+            "units": {"face_points": face_pts, "flop_per_face_point": fl_face, "nodes": nodes, "flop_per_node": fl_node},
+            "flop_counting": "algorithmic, from the formulas (bench.py alg_flops_face_point, alg_flops_node); the traces, "
+                             "derivatives and lifts run in two-float arithmetic on the FP32 pipe, about 63 FP64 "
+                             "instructions a face point and 25 a node remain",
             "hbm": kernel_bandwidths(w, preset, hbm_peak, hbm_note, flush, U0)}
 
     # ---- phase breakdown of one more step (events at the solver's own syncs) ----

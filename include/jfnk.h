@@ -119,18 +119,22 @@ typedef struct {
     int precond_prec;
     double sigma_fv, sigma_dg, c_ip;
     int use_graphs;
-    int tile_faces;      /* threads per block of the DG face kernel: 64, 128, 256 (0: 128) */
-    int tile_volume;     /* elements per DG volume block: 1 = ~64 threads, 2 = ~128 (0: 2) */
+    int tile_faces;      /* 64, 128, 256 (0: 128); accepted, without effect: face points share the
+                            blocks of tile_volume */
+    int tile_volume;     /* DG operator blocks: 1 = ~64 threads, 2 = ~128 (0: 2); smaller ones on
+                            grids that leave SMs without work */
     int tile_fv;         /* threads per block of the FV cell kernels: 64, 128, 256 (0: 128); the
                             face-once kernel of large levels takes 32 x 8 cells at 256, 32 x 4 else */
     int fv_split_cells;  /* FV levels with fewer cells than this run four lanes per cell (one
-                            per face), larger levels the face-once tile kernel (0: 65536) */
+                            per face), larger levels the face-once tile kernel (0: 65536); FP32
+                            levels of at most 4096 cells always run four lanes per cell */
     int profile;         /* 1: time the phases of implicit_step with CUDA events (jfnk_stats) */
     double precond_fd_eps;
     double time_budget_ms;
     int dg_fused;        /* FP32 tangent DG products of the preconditioner: 0 or 1 one fused
-                            launch per product (faces, volume and epilogue per element strip),
-                            2 a face launch and a volume launch */
+                            launch per product (faces, volume and epilogue per element strip;
+                            mu = 0: from flux derivatives the linearisation keeps), 2 a flux
+                            launch and a lift launch of the tangent fluxes */
     int rk_stages;       /* stages s of the pseudo-time smoother (Sec. 3.5), 1..4 (0: 1) */
     double rk_alpha[4];  /* its low-storage coefficients: one smoothing step is
                             w_k = w_0 + rk_alpha[k-1] dtau (b - g'w_{k-1}), k = 1..s; the
@@ -197,7 +201,10 @@ int dg_residual(jfnk_ctx *ctx, const double *U_dev, double *f_dev, void *stream)
 /* Jacobian-free product of Sec. 3.1 for G(U) = U - alpha_dt f(U) - Ubar_s:
  *   G'(U) y ~ y - alpha_dt (f(U + eps y) - f(U)) / eps,
  * eps = sqrt(eps_mach)/|y|_2 (eps_mach = 2^-52) when eps <= 0, else the given
- * eps.  fU_dev = f(U) may be NULL (then computed here).  y = 0 gives Jy = 0.
+ * eps.  fU_dev = f(U) may be NULL (then computed here; with eps <= 0 its states
+ * and fluxes are kept and the product takes the form of the solver's Arnoldi
+ * steps: fluxes at U + eps y minus those at U, linear parts applied to the
+ * differences).  y = 0 gives Jy = 0.  Nothing is copied or synchronised.
  * All vectors are N doubles on the device; Jy must not alias U, fU or y. */
 int jv_product(jfnk_ctx *ctx, const double *U_dev, const double *fU_dev, const double *y_dev,
                double alpha_dt, double eps, double *Jy_dev, void *stream);
@@ -345,13 +352,13 @@ int jfnk_eos_pressure(jfnk_ctx *ctx, const double *E_dev, size_t n, double *p_de
 int jfnk_tangent_product(jfnk_ctx *ctx, const double *U_dev, const double *y_dev, double alpha_dt,
                          double *out_dev, void *stream);
 
-/* Times the two kernels of one DG operator evaluation with CUDA events
- * recorded on `stream` around each launch: which 0 = FP64 residual,
- * 1 = FP64 finite-difference product with direction y (in the form the
- * solver's Arnoldi steps use: face traces of U stored by the residual at U,
- * plus eps times the traces of y), 2 = FP32 tangent product (contexts with
- * precond_prec < 64).  Runs `reps` evaluations;
- * ms[0], ms[1] receive the mean duration of the face and the volume kernel.
+/* Times the two launches of one DG operator evaluation with CUDA events
+ * recorded on `stream` around each: which 0 = FP64 residual, 1 = FP64
+ * finite-difference product with direction y (in the form the solver's Arnoldi
+ * steps use: about the linearisation the residual at U stores; y rounded to FP32
+ * when precond_prec < 64), 2 = FP32 tangent product (contexts with precond_prec
+ * < 64).  Runs `reps` evaluations; ms[0] receives the mean duration of the flux
+ * launch (face points and nodes), ms[1] of the lift launch.
  * which 3 (FP32 contexts with a preconditioner): the finest FV level's two
  * FP32 kernels linearised at U with alpha dt = 1 and x = b = y, ms[0] one
  * pseudo-time smoothing step, ms[1] the defect fused with the restriction;
@@ -361,9 +368,9 @@ int jfnk_tangent_product(jfnk_ctx *ctx, const double *U_dev, const double *y_dev
 int jfnk_time_operator(jfnk_ctx *ctx, int which, const double *U_dev, const double *y_dev, int reps,
                        double *ms_host, void *stream);
 
-/* Autotuner of the launch shapes: times every (tile_faces, tile_volume)
- * pair on `reps` FP64 FD products at state U with direction y (CUDA events on
- * `stream`), and every (tile_fv, fv_split_cells) pair on `reps` preconditioner
+/* Autotuner of the launch shapes: times every tile_volume on `reps` FP64 FD
+ * products at state U with direction y (CUDA events on `stream`; tile_faces has
+ * no effect and is kept), and every (tile_fv, fv_split_cells) pair on `reps` preconditioner
  * applications linearised at U (contexts with a preconditioner), keeps the
  * fastest in the context and writes them to best[0..3] = tile_faces,
  * tile_volume, tile_fv, fv_split_cells (host) and their times in ms to

@@ -722,26 +722,21 @@ int jfnk_autotune(jfnk_ctx *c, const double *U, const double *y, int reps, int *
     const int keep_sp = c->opts.fv_split_cells;
     jf_invalidate_graphs(c);   // captured graphs hold the old launch shapes
     double best_dg = 1e300;
-    int bf = keep_f, bv = keep_v;
-    const int fs[3] = {64, 128, 256}, vs[2] = {1, 2};
-    for (int fi = 0; fi < 3; ++fi)
-        for (int vi = 0; vi < 2; ++vi) {
-            c->opts.tile_faces = fs[fi];
-            c->opts.tile_volume = vs[vi];
-            double t[2];
-            int rc = jfnk_time_operator(c, 1, U, y, reps + 1, t, stream);   // first rep warms up
-            if (rc) {
-                c->opts.tile_faces = keep_f;
-                c->opts.tile_volume = keep_v;
-                return rc;
-            }
-            if (t[0] + t[1] < best_dg) {
-                best_dg = t[0] + t[1];
-                bf = fs[fi];
-                bv = vs[vi];
-            }
+    const int bf = keep_f;
+    int bv = keep_v;
+    for (int v = 1; v <= 2; ++v) {
+        c->opts.tile_volume = v;
+        double t[2];
+        int rc = jfnk_time_operator(c, 1, U, y, reps + 1, t, stream);   // first rep warms up
+        if (rc) {
+            c->opts.tile_volume = keep_v;
+            return rc;
         }
-    c->opts.tile_faces = bf;
+        if (t[0] + t[1] < best_dg) {
+            best_dg = t[0] + t[1];
+            bv = v;
+        }
+    }
     c->opts.tile_volume = bv;
     double best_mg = 0.0;
     int bfv = keep_fv, bsp = keep_sp;
