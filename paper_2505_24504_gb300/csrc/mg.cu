@@ -13,6 +13,7 @@
 //             pseudo-time step x + dtau (b - g'x), defect g'x - b.  g' is the
 //             FD quotient of Sec. 3.1 (FP64) or the exact tangent (FP32).
 //  k_restrict / k_prolong   agglomeration R and injection P (Sec. 3.4).
+//  k_map_eps    the same two and the first DG step of the FP64 form, with eps of what they write.
 //  mg_cycle   MG_l(x, b; u) of Sec. 3.4 on the host; every level's work is a few
 //             launches on the caller's stream, so an application can be captured
 //             in one CUDA graph.
@@ -854,6 +855,63 @@ struct TK {
     DGTab tab;
 };
 
+// ---- norm of what a kernel writes --------------------------------------------
+// The FP64 form's FD products need eps = cnum/|x| of the x their predecessor writes.
+// The writers reduce it themselves: a block adds up its squares, the block that takes
+// the last ticket adds the blocks' sums in block order and writes eps (out = nullptr:
+// nothing is reduced).  A dot product of its own cost a launch and a round of loads
+// more, seven times an application, and the defect's subtraction another launch: the
+// backward-Euler step of Q2 20x10 takes 12.34 ms against 12.81, Q2 62x29 14.07 against 14.34.
+struct EpsOut {
+    double *part;       // one sum per block
+    unsigned *ticket;   // back at zero after the launch
+    double *out;
+    double cnum;
+};
+// sum over the block's threads (TPB at most), valid in thread 0
+template <int TPB>
+__device__ __forceinline__ double eps_sum(double v) {
+    __shared__ double sv[TPB];
+    sv[threadIdx.x] = v;
+    __syncthreads();
+    double r = 0.0;
+    if (threadIdx.x < 32) {
+#pragma unroll 4
+        for (int k = threadIdx.x; k < blockDim.x; k += 32) r += sv[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+    }
+    __syncthreads();
+    return r;
+}
+// every thread of every block calls it (at least 32 threads a block)
+template <int TPB>
+__device__ __forceinline__ void eps_close(double sq, const EpsOut &E, unsigned bid, unsigned nblk) {
+    __shared__ bool last;
+    sq = eps_sum<TPB>(sq);
+    if (threadIdx.x == 0) {
+        E.part[bid] = sq;
+        __threadfence();
+        last = atomicAdd(E.ticket, 1u) == nblk - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double t = 0.0;
+    for (unsigned i = threadIdx.x; i < nblk; i += blockDim.x) t += __ldcg(E.part + i);
+    t = eps_sum<TPB>(t);
+    if (threadIdx.x == 0) {
+        *E.out = t > 0.0 ? div64(E.cnum, sqrt64(t)) : 0.0;
+        *E.ticket = 0u;
+    }
+}
+// what the FP64 transfers take besides: w is subtracted from u as it is read (the DG
+// defect r - G'z, which took a launch of its own), e reduces what is written
+struct XferX {
+    const double *w;
+    EpsOut e;
+};
+
 template <class Si, class So> struct RealOf { typedef float type; };
 template <> struct RealOf<double, double> { typedef double type; };
 
@@ -884,9 +942,10 @@ struct k_to_fv_b {
     static constexpr int TPB = 128, MINB = 0;
     static constexpr bool GROUP = std::is_same<So, float>::value;   // a grouped twin is built (lock-step ensembles)
     static constexpr bool LIN = std::is_same<Si, double>::value && std::is_same<So, float>::value;
+    static constexpr bool X64 = std::is_same<Si, double>::value && std::is_same<So, double>::value;
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<TK> K, JfArg<const Si *> u,
                                                JfArg<So *> v, JfArg<int> massfix, JfArg<So *> x0,
-                                               JfArg<const So *> dtau0, JfArg<LinOut> lo) {
+                                               JfArg<const So *> dtau0, JfArg<LinOut> lo, JfArg<XferX> xx) {
         jf_pdl_enter();
         typedef typename RealOf<Si, So>::type R;
         constexpr int NP = NP1 * NP1;
@@ -906,7 +965,9 @@ struct k_to_fv_b {
             float W[4];
             for (int q = 0; q < 4; ++q) {
                 const size_t gi = q * N1 + (size_t)e * NP + node;
-                const Si ui = u[gi];
+                Si ui = u[gi];
+                if constexpr (X64)
+                    if (xx.w) ui -= xx.w[gi];
                 su[le][q][node] = (R)ui;
                 if (LIN) {
                     lo.Ul[gi] = ui;
@@ -964,20 +1025,29 @@ struct k_to_fv_b {
             sc[le][q] = massfix ? (mfv / (R)NP - mnc) : (R)0;
         }
         __syncthreads();
-        if (!act) return;
+        if (!X64 && !act) return;
         const int ez = e / K.nx, ex = e % K.nx;
         const size_t I = (size_t)ex * NP1 + i, Jr = (size_t)ez * NP1 + j;
         const size_t n1 = (size_t)K.NX * K.NZ;
-        for (int q = 0; q < 4; ++q) {
-            const So val = (So)(Tu[q] - sc[le][q]);
-            v[q * n1 + Jr * K.NX + I] = val;
-            if (x0) x0[q * n1 + Jr * K.NX + I] = dtau0[Jr * K.NX + I] * val;   // first step from zero
-        }
+        double sq = 0.0;
+        if (act)
+            for (int q = 0; q < 4; ++q) {
+                const So val = (So)(Tu[q] - sc[le][q]);
+                v[q * n1 + Jr * K.NX + I] = val;
+                if (x0) {   // first step from zero
+                    const So xv = dtau0[Jr * K.NX + I] * val;
+                    x0[q * n1 + Jr * K.NX + I] = xv;
+                    if (X64) sq = fma((double)xv, (double)xv, sq);
+                }
+            }
+        if constexpr (X64)
+            if (xx.e.out) eps_close<128>(sq, xx.e, jf_bid, jf_nblk);
     }
 };
 template <class Si, class So, int NP1>
-__global__ void __launch_bounds__(128) k_to_fv(TK K, const Si *u, So *v, int massfix, So *x0, const So *dtau0, LinOut lo) {
-    k_to_fv_b<Si, So, NP1>::run(blockIdx.x, gridDim.x, K, u, v, massfix, x0, dtau0, lo);
+__global__ void __launch_bounds__(128) k_to_fv(TK K, const Si *u, So *v, int massfix, So *x0, const So *dtau0, LinOut lo,
+                                               XferX xx) {
+    k_to_fv_b<Si, So, NP1>::run(blockIdx.x, gridDim.x, K, u, v, massfix, x0, dtau0, lo, xx);
 }
 
 // T^-1_mf: FV (Si) -> DG (So); acc 0: store, 1: add
@@ -985,8 +1055,10 @@ template <class Si, class So, int NP1>
 struct k_to_dg_b {
     static constexpr int TPB = 128, MINB = 0;
     static constexpr bool GROUP = std::is_same<Si, float>::value;   // a grouped twin is built (lock-step ensembles)
+    static constexpr bool X64 = std::is_same<Si, double>::value && std::is_same<So, double>::value;
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<TK> K, JfArg<const Si *> v,
-                                               JfArg<So *> u, JfArg<int> massfix, JfArg<int> acc_mode) {
+                                               JfArg<So *> u, JfArg<int> massfix, JfArg<int> acc_mode,
+                                               JfArg<EpsOut> eo) {
         jf_pdl_enter();
         typedef typename RealOf<Si, So>::type R;
         constexpr int NP = NP1 * NP1;
@@ -1039,10 +1111,12 @@ struct k_to_dg_b {
                 sc[le][q][1][row] = w;
             }
         __syncthreads();
-        if (!act) return;
+        if (!X64 && !act) return;
         const size_t N1 = (size_t)K.n_el * NP;
+        double sq = 0.0;
     #pragma unroll
         for (int q = 0; q < 4; ++q) {
+            if (!act) break;
             const size_t gi = q * N1 + (size_t)e * NP + node;
             R shift = 0;
             if (massfix) {
@@ -1055,13 +1129,17 @@ struct k_to_dg_b {
                 shift -= mfv * ((R)1 / (R)NP);
             }
             const R val = Ti[q] - shift;
-            u[gi] = acc_mode ? (So)((R)u[gi] + val) : (So)val;
+            const So un = acc_mode ? (So)((R)u[gi] + val) : (So)val;
+            u[gi] = un;
+            if (X64) sq = fma((double)un, (double)un, sq);
         }
+        if constexpr (X64)
+            if (eo.out) eps_close<128>(sq, eo, jf_bid, jf_nblk);
     }
 };
 template <class Si, class So, int NP1>
-__global__ void __launch_bounds__(128) k_to_dg(TK K, const Si *v, So *u, int massfix, int acc_mode) {
-    k_to_dg_b<Si, So, NP1>::run(blockIdx.x, gridDim.x, K, v, u, massfix, acc_mode);
+__global__ void __launch_bounds__(128) k_to_dg(TK K, const Si *v, So *u, int massfix, int acc_mode, EpsOut eo) {
+    k_to_dg_b<Si, So, NP1>::run(blockIdx.x, gridDim.x, K, v, u, massfix, acc_mode, eo);
 }
 
 // R plus the coarse level's first pseudo-time step from zero: b_c = R r and,
@@ -1166,19 +1244,53 @@ __global__ void k_neg(S *x, const S *b, size_t n) {
     k_neg_b<S>::run(blockIdx.x, gridDim.x, x, b, n);
 }
 
-template <class S>
-struct k_sub_b {
-    static constexpr int TPB = 0, MINB = 0;
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const S *> r,
-                                               JfArg<const S *> w, JfArg<S *> d, JfArg<size_t> n) {
-        jf_pdl_enter();   // d = r - w
-        const size_t t = (size_t)jf_bid * blockDim.x + threadIdx.x;
-        if (t < n) d[t] = r[t] - w[t];
+// The FP64 form's elementwise writers of an x whose eps is needed next, with the
+// reduction (EpsOut): OP 0 first DG smoothing step z = dtau r, 1 restriction with the
+// coarse level's first step, 2 x -= P v_c.  32-bit indices (n < 2^31).  Latency bound on
+// the small levels; two elements a thread there, as in the dot product it replaces.
+struct MapA {
+    double *x, *b;        // x written; OP 1: b_c
+    const double *f, *dt; // OP 0: r and dtau of the elements; 1: fine defect, dtau_c; 2: v_c
+    unsigned n;           // elements of x
+    int NXf, NZf, fac;    // fine level (OP 0: fac = nodes of an element)
+    int zero;             // OP 2: x = 0 on entry
+    double mean;          // OP 1: 1/fac^2 where that is exact (fac a power of two), else 0
+};
+template <int OP>
+struct k_map_eps_b {
+    static constexpr int TPB = 256, MINB = 0;
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<MapA> A, JfArg<EpsOut> E) {
+        jf_pdl_enter();
+        const unsigned n1 = A.n / 4, NXf = A.NXf, NZf = A.NZf, fac = A.fac;
+        double sq = 0.0;
+        for (unsigned t = jf_bid * 256 + threadIdx.x; t < A.n; t += jf_nblk * 256) {
+            const unsigned q = t / n1, c = t - q * n1;
+            double xv;
+            if (OP == 0) {
+                xv = A.dt[c / fac] * A.f[t];
+            } else if (OP == 1) {
+                const unsigned NXc = NXf / fac, J = c / NXc, I = c - J * NXc;
+                const double *fq = A.f + (size_t)q * NXf * NZf + (size_t)J * fac * NXf + I * fac;
+                double acc = 0.0;
+                for (unsigned jj = 0; jj < fac; ++jj)
+                    for (unsigned ii = 0; ii < fac; ++ii) acc += fq[(size_t)jj * NXf + ii];
+                const double bv = A.mean != 0.0 ? acc * A.mean : acc / (double)(fac * fac);
+                A.b[t] = bv;
+                xv = A.dt[c] * bv;
+            } else {
+                const unsigned NXc = NXf / fac, NZc = NZf / fac, J = c / NXf, I = c - J * NXf;
+                const double pv = A.f[(size_t)q * NXc * NZc + (size_t)(J / fac) * NXc + I / fac];
+                xv = A.zero ? -pv : A.x[t] - pv;
+            }
+            A.x[t] = xv;
+            sq = fma(xv, xv, sq);
+        }
+        eps_close<256>(sq, E, jf_bid, jf_nblk);
     }
 };
-template <class S>
-__global__ void k_sub(const S *r, const S *w, S *d, size_t n) {
-    k_sub_b<S>::run(blockIdx.x, gridDim.x, r, w, d, n);
+template <int OP>
+__global__ void __launch_bounds__(256) k_map_eps(MapA A, EpsOut E) {
+    k_map_eps_b<OP>::run(blockIdx.x, gridDim.x, A, E);
 }
 
 __global__ void k_bg_fv(FVK K, double *hbx, double *hbxw, double *hbz) {
@@ -1267,18 +1379,42 @@ TK make_tk(jfnk_ctx *c) {
     return K;
 }
 
+// where a writer leaves eps of the preconditioner's FD products
+inline EpsOut eps_to(jfnk_ctx *c, double *out) {
+    return EpsOut{c->partial, c->ticket, out,
+                  c->opts.precond_fd_eps > 0.0 ? c->opts.precond_fd_eps : 1.4901161193847656e-08};
+}
+// OP of k_map_eps on n elements, eps to `out`; false (nothing launched) beyond 32-bit indices
+template <int OP>
+bool map_eps(jfnk_ctx *c, const MapA &A, size_t n, double *out, cudaStream_t s) {
+    if (n >= (1ull << 31)) return false;
+    const size_t per = n < (size_t)c->n_sm * 256 * 8 ? 2 : 8;
+    size_t g = (n + 256 * per - 1) / (256 * per);
+    if (g > (size_t)c->nb_red) g = c->nb_red;
+    jf_launch<k_map_eps_b<OP>>(k_map_eps<OP>, (unsigned)g, 256, 0, s, A, eps_to(c, out));
+    jf_launched();
+    return true;
+}
+
 template <class Si, class So>
 int to_fv(jfnk_ctx *c, const Si *u, So *v, cudaStream_t s, So *x0 = nullptr, const So *dtau0 = nullptr,
-          LinOut lo = LinOut{}) {
+          LinOut lo = LinOut{}, const double *w = nullptr, bool *eps = nullptr) {
     TK K = make_tk(c);
     const int NP = c->np1 * c->np1;
     const int EPB = (128 / NP) > 0 ? 128 / NP : 1;
     const unsigned g = (unsigned)((c->n_el + EPB - 1) / EPB);
+    // w: subtracted from u; eps: set when the launch also left eps of x0 (both FP64 only)
+    XferX xx = {};
+    xx.w = w;
+    if (eps && x0 && (long long)g <= c->nb_red) {
+        xx.e = eps_to(c, c->scal + S_EPSFV);
+        *eps = true;
+    }
     switch (c->np1) {
-        case 2: jf_launch<k_to_fv_b<Si, So, 2>>(k_to_fv<Si, So, 2>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo); jf_launched(); break;
-        case 3: jf_launch<k_to_fv_b<Si, So, 3>>(k_to_fv<Si, So, 3>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo); jf_launched(); break;
-        case 4: jf_launch<k_to_fv_b<Si, So, 4>>(k_to_fv<Si, So, 4>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo); jf_launched(); break;
-        case 5: jf_launch<k_to_fv_b<Si, So, 5>>(k_to_fv<Si, So, 5>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo); jf_launched(); break;
+        case 2: jf_launch<k_to_fv_b<Si, So, 2>>(k_to_fv<Si, So, 2>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo, xx); jf_launched(); break;
+        case 3: jf_launch<k_to_fv_b<Si, So, 3>>(k_to_fv<Si, So, 3>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo, xx); jf_launched(); break;
+        case 4: jf_launch<k_to_fv_b<Si, So, 4>>(k_to_fv<Si, So, 4>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo, xx); jf_launched(); break;
+        case 5: jf_launch<k_to_fv_b<Si, So, 5>>(k_to_fv<Si, So, 5>, g, EPB * NP, 0, s, K, u, v, c->opts.massfix && !c->opts.transfer_l2, x0, dtau0, lo, xx); jf_launched(); break;
         default: return JFNK_EINVAL;
     }
     JF_CK(cudaGetLastError());
@@ -1286,16 +1422,21 @@ int to_fv(jfnk_ctx *c, const Si *u, So *v, cudaStream_t s, So *x0 = nullptr, con
 }
 
 template <class Si, class So>
-int to_dg(jfnk_ctx *c, const Si *v, So *u, int acc, cudaStream_t s) {
+int to_dg(jfnk_ctx *c, const Si *v, So *u, int acc, cudaStream_t s, bool *eps = nullptr) {
     TK K = make_tk(c);
     const int NP = c->np1 * c->np1;
     const int EPB = (128 / NP) > 0 ? 128 / NP : 1;
     const unsigned g = (unsigned)((c->n_el + EPB - 1) / EPB);
+    EpsOut eo = {};   // eps: set when the launch also left eps of u (FP64 only)
+    if (eps && (long long)g <= c->nb_red) {
+        eo = eps_to(c, c->scal + S_EPSDG);
+        *eps = true;
+    }
     switch (c->np1) {
-        case 2: jf_launch<k_to_dg_b<Si, So, 2>>(k_to_dg<Si, So, 2>, g, EPB * NP, 0, s, K, v, u, c->opts.massfix && !c->opts.transfer_l2, acc); jf_launched(); break;
-        case 3: jf_launch<k_to_dg_b<Si, So, 3>>(k_to_dg<Si, So, 3>, g, EPB * NP, 0, s, K, v, u, c->opts.massfix && !c->opts.transfer_l2, acc); jf_launched(); break;
-        case 4: jf_launch<k_to_dg_b<Si, So, 4>>(k_to_dg<Si, So, 4>, g, EPB * NP, 0, s, K, v, u, c->opts.massfix && !c->opts.transfer_l2, acc); jf_launched(); break;
-        case 5: jf_launch<k_to_dg_b<Si, So, 5>>(k_to_dg<Si, So, 5>, g, EPB * NP, 0, s, K, v, u, c->opts.massfix && !c->opts.transfer_l2, acc); jf_launched(); break;
+        case 2: jf_launch<k_to_dg_b<Si, So, 2>>(k_to_dg<Si, So, 2>, g, EPB * NP, 0, s, K, v, u, c->opts.massfix && !c->opts.transfer_l2, acc, eo); jf_launched(); break;
+        case 3: jf_launch<k_to_dg_b<Si, So, 3>>(k_to_dg<Si, So, 3>, g, EPB * NP, 0, s, K, v, u, c->opts.massfix && !c->opts.transfer_l2, acc, eo); jf_launched(); break;
+        case 4: jf_launch<k_to_dg_b<Si, So, 4>>(k_to_dg<Si, So, 4>, g, EPB * NP, 0, s, K, v, u, c->opts.massfix && !c->opts.transfer_l2, acc, eo); jf_launched(); break;
+        case 5: jf_launch<k_to_dg_b<Si, So, 5>>(k_to_dg<Si, So, 5>, g, EPB * NP, 0, s, K, v, u, c->opts.massfix && !c->opts.transfer_l2, acc, eo); jf_launched(); break;
         default: return JFNK_EINVAL;
     }
     JF_CK(cudaGetLastError());
@@ -1336,9 +1477,10 @@ void launch_fv(bool l4, unsigned g, int tb, cudaStream_t s, const FVK &K, const 
 }
 #define JF_FV(T, IN, MODE, V, ...) launch_fv<T, IN, MODE, V>(l4, g, tb, s, __VA_ARGS__)
 // FV_RES: out = f_low(u) (FP64 only).  FV_SMOOTH / FV_DEFECT use the FD quotient
-// (prec 64, eps = sqrt(eps_mach)/|x| from an on-device norm) or the tangent (prec 32).
+// (prec 64, eps = sqrt(eps_mach)/|x| from an on-device norm, have_eps: the writer of x
+// left it) or the tangent (prec 32).
 int fv_op64(jfnk_ctx *c, int l, int mode, const double *u, const double *x, const double *b, double *out,
-            cudaStream_t s, RKS rk = RKS{nullptr, 0, 1.0, 1.0f}) {
+            cudaStream_t s, RKS rk = RKS{nullptr, 0, 1.0, 1.0f}, bool have_eps = false) {
     FVLev &L = c->lev[l];
     FVK K = make_fvk(c, l);
     const size_t n1 = (size_t)L.NX * L.NZ;
@@ -1353,7 +1495,7 @@ int fv_op64(jfnk_ctx *c, int l, int mode, const double *u, const double *x, cons
         else { JF_FV(D64, 0, FV_RES, false, K, ld, nullptr, nullptr, nullptr, nullptr, 0.0, out); }
     } else {
         double *epsp = c->scal + S_EPSFV + l;
-        JF_RET(red_dot(c, x, x, L.n, epsp, RED_EPSP, s));
+        if (!have_eps) JF_RET(red_dot(c, x, x, L.n, epsp, RED_EPSP, s));
         FLoad<D64, 1> ld{u, x, epsp, n1, 0.0};
         const double *dt = (const double *)L.dtau;
         const double *fu = (const double *)L.fu;
@@ -1421,10 +1563,10 @@ int fv_smooth32_corrected(jfnk_ctx *c, int l, const float *x, bool zero, const f
 }
 
 inline int fv_smooth_or_defect(jfnk_ctx *c, int l, int mode, const void *x, const void *b, void *out,
-                               cudaStream_t s, RKS rk = RKS{nullptr, 0, 1.0, 1.0f}) {
+                               cudaStream_t s, RKS rk = RKS{nullptr, 0, 1.0, 1.0f}, bool have_eps = false) {
     if (c->prec == 64)
         return fv_op64(c, l, mode, (const double *)c->lev[l].u, (const double *)x, (const double *)b,
-                       (double *)out, s, rk);
+                       (double *)out, s, rk, have_eps);
     return fv_op32(c, l, mode, (const float *)x, (const float *)b, (float *)out, s, rk);
 }
 
@@ -1529,9 +1671,11 @@ inline bool rk_multi(const jfnk_ctx *c) { return c->opts.rk_stages > 1 || c->opt
 // MG_l(x, b; u) of Sec. 3.4 on level l (0 = finest subgrid).  `zero`: x = 0 on
 // entry (products with x are skipped).  `first_done`: the caller already made
 // the first pre-smoothing step from zero (x = dtau b, fused into the transfer
-// or the restriction).
+// or the restriction).  have_eps (FP64): eps of the level's x is on the device, left by
+// the kernel that wrote x.
 template <class S>
-int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
+int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, bool have_eps, cudaStream_t s) {
+    constexpr bool D = sizeof(S) == 8;
     FVLev &L = c->lev[l];
     const size_t n1 = (size_t)L.NX * L.NZ;
     int pre = (l == 0) ? c->fine_pre : c->mid_pre;
@@ -1547,6 +1691,7 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
             if (rk) {
                 // stages x_k = x_0 + a_k dtau (b - g'x_{k-1}) through the level's x2 and r
                 // buffers (x_0 = L.x is kept until the last stage)
+                have_eps = false;
                 void *in = L.x, *out = L.x2, *spare = L.r;
                 for (int k = 0; k < ns; ++k) {
                     const double a = c->opts.rk_alpha[k];
@@ -1576,8 +1721,10 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
                           1.0);
                 jf_launched();
                 zero = false;
+                have_eps = false;
             } else {
-                JF_RET(fv_smooth_or_defect(c, l, FV_SMOOTH, L.x, L.b, L.x2, s));
+                JF_RET(fv_smooth_or_defect(c, l, FV_SMOOTH, L.x, L.b, L.x2, s, RKS{nullptr, 0, 1.0, 1.0f}, have_eps));
+                have_eps = false;
                 void *t = L.x;
                 L.x = L.x2;
                 L.x2 = t;
@@ -1590,24 +1737,32 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
     if (l < c->nlev - 1) {
         FVLev &C = c->lev[l + 1];
         const bool fuse = c->mid_pre >= 1 && !rk_multi(c);
+        bool eps_c = false;
         if (zero || c->prec == 64) {   // separate defect and restriction
             if (zero) {
                 jf_launch<k_neg_b<S>>(k_neg<S>, nblk(L.n, 256), 256, 0, s, (S *)L.r, (const S *)L.b, L.n);
                 jf_launched();
             } else {
-                JF_RET(fv_smooth_or_defect(c, l, FV_DEFECT, L.x, L.b, L.r, s));
+                JF_RET(fv_smooth_or_defect(c, l, FV_DEFECT, L.x, L.b, L.r, s, RKS{nullptr, 0, 1.0, 1.0f}, have_eps));
             }
-            jf_launch<k_restrict_b_b<S>>(k_restrict_b<S>, nblk(C.n, 256), 256, 0, s, (const S *)L.r, L.NX, L.NZ, L.fac, (S *)C.b,
-                                                           fuse ? (S *)C.x : nullptr, (const S *)C.dtau,
-                                                           (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0);
-            jf_launched();
+            if constexpr (D)
+                eps_c = fuse && map_eps<1>(c, MapA{(double *)C.x, (double *)C.b, (const double *)L.r, (const double *)C.dtau,
+                                                   (unsigned)C.n, L.NX, L.NZ, L.fac, 0,
+                                                   (L.fac & (L.fac - 1)) ? 0.0 : 1.0 / (L.fac * L.fac)}, C.n, c->scal + S_EPSFV + l + 1, s);
+            if (!eps_c) {
+                jf_launch<k_restrict_b_b<S>>(k_restrict_b<S>, nblk(C.n, 256), 256, 0, s, (const S *)L.r, L.NX, L.NZ, L.fac,
+                          (S *)C.b, fuse ? (S *)C.x : nullptr, (const S *)C.dtau,
+                          (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0);
+                jf_launched();
+            }
         } else {
             // defect and restriction (and the coarse first step) in one pass
             JF_RET(fv_defect_restrict(c, l, L.x, L.b, C.b, fuse ? C.x : nullptr, C.dtau, s));
         }
         bool vz = true, fd = fuse;
         for (int cyc = 0; cyc < c->cycles; ++cyc) {
-            JF_RET(mg_cycle_t<S>(c, l + 1, vz, fd, s));
+            JF_RET(mg_cycle_t<S>(c, l + 1, vz, fd, eps_c, s));
+            eps_c = false;
             vz = false;
             fd = false;
         }
@@ -1619,9 +1774,16 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
             L.x2 = t;
             post -= 1;
         } else {
-            jf_launch<k_prolong_b<S>>(k_prolong<S>, nblk(L.n, 256), 256, 0, s, (S *)L.x, (const S *)C.x, L.NX, L.NZ, L.fac,
-                      zero ? 1 : 0);
-            jf_launched();
+            have_eps = false;
+            if constexpr (D)
+                have_eps = post >= 1 && !rk_multi(c) &&
+                           map_eps<2>(c, MapA{(double *)L.x, nullptr, (const double *)C.x, nullptr, (unsigned)L.n, L.NX, L.NZ,
+                                              L.fac, zero ? 1 : 0, 0.0}, L.n, c->scal + S_EPSFV + l, s);
+            if (!have_eps) {
+                jf_launch<k_prolong_b<S>>(k_prolong<S>, nblk(L.n, 256), 256, 0, s, (S *)L.x, (const S *)C.x, L.NX, L.NZ, L.fac,
+                          zero ? 1 : 0);
+                jf_launched();
+            }
         }
         zero = false;
     }
@@ -1636,18 +1798,23 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, cudaStream_t s) {
 inline int fd_lin(const jfnk_ctx *c) { return c->opts.precond_fd_eps == 0.0; }
 
 template <class S>
-int dg_smooth_step(jfnk_ctx *c, const S *r, S *&z, S *&z2, bool &zero, cudaStream_t s, bool last = false);
+int dg_smooth_step(jfnk_ctx *c, const S *r, S *&z, S *&z2, bool &zero, cudaStream_t s, bool last, bool &have_eps);
 
 template <>
-int dg_smooth_step<double>(jfnk_ctx *c, const double *r, double *&z, double *&z2, bool &zero, cudaStream_t s, bool) {
+int dg_smooth_step<double>(jfnk_ctx *c, const double *r, double *&z, double *&z2, bool &zero, cudaStream_t s, bool, bool &have_eps) {
     const int NP = c->np1 * c->np1;
     if (zero) {
-        jf_launch<k_scale_dtau_dg_b<double>>(k_scale_dtau_dg<double>, nblk(c->N, 256), 256, 0, s, z, r, c->dtau_dg, c->npt, NP, 1.0); jf_launched();
+        have_eps = map_eps<0>(c, MapA{z, nullptr, r, c->dtau_dg, (unsigned)c->N, 0, 0, NP, 0, 0.0}, c->N, c->scal + S_EPSDG, s);
+        if (!have_eps) {
+            jf_launch<k_scale_dtau_dg_b<double>>(k_scale_dtau_dg<double>, nblk(c->N, 256), 256, 0, s, z, r, c->dtau_dg, c->npt, NP, 1.0);
+            jf_launched();
+        }
         zero = false;
         JF_CK(cudaGetLastError());
         return JFNK_OK;
     }
-    JF_RET(red_dot(c, z, z, c->N, c->scal + S_EPSDG, RED_EPSP, s));
+    if (!have_eps) JF_RET(red_dot(c, z, z, c->N, c->scal + S_EPSDG, RED_EPSP, s));
+    have_eps = false;
     DGArgs a = {};
     a.U = c->mg_U;
     a.y = z;
@@ -1666,7 +1833,7 @@ int dg_smooth_step<double>(jfnk_ctx *c, const double *r, double *&z, double *&z2
 }
 
 template <>
-int dg_smooth_step<float>(jfnk_ctx *c, const float *r, float *&z, float *&z2, bool &zero, cudaStream_t s, bool last) {
+int dg_smooth_step<float>(jfnk_ctx *c, const float *r, float *&z, float *&z2, bool &zero, cudaStream_t s, bool last, bool &) {
     const int NP = c->np1 * c->np1;
     if (zero) {
         jf_launch<k_scale_dtau_dg_b<float>>(k_scale_dtau_dg<float>, nblk(c->N, 256), 256, 0, s, z, r, c->dtau_dgf, c->npt, NP, 1.0); jf_launched();
@@ -1691,12 +1858,13 @@ int dg_smooth_step<float>(jfnk_ctx *c, const float *r, float *&z, float *&z2, bo
 }
 
 // d = r - G'z
+// DG defect r - G'z.  FP32: to d.  FP64: G'z to c->w2, the transfer subtracts it.
 template <class S>
-int dg_defect(jfnk_ctx *c, const S *r, const S *z, S *d, cudaStream_t s);
+int dg_defect(jfnk_ctx *c, const S *r, const S *z, S *d, cudaStream_t s, bool have_eps);
 
 template <>
-int dg_defect<double>(jfnk_ctx *c, const double *r, const double *z, double *d, cudaStream_t s) {
-    JF_RET(red_dot(c, z, z, c->N, c->scal + S_EPSDG, RED_EPSP, s));
+int dg_defect<double>(jfnk_ctx *c, const double *, const double *z, double *, cudaStream_t s, bool have_eps) {
+    if (!have_eps) JF_RET(red_dot(c, z, z, c->N, c->scal + S_EPSDG, RED_EPSP, s));
     DGArgs a = {};
     a.U = c->mg_U;
     a.y = z;
@@ -1706,13 +1874,11 @@ int dg_defect<double>(jfnk_ctx *c, const double *r, const double *z, double *d, 
     a.out0 = c->w2;
     a.lin = fd_lin(c);
     JF_RET(dg_apply(c, DG_JV, a, s));
-    jf_launch<k_sub_b<double>>(k_sub<double>, nblk(c->N, 256), 256, 0, s, r, c->w2, d, c->N); jf_launched();
-    JF_CK(cudaGetLastError());
     return JFNK_OK;
 }
 
 template <>
-int dg_defect<float>(jfnk_ctx *c, const float *r, const float *z, float *d, cudaStream_t s) {
+int dg_defect<float>(jfnk_ctx *c, const float *r, const float *z, float *d, cudaStream_t s, bool) {
     DGArgs a = {};
     a.U = c->mg_U;
     a.Uf = c->Usf;
@@ -1810,6 +1976,9 @@ int apply_t(jfnk_ctx *c, const S *r, S *zout, cudaStream_t s) {
     S *z = (S *)c->pz, *z2 = (S *)c->pz2, *z3 = (S *)c->pr;
     bool zero = true;
     const S *d = r;
+    constexpr bool D = sizeof(S) == 8;
+    const double *w = nullptr;        // FP64: subtracted from d by the transfer
+    bool eps_z = false, eps_x = false;   // FP64: eps of z / of the finest level's x is on the device
     const bool fuse0 = c->fine_pre >= 1 && !rk;
     bool transferred = false;
     if (sizeof(S) == 4 && c->dg_pre == 1 && c->opts.dg_fused != 2 && !rk) {
@@ -1842,17 +2011,20 @@ int apply_t(jfnk_ctx *c, const S *r, S *zout, cudaStream_t s) {
     } else {
         for (int i = 0; i < c->dg_pre; ++i) {
             if (rk) JF_RET(dg_rk_step<S>(c, r, z, z2, z3, zero, s, nullptr));
-            else JF_RET(dg_smooth_step<S>(c, r, z, z2, zero, s));
+            else JF_RET(dg_smooth_step<S>(c, r, z, z2, zero, s, false, eps_z));
         }
         if (!zero) {
-            JF_RET(dg_defect<S>(c, r, z, (S *)c->pd, s));
-            d = (const S *)c->pd;
+            JF_RET(dg_defect<S>(c, r, z, (S *)c->pd, s, eps_z));
+            if (D) w = c->w2;
+            else d = (const S *)c->pd;
         }
     }
     if (!transferred)
-        JF_RET(to_fv<S, S>(c, d, (S *)c->lev[0].b, s, fuse0 ? (S *)c->lev[0].x : nullptr, (const S *)c->lev[0].dtau));
-    JF_RET(mg_cycle_t<S>(c, 0, true, fuse0, s));
-    JF_RET(to_dg<S, S>(c, (const S *)c->lev[0].x, z, zero ? 0 : 1, s));
+        JF_RET(to_fv<S, S>(c, d, (S *)c->lev[0].b, s, fuse0 ? (S *)c->lev[0].x : nullptr, (const S *)c->lev[0].dtau,
+                            LinOut{}, w, D ? &eps_x : nullptr));
+    JF_RET(mg_cycle_t<S>(c, 0, true, fuse0, eps_x, s));
+    eps_z = false;
+    JF_RET(to_dg<S, S>(c, (const S *)c->lev[0].x, z, zero ? 0 : 1, s, D && c->dg_post >= 1 && !rk ? &eps_z : nullptr));
     zero = false;
     for (int i = 0; i < c->dg_post; ++i) {
         if (rk) {
@@ -1860,7 +2032,7 @@ int apply_t(jfnk_ctx *c, const S *r, S *zout, cudaStream_t s) {
             continue;
         }
         if (i == c->dg_post - 1) z2 = zout;   // the last step writes the output itself
-        JF_RET(dg_smooth_step<S>(c, r, z, z2, zero, s, i == c->dg_post - 1));
+        JF_RET(dg_smooth_step<S>(c, r, z, z2, zero, s, i == c->dg_post - 1, eps_z));
     }
     if (c->dg_post == 0) JF_CK(jf_memcpy(zout, z, c->N * sizeof(S), cudaMemcpyDeviceToDevice, s));
     for (int l = 0; l < c->nlev; ++l) {
