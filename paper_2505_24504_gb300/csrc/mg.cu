@@ -7,7 +7,8 @@
 //             with the element mass of the DG polynomial taken from the subcell
 //             values by the modified Newton-Cotes weights (Sec. 3.3, Appendix A).
 //  k_to_dg    T^-1: inverse tensor interpolation and the mass fix back.
-//  k_fv       f_low and the level products on one FV level, one thread per cell:
+//  k_fv       f_low and the level products on one FV level, four lanes per cell
+//             (k_fv_tile: face-once tiles on large levels):
 //             HLLC^pert on the four faces (background fluxes precomputed per
 //             row), gravity source, two-point viscous flux.  Modes: residual,
 //             pseudo-time step x + dtau (b - g'x), defect g'x - b.  g' is the
