@@ -29,6 +29,12 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// eight values as a tree: three dependent FP64 adds (64 clocks each) instead of eight
+__device__ __forceinline__ double tree8(const double *q, int stride) {
+    return ((q[0] + q[stride]) + (q[2 * stride] + q[3 * stride])) +
+           ((q[4 * stride] + q[5 * stride]) + (q[6 * stride] + q[7 * stride]));
+}
+
 // (through shared memory: 12 FP64 adds of one warp, where a shuffle tree in every warp
 // took 45 warp adds and two dependent trees of 110 clocks a step)
 __device__ __forceinline__ double block_sum(double v) {
@@ -38,19 +44,18 @@ __device__ __forceinline__ double block_sum(double v) {
     double r = 0.0;
     if (threadIdx.x < 32) {
         const double *q = sv + threadIdx.x;
-        r = ((q[0] + q[32]) + (q[64] + q[96])) + ((q[128] + q[160]) + (q[192] + q[224]));
-        r = warp_sum(r);
+        r = warp_sum(tree8(q, 32));
     }
     __syncthreads();
     return r;   // valid in thread 0
 }
 
 // true in the block that arrives last at the ticket (after its partials are
-// visible).  Partials are written by threads of the first warp only, so only
-// that warp fences.
+// visible).  Partials are written by threads of the first two warps only, so only
+// those fence.
 __device__ __forceinline__ bool last_block(unsigned *ticket, unsigned nblk) {
     __shared__ bool last;
-    if (threadIdx.x < 32) __threadfence();
+    if (threadIdx.x < 64) __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == nblk - 1;
     __syncthreads();
@@ -115,34 +120,42 @@ __device__ __forceinline__ double warp_sum_scatter(const double (&a)[NV], int la
 // h[j] = sum over blocks of part[j * nb + b] by the whole block, fixed order:
 // thread t sums the partials b = t mod RB of every vector (all loads of a round
 // issued together), then one warp-and-block reduction of the NV sums.
-// Thread j < NV returns its sum.
-template <int NV>
-__device__ __forceinline__ double finish_multi(const double *part, int nb, double *h) {
+// Thread j < NV returns its sum.  SQ: also row NV, which the second warp adds up
+// meanwhile, in *tot after the call (the whole block).
+template <int NV, bool SQ>
+__device__ __forceinline__ double finish_multi(const double *part, int nb, double *h, double *tot) {
     constexpr int P = NV <= 1 ? 1 : NV <= 2 ? 2 : NV <= 4 ? 4 : NV <= 8 ? 8 : NV <= 16 ? 16 : 32;
-    __shared__ double fw[NV][RB / 32];
-    double a[NV];
+    __shared__ double fw[NV][RB / 32], fs[SQ ? RB : 1], ft;
+    double a[NV], as = 0.0;
 #pragma unroll
     for (int j = 0; j < NV; ++j) a[j] = 0.0;
     for (int b = threadIdx.x; b < nb; b += RB) {
         double v[NV];
 #pragma unroll
         for (int j = 0; j < NV; ++j) v[j] = __ldcg(part + (size_t)j * nb + b);
+        if (SQ) as += __ldcg(part + (size_t)NV * nb + b);
 #pragma unroll
         for (int j = 0; j < NV; ++j) a[j] += v[j];
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (SQ) fs[threadIdx.x] = as;
     const double w = warp_sum_scatter<NV>(a, lane);
     const int j = lane / (32 / P);
     if (lane % (32 / P) == 0 && j < NV) fw[j][wid] = w;
     __syncthreads();
+    double r = 0.0;
     if (threadIdx.x < NV) {
-        double r = 0.0;
-#pragma unroll
-        for (int q = 0; q < RB / 32; ++q) r += fw[threadIdx.x][q];
+        r = tree8(fw[threadIdx.x], 1);
         h[threadIdx.x] = r;
-        return r;
+    } else if (SQ && wid == 1) {
+        const double t = warp_sum(tree8(fs + lane, 32));
+        if (lane == 0) ft = t;
     }
-    return 0.0;
+    if (SQ) {
+        __syncthreads();
+        *tot = ft;
+    }
+    return r;
 }
 // The close of pass 2 by the last block: with |w1|^2 = tot (thread 0) and lane j's h1, h2
 // (first warp), the second-pass flag, |w| and 1/|w|.
@@ -193,24 +206,29 @@ __device__ __forceinline__ double warp_sum_scatter(const double (&a)[NV], int la
     return s;
 }
 
-// block sums of NV accumulators into part[j * nblk + bid]
+// block sums of NV accumulators into part[j * nblk + bid] and of sq into row NV (by the
+// second warp, while the first adds up the vectors' warp sums)
 template <int NV>
-__device__ __forceinline__ void store_multi(const double (&acc)[NV], double *part, unsigned bid, unsigned nblk) {
+__device__ __forceinline__ void store_multi(const double (&acc)[NV], double sq, double *part, unsigned bid, unsigned nblk) {
     constexpr int P = NV <= 1 ? 1 : NV <= 2 ? 2 : NV <= 4 ? 4 : NV <= 8 ? 8 : NV <= 16 ? 16 : 32;
-    __shared__ double sw[NV][RB / 32];
+    __shared__ double sw[NV][RB / 32], ss[RB];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    ss[threadIdx.x] = sq;
     const double v = warp_sum_scatter<NV>(acc, lane);
     const int j = lane / (32 / P);
     if (lane % (32 / P) == 0 && j < NV) sw[j][wid] = v;
     __syncthreads();
     if (threadIdx.x < NV) {
-        double r = 0.0;
-#pragma unroll
-        for (int q = 0; q < RB / 32; ++q) r += sw[threadIdx.x][q];
-        part[(size_t)threadIdx.x * nblk + bid] = r;
+        part[(size_t)threadIdx.x * nblk + bid] = tree8(sw[threadIdx.x], 1);
+    } else if (wid == 1) {
+        const double r = warp_sum(tree8(ss + lane, 32));
+        if (lane == 0) part[(size_t)NV * nblk + bid] = r;
     }
 }
 
+// On short vectors bound by the latency of its reductions (8 us at 15,360 unknowns and one
+// vector): |w|^2 is summed by the second warp while the first sums h2, in the block and in
+// the closing block; in sequence a step took 1.2 % (15,360 unknowns) to 0.8 % (819,200) longer.
 // pass 2: w <- w - V h1, h2 = V^T w, w1sq = |w|^2, flag = (|w1| < |w0|/sqrt(2)),
 // nrm = |w| (final unless the third pass runs)
 template <int NV>
@@ -247,12 +265,10 @@ struct k_gs_update_dot_b {
     #pragma unroll
             for (int j = 0; j < NV; ++j) acc[j] = fma(v[j].y, a.y, fma(v[j].x, a.x, acc[j]));
         }
-        store_multi<NV>(acc, part, jf_bid, jf_nblk);
-        const double bs = block_sum(sq);
-        if (threadIdx.x == 0) part[(size_t)NV * jf_nblk + jf_bid] = bs;
+        store_multi<NV>(acc, sq, part, jf_bid, jf_nblk);
         if (!last_block(ticket, jf_nblk)) return;
-        const double r2 = finish_multi<NV>(part, jf_nblk, h2);
-        const double tot = sum_partials(part + (size_t)NV * jf_nblk, jf_nblk);
+        double tot;
+        const double r2 = finish_multi<NV, true>(part, jf_nblk, h2, &tot);
         close_update(tot, threadIdx.x < NV ? h1[threadIdx.x] : 0.0, r2, w1sq, nrm, flag, ticket);
     }
 };
@@ -272,6 +288,22 @@ __global__ void __launch_bounds__(RB) k_gs_update_dot(const double *V, size_t ld
 // branch into a select and run the FP64-pipe conversion for every element.
 __device__ __noinline__ float d2f_slow(double d) { return (float)d; }
 __device__ __noinline__ double f2d_slow(float f) { return (double)f; }
+
+// float -> double widening on the integer pipe, exact: binary64 re-biases the
+// binary32 exponent by 1023 - 127 = 896 and takes the 23 fraction bits as the
+// top of its 52 (IEEE 754 formats); zero keeps its sign.  Subnormal, infinite
+// and NaN inputs use the conversion instruction (an FP64-pipe operation, like
+// the DFMA), out of line.
+__device__ __forceinline__ double f2d_bits(float f) {
+    const unsigned b = __float_as_uint(f);
+    const unsigned e = (b >> 23) & 0xffu;
+    const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
+    if ((b & 0x7fffffffu) != 0u && (e == 0u || e == 0xffu)) return f2d_slow(f);   // subnormal, inf, NaN
+    const unsigned long long r = (b & 0x7fffffffu) == 0u ? sign
+                                                          : sign | ((unsigned long long)(e + 896u) << 52) |
+                                                                ((unsigned long long)(b & 0x7fffffu) << 29);
+    return __longlong_as_double((long long)r);
+}
 
 __device__ __forceinline__ float d2f_trunc(double d) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(d);
@@ -369,13 +401,13 @@ struct k_gs_dot32_b {
         }
         __syncthreads();
         if (threadIdx.x < NV) {
-            double r = 0.0;
+            double q8[RB / 32];   // widened on the integer pipe
     #pragma unroll
-            for (int q = 0; q < RB / 32; ++q) r += (double)sw[threadIdx.x][q];
-            part[(size_t)threadIdx.x * jf_nblk + jf_bid] = r;
+            for (int q = 0; q < RB / 32; ++q) q8[q] = f2d_bits(sw[threadIdx.x][q]);
+            part[(size_t)threadIdx.x * jf_nblk + jf_bid] = tree8(q8, 1);
         }
         if (!last_block(ticket, jf_nblk)) return;
-        finish_multi<NV>(part, jf_nblk, h);
+        finish_multi<NV, false>(part, jf_nblk, h, nullptr);
         __syncthreads();
         if (threadIdx.x == 0) *ticket = 0u;
     }
@@ -432,10 +464,10 @@ struct k_gsl_dot32_b {
         }
         __syncthreads();
         if (threadIdx.x < nv) {
-            double r = 0.0;
+            double q8[RB / 32];   // widened on the integer pipe
     #pragma unroll
-            for (int q = 0; q < RB / 32; ++q) r += (double)sw[threadIdx.x][q];
-            part[(size_t)threadIdx.x * jf_nblk + jf_bid] = r;
+            for (int q = 0; q < RB / 32; ++q) q8[q] = f2d_bits(sw[threadIdx.x][q]);
+            part[(size_t)threadIdx.x * jf_nblk + jf_bid] = tree8(q8, 1);
         }
         if (!last_block(ticket, jf_nblk)) return;
         sum_rows(part, nv, jf_nblk, h);
@@ -498,9 +530,7 @@ struct k_gsl_update_dot_b {
                     }
             });
         }
-        store_multi<LV>(acc, part, jf_bid, jf_nblk);
-        const double bs = block_sum(sq);
-        if (threadIdx.x == 0) part[(size_t)LV * jf_nblk + jf_bid] = bs;
+        store_multi<LV>(acc, sq, part, jf_bid, jf_nblk);
         if (!last_block(ticket, jf_nblk)) return;
         __shared__ double sh[LV];
         if (threadIdx.x < LV) sh[threadIdx.x] = 0.0;
@@ -782,22 +812,6 @@ __global__ void __launch_bounds__(RB) k_final_gs(const double *part, int nb, con
                                                  const double *flag_in, double *w1sq, double *nrm,
                                                  double *flag_out) {
     k_final_gs_b::run(blockIdx.x, gridDim.x, part, nb, h, nv, flag_in, w1sq, nrm, flag_out);
-}
-
-// float -> double widening on the integer pipe, exact: binary64 re-biases the
-// binary32 exponent by 1023 - 127 = 896 and takes the 23 fraction bits as the
-// top of its 52 (IEEE 754 formats); zero keeps its sign.  Subnormal, infinite
-// and NaN inputs use the conversion instruction (an FP64-pipe operation, like
-// the DFMA), out of line.
-__device__ __forceinline__ double f2d_bits(float f) {
-    const unsigned b = __float_as_uint(f);
-    const unsigned e = (b >> 23) & 0xffu;
-    const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
-    if ((b & 0x7fffffffu) != 0u && (e == 0u || e == 0xffu)) return f2d_slow(f);   // subnormal, inf, NaN
-    const unsigned long long r = (b & 0x7fffffffu) == 0u ? sign
-                                                          : sign | ((unsigned long long)(e + 896u) << 52) |
-                                                                ((unsigned long long)(b & 0x7fffffu) << 29);
-    return __longlong_as_double((long long)r);
 }
 
 // eps = sqrt(2^-52)/|x| of the FD product from an FP32 direction.  The squares are
