@@ -352,6 +352,16 @@ int jfnk_eos_pressure(jfnk_ctx *ctx, const double *E_dev, size_t n, double *p_de
 int jfnk_tangent_product(jfnk_ctx *ctx, const double *U_dev, const double *y_dev, double alpha_dt,
                          double *out_dev, void *stream);
 
+/* Diagnostic: the solver's Arnoldi process of nv columns (1..opts.gmres_restart)
+ * for G'(U) Q^-1 (Q^-1 = 1 without a preconditioner) from r: the basis
+ * v_0 = r/|r|, v_1, ..., v_nv to V_dev ((nv + 1) N doubles) and the Hessenberg
+ * columns to H_host, column j at H_host[j (nv + 1)], with the kernels and graphs of
+ * implicit_step.  Overwrites the context's linearisation and basis.
+ * Synchronises `stream` once a column.  JFNK_ENAN when |r| is 0 or a norm is not
+ * finite. */
+int jfnk_arnoldi(jfnk_ctx *ctx, const double *U_dev, double alpha_dt, const double *r_dev, int nv,
+                 double *V_dev, double *H_host, void *stream);
+
 /* Times the two launches of one DG operator evaluation with CUDA events
  * recorded on `stream` around each: which 0 = FP64 residual, 1 = FP64
  * finite-difference product with direction y (in the form the solver's Arnoldi

@@ -14,8 +14,8 @@
 // result and resets the counter.  Nothing waits on another block.
 // Gram-Schmidt twice (CGS2) in three passes over the basis: h1 = V^T w; then
 // w1 = w - V h1 fused with h2 = V^T w1 and |w1|^2 (so |w2|^2 = |w1|^2 - |h2|^2);
-// then, when the device-side test asks for it, w2 = w1 - V h2, fused with the
-// normalisation.
+// then w2 = w1 - V h2, fused with the normalisation (always after an FP32 pass 1,
+// otherwise when the device-side test asks for it).
 #include "internal.h"
 
 namespace {
@@ -158,14 +158,17 @@ __device__ __forceinline__ double finish_multi(const double *part, int nb, doubl
     return r;
 }
 // The close of pass 2 by the last block: with |w1|^2 = tot (thread 0) and lane j's h1, h2
-// (first warp), the second-pass flag, |w| and 1/|w|.
+// (first warp), the second-pass flag, |w| and 1/|w|.  P32: pass 1 ran in FP32, whose
+// rounding (some 1e-7 |h1|) stays in w1 however large w1 is, so the second pass always
+// runs; after an FP64 pass 1 it runs when the first took off more than half of |w|^2.
+template <bool P32>
 __device__ __forceinline__ void close_update(double tot, double h1, double h2, double *w1sq, double *nrm, double *flag,
                                              unsigned *ticket) {
     if (threadIdx.x >= 32) return;
     const double hh = warp_sum(h1 * h1), hh2 = warp_sum(h2 * h2);
     if (threadIdx.x != 0) return;
     *w1sq = tot;
-    const bool second = tot < 0.5 * (tot + hh);
+    const bool second = P32 || tot < 0.5 * (tot + hh);
     // |w2|^2 = |w1|^2 - |h2|^2 for w2 = w1 - V h2 with V orthonormal and h2 = V^T w1;
     // after the first pass h2 is tiny against |w1|, so the difference does not cancel
     const double nr = sqrt64(second ? fmax(tot - hh2, 0.0) : tot);
@@ -229,8 +232,8 @@ __device__ __forceinline__ void store_multi(const double (&acc)[NV], double sq, 
 // On short vectors bound by the latency of its reductions (8 us at 15,360 unknowns and one
 // vector): |w|^2 is summed by the second warp while the first sums h2, in the block and in
 // the closing block; in sequence a step took 1.2 % (15,360 unknowns) to 0.8 % (819,200) longer.
-// pass 2: w <- w - V h1, h2 = V^T w, w1sq = |w|^2, flag = (|w1| < |w0|/sqrt(2)),
-// nrm = |w| (final unless the third pass runs)
+// pass 2: w <- w - V h1, h2 = V^T w, w1sq = |w|^2, flag = 1 (close_update),
+// nrm = |w| after the third pass
 template <int NV>
 struct k_gs_update_dot_b {
     static constexpr int TPB = RB, MINB = 0;
@@ -269,7 +272,7 @@ struct k_gs_update_dot_b {
         if (!last_block(ticket, jf_nblk)) return;
         double tot;
         const double r2 = finish_multi<NV, true>(part, jf_nblk, h2, &tot);
-        close_update(tot, threadIdx.x < NV ? h1[threadIdx.x] : 0.0, r2, w1sq, nrm, flag, ticket);
+        close_update<true>(tot, threadIdx.x < NV ? h1[threadIdx.x] : 0.0, r2, w1sq, nrm, flag, ticket);
     }
 };
 template <int NV>
@@ -429,46 +432,31 @@ __device__ __forceinline__ void vec_groups(int nv, F f) {
     for (int j0 = 0; j0 < LV; j0 += 4)
         if (j0 < nv) f(j0);
 }
-struct k_gsl_dot32_b {
+// Pass 1 runs in FP64 here: h = V^T w.
+struct k_gsl_dot_b {
     static constexpr int TPB = RB, MINB = 0;
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const float *> V32, JfArg<int> nv,
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const double *> V, JfArg<int> nv,
                                                JfArg<size_t> ldv, JfArg<const double *> w, JfArg<size_t> n2,
                                                JfArg<double *> part, JfArg<unsigned *> ticket, JfArg<double *> h) {
         jf_pdl_enter();
         const double2 *w2 = reinterpret_cast<const double2 *>(w);
+        const double2 *V2 = reinterpret_cast<const double2 *>(V);
         const size_t l2 = ldv / 2;
-        const float2 *V2 = reinterpret_cast<const float2 *>(V32);
-        float acc[LV];
+        double acc[LV];
     #pragma unroll
-        for (int j = 0; j < LV; ++j) acc[j] = 0.0f;
+        for (int j = 0; j < LV; ++j) acc[j] = 0.0;
         for (size_t i = (size_t)jf_bid * RB + threadIdx.x; i < n2; i += (size_t)jf_nblk * RB) {
             const double2 a = w2[i];
-            const float ax = d2f_trunc(a.x), ay = d2f_trunc(a.y);
             vec_groups(nv, [&](int j0) {
     #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (j0 + j < nv) {
-                        const float2 v = V2[(size_t)(j0 + j) * l2 + i];
-                        acc[j0 + j] = fmaf(v.y, ay, fmaf(v.x, ax, acc[j0 + j]));
+                        const double2 v = V2[(size_t)(j0 + j) * l2 + i];
+                        acc[j0 + j] = fma(v.y, a.y, fma(v.x, a.x, acc[j0 + j]));
                     }
             });
         }
-        __shared__ float sw[LV][RB / 32];
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    #pragma unroll
-        for (int j = 0; j < LV; ++j) {
-            float v = acc[j];
-    #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) sw[j][wid] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < nv) {
-            double q8[RB / 32];   // widened on the integer pipe
-    #pragma unroll
-            for (int q = 0; q < RB / 32; ++q) q8[q] = f2d_bits(sw[threadIdx.x][q]);
-            part[(size_t)threadIdx.x * jf_nblk + jf_bid] = tree8(q8, 1);
-        }
+        store_multi<LV>(acc, 0.0, part, jf_bid, jf_nblk);
         if (!last_block(ticket, jf_nblk)) return;
         sum_rows(part, nv, jf_nblk, h);
         __syncthreads();
@@ -485,9 +473,9 @@ struct k_gsl_dot32_b {
         }
     }
 };
-__global__ void __launch_bounds__(RB) k_gsl_dot32(const float *V32, int nv, size_t ldv, const double *w, size_t n2,
-                                                  double *part, unsigned *ticket, double *h) {
-    k_gsl_dot32_b::run(blockIdx.x, gridDim.x, V32, nv, ldv, w, n2, part, ticket, h);
+__global__ void __launch_bounds__(RB) k_gsl_dot(const double *V, int nv, size_t ldv, const double *w, size_t n2,
+                                                double *part, unsigned *ticket, double *h) {
+    k_gsl_dot_b::run(blockIdx.x, gridDim.x, V, nv, ldv, w, n2, part, ticket, h);
 }
 struct k_gsl_update_dot_b {
     static constexpr int TPB = RB, MINB = 0;
@@ -535,11 +523,11 @@ struct k_gsl_update_dot_b {
         __shared__ double sh[LV];
         if (threadIdx.x < LV) sh[threadIdx.x] = 0.0;
         __syncthreads();
-        k_gsl_dot32_b::sum_rows(part, nv, jf_nblk, sh);
+        k_gsl_dot_b::sum_rows(part, nv, jf_nblk, sh);
         const double tot = sum_partials(part + (size_t)LV * jf_nblk, jf_nblk);   // synchronises
         const double r2 = threadIdx.x < LV ? sh[threadIdx.x] : 0.0;
         if (threadIdx.x < nv) h2[threadIdx.x] = r2;
-        close_update(tot, threadIdx.x < LV ? sc[threadIdx.x] : 0.0, r2, w1sq, nrm, flag, ticket);
+        close_update<false>(tot, threadIdx.x < LV ? sc[threadIdx.x] : 0.0, r2, w1sq, nrm, flag, ticket);
     }
 };
 __global__ void __launch_bounds__(RB) k_gsl_update_dot(const double *V, int nv, size_t ldv, double *w, size_t n2,
@@ -1005,9 +993,9 @@ int blas_cgs2(jfnk_ctx *c, const double *V, const float *V32, int nv, size_t ldv
     if (nv < 1 || nv > GS_FUSED_MAX || (n & 1) || (ldv & 1) || !V32) return JFNK_EINVAL;
     if (nv > 16) {
         const size_t n2 = n / 2;
-        const int g1 = one_wave(c, k_gsl_dot32, n2), g2 = one_wave(c, k_gsl_update_dot, n2),
+        const int g1 = one_wave(c, k_gsl_dot, n2), g2 = one_wave(c, k_gsl_update_dot, n2),
                   g3 = one_wave(c, k_gsl_update_scale, n2);
-        jf_launch<k_gsl_dot32_b>(k_gsl_dot32, g1, RB, 0, s, V32, nv, ldv, w, n2, c->partial, c->ticket, h1);
+        jf_launch<k_gsl_dot_b>(k_gsl_dot, g1, RB, 0, s, V, nv, ldv, w, n2, c->partial, c->ticket, h1);
         jf_launch<k_gsl_update_dot_b>(k_gsl_update_dot, g2, RB, 0, s, V, nv, ldv, w, n2, h1, c->partial, c->ticket, h2, w1sq, nrm, flag);
         jf_launch<k_gsl_update_scale_b>(k_gsl_update_scale, g3, RB, 0, s, V, nv, ldv, w, w32, n2, h2, flag, nrm + (S_INV - S_NORM));
         jf_launched(3);

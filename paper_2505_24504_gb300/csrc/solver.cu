@@ -175,6 +175,23 @@ int arnoldi_step(jfnk_ctx *c, const double *U, double adt, int j, cudaStream_t s
     return JFNK_OK;
 }
 
+// v_0 = r / beta and its float copy
+int arnoldi_start(jfnk_ctx *c, const double *r, double beta, cudaStream_t s) {
+    JF_CK(jf_memcpy(c->scal + S_NORM, &beta, sizeof(double), cudaMemcpyHostToDevice, s));
+    JF_RET(blas_scale_copy(r, c->scal + S_NORM, c->V, c->N, s));
+    JF_RET(blas_copy_d2f(c->V, c->V32, c->N, s));
+    JF_CK(jf_sync(s));   // beta lives on the host stack
+    return JFNK_OK;
+}
+
+// Hessenberg column j (j + 2 entries) from the pinned copy of the step's scalars: h1, plus
+// h2 when the second pass ran, and the norm of what was left
+void arnoldi_column(const jfnk_ctx *c, int j, double *h) {
+    const double *hp = c->h_pinned;
+    for (int i = 0; i <= j; ++i) h[i] = hp[S_H + i] + (hp[S_FLAG] != 0.0 ? hp[S_H2 + i] : 0.0);
+    h[j + 1] = hp[S_NORM];
+}
+
 // Solve G'(U) x = b from x = 0 until the residual estimate <= tol_abs.
 int fgmres(jfnk_ctx *c, const double *U, double adt, const double *b, double *x, double tol_abs, int *its,
            cudaStream_t s, Stats &st) {
@@ -182,7 +199,6 @@ int fgmres(jfnk_ctx *c, const double *U, double adt, const double *b, double *x,
     const size_t N = c->N;
     const int m = c->opts.gmres_restart;
     const int maxit = c->opts.gmres_max;
-    double *V = c->V;
     double H[65][64], cs[64], sn[64], g[65], y[64];
     JF_CK(jf_memset(x, 0, 8 * N, s));
     double beta;
@@ -192,10 +208,7 @@ int fgmres(jfnk_ctx *c, const double *U, double adt, const double *b, double *x,
     if (beta <= tol_abs || beta == 0.0) return JFNK_OK;
     const double *r = b;
     while (*its < maxit) {
-        JF_CK(jf_memcpy(c->scal + S_NORM, &beta, sizeof(double), cudaMemcpyHostToDevice, s));
-        JF_RET(blas_scale_copy(r, c->scal + S_NORM, V, N, s));
-        JF_RET(blas_copy_d2f(V, c->V32, N, s));
-        JF_CK(jf_sync(s));   // beta lives on the host stack
+        JF_RET(arnoldi_start(c, r, beta, s));
         memset(H, 0, sizeof(H));
         for (int i = 0; i <= m; ++i) g[i] = 0.0;
         g[0] = beta;
@@ -208,10 +221,10 @@ int fgmres(jfnk_ctx *c, const double *U, double adt, const double *b, double *x,
             st.t_pre += ph.ms(0, 1);
             st.t_jv += ph.ms(1, 2);
             st.t_orth += ph.ms(2, 3);
-            const double *hp = c->h_pinned;
-            if (hp[S_FLAG] != 0.0) ++st.reortho;
-            for (int i = 0; i <= j; ++i) H[i][j] = hp[S_H + i] + (hp[S_FLAG] != 0.0 ? hp[S_H2 + i] : 0.0);
-            H[j + 1][j] = hp[S_NORM];
+            if (c->h_pinned[S_FLAG] != 0.0) ++st.reortho;
+            double h[65];
+            arnoldi_column(c, j, h);
+            for (int i = 0; i <= j + 1; ++i) H[i][j] = h[i];
             if (!isfinite(H[j + 1][j])) return JFNK_ENAN;
             for (int i = 0; i < j; ++i) {
                 const double a0 = H[i][j], a1 = H[i + 1][j];
@@ -373,4 +386,32 @@ extern "C" int implicit_step(jfnk_ctx *c, double *U, double dt, int scheme, jfnk
         stats->reorth = st.reortho;
     }
     return rc;
+}
+
+extern "C" int jfnk_arnoldi(jfnk_ctx *c, const double *U, double adt, const double *r, int nv, double *V, double *H,
+                            void *stream) {
+    if (!c || !U || !r || !V || !H || nv < 1 || nv > c->opts.gmres_restart) return JFNK_EINVAL;
+    cudaStream_t s = (cudaStream_t)stream;
+    DGArgs a = {};
+    a.U = U;
+    a.out0 = c->fU;
+    a.lin_out = 1;
+    JF_RET(dg_apply(c, DG_RES, a, s));
+    if (c->mg_on) JF_RET(mg_linearize(c, U, adt, s));
+    else JF_CK(jf_memcpy(c->Ulin, U, 8 * c->N, cudaMemcpyDeviceToDevice, s));
+    double beta;
+    JF_RET(read_norm(c, r, &beta, s));
+    if (!isfinite(beta) || beta == 0.0) return JFNK_ENAN;
+    JF_RET(arnoldi_start(c, r, beta, s));
+    Phases ph(false);
+    for (int j = 0; j < nv; ++j) {
+        JF_RET(arnoldi_step(c, c->Ulin, adt, j, s, ph));
+        JF_CK(jf_sync(s));
+        double *h = H + (size_t)j * (nv + 1);
+        arnoldi_column(c, j, h);
+        for (int i = j + 2; i <= nv; ++i) h[i] = 0.0;
+        if (!isfinite(h[j + 1])) return JFNK_ENAN;
+    }
+    JF_CK(jf_memcpy(V, c->V, 8 * c->N * (size_t)(nv + 1), cudaMemcpyDeviceToDevice, s));
+    return JFNK_OK;
 }

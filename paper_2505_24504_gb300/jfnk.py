@@ -103,6 +103,7 @@ def _lib():
             "jfnk_norm2_noalloc": (I, [P, S, P, P]),
             "jfnk_time_operator": (I, [P, I, P, P, I, P, P]),
             "jfnk_tangent_product": (I, [P, P, P, D, P, P]),
+            "jfnk_arnoldi": (I, [P, P, D, P, I, P, P, P]),
             "jfnk_launch_count": (C.c_ulonglong, []),
             "jfnk_autotune": (I, [P, P, P, I, P, P, P]),
             "jfnk_strerror": (C.c_char_p, [I]),
@@ -331,6 +332,18 @@ class Context:
         self._states(U=U, y=y, out=out)
         _check(_lib().jfnk_tangent_product(self.h, _ptr(U), _ptr(y), float(adt), _ptr(out), _stream(stream)),
                "jfnk_tangent_product")
+
+    def arnoldi(self, U, alpha_dt, r, nv, stream=None):
+        """The solver's Arnoldi process of nv columns from r: the basis (nv + 1, N) on the
+        device and the Hessenberg matrix (nv + 1, nv) as a numpy array."""
+        import numpy as np
+        import torch
+        self._states(U=U, r=r)
+        V = torch.empty(nv + 1, self.N, dtype=torch.float64, device=U.device)
+        H = np.zeros((nv, nv + 1))
+        _check(_lib().jfnk_arnoldi(self.h, _ptr(U), float(alpha_dt), _ptr(r), int(nv), _ptr(V),
+                                   H.ctypes.data_as(C.c_void_p), _stream(stream)), "jfnk_arnoldi")
+        return V, H.T
 
     def time_operator(self, which, U, y, reps, stream=None):
         self._states(U=U, y=y)
