@@ -842,16 +842,16 @@ __global__ void __launch_bounds__(RB) k_eps32(const float *x, size_t n, double *
 // preconditioner's last smoothing step): one block
 struct k_eps_part_b {
     static constexpr int TPB = RB, MINB = 0;
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const float *> part, JfArg<int> nb,
+    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const double *> part, JfArg<int> nb,
                                                JfArg<double *> eps) {
         jf_pdl_enter();
         double acc = 0.0;
-        for (int i = threadIdx.x; i < nb; i += RB) acc += f2d_bits(part[i]);
+        for (int i = threadIdx.x; i < nb; i += RB) acc += part[i];
         acc = block_sum(acc);
         if (threadIdx.x == 0) *eps = finish_op(acc, RED_EPS);
     }
 };
-__global__ void __launch_bounds__(RB) k_eps_part(const float *part, int nb, double *eps) {
+__global__ void __launch_bounds__(RB) k_eps_part(const double *part, int nb, double *eps) {
     k_eps_part_b::run(blockIdx.x, gridDim.x, part, nb, eps);
 }
 
@@ -1191,7 +1191,7 @@ int blas_eps32(jfnk_ctx *c, const float *x, size_t n, double *eps_out, cudaStrea
     return JFNK_OK;
 }
 
-int blas_eps_part(jfnk_ctx *c, const float *part, int nb, double *eps_out, cudaStream_t s) {
+int blas_eps_part(jfnk_ctx *c, const double *part, int nb, double *eps_out, cudaStream_t s) {
     (void)c;
     jf_launch<k_eps_part_b>(k_eps_part, 1, RB, 0, s, part, nb, eps_out);
     jf_launched();

@@ -391,7 +391,7 @@ struct DGArgs {
     const void *z0;
     int z0mode;
     double alpha;
-    float *npart;          // FP32 smoothing: each block's sum of squares of the new z (may be null)
+    double *npart;         // FP32 smoothing: each block's sum of squares of the new z (may be null)
 };
 // Elements of a strip (block) of the fused FP32 tangent products: one thread per node
 // (viscous), and not more than 128 face points, (3 E + 1)(k + 1), where each thread also
@@ -442,7 +442,7 @@ int blas_eps32(jfnk_ctx *c, const float *x, size_t n, double *eps_out, cudaStrea
 int blas_scale_copy(const double *w, const double *nrm_dev, double *v, size_t n, cudaStream_t s);
 int blas_axpby(double a, const double *x, double b, const double *y, double *z, size_t n, cudaStream_t s);
 int blas_zcomb(const void *Z, int prec32, int nz, size_t n, const double *yv, double *x, cudaStream_t s);
-int blas_eps_part(jfnk_ctx *c, const float *part, int nb, double *eps_out, cudaStream_t s);
+int blas_eps_part(jfnk_ctx *c, const double *part, int nb, double *eps_out, cudaStream_t s);
 int blas_copy_d2f(const double *x, float *y, size_t n, cudaStream_t s);
 int blas_copy_f2d(const float *x, double *y, size_t n, cudaStream_t s);
 int blas_scale(double a, const double *x, double *y, size_t n, cudaStream_t s);

@@ -1850,7 +1850,7 @@ int dg_smooth_step<float>(jfnk_ctx *c, const float *r, float *&z, float *&z2, bo
     a.dtauf = c->dtau_dgf;
     a.adt = c->mg_adt;
     a.out0 = z2;
-    a.npart = last && mg_norm_blocks(c) ? (float *)c->partial : nullptr;
+    a.npart = last && mg_norm_blocks(c) ? c->partial : nullptr;
     JF_RET(dg_apply(c, DG_TLSMOOTH, a, s));
     float *t = z;
     z = z2;

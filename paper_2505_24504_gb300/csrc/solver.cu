@@ -59,7 +59,7 @@ struct Phases {
 int apply_jv(jfnk_ctx *c, const double *U, double adt, const double *y, const float *yf, double *w, cudaStream_t s) {
     // the FP32 preconditioner left the blocks' sums of squares of its output
     const int nb = yf ? mg_norm_blocks(c) : 0;
-    if (nb) JF_RET(blas_eps_part(c, (const float *)c->partial, nb, c->scal + S_EPS, s));
+    if (nb) JF_RET(blas_eps_part(c, c->partial, nb, c->scal + S_EPS, s));
     else if (yf) JF_RET(blas_eps32(c, yf, c->N, c->scal + S_EPS, s));
     else JF_RET(red_dot(c, y, y, c->N, c->scal + S_EPS, RED_EPS, s));
     DGArgs a = {};
