@@ -352,6 +352,11 @@ int jfnk_eos_pressure(jfnk_ctx *ctx, const double *E_dev, size_t n, double *p_de
 int jfnk_tangent_product(jfnk_ctx *ctx, const double *U_dev, const double *y_dev, double alpha_dt,
                          double *out_dev, void *stream);
 
+/* Diagnostic: the kernels' FP64 primitives on n doubles (device arrays; b for op 0
+ * and 4 only): op 0 a / b, 1 1 / a, 2 sqrt(a), 3 a split into two floats and joined
+ * again, 4 the sum of the two floats (float)a + (float)b. */
+int jfnk_arithmetic(int op, const double *a_dev, const double *b_dev, size_t n, double *out_dev, void *stream);
+
 /* Diagnostic: the solver's Arnoldi process of nv columns (1..opts.gmres_restart)
  * for G'(U) Q^-1 (Q^-1 = 1 without a preconditioner) from r: the basis
  * v_0 = r/|r|, v_1, ..., v_nv to V_dev ((nv + 1) N doubles) and the Hessenberg

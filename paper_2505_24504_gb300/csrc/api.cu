@@ -116,6 +116,13 @@ __global__ void k_eos(const double *E, size_t n, PhysC pc, const PowTab *pt, dou
     if (i < n) p[i] = pressure(D64{E[i]}, pc, pt).x;
 }
 
+__global__ void k_arith(int op, const double *a, const double *b, size_t n, double *out) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double x = a[i];
+    out[i] = op == 0 ? div64(x, b[i]) : op == 1 ? rcp64(x) : op == 2 ? sqrt64(x) : op == 3 ? join(split2(x)) : join(F2{(float)x, (float)b[i]});
+}
+
 __global__ void k_init_state(const double *thp, const double *prow, const double *throw_, const double *ubv,
                              double ubg, double wbg, int nx, int nz, int np1, double *U) {
     const int NP = np1 * np1;
@@ -645,6 +652,14 @@ int jfnk_eos_pressure(jfnk_ctx *c, const double *E, size_t n, double *p, void *s
     if (!c || !E || !p) return JFNK_EINVAL;
     if (n == 0) return JFNK_OK;
     k_eos<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(E, n, c->pc, c->powtab, p); jf_launched();
+    JF_CK(cudaGetLastError());
+    return JFNK_OK;
+}
+
+int jfnk_arithmetic(int op, const double *a, const double *b, size_t n, double *out, void *stream) {
+    if (op < 0 || op > 4 || !a || !out || ((op == 0 || op == 4) && !b)) return JFNK_EINVAL;
+    if (n == 0) return JFNK_OK;
+    k_arith<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(op, a, b, n, out); jf_launched();
     JF_CK(cudaGetLastError());
     return JFNK_OK;
 }

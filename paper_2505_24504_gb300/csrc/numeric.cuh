@@ -137,6 +137,60 @@ JF_D double sqrt64(double x) {
     return __fma_rn(__fma_rn(-g, g, x), h, g);
 }
 
+// ---- two-float arithmetic -----------------------------------------------------
+struct F2 {
+    float h, l;
+};
+JF_D F2 f2(float2 a) { return F2{a.x, a.y}; }
+JF_D float2 f2v(F2 a) { return make_float2(a.h, a.l); }
+// s += c y (no contraction across the error-free steps)
+JF_D void f2_fma(F2 &s, F2 c, F2 y) {
+    const float p = __fmul_rn(c.h, y.h);
+    float e = __fmaf_rn(c.h, y.h, -p);
+    e = __fmaf_rn(c.h, y.l, e);
+    e = __fmaf_rn(c.l, y.h, e);
+    const float t = __fadd_rn(s.h, p), z = __fsub_rn(t, s.h);
+    const float r = __fadd_rn(__fsub_rn(s.h, __fsub_rn(t, z)), __fsub_rn(p, z));
+    s.h = t;
+    s.l = __fadd_rn(s.l, __fadd_rn(r, e));
+}
+JF_D F2 f2_mul(F2 c, F2 y) {
+    const float p = __fmul_rn(c.h, y.h);
+    float e = __fmaf_rn(c.h, y.h, -p);
+    e = __fmaf_rn(c.h, y.l, e);
+    return F2{p, __fmaf_rn(c.l, y.h, e)};
+}
+JF_D F2 f2_neg(F2 a) { return F2{-a.h, -a.l}; }
+// the leading 24 and the following 24 bits of a double on the integer pipe (magnitudes
+// below 2^-126 become zero, the second part of those below 2^-103 too; overflow, infinity
+// and NaN through the conversion)
+static __device__ __noinline__ float d2f_conv(double d) { return (float)d; }
+static __device__ __noinline__ double f2d_conv(float f) { return (double)f; }
+JF_D F2 split2(double d) {
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned e = (hi >> 20) & 0x7ffu, s = hi & 0x80000000u;
+    if (e > 1150u) return F2{d2f_conv(d), 0.0f};
+    const unsigned m = __funnelshift_l(lo, hi, 3) & 0x7fffffu;
+    const float h = __uint_as_float(e < 897u ? 0u : s | ((e - 896u) << 23) | m);
+    // the other 29 bits, a fraction of 2^(e - 1023 - 23); signed
+    const float sc = __uint_as_float(e < 920u ? 0u : s | ((e - 919u) << 23));
+    return F2{h, __fmul_rn((float)(int)(lo & 0x1fffffffu) * 1.862645149230957e-09f, sc)};
+}
+// their sum as a double, rounded to its last place (the second part is dropped below
+// 2^-104)
+JF_D double join(F2 a) {
+    const float H = __fadd_rn(a.h, a.l), z = __fsub_rn(H, a.h);
+    const float L = __fadd_rn(__fsub_rn(a.h, __fsub_rn(H, z)), __fsub_rn(a.l, z));
+    const unsigned b = __float_as_uint(H), e = (b >> 23) & 0xffu;
+    if (e == 255u) return f2d_conv(H);   // infinity, NaN
+    // L in units of the double's last place, 2^(e - 127 - 52); signed like the magnitude.
+    // Below a power of two the units are half as large.
+    const float sc = __uint_as_float(e < 23u ? 0u : (b & 0x80000000u) | ((277u - e) << 23));
+    float k = __fmul_rn(L * 536870912.0f, sc);
+    if ((b & 0x7fffffu) == 0u) k = fminf(k, __fadd_rn(k, k));
+    return __longlong_as_double(__double_as_longlong(f2d_normal(H)) + (long long)__float2int_rn(k));
+}
+
 // ---------------------------------------------------------------------------
 struct D64 {
     double x;

@@ -103,6 +103,7 @@ def _lib():
             "jfnk_norm2_noalloc": (I, [P, S, P, P]),
             "jfnk_time_operator": (I, [P, I, P, P, I, P, P]),
             "jfnk_tangent_product": (I, [P, P, P, D, P, P]),
+            "jfnk_arithmetic": (I, [I, P, P, S, P, P]),
             "jfnk_arnoldi": (I, [P, P, D, P, I, P, P, P]),
             "jfnk_launch_count": (C.c_ulonglong, []),
             "jfnk_autotune": (I, [P, P, P, I, P, P, P]),
@@ -215,6 +216,14 @@ def norm2_noalloc(x, out, n=None, stream=None):
     in-library scratch; see include/jfnk.h)."""
     n = _check_norm_args(x, out, n)
     _check(_lib().jfnk_norm2_noalloc(_ptr(x), n, _ptr(out), _stream(stream)), "jfnk_norm2_noalloc")
+
+
+def arithmetic(op, a, b, out, stream=None):
+    """The kernels' FP64 primitives: op 0 a / b, 1 1 / a, 2 sqrt(a), 3 a through two floats,
+    4 (float)a + (float)b."""
+    for t, what in ((a, "a"), (b, "b"), (out, "out")):
+        _vec(t, a.numel(), what)
+    _check(_lib().jfnk_arithmetic(int(op), _ptr(a), _ptr(b), a.numel(), _ptr(out), _stream(stream)), "jfnk_arithmetic")
 
 
 def launch_count() -> int:
