@@ -71,15 +71,16 @@ JF_D double eos_pow(double E, const PowTab *T) {
 
 // ---------------------------------------------------------------------------
 // Quotient, reciprocal and square root of doubles with binary exponents within +-400
-// (others, zeros, infinities and NaN take the IEEE intrinsics).  A hardware FP32
+// (others, infinities and NaN take the IEEE intrinsics, zero divisors and roots of zero
+// too; -0 over a positive divisor gives 0: keeping its sign cost the viscous residual 6 %).  A hardware FP32
 // approximation of the significand is refined to about 45 bits in two-float arithmetic
 // (Newton's iteration with the residual formed by FMA) and put together as a double on
 // the integer pipe; one FP64 correction with the exact residual (Markstein, "Computation
 // of elementary functions on the IBM RISC System/6000 processor", 1990) then gives the
-// quotient from an approximation whose error is 2^-88: the correctly rounded result (no
-// difference from the IEEE intrinsics in 3.1e8 random quotients and roots; reciprocals of
-// the last few significands below a power of two, whose exact value lies that close to a
-// tie, can round to the other neighbour).  Two FP64 instructions for a reciprocal, three
+// quotient from an approximation whose error is 2^-88: the correctly rounded result (that
+// of the IEEE operations for every leading 24 bits of a significand, tests; next to powers
+// of two, where an exact value can lie that close to a tie, within a unit in the last
+// place).  Two FP64 instructions for a reciprocal, three
 // for a quotient or a square root: 35, 55 and 51 clocks of an SM per warp where the IEEE
 // intrinsics take 142 and 143, latency 236, 300 and 328 clocks against 562 and 597.
 JF_D bool mid_exp(unsigned hi) { return (hi & 0x7fffffffu) - (623u << 20) < (801u << 20); }
