@@ -138,38 +138,39 @@ __global__ void k_init_state(const double *thp, const double *prow, const double
     for (int v = 0; v < 4; ++v) U[v * N1 + i] = Uv[v] - ubv[v * nrow + J];
 }
 
-size_t workspace(const jfnk_grid *g, int k, const jfnk_opts *o, const jfnk_physics *ph, int *nlev_out) {
+bool multi_stage(const jfnk_opts &o) { return o.rk_stages > 1 || (o.rk_stages == 1 && o.rk_alpha[0] != 1.0); }
+
+// bytes of a context's device arrays (create_locked allocates these and no others)
+size_t workspace(const jfnk_grid *g, int k, const jfnk_opts *o, bool visc) {
     const int n1 = k + 1;
-    const size_t npt = (size_t)g->nx * g->nz * n1 * n1, N = 4 * npt;
+    const size_t npt = (size_t)g->nx * g->nz * n1 * n1, N = 4 * npt, n_el = (size_t)g->nx * g->nz;
     const int m = o->gmres_restart;
-    const int prec = o->precond_prec;
-    const size_t sS = prec == 64 ? 8 : 4;
-    size_t b = 0;
-    b += sizeof(PowTab);
-    const size_t nrow = (size_t)g->nz * n1;
-    b += 8 * (4 * nrow * 6 + 4 * (size_t)(g->nz + 1) * 3 + nrow * 2);
-    const size_t fx = (size_t)g->nz * (g->nx + 1) * n1, fz = (size_t)(g->nz + 1) * g->nx * n1;
-    const bool visc = ph ? ph->mu != 0.0 : true;
-    b += 8 * (4 + (visc ? 6 : 0)) * (fx + fz);
-    if (prec != 64) b += 4 * (4 + (visc ? 6 : 0)) * (fx + fz);
-    if (prec != 64 && o->dg_fused != 2 && !(ph && visc)) b += 128 * (fx + fz) + 4 * N;   // FP32 flux derivatives
-    b += 8 * N * 9;                        // DG work vectors
-    b += 12 * N * (size_t)(m + 1);         // V and its float copy
-    const bool mg_on = o->mg_key[0] != 0;
-    b += ((prec == 64 || !mg_on) ? 8 : 4) * N * (size_t)m;   // Z
-    b += sS * N * 6;                       // pz, pz2, pd, pr, pin, pout
-    b += 8 * (size_t)g->nx * g->nz;        // dtau_dg
+    const bool p64 = o->precond_prec == 64, mg_on = o->mg_key[0] != 0;
+    const size_t sS = p64 ? 8 : 4;
+    const size_t nrow = (size_t)g->nz * n1, nf = (size_t)g->nz + 1;
+    const size_t nfp = (size_t)g->nz * (g->nx + 1) * n1 + nf * g->nx * n1;
+    size_t b = sizeof(PowTab) + 8 * (30 * nrow + 12 * nf);
+    b += 8 * (4 + (visc ? 6 : 0)) * nfp;
+    if (!p64) {
+        if (o->dg_fused == 2) b += 4 * (4 + (visc ? 6 : 0)) * nfp;
+        else if (!visc) b += 128 * nfp + 4 * N;   // FP32 flux derivatives
+        b += 4 * n_el + 4 * N + 32 * (nrow + nf);   // step sizes, state and background in FP32
+    }
+    b += 8 * N * 5;                                                  // fU, Ubs, Usave, G, dU
+    b += 8 * N * (size_t)(m + 1) + 4 * N * v32_slots(m);             // V and its float copies
+    b += (p64 || !mg_on ? 8 : 4) * N * (size_t)m;                    // Z
+    b += sS * N * (size_t)(3 + multi_stage(*o)) + 8 * n_el;          // pz, pz2, pd, pr; dtau_dg
+    if (p64) b += 8 * N + (mg_on && o->precond_fd_eps > 0.0 ? 8 * N : 0);   // pout, Ulin
     int NX[JF_MAXLEV], NZ[JF_MAXLEV], fac[JF_MAXLEV];
     const int nl = hierarchy(g->nx, g->nz, k, o->fv_levels < 1 ? 1 : o->fv_levels, NX, NZ, fac);
     for (int l = 0; l < nl; ++l) {
         const size_t n = 4 * (size_t)NX[l] * NZ[l];
-        b += 8 * (4 * (size_t)NZ[l] * 4 + 4);
-        b += sS * n * 6 + sS * n / 4;
-        if (prec != 64 && n / 4 <= FV_STORED) b += 320 * (n / 4);   // stored stencil
+        b += (8 * 16 + 4 * 4) * (size_t)NZ[l] + 8 * 4 * (size_t)(NZ[l] + 1);
+        b += sS * n * (size_t)(4 + (l > 0) + p64) + sS * n / 4;      // u, x, x2, b, r below the finest, fu; dtau
+        if (!p64 && n / 4 <= FV_STORED) b += 320 * (n / 4);          // stored stencil
     }
-    b += 8 * 4096 * 32 + 8 * 256;
-    b += 8 * (fx + fz) * (visc ? 33 : 12) + 8 * N + 8 * npt * (visc ? 19 : 5);   // linearisation of the DG operator
-    if (nlev_out) *nlev_out = nl;
+    b += 8 * n_partials(N) + 8 * S_COUNT + 256;
+    b += 8 * nfp * (visc ? 33 : 12) + 8 * N + 8 * npt * (visc ? 19 : 5);   // linearisation of the DG operator
     return b;
 }
 
@@ -222,7 +223,9 @@ size_t jfnk_workspace_bytes(const jfnk_grid *g, int k, const jfnk_opts *opts) {
     if (opts) o = *opts;
     else jfnk_default_opts(&o);
     if (!g || k < 1 || k > 4 || g->nx < 1 || g->nz < 1) return 0;
-    return workspace(g, k, &o, nullptr, nullptr);
+    // (the viscosity is not known here: the larger of the two)
+    const size_t v = workspace(g, k, &o, true), i = workspace(g, k, &o, false);
+    return v > i ? v : i;
 }
 
 static void destroy_unlocked(jfnk_ctx *c);
@@ -411,7 +414,7 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
         A_(c->symx, 8 * 6 * fx);
         A_(c->symz, 8 * 6 * fz);
     }
-    if (c->prec != 64) {
+    if (c->prec != 64 && o.dg_fused == 2) {
         A_(c->phixf, 4 * 4 * fx);
         A_(c->phizf, 4 * 4 * fz);
         if (visc) {
@@ -421,28 +424,30 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
     }
     const size_t N = c->N;
     A_(c->fU, 8 * N);
-    A_(c->w1, 8 * N);
-    A_(c->w2, 8 * N);
     A_(c->Ubs, 8 * N);
-    A_(c->Un, 8 * N);
     A_(c->Usave, 8 * N);
     A_(c->G, 8 * N);
     A_(c->dU, 8 * N);
-    A_(c->Ulin, 8 * N);
     const int m = o.gmres_restart;
     const size_t sS = c->prec == 64 ? 8 : 4;
     // FGMRES stores z_j = Q^-1 v_j in the preconditioner's precision; without a
     // preconditioner z_j = v_j is copied in FP64
     const size_t sZ = (c->prec == 64 || !c->mg_on) ? 8 : 4;
     A_(c->V, 8 * N * (size_t)(m + 1));
-    A_(c->V32, 4 * N * (size_t)(m + 1));
+    A_(c->V32, 4 * N * v32_slots(m));
     A_(c->Z, sZ * N * (size_t)m);
     A_(c->pz, sS * N);
     A_(c->pz2, sS * N);
     A_(c->pd, sS * N);
-    A_(c->pr, sS * N);
-    A_(c->pin, sS * N);
-    A_(c->pout, sS * N);
+    if (multi_stage(o)) A_(c->pr, sS * N);
+    c->pin = c->V + (size_t)m * N;
+    if (c->prec == 64) {
+        c->w2 = (double *)c->pd;
+        A_(c->pout, 8 * N);
+        if (c->mg_on && o.precond_fd_eps > 0.0) A_(c->Ulin, 8 * N);
+    } else {
+        c->pout = (float *)c->pin + N;
+    }
     A_(c->dtau_dg, 8 * (size_t)c->n_el);
     if (c->prec != 64) {
         A_(c->dtau_dgf, 4 * (size_t)c->n_el);
@@ -481,11 +486,12 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
         A_(L.hbxw, 8 * 8 * (size_t)NZ[l]);
         A_(L.hbz, 8 * 4 * (size_t)(NZ[l] + 1));
         A_(L.u, sS * L.n);
-        A_(L.fu, 8 * L.n);
+        if (c->prec == 64) A_(L.fu, 8 * L.n);
         A_(L.x, sS * L.n);
         A_(L.x2, sS * L.n);
         A_(L.b, sS * L.n);
-        A_(L.r, sS * L.n);
+        if (l == 0) L.r = c->pd;   // (L.n = N)
+        else A_(L.r, sS * L.n);
         A_(L.dtau, sS * L.n / 4);
         if (c->prec != 64 && L.n / 4 <= FV_STORED) A_(L.st, 320 * (L.n / 4));
         std::vector<double> ub(4 * (size_t)NZ[l]);
@@ -501,7 +507,7 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
             return JFNK_ECUDA;
         }
     }
-    c->nb_red = 4096;
+    c->nb_red = NB_RED;
     {
         int dev = 0, nsm = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -512,7 +518,7 @@ static int create_locked(const jfnk_grid *g, int k, const jfnk_physics *ph, cons
         }
         c->n_sm = nsm;
     }
-    A_(c->partial, 8 * (size_t)c->nb_red * 32);
+    A_(c->partial, 8 * n_partials(N));
     {
         const size_t nfp = (size_t)g->nz * (g->nx + 1) * c->np1 + (size_t)(g->nz + 1) * g->nx * c->np1;
         A_(c->lin.tr, 8 * nfp * (visc ? 20 : 8));
@@ -718,7 +724,7 @@ int jfnk_time_operator(jfnk_ctx *c, int which, const double *U, const double *y,
         a.Uf = c->Usf;
         if (!rc && c->jac) rc = dg_apply(c, DG_TLLIN, a, s);
     }
-    a.out0 = which == 2 ? (void *)c->pz2 : (void *)c->w2;
+    a.out0 = which == 2 ? (void *)c->pz2 : (void *)c->dU;
     c->t_faces_ms = c->t_volume_ms = 0.0;
     c->timing = 1;
     for (int r = 0; r < reps && rc == JFNK_OK; ++r)

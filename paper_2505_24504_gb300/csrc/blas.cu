@@ -991,7 +991,7 @@ static void cgs2_t(jfnk_ctx *c, const double *V, const float *V32, size_t ldv, d
 int blas_cgs2(jfnk_ctx *c, const double *V, const float *V32, int nv, size_t ldv, double *w, float *w32, size_t n,
               double *h1, double *h2, double *w1sq, double *nrm, double *flag, cudaStream_t s) {
     if (nv < 1 || nv > GS_FUSED_MAX || (n & 1) || (ldv & 1) || !V32) return JFNK_EINVAL;
-    if (nv > 16) {
+    if (nv > GS_FP32_MAX) {
         const size_t n2 = n / 2;
         const int g1 = one_wave(c, k_gsl_dot, n2), g2 = one_wave(c, k_gsl_update_dot, n2),
                   g3 = one_wave(c, k_gsl_update_scale, n2);

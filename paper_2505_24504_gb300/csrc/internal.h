@@ -203,6 +203,15 @@ struct DGTab {
 // against 16.86.  At 51,200 cells reading the stencil costs more than the fluxes it
 // saves (preconditioner of the warm bubble 169 us against 155), at 12,800 the two agree.
 constexpr size_t FV_STORED = 4096;
+constexpr int NB_RED = 4096;   // partial-sum blocks of the reductions
+// Partial sums of a context of N unknowns: a row of NB_RED (a reduction over any length),
+// 33 rows of the blocks that two elements a thread give N (Gram-Schmidt against 32 vectors
+// and |w|^2; on long vectors its blocks fit one wave), 16 rows of NB_RED (the general
+// multi-dot), and one of each block of the DG smoothing step (mg_norm_blocks looks).
+inline size_t n_partials(size_t N) {
+    const size_t rows = 33 * ((N + 511) / 512), lo = NB_RED, hi = 32 * (size_t)NB_RED;
+    return rows < lo ? lo : rows > hi ? hi : rows;
+}
 struct FVLev {
     int NX, NZ;
     int fac;             // agglomeration factor to the next coarser level (0: coarsest)
@@ -255,13 +264,16 @@ struct jfnk_ctx {
     double *phix, *symx, *phiz, *symz;
     float *phixf, *symxf, *phizf, *symzf;
     // DG work vectors (FP64, N each)
-    double *fU, *w1, *w2, *Ubs, *Un, *Usave, *G, *dU;
+    double *fU, *Ubs, *Usave, *G, *dU;
+    double *w2;          // G'z of the FP64 preconditioner's DG defect (prec 64)
     // Krylov basis: V (m+1) N doubles, Z m N of the preconditioner's type
     double *V;
-    float *V32;          // float copy of V (first Gram-Schmidt pass)
+    float *V32;          // float copy of v_j at v32_slot(j)
     void *Z;
     // preconditioner DG vectors (type of the preconditioner)
-    void *pz, *pz2, *pd, *pr;
+    void *pz, *pz2;
+    void *pd;            // DG defect; once it is transferred, the finest FV level's defect
+    void *pr;            // multi-stage smoothers only
     double *dtau_dg;     // [n_el]
     float *dtau_dgf;     // [n_el] FP32 copy (prec 32)
     float *jac, *jacn;   // FP32 derivatives of the face fluxes (32 a face point) and node values
@@ -274,14 +286,14 @@ struct jfnk_ctx {
     LinPtr lin;          // linearisation of the DG operator at the state of the last residual
     int lin_valid;       // lin and fU come from the same residual evaluation
     unsigned *ticket;    // arrival counter of the single-launch reductions (0 between launches)
-    int nb_red;          // partial-sum blocks
+    int nb_red;          // blocks of a reduction at most
     int n_sm;            // streaming multiprocessors of the context's device
     double *scal;        // device scalars (norms, eps)
     double *h_pinned;    // host pinned scratch for Hessenberg columns
     // linearisation of the preconditioner (set by mg_linearize)
     double mg_adt;
-    const double *mg_U;  // = Ulin, the context's copy of the linearisation state
-    double *Ulin;
+    double *Ulin;        // copy of the state where the general FP64 products need it (prec 64 with a
+                         // given precond_fd_eps)
     // counters of the current call
     long long dg_calls, fv_calls;
     double deadline;     // steady-clock seconds at which the current implicit step times out (0: none)
@@ -293,7 +305,9 @@ struct jfnk_ctx {
     double mg_graph_adt;
     unsigned long long graph_launches;   // kernels in the graph
     long long graph_dg_calls, graph_fv_calls;
-    void *pin, *pout;                    // fixed input / output of the graph
+    void *pin, *pout;                    // fixed input / output of the graph: pin, and pout in FP32, lie in
+                                         // the basis' last vector, which an Arnoldi step writes only after
+                                         // its preconditioner application
     int mg_graph_gen;                    // incremented at every capture of the preconditioner
     int capturing;                       // 1 while an Arnoldi step is being captured
     // one graph per Arnoldi step index j (preconditioner child graph, FD
@@ -409,7 +423,7 @@ inline int dgtl_blocks(const jfnk_ctx *c) {
 // output (0: none; eps of the FD product then takes a pass over z)
 inline int mg_norm_blocks(const jfnk_ctx *c) {
     const bool ok = c->mg_on && c->prec != 64 && c->dg_post > 0 && c->opts.dg_fused != 2 && c->opts.rk_stages == 1 &&
-                    c->opts.rk_alpha[0] == 1.0 && dgtl_blocks(c) <= c->nb_red * 32;
+                    c->opts.rk_alpha[0] == 1.0 && (size_t)dgtl_blocks(c) <= n_partials(c->N);
     return ok ? dgtl_blocks(c) : 0;
 }
 
@@ -433,6 +447,11 @@ int blas_mupdate_norm(jfnk_ctx *c, const double *V, int nv, size_t ldv, const do
                       double sign, const double *flag_in, double *w1sq, double *nrm, double *flag_out,
                       cudaStream_t s);
 constexpr int GS_FUSED_MAX = 32;   // basis vectors of the fused CGS2 kernels
+constexpr int GS_FP32_MAX = 16;    // of those whose first pass runs in FP32
+// where the float copy of v_j lies: the first pass reads v_0 .. v_15, the preconditioner
+// the current vector, so the later ones share a slot
+inline size_t v32_slot(int j) { return (size_t)(j < GS_FP32_MAX ? j : GS_FP32_MAX); }
+inline size_t v32_slots(int restart) { return v32_slot(restart) + 1; }
 // V32: float copy of the basis (first pass in FP32); w32: where the
 // float copy of the normalised w goes (may be null)
 int blas_cgs2(jfnk_ctx *c, const double *V, const float *V32, int nv, size_t ldv, double *w, float *w32, size_t n,

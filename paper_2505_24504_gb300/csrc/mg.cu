@@ -925,11 +925,10 @@ __device__ __forceinline__ void load_ttab(const TK &K, R sV[NP1][NP1], R sVi[NP1
     for (int t = threadIdx.x; t < NP1; t += blockDim.x) som[t] = (R)K.tab.om[t];
 }
 
-// What the FP32 linearisation takes along with the transfer of the state: the context's
-// FP64 and FP32 copies of U and the DG pseudo-time steps.  One launch instead of a copy, a
-// conversion, the step sizes and the transfer, each a pass over the state.
+// What the FP32 linearisation takes along with the transfer of the state: the FP32 copy of
+// U and the DG pseudo-time steps.  One launch instead of a conversion, the step sizes and
+// the transfer, each a pass over the state.
 struct LinOut {
-    double *Ul;          // null: a plain transfer
     float *Uf, *dtauf;
     const float *ubvf;
     PhysC pc;
@@ -971,7 +970,6 @@ struct k_to_fv_b {
                     if (xx.w) ui -= xx.w[gi];
                 su[le][q][node] = (R)ui;
                 if (LIN) {
-                    lo.Ul[gi] = ui;
                     lo.Uf[gi] = (float)ui;
                     W[q] = (float)ui + lo.ubvf[q * (K.nz * NP1) + (e / K.nx) * NP1 + node / NP1];
                 }
@@ -1817,7 +1815,7 @@ int dg_smooth_step<double>(jfnk_ctx *c, const double *r, double *&z, double *&z2
     if (!have_eps) JF_RET(red_dot(c, z, z, c->N, c->scal + S_EPSDG, RED_EPSP, s));
     have_eps = false;
     DGArgs a = {};
-    a.U = c->mg_U;
+    a.U = c->Ulin;
     a.y = z;
     a.fU = c->fU;
     a.r = r;
@@ -1843,7 +1841,6 @@ int dg_smooth_step<float>(jfnk_ctx *c, const float *r, float *&z, float *&z2, bo
         return JFNK_OK;
     }
     DGArgs a = {};
-    a.U = c->mg_U;
     a.Uf = c->Usf;
     a.yf = z;
     a.rf = r;
@@ -1867,7 +1864,7 @@ template <>
 int dg_defect<double>(jfnk_ctx *c, const double *, const double *z, double *, cudaStream_t s, bool have_eps) {
     if (!have_eps) JF_RET(red_dot(c, z, z, c->N, c->scal + S_EPSDG, RED_EPSP, s));
     DGArgs a = {};
-    a.U = c->mg_U;
+    a.U = c->Ulin;
     a.y = z;
     a.fU = c->fU;
     a.eps = c->scal + S_EPSDG;
@@ -1881,7 +1878,6 @@ int dg_defect<double>(jfnk_ctx *c, const double *, const double *z, double *, cu
 template <>
 int dg_defect<float>(jfnk_ctx *c, const float *r, const float *z, float *d, cudaStream_t s, bool) {
     DGArgs a = {};
-    a.U = c->mg_U;
     a.Uf = c->Usf;
     a.yf = z;
     a.rf = r;   // the tangent product's epilogue forms d = r - G'z
@@ -1896,7 +1892,6 @@ int dg_first_step_defect32(jfnk_ctx *c, const float *r, float *z, float *d, cuda
                            const TransferOut *tro = nullptr) {
     DGArgs a = {};
     a.tro = tro;
-    a.U = c->mg_U;
     a.Uf = c->Usf;
     a.rf = r;
     a.dtauf = c->dtau_dgf;
@@ -1925,7 +1920,7 @@ int dg_rk_step(jfnk_ctx *c, const S *r, S *&z, S *&z2, S *&z3, bool &zero, cudaS
             JF_CK(cudaGetLastError());
         } else {
             DGArgs A = {};
-            A.U = c->mg_U;
+            A.U = c->Ulin;
             A.adt = c->mg_adt;
             A.out0 = out;
             A.z0 = zero ? nullptr : z;
@@ -2058,22 +2053,21 @@ int fv_setup_background(jfnk_ctx *c, cudaStream_t s) {
 }
 
 int mg_linearize(jfnk_ctx *c, const double *Uin, double adt, cudaStream_t s) {
-    // every pointer the captured graph holds is context-owned: Ulin is the copy of U
+    // every pointer the captured graph holds is context-owned: Ulin is the copy of U (the
+    // products about the stored linearisation need none)
     c->mg_adt = adt;
-    c->mg_U = c->Ulin;
     if (c->prec == 64) {
-        JF_CK(jf_memcpy(c->Ulin, Uin, 8 * c->N, cudaMemcpyDeviceToDevice, s));
-        const double *U = c->Ulin;
+        if (c->Ulin) JF_CK(jf_memcpy(c->Ulin, Uin, 8 * c->N, cudaMemcpyDeviceToDevice, s));
         const int epb = 256 / (c->np1 * c->np1);
-        jf_launch<k_dg_dtau_b>(k_dg_dtau, (unsigned)((c->n_el + epb - 1) / epb), 256, 0, s, U, (const double *)c->ubv, c->grid.nx,
+        jf_launch<k_dg_dtau_b>(k_dg_dtau, (unsigned)((c->n_el + epb - 1) / epb), 256, 0, s, Uin, (const double *)c->ubv, c->grid.nx,
                   c->grid.nz, c->np1, c->pc, c->powtab, 1.0 / c->hx, 1.0 / c->hz, c->phys.mu, adt, c->opts.sigma_dg,
                   c->dtau_dg);
         jf_launched();
         JF_CK(cudaGetLastError());
-        JF_RET(to_fv<double, double>(c, U, (double *)c->lev[0].u, s));
+        JF_RET(to_fv<double, double>(c, Uin, (double *)c->lev[0].u, s));
     } else {
         JF_RET(to_fv<double, float>(c, Uin, (float *)c->lev[0].u, s, nullptr, nullptr,
-                                    LinOut{c->Ulin, c->Usf, c->dtau_dgf, c->ubvf, c->pc, 1.0 / c->hx, 1.0 / c->hz,
+                                    LinOut{c->Usf, c->dtau_dgf, c->ubvf, c->pc, 1.0 / c->hx, 1.0 / c->hz,
                                            c->phys.mu, adt, c->opts.sigma_dg}));
         if (c->jac && (c->dg_pre || c->dg_post)) {
             DGArgs a = {};

@@ -53,17 +53,16 @@ struct Phases {
     }
 };
 
-// w = G'(U) y about the linearisation of the last residual (U is its state), with
+// w = G'(U) y about the linearisation of the last residual (U its state), with
 // eps = sqrt(eps_mach)/|y| computed on the device; y in FP64, or in FP32 (yf) as the FP32
 // preconditioner writes it
-int apply_jv(jfnk_ctx *c, const double *U, double adt, const double *y, const float *yf, double *w, cudaStream_t s) {
+int apply_jv(jfnk_ctx *c, double adt, const double *y, const float *yf, double *w, cudaStream_t s) {
     // the FP32 preconditioner left the blocks' sums of squares of its output
     const int nb = yf ? mg_norm_blocks(c) : 0;
     if (nb) JF_RET(blas_eps_part(c, c->partial, nb, c->scal + S_EPS, s));
     else if (yf) JF_RET(blas_eps32(c, yf, c->N, c->scal + S_EPS, s));
     else JF_RET(red_dot(c, y, y, c->N, c->scal + S_EPS, RED_EPS, s));
     DGArgs a = {};
-    a.U = U;
     a.y = y;
     a.yf = yf;
     a.fU = c->fU;
@@ -86,26 +85,26 @@ int read_norm(jfnk_ctx *c, const double *x, double *out, cudaStream_t s) {
 // Gram-Schmidt (second pass decided on the device), normalisation, and the
 // copy of the Hessenberg column to pinned host memory.  No host decisions, so
 // it can be captured.
-int arnoldi_step_work(jfnk_ctx *c, const double *U, double adt, int j, cudaStream_t s, Phases *ph) {
+int arnoldi_step_work(jfnk_ctx *c, double adt, int j, cudaStream_t s, Phases *ph) {
     const size_t N = c->N;
     double *V = c->V;
     double *vj = V + (size_t)j * N, *w = V + (size_t)(j + 1) * N;
     if (ph) ph->mark(0, s);
     if (c->mg_on) {
         JF_RET(mg_apply(c, vj, (char *)c->Z + (size_t)j * N * (c->prec == 64 ? 8 : 4), s,
-                        c->prec == 64 ? nullptr : c->V32 + (size_t)j * N));
+                        c->prec == 64 ? nullptr : c->V32 + v32_slot(j) * N));
     } else {
         JF_CK(jf_memcpy((double *)c->Z + (size_t)j * N, vj, 8 * N, cudaMemcpyDeviceToDevice, s));
     }
     if (ph) ph->mark(1, s);
-    if (c->prec == 64 || !c->mg_on) JF_RET(apply_jv(c, U, adt, (const double *)c->Z + (size_t)j * N, nullptr, w, s));
-    else JF_RET(apply_jv(c, U, adt, nullptr, (const float *)c->Z + (size_t)j * N, w, s));
+    if (c->prec == 64 || !c->mg_on) JF_RET(apply_jv(c, adt, (const double *)c->Z + (size_t)j * N, nullptr, w, s));
+    else JF_RET(apply_jv(c, adt, nullptr, (const float *)c->Z + (size_t)j * N, w, s));
     if (ph) ph->mark(2, s);
     // classical Gram-Schmidt; the update kernel also reduces |w|^2, and a
     // second pass runs only when the first lost more than half of |w|
     // (decided on the device)
     if (j + 1 <= GS_FUSED_MAX && (N & 1) == 0) {
-        JF_RET(blas_cgs2(c, V, c->V32, j + 1, N, w, c->V32 + (size_t)(j + 1) * N, N, c->scal + S_H, c->scal + S_H2,
+        JF_RET(blas_cgs2(c, V, c->V32, j + 1, N, w, c->V32 + v32_slot(j + 1) * N, N, c->scal + S_H, c->scal + S_H2,
                          c->scal + S_W1, c->scal + S_NORM, c->scal + S_FLAG, s));   // normalises w too
         if (ph) ph->mark(3, s);
         JF_CK(jf_memcpy(c->h_pinned, c->scal, 8 * S_COUNT, cudaMemcpyDeviceToHost, s));
@@ -118,17 +117,17 @@ int arnoldi_step_work(jfnk_ctx *c, const double *U, double adt, int j, cudaStrea
     JF_RET(blas_mupdate_norm(c, V, j + 1, N, c->scal + S_H2, w, N, -1.0, c->scal + S_FLAG, nullptr,
                              c->scal + S_NORM, nullptr, s));
     JF_RET(blas_scale_copy(w, c->scal + S_NORM, w, N, s));
-    JF_RET(blas_copy_d2f(w, c->V32 + (size_t)(j + 1) * N, N, s));   // float copy of the basis
+    JF_RET(blas_copy_d2f(w, c->V32 + v32_slot(j + 1) * N, N, s));   // float copy of the basis
     if (ph) ph->mark(3, s);
     JF_CK(jf_memcpy(c->h_pinned, c->scal, 8 * S_COUNT, cudaMemcpyDeviceToHost, s));
     return JFNK_OK;
 }
 
 // Arnoldi step j, replayed from a graph captured per j (pointers are all
-// context-owned: U is the context's copy of the Newton iterate).
-int arnoldi_step(jfnk_ctx *c, const double *U, double adt, int j, cudaStream_t s, Phases &ph) {
-    const bool graphs = c->opts.use_graphs && !ph.on && U == c->Ulin && j < 64 && !t_jf_rec;
-    if (!graphs) return arnoldi_step_work(c, U, adt, j, s, ph.on ? &ph : nullptr);
+// context-owned: the products take the stored linearisation, not U).
+int arnoldi_step(jfnk_ctx *c, double adt, int j, cudaStream_t s, Phases &ph) {
+    const bool graphs = c->opts.use_graphs && !ph.on && j < 64 && !t_jf_rec;
+    if (!graphs) return arnoldi_step_work(c, adt, j, s, ph.on ? &ph : nullptr);
     if (c->arn_adt != adt) {
         for (int i = 0; i < 64; ++i)
             if (c->arn_valid[i]) {
@@ -144,7 +143,7 @@ int arnoldi_step(jfnk_ctx *c, const double *U, double adt, int j, cudaStream_t s
         const long long d0 = c->dg_calls, f0 = c->fv_calls;
         JF_CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
         c->capturing = 1;   // the preconditioner's kernels are captured inline
-        const int rc = arnoldi_step_work(c, U, adt, j, c->cap_stream, nullptr);
+        const int rc = arnoldi_step_work(c, adt, j, c->cap_stream, nullptr);
         c->capturing = 0;
         cudaGraph_t g = nullptr;
         const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
@@ -193,7 +192,7 @@ void arnoldi_column(const jfnk_ctx *c, int j, double *h) {
 }
 
 // Solve G'(U) x = b from x = 0 until the residual estimate <= tol_abs.
-int fgmres(jfnk_ctx *c, const double *U, double adt, const double *b, double *x, double tol_abs, int *its,
+int fgmres(jfnk_ctx *c, double adt, const double *b, double *x, double tol_abs, int *its,
            cudaStream_t s, Stats &st) {
     Phases ph(c->opts.profile != 0);
     const size_t N = c->N;
@@ -215,7 +214,7 @@ int fgmres(jfnk_ctx *c, const double *U, double adt, const double *b, double *x,
         int jd = 0;
         bool conv = false;
         for (int j = 0; j < m; ++j) {
-            JF_RET(arnoldi_step(c, U, adt, j, s, ph));
+            JF_RET(arnoldi_step(c, adt, j, s, ph));
             JF_CK(jf_sync(s));
             if (out_of_time(c)) return JFNK_ETIMEOUT;
             st.t_pre += ph.ms(0, 1);
@@ -260,10 +259,11 @@ int fgmres(jfnk_ctx *c, const double *U, double adt, const double *b, double *x,
         JF_RET(blas_zcomb(c->Z, (c->prec != 64 && c->mg_on) ? 1 : 0, jd, N, y, x, s));
         if (conv) return JFNK_OK;
         if (*its >= maxit) return JFNK_ENOTCONV;
-        // restart from the true residual r = b - G'x
-        JF_RET(apply_jv(c, U, adt, x, nullptr, c->w2, s));
-        JF_RET(blas_axpby(1.0, b, -1.0, c->w2, c->w2, N, s));
-        r = c->w2;
+        // restart from the true residual r = b - G'x (in the basis' last vector: the basis is done with)
+        double *w = c->V + (size_t)m * N;
+        JF_RET(apply_jv(c, adt, x, nullptr, w, s));
+        JF_RET(blas_axpby(1.0, b, -1.0, w, w, N, s));
+        r = w;
         JF_RET(read_norm(c, r, &beta, s));
         if (!isfinite(beta)) return JFNK_ENAN;
         if (beta <= tol_abs) return JFNK_OK;
@@ -307,13 +307,11 @@ int newton(jfnk_ctx *c, double *U, double adt, Stats &st, cudaStream_t s) {
         }
         Phases ph(c->opts.profile != 0);
         ph.mark(0, s);
-        // the context's copy of U^k: the captured Arnoldi graphs hold this pointer
         if (c->mg_on) JF_RET(mg_linearize(c, U, adt, s));
-        else JF_CK(jf_memcpy(c->Ulin, U, 8 * c->N, cudaMemcpyDeviceToDevice, s));
         ph.mark(1, s);
         JF_RET(blas_scale(-1.0, c->G, c->G, c->N, s));
         int its = 0;
-        int rc = fgmres(c, c->Ulin, adt, c->G, c->dU, eta * nk, &its, s, st);
+        int rc = fgmres(c, adt, c->G, c->dU, eta * nk, &its, s, st);
         st.gmres_its += its;
         if (rc != JFNK_OK && rc != JFNK_ENOTCONV) return rc;
         JF_RET(blas_axpby(1.0, U, 1.0, c->dU, U, c->N, s));
@@ -358,8 +356,7 @@ extern "C" int implicit_step(jfnk_ctx *c, double *U, double dt, int scheme, jfnk
         if (rc == JFNK_OK) {
             // Ubar_2 = U^n + (1 - alpha) dt f(U_1); f(U_1) is the last residual's f
             stages = 2;
-            JF_CK(jf_memcpy(c->w1, c->fU, 8 * N, cudaMemcpyDeviceToDevice, s));
-            rc = blas_axpby(1.0, c->Usave, (1.0 - a) * dt, c->w1, c->Ubs, N, s);
+            rc = blas_axpby(1.0, c->Usave, (1.0 - a) * dt, c->fU, c->Ubs, N, s);
             if (rc == JFNK_OK) rc = jf_memcpy(U, c->Ubs, 8 * N, cudaMemcpyDeviceToDevice, s) == cudaSuccess
                                         ? JFNK_OK
                                         : JFNK_ECUDA;
@@ -398,14 +395,13 @@ extern "C" int jfnk_arnoldi(jfnk_ctx *c, const double *U, double adt, const doub
     a.lin_out = 1;
     JF_RET(dg_apply(c, DG_RES, a, s));
     if (c->mg_on) JF_RET(mg_linearize(c, U, adt, s));
-    else JF_CK(jf_memcpy(c->Ulin, U, 8 * c->N, cudaMemcpyDeviceToDevice, s));
     double beta;
     JF_RET(read_norm(c, r, &beta, s));
     if (!isfinite(beta) || beta == 0.0) return JFNK_ENAN;
     JF_RET(arnoldi_start(c, r, beta, s));
     Phases ph(false);
     for (int j = 0; j < nv; ++j) {
-        JF_RET(arnoldi_step(c, c->Ulin, adt, j, s, ph));
+        JF_RET(arnoldi_step(c, adt, j, s, ph));
         JF_CK(jf_sync(s));
         double *h = H + (size_t)j * (nv + 1);
         arnoldi_column(c, j, h);
