@@ -234,25 +234,50 @@ def timed_once(ctx, U, w, **kw):
 
 
 # ---------------------------------------------------------------------------
-# Algorithmic flops of the FD product about a stored linearisation, from the formulas (a
-# divide, square root or x^gamma counts one flop, an FMA two, compares and selects none):
-#  face point, stored states of U plus eps times the traces of y:
-#    traces of y: 2 sides x 4 variables x (k+1) FMA; U + eps tr(y): 8 FMA; HLLC in
-#    contact form: 1/rho 2, velocities 2, pressures 2 x 3, sound speeds 2 x 3, their
-#    differences 3, rho (S - u) 2, contact speed 7, star mass 3, side factors 1, flux 6
-#    (38); minus the stored flux: 4
+# Algorithmic work of the FD product about a stored linearisation, from the formulas, by the
+# pipe that does it (a divide, square root or x^gamma counts one flop, an FMA two, compares
+# and selects none).
+# FP64 pipe:
+#  face point: U + eps tr(y) 8 FMA; HLLC in contact form: 1/rho 2, velocities 2, pressures
+#    2 x 3, sound speeds 2 x 3, their differences 3, rho (S - u) 2, contact speed 7, star
+#    mass 3, side factors 1, flux 6 (38); minus the stored flux 4
 #  node: U + eps y 4 FMA; 1/rho 1; pressure 3; velocities 2; fluxes 7; minus the stored
-#    fluxes 5; sum factorisation 4 variables x 2 directions x (k+1) FMA; gravity 2; lift
-#    of the four face terms 4 x 4 FMA; quotient and update 1 FMA per variable
+#    fluxes 5; quotient and update 1 FMA per variable
+# two-float FMAs on the FP32 pipe (TWO_FLOAT_FMA instructions each):
+#  face point: traces of y 2 sides x 4 variables x (k+1)
+#  node: sum factorisation 4 variables x 2 directions x (k+1); gravity 1; lift of the four
+#    face terms 4 x 4
 HLLC_FLOPS = 38
+TWO_FLOAT_FMA = 12   # product with its error 4, TwoSum 6, low parts 2
+FP32_LANES_PER_SM = 128
 
 
-def alg_flops_face_point(k):
-    return 2 * (2 * 4 * (k + 1)) + 2 * 8 + HLLC_FLOPS + 4
+def fp64_flops_face_point():
+    return 2 * 8 + HLLC_FLOPS + 4
 
 
-def alg_flops_node(k):
-    return 2 * 4 + 1 + 3 + 2 + 7 + 5 + 2 * (4 * 2 * (k + 1)) + 2 + 2 * 16 + 2 * 4
+def fp64_flops_node():
+    return 2 * 4 + 1 + 3 + 2 + 7 + 5 + 2 * 4
+
+
+def two_float_fma_face_point(k):
+    return 2 * 4 * (k + 1)
+
+
+def two_float_fma_node(k):
+    return 4 * 2 * (k + 1) + 1 + 4 * 4
+
+
+def fd_product_roofline(k, face_pts, nodes, ms, peak64, nsm, sm_mhz):
+    """Work of one FD product on each pipe over the product's time, against that pipe's rate."""
+    flops = fp64_flops_face_point() * face_pts + fp64_flops_node() * nodes
+    fma = two_float_fma_face_point(k) * face_pts + two_float_fma_node(k) * nodes
+    ach = flops / (ms * 1e-3) / 1e12
+    issue = TWO_FLOAT_FMA * fma / (ms * 1e-3) / (nsm * FP32_LANES_PER_SM * sm_mhz * 1e6)
+    return {"achieved": ach, "peak": peak64, "unit": "TFLOP/s", "frac": ach / peak64, "flop": flops,
+            "units": {"face_points": face_pts, "flop_per_face_point": fp64_flops_face_point(),
+                      "nodes": nodes, "flop_per_node": fp64_flops_node()},
+            "two_float": {"fma": fma, "fp32_instructions_per_fma": TWO_FLOAT_FMA, "frac_of_fp32_issue": issue}}
 
 
 def fp64_peak_tflops(sm_mhz):
@@ -961,18 +986,14 @@ def main():
     n1 = w.k + 1
     face_pts = (w.nz * (w.nx + 1) + (w.nz + 1) * w.nx) * n1
     nodes = w.n_el * n1 * n1
-    fl_face, fl_node = alg_flops_face_point(w.k), alg_flops_node(w.k)
-    flops = fl_face * face_pts + fl_node * nodes
-    ach = flops / ((fm + vm) * 1e-3) / 1e12
     roof = {"bound": "alu", "kernel": "k_fd_flux + k_fd_lift: one FD product about the stored linearisation",
-            "achieved": ach, "peak": peak64, "unit": "TFLOP/s", "frac": ach / peak64, "traffic": TRAFFIC_FD,
+            **fd_product_roofline(w.k, face_pts, nodes, fm + vm, peak64, nsm, sm_mhz), "traffic": TRAFFIC_FD,
             "peak_source": (f"derived, not measured: {nsm} SMs (device properties) x {FP64_FLOP_PER_SM_CLK:g} FP64 "
                             f"flop/SM/clock x {sm_mhz:g} MHz"),
-            "flux_launch_ms": fm, "lift_launch_ms": vm, "flop": flops,
-            "units": {"face_points": face_pts, "flop_per_face_point": fl_face, "nodes": nodes, "flop_per_node": fl_node},
-            "flop_counting": "algorithmic, from the formulas (bench.py alg_flops_face_point, alg_flops_node); the traces, "
-                             "derivatives and lifts run in two-float arithmetic on the FP32 pipe, about 63 FP64 "
-                             "instructions a face point and 25 a node remain",
+            "flux_launch_ms": fm, "lift_launch_ms": vm,
+            "flop_counting": "algorithmic FP64-pipe work from the formulas (bench.py fp64_flops_*) over the time of both "
+                             "launches; the traces, derivatives and lifts run in two-float arithmetic on the FP32 pipe "
+                             "and are counted under two_float only",
             "hbm": kernel_bandwidths(w, preset, hbm_peak, hbm_note, flush, U0)}
 
     # ---- phase breakdown of one more step (events at the solver's own syncs) ----
