@@ -70,11 +70,11 @@ __device__ __forceinline__ double sum_partials(const double *part, int nb) {
     return block_sum(acc);
 }
 
-// cnum: numerator of the eps ops (sqrt(2^-52) for RED_EPS, sqrt(2^-23) for
-// RED_EPS32, the preconditioner's choice for RED_EPSP)
+// cnum: numerator of the eps ops (sqrt(2^-52) for RED_EPS, the preconditioner's choice
+// for RED_EPSP)
 __device__ __forceinline__ double finish_op(double acc, int op, double cnum = 1.4901161193847656e-08) {
     if (op == RED_SQRT) return sqrt64(acc);
-    if (op == RED_EPS || op == RED_EPS32 || op == RED_EPSP) return acc > 0.0 ? div64(cnum, sqrt64(acc)) : 0.0;
+    if (op == RED_EPS || op == RED_EPSP) return acc > 0.0 ? div64(cnum, sqrt64(acc)) : 0.0;
     return acc;
 }
 
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(RB) k_dot_partial(const S *x, const S *y, size
 }
 
 // op (single-launch reductions): RED_SUM -> sum; RED_SQRT -> sqrt(sum);
-// RED_EPS -> sqrt(2^-52)/sqrt(sum) (0 if sum == 0); RED_EPS32 -> sqrt(2^-23)/sqrt(sum)
+// RED_EPS, RED_EPSP -> cnum/sqrt(sum) (0 if sum == 0)
 
 // h_j partials for NV basis vectors at once: accumulators are compile-time
 // indexed (registers), warp sums go through one shared-memory pass.
@@ -934,7 +934,6 @@ inline int nblocks_red(jfnk_ctx *c, size_t n) {
 }  // namespace
 
 static double eps_numerator(const jfnk_ctx *c, int op) {
-    if (op == RED_EPS32) return 3.4526698300124393e-04;   // sqrt(2^-23)
     if (op == RED_EPSP && c->opts.precond_fd_eps > 0.0) return c->opts.precond_fd_eps;
     return 1.4901161193847656e-08;                         // sqrt(2^-52)
 }
@@ -942,14 +941,6 @@ static double eps_numerator(const jfnk_ctx *c, int op) {
 int red_dot(jfnk_ctx *c, const double *x, const double *y, size_t n, double *out, int op, cudaStream_t s) {
     const int nb = nblocks_red(c, n);
     jf_launch<k_dot1_b<double>>(k_dot1<double>, nb, RB, 0, s, x, y, n, c->partial, c->ticket, out, op, eps_numerator(c, op));
-    jf_launched();
-    JF_CK(cudaGetLastError());
-    return JFNK_OK;
-}
-
-int red_dotf(jfnk_ctx *c, const float *x, const float *y, size_t n, double *out, int op, cudaStream_t s) {
-    const int nb = nblocks_red(c, n);
-    jf_launch<k_dot1_b<float>>(k_dot1<float>, nb, RB, 0, s, x, y, n, c->partial, c->ticket, out, op, eps_numerator(c, op));
     jf_launched();
     JF_CK(cudaGetLastError());
     return JFNK_OK;
@@ -1131,31 +1122,6 @@ int blas_zcomb(const void *Z, int prec32, int nzv, size_t n, const double *yv, d
             jf_launch<k_zcomb_b<double>>(k_zcomb<double>, grid_for(n), 256, 0, s, (const double *)Z + (size_t)j0 * n, m, n, y, x);
         jf_launched();
     }
-    JF_CK(cudaGetLastError());
-    return JFNK_OK;
-}
-
-// Second Gram-Schmidt pass needed?  With w1 = w0 - V h the first pass left
-// |w1|^2 of |w0|^2 = |w1|^2 + |h|^2; reorthogonalise when |w1| < |w0| / sqrt(2)
-// ("twice is enough").  flag = 1.0 or 0.0, decided on the device.
-struct k_reortho_flag_b {
-    static constexpr int TPB = 0, MINB = 0;
-    static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<const double *> w1sq,
-                                               JfArg<const double *> h, JfArg<int> nv, JfArg<double *> flag) {
-        jf_pdl_enter();
-        double hh = 0.0;
-        for (int i = threadIdx.x; i < nv; i += 32) hh += h[i] * h[i];
-        hh = warp_sum(hh);
-        if (threadIdx.x == 0) *flag = (*w1sq < 0.5 * (*w1sq + hh)) ? 1.0 : 0.0;
-    }
-};
-__global__ void k_reortho_flag(const double *w1sq, const double *h, int nv, double *flag) {
-    k_reortho_flag_b::run(blockIdx.x, gridDim.x, w1sq, h, nv, flag);
-}
-
-int blas_reortho_flag(const double *w1sq, const double *h, int nv, double *flag, cudaStream_t s) {
-    jf_launch<k_reortho_flag_b>(k_reortho_flag, 1, 32, 0, s, w1sq, h, nv, flag);
-    jf_launched();
     JF_CK(cudaGetLastError());
     return JFNK_OK;
 }

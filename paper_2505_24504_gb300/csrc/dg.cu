@@ -586,15 +586,15 @@ __device__ __forceinline__ void block_squares(float sq, int n, double *out) {
     if (threadIdx.x == 0) *out = r;
 }
 
-template <int NP1, bool VISC, int MODE, int FIRST>
+template <int NP1, int MODE, int FIRST>
 struct k_dgtl_b {
-    static constexpr int TPB = 128, MINB = VISC ? 5 : 8;
-    static constexpr bool GROUP = !VISC;   // a grouped twin is built (lock-step ensembles)
+    static constexpr int TPB = 128, MINB = 5;
+    static constexpr bool GROUP = false;   // (lock-step members of viscous ensembles replay one at a time)
     static __device__ __forceinline__ void run(unsigned jf_bid, unsigned jf_nblk, JfArg<DGK> K, JfArg<DGArgs> A,
                                                JfArg<float *> out1f, JfArg<TransferOut> TR) {
         jf_pdl_enter();
         constexpr int NP = NP1 * NP1;
-        constexpr int E = strip_elems(NP1, VISC);
+        constexpr int E = strip_elems(NP1, true);
         // U' (value, tangent) of the strip's elements [1], of the elements below [0] and
         // above [2] them, and of the strip's west [0] and east [1] neighbours: every
         // trace the faces need comes from shared memory, loaded coalesced up front
@@ -605,8 +605,8 @@ struct k_dgtl_b {
         __shared__ float sg[2][E][4][NP];              // volume fluxes (tangent part)
         __shared__ float sPx[E + 1][4][NP1];           // x-face terms Phi (face f west of strip element f)
         __shared__ float sPz[2][E][4][NP1];            // z-face terms: [0] bottom, [1] top of element le
-        __shared__ float sSx[VISC ? E + 1 : 1][6][NP1];   // viscous symmetry terms (L side 0..2, R side 3..5)
-        __shared__ float sSz[VISC ? 2 : 1][VISC ? E : 1][6][NP1];
+        __shared__ float sSx[E + 1][6][NP1];   // viscous symmetry terms (L side 0..2, R side 3..5)
+        __shared__ float sSz[2][E][6][NP1];
         __shared__ float sDx[NP1][NP1], sDz[NP1][NP1], sDn[NP1][NP1], sl[8][NP1];
         __shared__ float sdf[FIRST ? E : 1][4][NP];    // the defect, for the transfer (FIRST)
         __shared__ float smf[FIRST ? E : 1][4][2][NP1];   // row sums of the mass fix
@@ -670,26 +670,24 @@ struct k_dgtl_b {
             const TL32 u = U[1] * ir, w = U[2] * ir;
             TL32 Fx[4], Fz[4];
             flux_xz(U, u, w, p, Fx, Fz);
-            if (VISC) {
-                TL32 dx[4], dz[4];
+            TL32 dx[4], dz[4];
     #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    TL32 sx = mk(0.0, TL32{}), sz = mk(0.0, TL32{});
+            for (int v = 0; v < 4; ++v) {
+                TL32 sx = mk(0.0, TL32{}), sz = mk(0.0, TL32{});
     #pragma unroll
-                    for (int q = 0; q < NP1; ++q) {
-                        sx = jfma(TLc{sDn[a][q]}, sn[1][le][v * NP + b * NP1 + q], sx);
-                        sz = jfma(TLc{sDn[b][q]}, sn[1][le][v * NP + q * NP1 + a], sz);
-                    }
-                    dx[v] = TLc{K.two_hxf} * sx;
-                    dz[v] = TLc{K.two_hzf} * sz + TLc{K.dubvf[v * nrow + J]};
+                for (int q = 0; q < NP1; ++q) {
+                    sx = jfma(TLc{sDn[a][q]}, sn[1][le][v * NP + b * NP1 + q], sx);
+                    sz = jfma(TLc{sDn[b][q]}, sn[1][le][v * NP + q * NP1 + a], sz);
                 }
-                const TLc mu = TLc{K.pc.muf};
-                const TL32 phi[4] = {u, u, w, U[3] * ir};
+                dx[v] = TLc{K.two_hxf} * sx;
+                dz[v] = TLc{K.two_hzf} * sz + TLc{K.dubvf[v * nrow + J]};
+            }
+            const TLc mu = TLc{K.pc.muf};
+            const TL32 phi[4] = {u, u, w, U[3] * ir};
     #pragma unroll
-                for (int v = 1; v < 4; ++v) {
-                    Fx[v] = Fx[v] - mu * visc_c(phi[v], dx[0], dx[v]);
-                    Fz[v] = Fz[v] - mu * visc_c(phi[v], dz[0], dz[v]);
-                }
+            for (int v = 1; v < 4; ++v) {
+                Fx[v] = Fx[v] - mu * visc_c(phi[v], dx[0], dx[v]);
+                Fz[v] = Fz[v] - mu * visc_c(phi[v], dz[0], dz[v]);
             }
     #pragma unroll
             for (int v = 0; v < 4; ++v) {
@@ -708,7 +706,7 @@ struct k_dgtl_b {
             for (int q = 0; q < NP1; ++q) {
                 const TL32 u = src[v * NP + i0 + q * st];
                 tv = jfma(TLc{pa[q]}, u, tv);
-                if (VISC) td = jfma(TLc{pd[q]}, u, td);
+                td = jfma(TLc{pd[q]}, u, td);
             }
         };
         const int nxf = (Ev + 1) * NP1, nzf = 2 * Ev * NP1;
@@ -741,7 +739,7 @@ struct k_dgtl_b {
                 hllc_s<TL32, 0>(SL, SR, H);
     #pragma unroll
                 for (int v = 0; v < 4; ++v) Phi[v] = H[v];
-                if (VISC && !wallL && !wallR) {
+                if (!wallL && !wallR) {
                     const TLc hmu = TLc{0.5f * K.pc.muf};
                     const TL32 J0 = trL[0] - trR[0];
     #pragma unroll
@@ -759,12 +757,10 @@ struct k_dgtl_b {
                 }
     #pragma unroll
                 for (int v = 0; v < 4; ++v) sPx[f][v][sp] = Phi[v].d;
-                if (VISC) {
     #pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        sSx[f][q][sp] = sLv[q].d;
-                        sSx[f][3 + q][sp] = sRv[q].d;
-                    }
+                for (int q = 0; q < 3; ++q) {
+                    sSx[f][q][sp] = sLv[q].d;
+                    sSx[f][3 + q][sp] = sRv[q].d;
                 }
             } else {
                 const int u = t - nxf;
@@ -799,7 +795,7 @@ struct k_dgtl_b {
                 hllc_s<TL32, 1>(SL, SR, H);
     #pragma unroll
                 for (int v = 0; v < 4; ++v) Phi[v] = H[v];
-                if (VISC && !wallB && !wallT) {
+                if (!wallB && !wallT) {
                     const TLc hmu = TLc{0.5f * K.pc.muf};
                     const TL32 J0 = trL[0] - trR[0];
     #pragma unroll
@@ -817,12 +813,10 @@ struct k_dgtl_b {
                 }
     #pragma unroll
                 for (int v = 0; v < 4; ++v) sPz[top][l][v][sp] = Phi[v].d;
-                if (VISC) {
     #pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        sSz[top][l][q][sp] = sLv[q].d;
-                        sSz[top][l][3 + q][sp] = sRv[q].d;
-                    }
+                for (int q = 0; q < 3; ++q) {
+                    sSz[top][l][q][sp] = sLv[q].d;
+                    sSz[top][l][3 + q][sp] = sRv[q].d;
                 }
             }
         }
@@ -845,7 +839,7 @@ struct k_dgtl_b {
             f = fmaf(-lpxa, sPx[le + 1][v][b], f);
             f = fmaf(lmzb, sPz[0][le][v][a], f);
             f = fmaf(-lpzb, sPz[1][le][v][a], f);
-            if (VISC && v > 0) {
+            if (v > 0) {
                 const int q = v - 1;
                 f = fmaf(dlmxa, sSx[le][3 + q][b], f);
                 f = fmaf(dlpxa, sSx[le + 1][q][b], f);
@@ -878,9 +872,9 @@ struct k_dgtl_b {
         if (FIRST && TR.b) dgtl_transfer<NP1, E>(TR, sdf, smf, sg[0], le, node, ez, ex0 + le, active);
     }
 };
-template <int NP1, bool VISC, int MODE, int FIRST>
-__global__ void __launch_bounds__(128, VISC ? 5 : 8) k_dgtl(DGK K, DGArgs A, float *out1f, TransferOut TR) {
-    k_dgtl_b<NP1, VISC, MODE, FIRST>::run(blockIdx.x, gridDim.x, K, A, out1f, TR);
+template <int NP1, int MODE, int FIRST>
+__global__ void __launch_bounds__(128, 5) k_dgtl(DGK K, DGArgs A, float *out1f, TransferOut TR) {
+    k_dgtl_b<NP1, MODE, FIRST>::run(blockIdx.x, gridDim.x, K, A, out1f, TR);
 }
 
 // ---------------------------------------------------------------------------
@@ -1344,10 +1338,10 @@ int launch_tl(jfnk_ctx *c, const DGK &K, const DGArgs &a, cudaStream_t s) {
     if constexpr (VISC) {
         const int threads = E * NP1 * NP1;
         if (MODE == DG_TLJV && a.out1f)
-            jf_launch<k_dgtl_b<NP1, VISC, MODE, 1>>(k_dgtl<NP1, VISC, MODE, 1>, nb, threads, 0, s, K, a, a.out1f,
+            jf_launch<k_dgtl_b<NP1, MODE, 1>>(k_dgtl<NP1, MODE, 1>, nb, threads, 0, s, K, a, a.out1f,
                       a.tro ? *a.tro : TransferOut{});
         else
-            jf_launch<k_dgtl_b<NP1, VISC, MODE, 0>>(k_dgtl<NP1, VISC, MODE, 0>, nb, threads, 0, s, K, a, (float *)nullptr, TransferOut{});
+            jf_launch<k_dgtl_b<NP1, MODE, 0>>(k_dgtl<NP1, MODE, 0>, nb, threads, 0, s, K, a, (float *)nullptr, TransferOut{});
     } else {
         const float4 *J = (const float4 *)c->jac, *Jn = (const float4 *)c->jacn;
         if (MODE == DG_TLJV && a.out1f)

@@ -434,15 +434,13 @@ int dg_residual_grouped(jfnk_ctx *const *ctx, int n, const double *const *U, dou
 
 // reductions / BLAS-1 (blas.cu)
 int red_dot(jfnk_ctx *c, const double *x, const double *y, size_t n, double *out_dev, int op, cudaStream_t s);
-int red_dotf(jfnk_ctx *c, const float *x, const float *y, size_t n, double *out_dev, int op, cudaStream_t s);
 // RED_EPSP: eps of the preconditioner's FD products, numerator opts.precond_fd_eps
 // (sqrt(eps_mach) when 0)
-enum { RED_SUM = 0, RED_SQRT = 1, RED_EPS = 2, RED_EPS32 = 3, RED_EPSP = 4 };
+enum { RED_SUM = 0, RED_SQRT = 1, RED_EPS = 2, RED_EPSP = 3 };
 int blas_mdot(jfnk_ctx *c, const double *V, int nv, size_t ldv, const double *w, size_t n, double *h_dev, cudaStream_t s,
               const double *flag = nullptr);
 int blas_mupdate(jfnk_ctx *c, const double *V, int nv, size_t ldv, const double *h_dev, double *w, size_t n, double sign,
                  cudaStream_t s, const double *flag = nullptr);
-int blas_reortho_flag(const double *w1sq, const double *h, int nv, double *flag, cudaStream_t s);
 int blas_mupdate_norm(jfnk_ctx *c, const double *V, int nv, size_t ldv, const double *h, double *w, size_t n,
                       double sign, const double *flag_in, double *w1sq, double *nrm, double *flag_out,
                       cudaStream_t s);

@@ -1569,10 +1569,10 @@ inline int fv_smooth_or_defect(jfnk_ctx *c, int l, int mode, const void *x, cons
     return fv_op32(c, l, mode, (const float *)x, (const float *)b, (float *)out, s, rk);
 }
 
-// defect g'x - b on level l restricted to level l+1 (b_{l+1}, and x_{l+1} = dtau b
+// FP32 defect g'x - b on level l restricted to level l+1 (b_{l+1}, and x_{l+1} = dtau b
 // when xc is given)
-int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *bc, void *xc, const void *dtc,
-                       cudaStream_t s) {
+int fv_defect_restrict32(jfnk_ctx *c, int l, const float *x, const float *b, float *bc, float *xc, const float *dtc,
+                         cudaStream_t s) {
     FVLev &L = c->lev[l];
     FVLev &C = c->lev[l + 1];
     FVK K = make_fvk(c, l);
@@ -1582,83 +1582,39 @@ int fv_defect_restrict(jfnk_ctx *c, int l, const void *x, const void *b, void *b
     const int tb = c->opts.tile_fv;
     const bool l4 = L.st || fv_four_lanes(c, n1);
     const bool f2 = L.fac == 2;
-    const unsigned g = nblk((f2 ? 16 : 4) * nc, tb);   // lanes per coarse cell
-    c->fv_calls++;
+    const int bf = (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0;   // BF16 coarsest level
+    const FLoad<TL32, 2> ld{(const float *)L.u, x, n1};
     if (!l4 && !f2) {
         // large levels agglomerated by 3 or 5 (odd k + 1): separate defect and restriction
         // (the fused kernel would run fac^2 cells one after another per coarse cell)
-        c->fv_calls--;   // counted by the defect
-        JF_RET(fv_smooth_or_defect(c, l, FV_DEFECT, x, b, L.r, s));
-        if (c->prec == 64)
-            jf_launch<k_restrict_b_b<double>>(k_restrict_b<double>, nblk(C.n, 256), 256, 0, s, (const double *)L.r, L.NX, L.NZ, L.fac,
-                      (double *)bc, (double *)xc, (const double *)dtc, 0);
-        else
-            jf_launch<k_restrict_b_b<float>>(k_restrict_b<float>, nblk(C.n, 256), 256, 0, s, (const float *)L.r, L.NX, L.NZ, L.fac,
-                      (float *)bc, (float *)xc, (const float *)dtc, (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0);
-        jf_launched();
-        JF_CK(cudaGetLastError());
-        return JFNK_OK;
-    }
-#define JF_DR(T, IN, V, F2, ST, ...) jf_launch<k_fv_defect_restrict_b<T, IN, V, F2, ST>>(k_fv_defect_restrict<T, IN, V, F2, ST>, g, tb, 0, s, __VA_ARGS__)
-#define JF_DR2(T, IN, V, ST, ...)                            \
-    do {                                                     \
-        if (f2) JF_DR(T, IN, V, true, ST, __VA_ARGS__);      \
-        else JF_DR(T, IN, V, false, ST, __VA_ARGS__);        \
-    } while (0)
-    // large levels with 2 x 2 agglomeration: the face-once tile kernel
-    const int tz = tb >= 256 ? 8 : 4;   // tile rows follow the block size
-    const unsigned gt = (unsigned)(((L.NX + FV_TX - 1) / FV_TX) * ((L.NZ + tz - 1) / tz));
-#define JF_DRT(T, IN, V, ld, bb, fuu, outc, xcc, dtc_, bff)                                                     \
-    do {                                                                                                        \
-        if (tz == 8)                                                                                            \
-            jf_launch<k_fv_tile_b<T, IN, FV_DEFRES, V, 8>>(k_fv_tile<T, IN, FV_DEFRES, V, 8>, gt, FV_TX * 8, 0, s, K, ld, bb, nullptr, fuu, c->mg_adt, \
-                      outc, xcc, dtc_, bff, RKS{nullptr, 0, 1.0, 1.0f});                                                                    \
-        else                                                                                                    \
-            jf_launch<k_fv_tile_b<T, IN, FV_DEFRES, V, 4>>(k_fv_tile<T, IN, FV_DEFRES, V, 4>, gt, FV_TX * 4, 0, s, K, ld, bb, nullptr, fuu, c->mg_adt, \
-                      outc, xcc, dtc_, bff, RKS{nullptr, 0, 1.0, 1.0f});                                                                    \
-    } while (0)
-    if (!l4 && f2) {
-        if (c->prec == 64) {
-            double *epsp = c->scal + S_EPSFV + l;
-            JF_RET(red_dot(c, (const double *)x, (const double *)x, L.n, epsp, RED_EPSP, s));
-            FLoad<D64, 1> ld{(const double *)L.u, (const double *)x, epsp, n1, 0.0};
-            if (visc) JF_DRT(D64, 1, true, ld, (const double *)b, (const double *)L.fu, (double *)bc, (double *)xc, (const double *)dtc, 0);
-            else JF_DRT(D64, 1, false, ld, (const double *)b, (const double *)L.fu, (double *)bc, (double *)xc, (const double *)dtc, 0);
-        } else {
-            FLoad<TL32, 2> ld{(const float *)L.u, (const float *)x, n1};
-            const int bf = (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0;
-            if (visc) JF_DRT(TL32, 2, true, ld, (const float *)b, nullptr, (float *)bc, (float *)xc, (const float *)dtc, bf);
-            else JF_DRT(TL32, 2, false, ld, (const float *)b, nullptr, (float *)bc, (float *)xc, (const float *)dtc, bf);
-        }
-        jf_launched();
-        JF_CK(cudaGetLastError());
-        return JFNK_OK;
-    }
+        JF_RET(fv_op32(c, l, FV_DEFECT, x, b, (float *)L.r, s));
+        jf_launch<k_restrict_b_b<float>>(k_restrict_b<float>, nblk(C.n, 256), 256, 0, s, (const float *)L.r, L.NX, L.NZ, L.fac, bc,
+                  xc, dtc, bf);
+    } else if (!l4) {
+        // large levels with 2 x 2 agglomeration: the face-once tile kernel
+        c->fv_calls++;
+        const int tz = tb >= 256 ? 8 : 4;   // tile rows follow the block size
+        const unsigned gt = (unsigned)(((L.NX + FV_TX - 1) / FV_TX) * ((L.NZ + tz - 1) / tz));
+        auto tile = [&](auto body, auto kernel) {
+            jf_launch<decltype(body)>(kernel, gt, FV_TX * tz, 0, s, K, ld, b, nullptr, nullptr, c->mg_adt, bc, xc, dtc, bf,
+                      RKS{nullptr, 0, 1.0, 1.0f});
+        };
+#define JF_DRT(V, TZ) tile(k_fv_tile_b<TL32, 2, FV_DEFRES, V, TZ>{}, k_fv_tile<TL32, 2, FV_DEFRES, V, TZ>)
+        if (visc) tz == 8 ? JF_DRT(true, 8) : JF_DRT(true, 4);
+        else tz == 8 ? JF_DRT(false, 8) : JF_DRT(false, 4);
 #undef JF_DRT
-#define JF_DR4(T, IN, ...)                                   \
-    do {                                                     \
-        if (visc) JF_DR2(T, IN, true, false, __VA_ARGS__);   \
-        else JF_DR2(T, IN, false, false, __VA_ARGS__);       \
-    } while (0)
-    if (c->prec == 64) {
-        double *epsp = c->scal + S_EPSFV + l;
-        JF_RET(red_dot(c, (const double *)x, (const double *)x, L.n, epsp, RED_EPSP, s));
-        FLoad<D64, 1> ld{(const double *)L.u, (const double *)x, epsp, n1, 0.0};
-        JF_DR4(D64, 1, K, ld, (const double *)b, (const double *)L.fu, c->mg_adt, L.fac, (double *)bc, (double *)xc,
-               (const double *)dtc, 0);
     } else {
-        FLoad<TL32, 2> ld{(const float *)L.u, (const float *)x, n1};
-        const int bf = (c->prec == 16 && l + 1 == c->nlev - 1) ? 1 : 0;   // BF16 coarsest level
-        if (K.st)
-            JF_DR2(TL32, 2, false, true, K, ld, (const float *)b, nullptr, c->mg_adt, L.fac, (float *)bc, (float *)xc,
-                   (const float *)dtc, bf);
-        else
-            JF_DR4(TL32, 2, K, ld, (const float *)b, nullptr, c->mg_adt, L.fac, (float *)bc, (float *)xc,
-                   (const float *)dtc, bf);
-    }
-#undef JF_DR4
-#undef JF_DR2
+        c->fv_calls++;
+        const unsigned g = nblk((f2 ? 16 : 4) * nc, tb);   // lanes per coarse cell
+        auto lanes = [&](auto body, auto kernel) {
+            jf_launch<decltype(body)>(kernel, g, tb, 0, s, K, ld, b, nullptr, c->mg_adt, L.fac, bc, xc, dtc, bf);
+        };
+#define JF_DR(V, F2, ST) lanes(k_fv_defect_restrict_b<TL32, 2, V, F2, ST>{}, k_fv_defect_restrict<TL32, 2, V, F2, ST>)
+        if (K.st) f2 ? JF_DR(false, true, true) : JF_DR(false, false, true);
+        else if (visc) f2 ? JF_DR(true, true, false) : JF_DR(true, false, false);
+        else f2 ? JF_DR(false, true, false) : JF_DR(false, false, false);
 #undef JF_DR
+    }
     jf_launched();
     JF_CK(cudaGetLastError());
     return JFNK_OK;
@@ -1737,7 +1693,7 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, bool have_eps, cu
         FVLev &C = c->lev[l + 1];
         const bool fuse = c->mid_pre >= 1 && !rk_multi(c);
         bool eps_c = false;
-        if (zero || c->prec == 64) {   // separate defect and restriction
+        if (zero || D) {   // separate defect and restriction
             if (zero) {
                 jf_launch<k_neg_b<S>>(k_neg<S>, nblk(L.n, 256), 256, 0, s, (S *)L.r, (const S *)L.b, L.n);
                 jf_launched();
@@ -1756,7 +1712,8 @@ int mg_cycle_t(jfnk_ctx *c, int l, bool zero, bool first_done, bool have_eps, cu
             }
         } else {
             // defect and restriction (and the coarse first step) in one pass
-            JF_RET(fv_defect_restrict(c, l, L.x, L.b, C.b, fuse ? C.x : nullptr, C.dtau, s));
+            JF_RET(fv_defect_restrict32(c, l, (const float *)L.x, (const float *)L.b, (float *)C.b,
+                                        fuse ? (float *)C.x : nullptr, (const float *)C.dtau, s));
         }
         bool vz = true, fd = fuse;
         for (int cyc = 0; cyc < c->cycles; ++cyc) {
@@ -2203,7 +2160,8 @@ int mg_time_fv_level0(jfnk_ctx *c, const double *U, const double *y, int reps, d
         cudaEventRecord(e[0], s);
         rc = fv_op32(c, 0, FV_SMOOTH, (const float *)L.x, (const float *)L.b, (float *)L.x2, s);
         cudaEventRecord(e[1], s);
-        if (rc == JFNK_OK) rc = fv_defect_restrict(c, 0, L.x, L.b, C.b, C.x, C.dtau, s);
+        if (rc == JFNK_OK)
+            rc = fv_defect_restrict32(c, 0, (const float *)L.x, (const float *)L.b, (float *)C.b, (float *)C.x, (const float *)C.dtau, s);
         cudaEventRecord(e[2], s);
         if (cudaEventSynchronize(e[2]) != cudaSuccess) rc = JFNK_ECUDA;
         float m0 = 0.f, m1 = 0.f;
