@@ -424,7 +424,8 @@ __global__ void __launch_bounds__(RB) k_gs_dot32(const float *V32, size_t ldv, c
 // The three passes for 17 to 32 basis vectors (nv at run time): the sums stay in
 // registers, the vectors are read in groups of four, in pass 2 once for the update and
 // again (from L1 / L2) for the sums.  The general multi-dot path took eight launches and
-// some 110 us of latency for such a column on a grid of 7,200 unknowns, these three 40.
+// some 110 us of latency for such a column on a grid of 7,200 unknowns, these three 40
+// (with pass 1 in FP32; in FP64 a step of that grid takes the same 12.0 ms).
 constexpr int LV = 32;
 template <class F>
 __device__ __forceinline__ void vec_groups(int nv, F f) {
@@ -1004,8 +1005,7 @@ int blas_cgs2(jfnk_ctx *c, const double *V, const float *V32, int nv, size_t ldv
 }
 
 // Diagnostic timing of the three CGS2 launches with 8 basis vectors on the
-// context's basis buffers (filled with a fixed byte pattern, so the second pass
-// is always taken, as on the solver's problems).  ms[0]: pass 1 (FP32 multi-dot),
+// context's basis buffers (filled with a fixed byte pattern).  ms[0]: pass 1 (FP32 multi-dot),
 // ms[1]: passes 2 and 3 (update + dot, update + normalisation); means over reps.
 int blas_time_cgs2(jfnk_ctx *c, int reps, double *ms, cudaStream_t s) {
     constexpr int NV = 8;

@@ -5,10 +5,11 @@
 // f is linear in its numerical and node fluxes, f = L(F), so f(U + eps y) - f(U) =
 // L(F(U + eps y) - F(U)).  The residual at U keeps what does not depend on y: the states
 // and (viscous) gradients at the face points and nodes, and the fluxes there.  A product
-// then evaluates the fluxes at U + eps y in FP64, subtracts the stored ones (exact: the
-// two are within a factor of two of each other), and applies L, the traces and the
-// gradients of y in two-float arithmetic (an unevaluated sum of two floats, about 46
-// bits; products by FMA, sums by Knuth's TwoSum) on the FP32 pipe.
+// then evaluates the fluxes at U + eps y in FP64, subtracts the stored ones (one rounding;
+// none where the two are within a factor of two of each other, as they are except near
+// zero), and applies L, the traces and the gradients of y in two-float arithmetic (an
+// unevaluated sum of two floats, about 46 bits; products by FMA, sums by Knuth's TwoSum)
+// on the FP32 pipe.
 // What bounds it: FP64 instructions, as in the general form (19 clocks of an SM each per
 // warp, where an FP32 one takes 0.25).  Per Q3 face point 63 of them against 103, per
 // node 25 against 85.  Accuracy: the differences are formed before anything is summed, so
@@ -16,10 +17,12 @@
 // about 1/eps larger; 46 bits are far below the noise of the fluxes themselves.  The
 // form holds for eps = sqrt(eps_mach)/|y| (the differences keep 2^-26 of U at most); a
 // caller's own, larger eps takes the general form.
-// Measured on GB300 (events around the launches): Q3 160 x 80 elements 31.8 + 11.6 us,
-// the general form 33.0 + 40.7 (and 48.8 + 47.4 before the primitives of numeric.cuh);
-// viscous Q2 256 x 32 31.3 + 8.7 against 49.0 + 30.9, Q4 320 x 160 150 + 37 against
-// 191 + 267.  The 103,360 face points and 204,800 nodes take 21.5 us of FP64 issue.
+// Measured on GB300 (events around the launches; FP32 directions): Q3 160 x 80 elements
+// 32.3 + 11.9 us, the general form as a face and a volume launch 33.0 + 40.7 (and
+// 48.8 + 47.4 before the primitives of numeric.cuh); viscous Q2 256 x 32 31.6 + 9.1 against
+// 49.0 + 30.9, Q4 320 x 160 151 + 37 against 191 + 267.  FP64 directions are scaled and
+// split: 35.7, 34.8 and 178 us for the flux launch.  The 103,360 face points and 204,800
+// nodes take 21.5 us of FP64 issue.
 
 // Direction entries as two floats.  FP32 vectors are exact in the first part.  FP64 ones
 // are scaled by the power of two that brings |y| (from eps = sqrt(eps_mach)/|y|) to about

@@ -86,10 +86,10 @@ JF_D bool faster(TL32 uL, TL32 cL, TL32 uR, TL32 cR, TL32) { return le(uR + cR, 
 // S* - u_L = ((p_R - p_L) - d q_R) / (q_L - q_R).  In this form nothing large cancels
 // (F_K and S_K (U*_K - U_K) do in the textbook one), and the whole flux takes about 51
 // FP64 instructions instead of 119.
-// With the quotients, roots and powers of numeric.cuh the FP64 residual's face kernel
-// fell from 48.6 to 28.0 us on 103,360 Q3 face points, from 46.9 to 26.0 us on the
-// 50,016 viscous Q2 ones, and from 26 to 15 us where one SM's latency chain sets the
-// time (20 x 10 elements, Q2).
+// With the quotients, roots and powers of numeric.cuh the faces of the FP64 residual, then
+// a launch of their own, fell from 48.6 to 28.0 us on 103,360 Q3 face points, from 46.9 to
+// 26.0 us on the 50,016 viscous Q2 ones, and from 26 to 15 us where one SM's latency chain
+// sets the time (20 x 10 elements, Q2).  (Faces and nodes in one launch: k_dg_flux.)
 template <class T, int D>
 JF_D void hllc_s(const Side<T> &L, const Side<T> &R, T H[4]) {
     constexpr int iN = 1 + D, iT = 2 - D;

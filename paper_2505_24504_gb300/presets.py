@@ -6,7 +6,8 @@ implicit steps per candidate (`autotune.tuned_schedule_context` searches the
 same candidates: keys, then sigma_fv, then sigma_dg) and the kernels per launch
 shape (`jfnk_autotune`).  They are recorded here so that the benchmark, the parity tests
 at full size and the CPU reference all run the same configuration;
-`bench.py --tune` runs the autotuner again and reports what it picks.  None of
+`bench.py --tune` runs the autotuner again and reports what it picks.  (The launch
+shapes were picked with earlier kernels; tile_faces has no effect on the present ones.)  None of
 these choices changes the converged answer (the Newton tolerance decides it);
 they change iteration counts and speed only.
 """
