@@ -176,7 +176,8 @@ void jfnk_destroy(jfnk_ctx *ctx);
 size_t jfnk_num_unknowns(const jfnk_ctx *ctx);
 
 /* Device bytes jfnk_create would allocate for these arguments (HBM
- * admission); 0 on invalid arguments. */
+ * admission), the larger of the inviscid and the viscous context; 0 on invalid
+ * arguments. */
 size_t jfnk_workspace_bytes(const jfnk_grid *grid, int k, const jfnk_opts *opts);
 
 /* Node coordinates in the DG layout without the variable index:
